@@ -1,13 +1,15 @@
 // Rigid-body and surface-site kernels (Sec. II.B and II.B.2 of arXiv 2604.14307).
 //
-// k_body_md     first velocity-Verlet half kick, drift of R, and the Miller et
-//               al. NO_SQUISH free-rotor sequence 3-2-1-2-3 for q and its
-//               conjugate momentum p = 2 q (x) (0, L_body), formed from the
-//               stored space-frame L and converted back; one thread per body.
-// k_body_centres the space-frame offsets Q c of every WCA centre, once per pose.
+// k_body_md     (the transfer's sum,) first velocity-Verlet half kick, drift of R,
+//               and the Miller et al. NO_SQUISH free-rotor sequence 3-2-1-2-3 for
+//               q and its conjugate momentum p = 2 q (x) (0, L_body), formed from
+//               the stored space-frame L and converted back; four lanes per body.
+//               Finishes the force pass where no two bodies share a box.
+// k_body_centres the space-frame offsets Q c of every WCA centre, once per pose
+//               (k_body_md writes them for shapes of one or two centres).
 // k_body_force  core-shifted WCA (Eq. 1) between the centres of different
 //               bodies of a replica, with torques, over Verlet neighbour lists
-//               (FP32 bounding-sphere prefilter); one thread per body for
+//               (FP32 bounding-sphere prefilter); eight lanes per body for
 //               shapes of one or two centres, one warp per body otherwise;
 //               the pair arithmetic in the form's precision (FP32 for P32),
 //               forces and torques summed in FP64; optional second kick.
@@ -42,14 +44,6 @@ __device__ __forceinline__ bool site_owned(const StepArgs &a, Real z)
 
 
 // ------------------------------------------------------------- quaternions
-__device__ __forceinline__ void quat_mul(const double a[4], const double b[4], double o[4])
-{
-    o[0] = a[0] * b[0] - a[1] * b[1] - a[2] * b[2] - a[3] * b[3];
-    o[1] = a[0] * b[1] + a[1] * b[0] + a[2] * b[3] - a[3] * b[2];
-    o[2] = a[0] * b[2] - a[1] * b[3] + a[2] * b[0] + a[3] * b[1];
-    o[3] = a[0] * b[3] + a[1] * b[2] - a[2] * b[1] + a[3] * b[0];
-}
-
 // rotation matrix of a unit quaternion (w, x, y, z), body -> space
 __device__ __forceinline__ void rotmat(const double q[4], double Q[9])
 {
@@ -69,71 +63,6 @@ __device__ __forceinline__ void mtv(const double Q[9], const double x[3], double
     for (int a = 0; a < 3; ++a) o[a] = (Q[a] * x[0] + Q[3 + a] * x[1]) + Q[6 + a] * x[2];
 }
 
-// body-frame angular momentum from p: L_body = vec(q* (x) p) / 2
-__device__ __forceinline__ void body_L(const double q[4], const double p[4], double Lb[3])
-{
-    double qc[4] = {q[0], -q[1], -q[2], -q[3]}, t[4];
-    quat_mul(qc, p, t);
-    Lb[0] = 0.5 * t[1]; Lb[1] = 0.5 * t[2]; Lb[2] = 0.5 * t[3];
-}
-__device__ __forceinline__ void p_from_Lb(const double q[4], const double Lb[3], double p[4])
-{
-    double v[4] = {0.0, Lb[0], Lb[1], Lb[2]}, t[4];
-    quat_mul(q, v, t);
-    for (int a = 0; a < 4; ++a) p[a] = 2.0 * t[a];
-}
-
-__device__ __forceinline__ void L_to_p(const double q[4], const double Lm[3], double p[4])
-{
-    double Q[9], Lb[3];
-    rotmat(q, Q);
-    mtv(Q, Lm, Lb);
-    p_from_Lb(q, Lb, p);
-}
-__device__ __forceinline__ void p_to_L(const double q[4], const double p[4], double Lm[3])
-{
-    double Q[9], Lb[3];
-    body_L(q, p, Lb);
-    rotmat(q, Q);
-    mv(Q, Lb, Lm);
-}
-
-// p += 2 h q (x) (0, Q^T tau): torque kick over a half step h
-__device__ __forceinline__ void torque_kick(const double q[4], double p[4], const double T[3], double h)
-{
-    double Q[9], tb[3];
-    rotmat(q, Q);
-    mtv(Q, T, tb);
-    double v[4] = {0.0, tb[0], tb[1], tb[2]}, t[4];
-    quat_mul(q, v, t);
-    for (int a = 0; a < 4; ++a) p[a] += 2.0 * h * t[a];
-}
-
-// free rotation about body axis k (1..3) for time h (Miller et al. 2002)
-__device__ __forceinline__ void rotor(double q[4], double p[4], int k, double h, const double Ih[3])
-{
-    if (Ih[k - 1] == 0.0) return;
-    double Pq[4], Pp[4];
-    if (k == 1) {
-        Pq[0] = -q[1]; Pq[1] = q[0]; Pq[2] = q[3]; Pq[3] = -q[2];
-        Pp[0] = -p[1]; Pp[1] = p[0]; Pp[2] = p[3]; Pp[3] = -p[2];
-    } else if (k == 2) {
-        Pq[0] = -q[2]; Pq[1] = -q[3]; Pq[2] = q[0]; Pq[3] = q[1];
-        Pp[0] = -p[2]; Pp[1] = -p[3]; Pp[2] = p[0]; Pp[3] = p[1];
-    } else {
-        Pq[0] = -q[3]; Pq[1] = q[2]; Pq[2] = -q[1]; Pq[3] = q[0];
-        Pp[0] = -p[3]; Pp[1] = p[2]; Pp[2] = -p[1]; Pp[3] = p[0];
-    }
-    double zeta = (p[0] * Pq[0] + p[1] * Pq[1] + p[2] * Pq[2] + p[3] * Pq[3]) / (4.0 * Ih[k - 1]);
-    double c = cos(zeta * h), s = sin(zeta * h);
-    for (int a = 0; a < 4; ++a) {
-        double nq = c * q[a] + s * Pq[a];
-        double np = c * p[a] + s * Pp[a];
-        q[a] = nq;
-        p[a] = np;
-    }
-}
-
 __device__ __forceinline__ double wrapd(double y, double L, int &bad)
 {
     if (y >= L) y = y - L;
@@ -149,49 +78,205 @@ __device__ __forceinline__ float wrapf(float y, float L, int &bad)
     return y;
 }
 
-// --------------------------------------------------------------- body MD
-__global__ void k_body_md(StepArgs a)
+// ------------------------------------------------- bodies, lane parallel
+// A warp-wide FP64 instruction takes 64 cycles of its SM sub-partition however
+// many lanes it has (measured: 64.2 cycles with 1 to 32 active lanes, four
+// warps on four sub-partitions at once), so the rigid-body arithmetic is
+// bound by the number of FP64 instructions a warp executes one after another,
+// not by its operations.  A body is therefore spread over four lanes: lane c
+// holds component c of its quaternion and conjugate momentum and component c of
+// its vectors (lane 3 repeats lane 0's vector work), each component is formed
+// by the expression of the scalar form, in the same order, and components of
+// the other lanes come by shuffles.  The body step of one body went from 27 to
+// 12 us with the transfer's sum and the centres in the same launch (36 us in three).
+__device__ __forceinline__ double lane4(double v, int c) { return __shfl_sync(0xffffffffu, v, c, 4); }
+__device__ __forceinline__ float lane4(float v, int c) { return __shfl_sync(0xffffffffu, v, c, 4); }
+__device__ __forceinline__ double flip(double v, bool neg)   // -v if neg, exactly
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n_bodies) return;
-    DevBody b = a.bodies[i];
-    const DevShape sh = a.shapes[b.shape];
-    const DevReplica r = a.reps[b.rep];
+    return __hiloint2double(__double2hiint(v) ^ (neg ? 0x80000000 : 0), __double2loint(v));
+}
+
+// a / b with rb = RN(1 / b): Markstein's correction (IBM J. Res. Dev. 34, 111
+// (1990)) applied twice.  The first makes the quotient faithful, the second
+// rounds it correctly, so the result is that of the IEEE division (no overflow
+// or underflow in between), in 5 instructions of 64 cycles instead of about 11.
+__device__ __forceinline__ double div_by(double a, double b, double rb)
+{
+    double q = a * rb;
+    q = fma(fma(-b, q, a), rb, q);
+    return fma(fma(-b, q, a), rb, q);
+}
+
+// component c of the quaternion product (quat_mul); a, b: lane c's component
+__device__ __forceinline__ double lane_qmul(double a, double b, int c)
+{
+    const double t0 = lane4(a, 0) * lane4(b, c), t1 = lane4(a, 1) * lane4(b, c ^ 1);
+    const double t2 = lane4(a, 2) * lane4(b, c ^ 2), t3 = lane4(a, 3) * lane4(b, c ^ 3);
+    return ((t0 + flip(t1, c == 0 || c == 2)) + flip(t2, c == 0 || c == 3)) + flip(t3, c < 2);
+}
+// (0, v) as a quaternion from vector component lanes, and back (lane 3: component 0)
+__device__ __forceinline__ double lane_vec_to_quat(double v, int c)
+{
+    const double t = lane4(v, (c + 3) & 3);
+    return c == 0 ? 0.0 : t;
+}
+__device__ __forceinline__ double lane_quat_to_vec(double t, int c) { return lane4(t, c == 3 ? 1 : c + 1); }
+
+// row and column c of the rotation matrix (rotmat) of the quaternion q
+struct LaneRot { double r[3], c[3]; };
+__device__ __forceinline__ LaneRot lane_rot(double q, int c)
+{
+    const int i = c == 3 ? 0 : c, j = i == 2 ? 0 : i + 1, l = i == 0 ? 2 : i - 1;
+    const double w = lane4(q, 0), qi = lane4(q, 1 + i), qj = lane4(q, 1 + j), ql = lane4(q, 1 + l);
+    const double dii = 1.0 - 2.0 * (qj * qj + ql * ql);
+    const double ij = qi * qj, il = qi * ql, wl = w * ql, wj = w * qj;
+    const double rij = 2.0 * (ij - wl), ril = 2.0 * (il + wj), cji = 2.0 * (ij + wl), cli = 2.0 * (il - wj);
+    LaneRot o;
+    o.r[0] = i == 0 ? dii : (i == 1 ? ril : rij); o.c[0] = i == 0 ? dii : (i == 1 ? cli : cji);
+    o.r[1] = i == 0 ? rij : (i == 1 ? dii : ril); o.c[1] = i == 0 ? cji : (i == 1 ? dii : cli);
+    o.r[2] = i == 0 ? ril : (i == 1 ? rij : dii); o.c[2] = i == 0 ? cli : (i == 1 ? cji : dii);
+    return o;
+}
+__device__ __forceinline__ double lane_dot(const double (&m)[3], double x)
+{
+    return (m[0] * lane4(x, 0) + m[1] * lane4(x, 1)) + m[2] * lane4(x, 2);
+}
+__device__ __forceinline__ double lane_mv(const LaneRot &Q, double x) { return lane_dot(Q.r, x); }
+__device__ __forceinline__ double lane_mtv(const LaneRot &Q, double x) { return lane_dot(Q.c, x); }
+
+__device__ __forceinline__ double lane_L_to_p(double q, const LaneRot &Q, double L, int c)
+{
+    return 2.0 * lane_qmul(q, lane_vec_to_quat(lane_mtv(Q, L), c), c);
+}
+__device__ __forceinline__ double lane_p_to_Lb(double q, double p, int c)   // vec(q* (x) p) / 2
+{
+    return 0.5 * lane_quat_to_vec(lane_qmul(flip(q, c != 0), p, c), c);
+}
+__device__ __forceinline__ double lane_torque_kick(double q, const LaneRot &Q, double T, double h, int c)
+{
+    return 2.0 * h * lane_qmul(q, lane_vec_to_quat(lane_mtv(Q, T), c), c);
+}
+// free rotation about body axis k (rotor); Ih its moment, r4 = RN(1 / (4 Ih))
+__device__ __forceinline__ void lane_rotor(double &q, double &p, int k, double h, double Ih, double r4, int c)
+{
+    if (Ih == 0.0) return;   // the same for all lanes of the body
+    const bool neg = k == 1 ? (c == 0 || c == 3) : (k == 2 ? c < 2 : (c == 0 || c == 2));
+    const double Pq = flip(lane4(q, c ^ k), neg), Pp = flip(lane4(p, c ^ k), neg);
+    const double t = p * Pq;
+    const double dot = ((lane4(t, 0) + lane4(t, 1)) + lane4(t, 2)) + lane4(t, 3);
+    const double zeta = div_by(dot, 4.0 * Ih, r4);
+    double sn, cs;
+    sincos(zeta * h, &sn, &cs);
+    q = cs * q + sn * Pq;
+    p = cs * p + sn * Pp;
+}
+
+// Forces done: external force, stored F and T, the second half kick (kick)
+// and the pose record the site kernels read.  Component c of every vector on
+// lane c; store: this lane writes (lane 3 and repeated lanes do not).
+__device__ __forceinline__ void lane_force_finish(const StepArgs &a, int64_t i, const DevShape &sh, double q, double R,
+                                                  double P, double L, double F, double T, int kick, int c, bool store)
+{
+    const int k = c == 3 ? 0 : c;
+    F += a.fext[k];   // external force at the centre of mass (no torque)
+    const LaneRot Q = lane_rot(q, c);
+    DevBody *o = a.bodies + i;
+    if (kick) {
+        double p = lane_L_to_p(q, Q, L, c);
+        P = P + 0.5 * a.dt * F;
+        p += lane_torque_kick(q, Q, T, 0.5 * a.dt, c);
+        L = lane_mv(Q, lane_p_to_Lb(q, p, c));
+    }
+    // pose: Q, R, V = P/M, omega = Q Ihat^-1 Q^T L (Eq. 5)
+    const double V = div_by(P, sh.M, sh.rM);
+    const double Lb = lane_mtv(Q, L);
+    const double wb = sh.Ihat[k] > 0.0 ? div_by(Lb, sh.Ihat[k], sh.rI[k]) : 0.0;
+    const double W = lane_mv(Q, wb);
+    if (!store) return;
+    o->F[k] = F;
+    o->T[k] = T;
+    if (kick) { o->P[k] = P; o->Lm[k] = L; }
+    double *p64 = a.pose64 + i * POSE_W;
+    float *p32 = a.pose32 + i * POSE_W;
+    for (int m = 0; m < 3; ++m) { p64[3 * k + m] = Q.r[m]; p32[3 * k + m] = (float)Q.r[m]; }
+    p64[9 + k] = R; p32[9 + k] = (float)R;
+    p64[12 + k] = V; p32[12 + k] = (float)V;
+    p64[15 + k] = W; p32[15 + k] = (float)W;
+}
+
+// --------------------------------------------------------------- body MD
+// IMPULSE: first adds the transfer's per-warp partial sums (the work of
+// k_body_impulse, for the step pipeline, where nothing stands between the two).
+// LONE: every replica has one body at most, so no force acts between bodies and
+// the force pass is finished here.  Also writes the space-frame WCA centres of
+// shapes with one or two of them.
+template <typename Real, bool IMPULSE, bool LONE>
+__global__ void __launch_bounds__(64) k_body_md(StepArgs a)
+{
+    const int g = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 2);
+    const int c = threadIdx.x & 3, k = c == 3 ? 0 : c;
+    const bool valid = g < a.n_bodies;
+    const int i = valid ? g : a.n_bodies - 1;   // every lane takes part in the shuffles
+    const bool store = valid && c < 3;
+    DevBody *o = a.bodies + i;
+    const DevShape &sh = a.shapes[o->shape];
+    const DevReplica &r = a.reps[o->rep];
     const double dt = a.dt;
     int bad = 0;
-    double p[4];
-    L_to_p(b.q, b.Lm, p);
-    for (int k = 0; k < 3; ++k) b.P[k] += 0.5 * dt * b.F[k];
-    torque_kick(b.q, p, b.T, 0.5 * dt);
-    for (int k = 0; k < 3; ++k) {
-        const double d = dt * (b.P[k] / sh.M);
-        b.D[k] += d;
-        b.R[k] = wrapd(b.R[k] + d, (double)r.L[k], bad);
+    double q = o->q[c], P = o->P[k], L = o->Lm[k], R = o->R[k];
+    if (IMPULSE) {
+        const Real *in = reinterpret_cast<const Real *>(a.partial) + (int64_t)i * SITE_WARPS * 6;
+        double sP = 0.0, sL = 0.0;
+        for (int w = 0; w < SITE_WARPS; ++w) {
+            sP += (double)in[w * 6 + k];
+            sL += (double)in[w * 6 + 3 + k];
+        }
+        P += sP;
+        L += sL;
     }
-    rotor(b.q, p, 3, 0.5 * dt, sh.Ihat);
-    rotor(b.q, p, 2, 0.5 * dt, sh.Ihat);
-    rotor(b.q, p, 1, dt, sh.Ihat);
-    rotor(b.q, p, 2, 0.5 * dt, sh.Ihat);
-    rotor(b.q, p, 3, 0.5 * dt, sh.Ihat);
-    double nq = sqrt(b.q[0] * b.q[0] + b.q[1] * b.q[1] + b.q[2] * b.q[2] + b.q[3] * b.q[3]);
-    for (int k = 0; k < 4; ++k) b.q[k] /= nq;
-    p_to_L(b.q, p, b.Lm);
-    DevBody *o = a.bodies + i;
-    for (int k = 0; k < 3; ++k) { o->R[k] = b.R[k]; o->P[k] = b.P[k]; o->Lm[k] = b.Lm[k]; o->D[k] = b.D[k]; }
-    for (int k = 0; k < 4; ++k) o->q[k] = b.q[k];
-    a.bpos[i] = make_float4((float)b.R[0], (float)b.R[1], (float)b.R[2], (float)sh.bound);
+    LaneRot Q = lane_rot(q, c);
+    double p = lane_L_to_p(q, Q, L, c);
+    P += 0.5 * dt * o->F[k];
+    p += lane_torque_kick(q, Q, o->T[k], 0.5 * dt, c);
+    const double d = dt * div_by(P, sh.M, sh.rM);
+    const double D = o->D[k] + d;
+    R = wrapd(R + d, (double)r.L[k], bad);
+#pragma unroll 1
+    for (int e = 0; e < 5; ++e) {   // axes 3, 2, 1, 2, 3
+        const int ax = e < 3 ? 3 - e : e - 1;
+        lane_rotor(q, p, ax, e == 2 ? dt : 0.5 * dt, sh.Ihat[ax - 1], sh.r4I[ax - 1], c);
+    }
+    const double qq = q * q;
+    q /= sqrt(((lane4(qq, 0) + lane4(qq, 1)) + lane4(qq, 2)) + lane4(qq, 3));
+    Q = lane_rot(q, c);
+    L = lane_mv(Q, lane_p_to_Lb(q, p, c));
+    if (store) { o->R[k] = R; o->D[k] = D; }
+    if (store && !LONE) { o->P[k] = P; o->Lm[k] = L; }
+    if (valid) o->q[c] = q;
+    if (a.max_cent <= 2)
+        for (int e = 0; e < sh.n_cent; ++e) {
+            const double *t = a.tcent + 3 * (sh.cent_begin + e);
+            const double x = (Q.r[0] * t[0] + Q.r[1] * t[1]) + Q.r[2] * t[2];
+            if (store) {
+                a.cent64[3 * (o->cent_begin + e) + k] = x;
+                reinterpret_cast<float *>(a.cent32 + o->cent_begin + e)[k] = (float)x;
+            }
+        }
     // neighbour lists stay valid while every body is within half the skin of
     // its position at the last build
+    const float Rf = (float)R, h = 0.5f * r.L[k];
     const float4 p0 = a.bpos_build[i];
-    float d2 = 0.0f;
-    const float Rf[3] = {(float)b.R[0], (float)b.R[1], (float)b.R[2]}, R0[3] = {p0.x, p0.y, p0.z};
-    for (int k = 0; k < 3; ++k) {
-        float d = Rf[k] - R0[k], h = 0.5f * r.L[k];
-        d = d > h ? d - r.L[k] : (d < -h ? d + r.L[k] : d);
-        d2 += d * d;
+    float dx = Rf - (k == 0 ? p0.x : (k == 1 ? p0.y : p0.z));
+    dx = dx > h ? dx - r.L[k] : (dx < -h ? dx + r.L[k] : dx);
+    const float x2 = dx * dx;
+    const float d2 = ((0.0f + lane4(x2, 0)) + lane4(x2, 1)) + lane4(x2, 2);
+    const float4 at = make_float4(lane4(Rf, 0), lane4(Rf, 1), lane4(Rf, 2), (float)sh.bound);
+    if (valid && c == 3) {
+        a.bpos[i] = at;
+        if (!LONE && d2 > 0.25f * NLIST_SKIN * NLIST_SKIN) atomicOr(a.nl_dirty, 1);
     }
-    if (d2 > 0.25f * NLIST_SKIN * NLIST_SKIN) atomicOr(a.nl_dirty, 1);
-    if (bad) atomicOr(a.d_err, ERR_POSITION);
+    if (store && bad) atomicOr(a.d_err, ERR_POSITION);
+    if (LONE) lane_force_finish(a, i, sh, q, R, P, L, 0.0, 0.0, 1, c, store);
 }
 
 __global__ void k_body_pos(StepArgs a)
@@ -202,33 +287,41 @@ __global__ void k_body_pos(StepArgs a)
     a.bpos[i] = make_float4((float)b.R[0], (float)b.R[1], (float)b.R[2], (float)a.shapes[b.shape].bound);
 }
 
-void launch_body_md(const StepArgs &a, cudaStream_t s)
+template <typename Real>
+static void body_md(const StepArgs &a, bool impulse, cudaStream_t s)
 {
-    if (a.n_bodies == 0) return;
-    k_body_md<<<(a.n_bodies + 127) / 128, 128, 0, s>>>(a);
-}
-
-// ------------------------------------------------------------ WCA forces
-__device__ __forceinline__ void min_image(double d[3], const int32_t L[3])
-{
-    for (int k = 0; k < 3; ++k) {
-        double h = 0.5 * L[k];
-        if (d[k] > h) d[k] -= L[k];
-        else if (d[k] < -h) d[k] += L[k];
+    const unsigned grid = (unsigned)((a.n_bodies + 15) / 16);   // 64 threads, four lanes per body
+    if (a.lone_bodies) {
+        if (impulse) k_body_md<Real, true, true><<<grid, 64, 0, s>>>(a);
+        else k_body_md<Real, false, true><<<grid, 64, 0, s>>>(a);
+    } else {
+        if (impulse) k_body_md<Real, true, false><<<grid, 64, 0, s>>>(a);
+        else k_body_md<Real, false, false><<<grid, 64, 0, s>>>(a);
     }
 }
 
+void launch_body_md(const StepArgs &a, bool impulse, cudaStream_t s)
+{
+    if (a.n_bodies == 0) return;
+    if (a.precision == 1) body_md<float>(a, impulse, s);
+    else body_md<double>(a, impulse, s);
+}
+
+// ------------------------------------------------------------ WCA forces
 // Rotated WCA centres of every body, Q c in the space frame, once per pose (in
 // FP64 and rounded to float), so that the pair loop below only adds offsets.
-__global__ void k_body_centres(StepArgs a)
+// One warp per body, one centre per lane: the rotation matrix is formed once
+// for all of them (1120 bodies of up to 19 centres: 6.6 us, 19.6 with one
+// thread per body).
+__global__ void __launch_bounds__(128) k_body_centres(StepArgs a)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     if (i >= a.n_bodies) return;
     const DevBody &b = a.bodies[i];
     const DevShape &sh = a.shapes[b.shape];
     double Q[9];
     rotmat(b.q, Q);
-    for (int c = 0; c < sh.n_cent; ++c) {
+    for (int c = threadIdx.x & 31; c < sh.n_cent; c += 32) {
         double d[3];
         mv(Q, a.tcent + 3 * (sh.cent_begin + c), d);
         const int64_t g = b.cent_begin + c;
@@ -252,38 +345,30 @@ template <> struct CentreOf<double> {
     }
 };
 
-// WCA force (Eq. 1) between centre ca of body i and centre cc of body j, added
-// to F and the torque c_a x f to T.  The centre-pair vector
-// (R_i + c_a) - (R_j + c_c) takes its own minimum image.  Real = float for the
-// P32 form (R_i - R_j formed in FP64, then the pair arithmetic in FP32), double
-// for the P64 form; F and T accumulate in FP64.
+// WCA force (Eq. 1) between centre c_a of body i and centre c_c of body j; dR =
+// R_i - R_j, formed in FP64 and rounded to the form's precision.  The
+// centre-pair vector dR + (c_a - c_c) takes its own minimum image.  Real =
+// float for the P32 form, double for the P64 form.  False beyond the cutoff.
 template <typename Real>
-__device__ __forceinline__ void centre_pair(const StepArgs &a, const DevBody &bi, const DevShape &si, int ca,
-                                            const DevBody &bj, const DevShape &sj, int cc, const DevReplica &r,
-                                            double F[3], double T[3])
+__device__ __forceinline__ bool centre_force(Real dij, const Real (&dR)[3], const Real (&c_a)[3], const Real (&c_c)[3],
+                                             const DevReplica &r, Real (&f)[3])
 {
     const Real rc_extra = Real(1.122462048309373);   // 2^(1/6) sigma
-    const Real dij = Real(0.5 * (si.wca_d + sj.wca_d));
     const Real delta = dij - Real(1), rcut = delta + rc_extra;
-    Real c_a[3], c_c[3], dv[3];
-    CentreOf<Real>::get(a, bi.cent_begin + ca, c_a);
-    CentreOf<Real>::get(a, bj.cent_begin + cc, c_c);
+    Real dv[3];
     for (int k = 0; k < 3; ++k) {
-        dv[k] = (Real)(bi.R[k] - bj.R[k]) + (c_a[k] - c_c[k]);
+        dv[k] = dR[k] + (c_a[k] - c_c[k]);
         const Real L = (Real)r.L[k], h = Real(0.5) * L;
         if (dv[k] > h) dv[k] -= L;
         else if (dv[k] < -h) dv[k] += L;
     }
     const Real rr = sqrt(dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2]);
-    if (!(rr <= rcut)) return;
+    if (!(rr <= rcut)) return false;
     const Real sdl = Real(1) / (rr - delta);
     const Real s6 = sdl * sdl * sdl * sdl * sdl * sdl;
     const Real fm = Real(4) * (Real(12) * s6 * s6 - Real(6) * s6) / (rr - delta);
-    const double f[3] = {(double)(fm * dv[0] / rr), (double)(fm * dv[1] / rr), (double)(fm * dv[2] / rr)};
-    F[0] += f[0]; F[1] += f[1]; F[2] += f[2];
-    T[0] += (double)c_a[1] * f[2] - (double)c_a[2] * f[1];
-    T[1] += (double)c_a[2] * f[0] - (double)c_a[0] * f[2];
-    T[2] += (double)c_a[0] * f[1] - (double)c_a[1] * f[0];
+    for (int k = 0; k < 3; ++k) f[k] = fm * dv[k] / rr;
+    return true;
 }
 
 __device__ __forceinline__ bool may_interact(const StepArgs &a, const float4 &pi, const float4 &pj,
@@ -325,94 +410,151 @@ __global__ void k_nlist_build(StepArgs a)
     }
 }
 
-// Forces done: external force, stored F and T, the second half kick (kick)
-// and the pose record the site kernels read (FP64).
-__device__ __forceinline__ void body_force_finish(const StepArgs &a, int64_t i, const DevBody &bi, const DevShape &si,
-                                                  double F[3], const double T[3], int kick)
-{
-    for (int k = 0; k < 3; ++k) F[k] += a.fext[k];   // external force at the centre of mass (no torque)
-    double Qi[9];
-    rotmat(bi.q, Qi);
-    DevBody *o = a.bodies + i;
-    double P[3] = {bi.P[0], bi.P[1], bi.P[2]}, L[3] = {bi.Lm[0], bi.Lm[1], bi.Lm[2]};
-    for (int k = 0; k < 3; ++k) { o->F[k] = F[k]; o->T[k] = T[k]; }
-    if (kick) {
-        double p[4];
-        L_to_p(bi.q, L, p);
-        for (int k = 0; k < 3; ++k) P[k] = bi.P[k] + 0.5 * a.dt * F[k];
-        torque_kick(bi.q, p, T, 0.5 * a.dt);
-        p_to_L(bi.q, p, L);
-        for (int k = 0; k < 3; ++k) { o->P[k] = P[k]; o->Lm[k] = L[k]; }
-    }
-    // pose: Q, R, V = P/M, omega = Q Ihat^-1 Q^T L (Eq. 5)
-    double V[3], Lb[3], wb[3], W[3];
-    for (int k = 0; k < 3; ++k) V[k] = P[k] / si.M;
-    mtv(Qi, L, Lb);
-    for (int k = 0; k < 3; ++k) wb[k] = si.Ihat[k] > 0.0 ? Lb[k] / si.Ihat[k] : 0.0;
-    mv(Qi, wb, W);
-    double *p64 = a.pose64 + i * POSE_W;
-    float *p32 = a.pose32 + i * POSE_W;
-    for (int k = 0; k < 9; ++k) { p64[k] = Qi[k]; p32[k] = (float)Qi[k]; }
-    for (int k = 0; k < 3; ++k) {
-        p64[9 + k] = bi.R[k]; p32[9 + k] = (float)bi.R[k];
-        p64[12 + k] = V[k]; p32[12 + k] = (float)V[k];
-        p64[15 + k] = W[k]; p32[15 + k] = (float)W[k];
-    }
-    if (i == 0) *a.nl_dirty = 0;   // the lists used by this step are fresh
-}
-
-// One thread per body (shapes of one or two centres): the candidates in
-// ascending order, each centre pair in turn.
-template <typename Real>
+// Shapes of one or two centres (spheres, dumbbells): eight lanes per body.
+// The lanes take the body's candidates eight at a time, one candidate each;
+// the forces of those in reach are then added in candidate order, component k
+// on lane k, so the sums are those of a serial loop.  Rebuilds the body's
+// candidate list first when the lists are out of date (the flag is cleared by
+// the next site PRE pass).  One thread per body, in turn over its candidates,
+// took 7.5 us for a body without any and 11-16 us at 221 bodies (with the list
+// pass and the centres in launches of their own); now 5.5 and 9.5 us in all.
+template <typename Real, int MAXC>
 __global__ void __launch_bounds__(128) k_body_force(StepArgs a, int kick)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n_bodies) return;
-    const DevBody bi = a.bodies[i];
-    const DevShape si = a.shapes[bi.shape];
+    constexpr int NP = MAXC * MAXC;
+    const unsigned full = 0xffffffffu;
+    const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+    const int sub = threadIdx.x & 7, gsh = threadIdx.x & 24;   // lane of the body, its first lane in the warp
+    const int c = sub & 3, k = c == 3 ? 0 : c, k1 = k == 2 ? 0 : k + 1, k2 = k == 0 ? 2 : k - 1;
+    const bool valid = g < a.n_bodies;
+    const int64_t i = valid ? g : a.n_bodies - 1;   // every lane takes part in the votes and shuffles
+    const DevBody &bi = a.bodies[i];
+    const DevShape &si = a.shapes[bi.shape];
     const DevReplica r = a.reps[bi.rep];
-    double F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
-    const int n = a.ncount[i];
-    if (n >= 0 && n <= NLIST_MAX) {
-        for (int e = 0; e < n; ++e) {
-            const int64_t j = a.nlist[i * NLIST_MAX + e];
-            if (j < r.body_begin || j >= r.body_end) continue;
-            const DevBody &bj = a.bodies[j];
-            const DevShape &sj = a.shapes[bj.shape];
-            for (int ca = 0; ca < si.n_cent; ++ca)
-                for (int cc = 0; cc < sj.n_cent; ++cc) centre_pair<Real>(a, bi, si, ca, bj, sj, cc, r, F, T);
+    const float4 pi = a.bpos[i];
+    const float cut = (float)(0.5 * (si.wca_d + a.max_wca_d) - 1.0 + 1.122462048309373);
+    int n;
+    if (*a.nl_dirty) {
+        // candidates within the bounding spheres + cutoff + skin, ascending
+        const float reach = cut + NLIST_SKIN + 1e-2f;
+        n = 0;
+        constexpr int U = 4;   // position loads in flight per lane
+        for (int64_t j0 = r.body_begin; __any_sync(full, j0 < r.body_end); j0 += 8 * U) {
+            float4 pj[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) pj[u] = a.bpos[min(j0 + 8 * u + sub, r.body_end - 1)];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t j = j0 + 8 * u + sub;
+                const bool hit = j < r.body_end && j != i && may_interact(a, pi, pj[u], r, reach);
+                const unsigned m = (__ballot_sync(full, hit) >> gsh) & 0xffu;
+                const int slot = n + __popc(m & ((1u << sub) - 1u));
+                if (valid && hit && slot < NLIST_MAX) a.nlist[i * NLIST_MAX + slot] = (int32_t)j;
+                n += __popc(m);
+            }
         }
+        n = n <= NLIST_MAX ? n : -1;
+        if (valid && sub == 0) {
+            a.ncount[i] = n;
+            a.bpos_build[i] = pi;
+        }
+        __syncwarp();   // the list is read by the body's other lanes
     } else {
-        const float4 pi = a.bpos[i];
-        const float reach = (float)(0.5 * (si.wca_d + a.max_wca_d) - 1.0 + 1.122462048309373) + 1e-2f;
-        for (int64_t j = r.body_begin; j < r.body_end; ++j) {
-            if (j == i || !may_interact(a, pi, a.bpos[j], r, reach)) continue;
-            const DevBody &bj = a.bodies[j];
+        n = a.ncount[i];
+    }
+    const bool listed = n >= 0 && n <= NLIST_MAX;
+    const int64_t total = !valid ? 0 : (listed ? n : r.body_end - r.body_begin);
+    double F = 0.0, T = 0.0;
+    for (int64_t e0 = 0; __any_sync(full, e0 < total); e0 += 8) {
+        const int64_t e = e0 + sub;
+        bool on = e < total;
+        int64_t j = i;
+        if (on) {
+            j = listed ? (int64_t)a.nlist[i * NLIST_MAX + e] : r.body_begin + e;
+            on = j >= r.body_begin && j < r.body_end;
+            if (!listed) on = on && j != i && may_interact(a, pi, a.bpos[j], r, cut + 1e-2f);
+        }
+        Real f[NP][3];
+        unsigned near[NP], some = 0;
+        {
+            const DevBody &bj = a.bodies[on ? j : i];
             const DevShape &sj = a.shapes[bj.shape];
-            for (int ca = 0; ca < si.n_cent; ++ca)
-                for (int cc = 0; cc < sj.n_cent; ++cc) centre_pair<Real>(a, bi, si, ca, bj, sj, cc, r, F, T);
+            const Real dij = Real(0.5 * (si.wca_d + sj.wca_d));
+            Real dR[3];
+            for (int m = 0; m < 3; ++m) dR[m] = (Real)(bi.R[m] - bj.R[m]);
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                const int ca = p / MAXC, cc = p % MAXC;
+                bool hit = on && ca < si.n_cent && cc < sj.n_cent;
+                if (hit) {
+                    Real ci[3], cj[3];
+                    CentreOf<Real>::get(a, bi.cent_begin + ca, ci);
+                    CentreOf<Real>::get(a, bj.cent_begin + cc, cj);
+                    hit = centre_force<Real>(dij, dR, ci, cj, r, f[p]);
+                }
+                near[p] = (__ballot_sync(full, hit) >> gsh) & 0xffu;
+                some |= near[p];
+            }
+        }
+        while (__any_sync(full, some != 0)) {   // the body's candidates in reach, in order
+            const int src = some ? __ffs(some) - 1 : 0;
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                Real t[3];
+                for (int m = 0; m < 3; ++m) t[m] = __shfl_sync(full, f[p][m], src, 8);
+                if (some && (near[p] >> src & 1u)) {
+                    Real ci[3];
+                    CentreOf<Real>::get(a, bi.cent_begin + p / MAXC, ci);
+                    const double f1 = (double)(k == 0 ? t[1] : (k == 1 ? t[2] : t[0]));
+                    const double f2 = (double)(k == 0 ? t[2] : (k == 1 ? t[0] : t[1]));
+                    F += (double)(k == 0 ? t[0] : (k == 1 ? t[1] : t[2]));
+                    T += (double)ci[k1] * f2 - (double)ci[k2] * f1;
+                }
+            }
+            some &= some - 1;
         }
     }
-    body_force_finish(a, i, bi, si, F, T, kick);
+    lane_force_finish(a, i, si, bi.q[c], bi.R[k], bi.P[k], bi.Lm[k], F, T, kick, c, valid && sub < 3);
 }
 
 // One warp per body (shapes with many centres, e.g. rods): the lanes take the
 // (neighbour, centre, centre) triples of the body's candidates in turn, each
 // lane summing its triples in order, and a fixed shuffle tree adds the lanes,
-// so the result depends only on the candidate list.
+// so the result depends only on the candidate list.  R_i - R_j is formed once
+// per candidate and kept in shared memory (formed for every triple, its FP64
+// subtractions and conversions were most of the pass: 200 us against 147 for
+// 1120 bodies of up to 19 centres).
+constexpr int WARP_BODIES = 4;   // bodies (warps) per CTA
 template <typename Real>
-__global__ void __launch_bounds__(128) k_body_force_warp(StepArgs a, int kick)
+__global__ void __launch_bounds__(32 * WARP_BODIES) k_body_force_warp(StepArgs a, int kick)
 {
+    __shared__ Real sdR[WARP_BODIES][NLIST_MAX][3];
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (i >= a.n_bodies) return;   // uniform over the warp
-    const DevBody bi = a.bodies[i];
-    const DevShape si = a.shapes[bi.shape];
+    const DevBody &bi = a.bodies[i];
+    const DevShape &si = a.shapes[bi.shape];
     const DevReplica r = a.reps[bi.rep];
     double F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
+    auto pair = [&](const Real (&dR)[3], const DevBody &bj, const DevShape &sj, int ca, int cc) {
+        Real ci[3], cj[3], f[3];
+        CentreOf<Real>::get(a, bi.cent_begin + ca, ci);
+        CentreOf<Real>::get(a, bj.cent_begin + cc, cj);
+        if (!centre_force<Real>(Real(0.5 * (si.wca_d + sj.wca_d)), dR, ci, cj, r, f)) return;
+        for (int k = 0; k < 3; ++k) F[k] += (double)f[k];
+        T[0] += (double)ci[1] * (double)f[2] - (double)ci[2] * (double)f[1];
+        T[1] += (double)ci[2] * (double)f[0] - (double)ci[0] * (double)f[2];
+        T[2] += (double)ci[0] * (double)f[1] - (double)ci[1] * (double)f[0];
+    };
     const int n = a.ncount[i];
     const int nci = si.n_cent, maxc = max(a.max_cent, 1);
     if (n >= 0 && n <= NLIST_MAX) {
+        for (int e = lane; e < n; e += 32) {
+            const int64_t j = a.nlist[i * NLIST_MAX + e];
+            const bool on = j >= r.body_begin && j < r.body_end;
+            for (int k = 0; k < 3; ++k) sdR[wid][e][k] = on ? (Real)(bi.R[k] - a.bodies[j].R[k]) : Real(0);
+        }
+        __syncwarp();
         const int per = nci * maxc;
         for (int t = lane; t < n * per; t += 32) {
             const int e = t / per, rem = t - e * per, ca = rem / maxc, cc = rem - ca * maxc;
@@ -420,7 +562,7 @@ __global__ void __launch_bounds__(128) k_body_force_warp(StepArgs a, int kick)
             if (j < r.body_begin || j >= r.body_end) continue;
             const DevBody &bj = a.bodies[j];
             const DevShape &sj = a.shapes[bj.shape];
-            if (cc < sj.n_cent) centre_pair<Real>(a, bi, si, ca, bj, sj, cc, r, F, T);
+            if (cc < sj.n_cent) pair(sdR[wid][e], bj, sj, ca, cc);
         }
     } else {
         // the list overflowed: every body of the replica, prefiltered
@@ -430,8 +572,10 @@ __global__ void __launch_bounds__(128) k_body_force_warp(StepArgs a, int kick)
             if (j == i || !may_interact(a, pi, a.bpos[j], r, reach)) continue;
             const DevBody &bj = a.bodies[j];
             const DevShape &sj = a.shapes[bj.shape];
+            Real dR[3];
+            for (int k = 0; k < 3; ++k) dR[k] = (Real)(bi.R[k] - bj.R[k]);
             for (int ca = 0; ca < nci; ++ca)
-                for (int cc = 0; cc < sj.n_cent; ++cc) centre_pair<Real>(a, bi, si, ca, bj, sj, cc, r, F, T);
+                for (int cc = 0; cc < sj.n_cent; ++cc) pair(dR, bj, sj, ca, cc);
         }
     }
 #pragma unroll
@@ -441,24 +585,36 @@ __global__ void __launch_bounds__(128) k_body_force_warp(StepArgs a, int kick)
             F[k] += __shfl_down_sync(0xffffffffu, F[k], o);
             T[k] += __shfl_down_sync(0xffffffffu, T[k], o);
         }
-    if (lane == 0) body_force_finish(a, i, bi, si, F, T, kick);
+    const int c = lane & 3, k = c == 3 ? 0 : c;
+    double Fk = 0.0, Tk = 0.0;
+    for (int m = 0; m < 3; ++m) {   // lane 0's sums, component k to lane k
+        const double f = __shfl_sync(0xffffffffu, F[m], 0), t = __shfl_sync(0xffffffffu, T[m], 0);
+        if (m == k) { Fk = f; Tk = t; }
+    }
+    lane_force_finish(a, i, si, bi.q[c], bi.R[k], bi.P[k], bi.Lm[k], Fk, Tk, kick, c, lane < 3);
+    if (i == 0 && lane == 0) *a.nl_dirty = 0;   // the lists used by this step are fresh
 }
 
 void launch_body_force(const StepArgs &a, int kick, cudaStream_t s)
 {
     if (a.n_bodies == 0) return;
+    if (kick && a.lone_bodies) return;   // finished by k_body_md
+    const unsigned warps = (unsigned)((a.n_bodies + WARP_BODIES - 1) / WARP_BODIES);
     if (!kick) k_body_pos<<<(a.n_bodies + 127) / 128, 128, 0, s>>>(a);
-    k_body_centres<<<(a.n_bodies + 127) / 128, 128, 0, s>>>(a);
-    const int wpb = 4;
-    k_nlist_build<<<(a.n_bodies + wpb - 1) / wpb, 32 * wpb, 0, s>>>(a);
-    if (a.max_cent <= 2) {   // spheres, dumbbells: one thread per body
-        const unsigned grid = (unsigned)((a.n_bodies + 127) / 128);
-        if (a.precision == 1) k_body_force<float><<<grid, 128, 0, s>>>(a, kick);
-        else k_body_force<double><<<grid, 128, 0, s>>>(a, kick);
+    if (!kick || a.max_cent > 2) k_body_centres<<<warps, 32 * WARP_BODIES, 0, s>>>(a);
+    if (a.max_cent <= 2) {   // spheres, dumbbells: eight lanes per body
+        const unsigned grid = (unsigned)((a.n_bodies + 15) / 16);
+        if (a.precision == 1) {
+            if (a.max_cent <= 1) k_body_force<float, 1><<<grid, 128, 0, s>>>(a, kick);
+            else k_body_force<float, 2><<<grid, 128, 0, s>>>(a, kick);
+        } else {
+            if (a.max_cent <= 1) k_body_force<double, 1><<<grid, 128, 0, s>>>(a, kick);
+            else k_body_force<double, 2><<<grid, 128, 0, s>>>(a, kick);
+        }
     } else {                 // many centres: one warp per body
-        const unsigned grid = (unsigned)((a.n_bodies + wpb - 1) / wpb);
-        if (a.precision == 1) k_body_force_warp<float><<<grid, 32 * wpb, 0, s>>>(a, kick);
-        else k_body_force_warp<double><<<grid, 32 * wpb, 0, s>>>(a, kick);
+        k_nlist_build<<<warps, 32 * WARP_BODIES, 0, s>>>(a);
+        if (a.precision == 1) k_body_force_warp<float><<<warps, 32 * WARP_BODIES, 0, s>>>(a, kick);
+        else k_body_force_warp<double><<<warps, 32 * WARP_BODIES, 0, s>>>(a, kick);
     }
 }
 
@@ -606,6 +762,8 @@ __global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_sites_
     const DevShape sh = a.shapes[shape];
     const DevReplica r = a.reps[rep];
     const int64_t step = *a.d_step + a.step_offset;
+    // the force pass of this pose is done: its neighbour lists are fresh
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.nl_dirty = 0;
     if (threadIdx.x < POSE_W) sPose[threadIdx.x] = pose_ptr(a, blockIdx.x, Real(0))[threadIdx.x];
     if (threadIdx.x == 0) grid_shift(r, step, sS);
     __syncthreads();

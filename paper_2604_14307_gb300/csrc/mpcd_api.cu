@@ -75,6 +75,7 @@ struct mpcd_ctx {
     float4 *d_cent32 = nullptr;
     int64_t n_cent_bodies = 0;                  // WCA centres over all bodies
     int max_cent = 0;                           // most centres of any shape
+    bool lone_bodies = true;                    // no replica has more than one body
     float *d_tbf = nullptr, *d_tmf = nullptr;
     void *sol[2][6] = {};
     uint32_t *tag[2] = {nullptr, nullptr};
@@ -253,6 +254,7 @@ StepArgs make_args(const mpcd_ctx *c)
     a.tcent = c->d_tcent;
     a.max_wca_d = c->max_wca_d;
     a.max_cent = c->max_cent;
+    a.lone_bodies = c->lone_bodies ? 1 : 0;
     a.cent64 = c->d_cent64;
     a.cent32 = c->d_cent32;
     a.site_v = c->site_v;
@@ -414,6 +416,40 @@ bool staged_fits(const mpcd_ctx *c, int tile, int mode, int block)
     return ring_bytes(c, mode, tile, block) <= lim;
 }
 
+// Default launch form of the solvent pass (mpcd_autotune measures instead).
+// FP32, at least four 1024-particle tiles for each of three CTAs per SM: the
+// staged pass, whose work counter evens out the SMs that the site/body chain
+// shares (us per step, per-warp ring against staged: 80 M particles 1940 and
+// 1794, 17 M in 512 boxes 450 and 398, 17 M of solvent alone 504 and 462, 9 M
+// MPCD-AT 736 and 559, 2.6 M 110 and 104; 0.6 M MPCD-AT 65 and 69).  Boxes that
+// cut the tiles short keep the ring.  Otherwise FP32 takes a ring per warp of
+// 128-particle tiles; MPCD-AT beside colloids with 384 threads, because 512 of
+// its 128 registers fill the SM and the site/body chain then waits for the
+// whole pass (0.6 M particles, 221 bodies: 144 and 65 us per step).  FP64 takes
+// the warp-specialised pass with the largest tile whose ring fits, else direct
+// loads.
+void default_tuning(mpcd_ctx *c)
+{
+    const int period = c->tune.sort_period;
+    const bool p32 = c->prm.precision == MPCD_P32;
+    if (p32 && c->Ns >= (int64_t)4 * 3 * c->num_sms * 1024 && c->Ns >= (int64_t)4096 * c->nrep &&
+        staged_fits(c, 1024, 1, 128)) {
+        c->tune = mpcd_tuning{128, 1024, 3, period, 1};
+        return;
+    }
+    if (staged_fits(c, 128, 3, 512)) {
+        c->tune = mpcd_tuning{c->prm.rule == MPCD_AT && c->B > 0 ? 384 : 512, 128, 1, period, 3};
+        return;
+    }
+    c->tune = mpcd_tuning{512, 2048, 1, period, 0};
+    for (int t : {2048, 1536, 1024, 512})
+        if (staged_fits(c, t, 2, 512)) {
+            c->tune.tile = t;
+            c->tune.staged = 2;
+            break;
+        }
+}
+
 LaunchCfg solvent_cfg(const mpcd_ctx *c)
 {
     const int mode =
@@ -436,15 +472,17 @@ int k_stream(mpcd_ctx *c, cudaStream_t s)
     LaunchCfg cfg = solvent_cfg(c);
     int e = timed(c, "solvent_stream", solvent_bytes(c, SOLV_STREAM), s, [&] { launch_solvent(a, SOLV_STREAM, cfg, s); });
     if (e) return e;
-    e = timed(c, "body_md", 0, s, [&] { launch_body_md(a, s); });
+    e = timed(c, "body_md", 0, s, [&] { launch_body_md(a, false, s); });
     if (e) return e;
     return timed(c, "body_force", 0, s, [&] { launch_body_force(a, 1, s); });
 }
 
-int k_bodies(mpcd_ctx *c, cudaStream_t s)
+// the body step; impulse: with the transfer of the POST coupling before it
+// (k_post without its impulse pass)
+int k_bodies(mpcd_ctx *c, cudaStream_t s, bool impulse = false)
 {
     StepArgs a = make_args(c);
-    int e = timed(c, "body_md", 0, s, [&] { launch_body_md(a, s); });
+    int e = timed(c, "body_md", 0, s, [&] { launch_body_md(a, impulse, s); });
     if (e) return e;
     return timed(c, "body_force", 0, s, [&] { launch_body_force(a, 1, s); });
 }
@@ -464,12 +502,12 @@ int k_params(mpcd_ctx *c, cudaStream_t s)
     return timed(c, "cell_params", bytes, s, [&] { launch_params(a, c->num_sms * 8, s); });
 }
 
-int k_post(mpcd_ctx *c, cudaStream_t s)
+int k_post(mpcd_ctx *c, cudaStream_t s, bool impulse = true)
 {
     StepArgs a = make_args(c);
     double bytes = (double)c->Nsite * (3.0 * c->realsz + 4.0);
     int e = timed(c, "sites_post", bytes, s, [&] { launch_sites_post(a, c->max_sites, s); });
-    if (e) return e;
+    if (e || !impulse) return e;
     return timed(c, "body_impulse", 0, s, [&] { launch_body_impulse(a, s); });
 }
 
@@ -656,9 +694,11 @@ int run_steps(mpcd_ctx *c, int64_t n, cudaStream_t s)
         } else {
             CK(c, cudaEventRecord(c->side_ev[0], s));
             CK(c, cudaStreamWaitEvent(c->side, c->side_ev[0], 0));
-            if ((e = k_post(c, c->side))) break;
+            // the transfer is added by the body step, unless it is sampled in between
+            const bool apart = c->vacf.n_lags > 0;
+            if ((e = k_post(c, c->side, apart))) break;
             if ((e = k_vacf(c, c->side))) break;
-            if ((e = k_bodies(c, c->side))) break;
+            if ((e = k_bodies(c, c->side, !apart))) break;
             if ((e = k_pre(c, c->side, 1))) break;   // step k+1, before the counter advances
             CK(c, cudaEventRecord(c->side_ev[1], c->side));
             if ((e = k_solvent(c, SOLV_COLLIDE | SOLV_STREAM | SOLV_BIN, s))) break;
@@ -796,7 +836,12 @@ int mpcd_create(const mpcd_params *params, int32_t n_shapes, const mpcd_shape_de
         }
         (void)off;
         S.M = M;
-        for (int k = 0; k < 3; ++k) S.Ihat[k] = I[k];
+        S.rM = 1.0 / M;
+        for (int k = 0; k < 3; ++k) {
+            S.Ihat[k] = I[k];
+            S.rI[k] = I[k] > 0.0 ? 1.0 / I[k] : 0.0;
+            S.r4I[k] = I[k] > 0.0 ? 1.0 / (4.0 * I[k]) : 0.0;
+        }
         double bound = 0;
         for (int j = 0; j < d.n_centres; ++j) {
             const double *x = d.centres + 3 * j;
@@ -853,6 +898,7 @@ int mpcd_create(const mpcd_params *params, int32_t n_shapes, const mpcd_shape_de
         cells += (int64_t)d.L[0] * d.L[1] * d.L[2];
         slot += (d.n_solvent + 7) & ~(int64_t)7;
         bodies += d.n_bodies;
+        if (d.n_bodies > 1) c->lone_bodies = false;
         rows += d.n_solvent;
         c->reps.push_back(R);
     }
@@ -979,20 +1025,7 @@ int mpcd_create(const mpcd_params *params, int32_t n_shapes, const mpcd_shape_de
     if (cudaMemset(c->d_bpos_build, 0, std::max<int64_t>(1, c->B) * sizeof(float4)) != cudaSuccess) st = MPCD_ERR_CUDA;
     if (cudaMemset(c->d_nl_dirty, 0xFF, sizeof(int)) != cudaSuccess) st = MPCD_ERR_CUDA;
     if (cudaMemset(c->d_err, 0, 8) != cudaSuccess) st = MPCD_ERR_CUDA;
-    // default launch form: a ring per warp of 128-particle tiles, else the
-    // warp-specialised pass with the largest tile whose ring fits in shared
-    // memory (the FP64 form), else direct loads
-    if (staged_fits(c, 128, 3, 512)) {
-        c->tune = mpcd_tuning{512, 128, 1, c->tune.sort_period, 3};
-    } else {
-        c->tune = mpcd_tuning{512, 2048, 1, c->tune.sort_period, 0};
-        for (int t : {2048, 1536, 1024, 512})
-            if (staged_fits(c, t, 2, 512)) {
-                c->tune.tile = t;
-                c->tune.staged = 2;
-                break;
-            }
-    }
+    default_tuning(c);
     build_tiles(c);
     build_ctiles(c);
     if (!st) st = upload_tiles(c);

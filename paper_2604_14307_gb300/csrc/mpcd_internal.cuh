@@ -68,6 +68,7 @@ struct DevShape {
     int32_t n_sites, n_cent;
     double M;               // total site mass
     double Ihat[3];         // principal moments of the sites
+    double rM, rI[3], r4I[3];   // RN(1 / M), RN(1 / Ihat), RN(1 / (4 Ihat)) (0 for a zero moment)
     double wca_d;           // centre diameter
     double bound;           // largest centre distance from the COM
 };
@@ -124,6 +125,7 @@ struct StepArgs {
     const double *tcent;            // WCA centres [centres][3]
     double max_wca_d;               // largest centre diameter of any shape
     int32_t max_cent;               // most WCA centres of any shape
+    int32_t lone_bodies;            // every replica has one body at most: no force between bodies
     double *cent64;                 // per body centre: Q c in the space frame [n][3] (this step's pose)
     float4 *cent32;                 // the same rounded to float
     void *site_v;                   // [3][n_sites] SoA
@@ -504,7 +506,8 @@ void launch_body_partial(const StepArgs &a, double *out, cudaStream_t s);
 void launch_body_apply(const StepArgs &a, const double *dpl, cudaStream_t s);
 
 // bodies and sites (kernels_bodies.cu)
-void launch_body_md(const StepArgs &a, cudaStream_t s);
+// impulse: with the transfer's sums (launch_body_impulse) added first
+void launch_body_md(const StepArgs &a, bool impulse, cudaStream_t s);
 void launch_body_force(const StepArgs &a, int kick, cudaStream_t s);
 void launch_sites_pre(const StepArgs &a, int max_sites, cudaStream_t s);
 void launch_sites_post(const StepArgs &a, int max_sites, cudaStream_t s);
