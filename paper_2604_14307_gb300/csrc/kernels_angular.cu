@@ -72,7 +72,7 @@ __global__ void k_ang_shift(StepArgs a, int4 *shifts)
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= a.n_rep) return;
     int32_t S[3];
-    grid_shift(a.reps[r], *a.d_step, S);
+    grid_shift(a.reps[r], current_step(a), S);
     shifts[r] = make_int4(S[0], S[1], S[2], 0);
 }
 

@@ -761,7 +761,7 @@ __global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_sites_
     const int64_t site_begin = B.site_begin;
     const DevShape sh = a.shapes[shape];
     const DevReplica r = a.reps[rep];
-    const int64_t step = *a.d_step + a.step_offset;
+    const int64_t step = current_step(a);
     // the force pass of this pose is done: its neighbour lists are fresh
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.nl_dirty = 0;
     if (threadIdx.x < POSE_W) sPose[threadIdx.x] = pose_ptr(a, blockIdx.x, Real(0))[threadIdx.x];
@@ -910,7 +910,7 @@ __global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_sites_
     const int64_t site_begin = B.site_begin;
     const DevShape sh = a.shapes[B.shape];
     const DevReplica r = a.reps[B.rep];
-    const int64_t step = *a.d_step;
+    const int64_t step = current_step(a);
     if (threadIdx.x < POSE_W) sPose[threadIdx.x] = pose_ptr(a, blockIdx.x, Real(0))[threadIdx.x];
     __syncthreads();
     Pose<Real> P;
@@ -1018,7 +1018,7 @@ __global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_ang_si
     const int64_t site_begin = B.site_begin;
     const DevShape sh = a.shapes[B.shape];
     const DevReplica r = a.reps[B.rep];
-    const int64_t step = *a.d_step;
+    const int64_t step = current_step(a);
     const int4 S = a.ang_shift[B.rep];
     W *w = reinterpret_cast<W *>(a.ang_words);
     const int64_t C = a.n_cells;
@@ -1088,11 +1088,11 @@ void launch_body_impulse(const StepArgs &a, cudaStream_t s)
     else k_body_impulse<double><<<(a.n_bodies + 127) / 128, 128, 0, s>>>(a);
 }
 
-__global__ void k_advance_step(int64_t *step) { *step += 1; }
+__global__ void k_advance_step(int64_t *step, int64_t n) { *step += n; }
 
-void launch_advance_step(const StepArgs &a, cudaStream_t s)
+void launch_advance_step(const StepArgs &a, int64_t n, cudaStream_t s)
 {
-    k_advance_step<<<1, 1, 0, s>>>(const_cast<int64_t *>(a.d_step));
+    k_advance_step<<<1, 1, 0, s>>>(const_cast<int64_t *>(a.d_step), n);
 }
 
 // FP64 body diagnostics: sum P, sum |P|^2/2M, sum L_b.Ihat^-1.L_b/2 (L_b = Q^T L)
@@ -1130,7 +1130,7 @@ void launch_body_diag(const StepArgs &a, double *acc, cudaStream_t s)
 // angular velocity Q Ihat^-1 Q^T L.  FP64, one thread per body.
 __global__ void k_vacf_sample(StepArgs a, VacfArgs g)
 {
-    const int64_t done = *a.d_step + 1 - g.start;   // steps completed since the start
+    const int64_t done = current_step(a) + 1 - g.start;   // steps completed since the start
     if (done <= 0 || done % g.every != 0) return;
     const int64_t smp = done / g.every - 1;          // this sample's index
     const int nk = (int)(smp + 1 < g.n_lags ? smp + 1 : g.n_lags);

@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(512) k_solvent(StepArgs a)
     __shared__ int64_t sbeg, send;
     __shared__ uint32_t skey[2];
 
-    const int64_t step = *a.d_step;
+    const int64_t step = current_step(a);
     const Real dt = Consts<Real>::dt(a), m = Consts<Real>::m(a), kT = Consts<Real>::kT(a);
     const Real ca = Consts<Real>::ca(a), sa = Consts<Real>::sa(a);
     const Real sc = sqrt(kT / m);
@@ -558,7 +558,7 @@ __global__ void __maxnreg__((StRegs<Real, RULE>::n)) k_solvent_staged(StepArgs a
     __shared__ int stile[ST_STAGES];   // tile in each stage (-1: none, the pass is done)
 
     const size_t SB = stage_bytes<Real, RULE>(cap);
-    const int64_t step = *a.d_step;
+    const int64_t step = current_step(a);
     const Real dt = Consts<Real>::dt(a), m = Consts<Real>::m(a), kT = Consts<Real>::kT(a);
     const Real ca = Consts<Real>::ca(a), sa = Consts<Real>::sa(a);
     const Real sc = sqrt(kT / m);
@@ -782,7 +782,7 @@ __global__ void __launch_bounds__(544) k_solvent_ws(StepArgs a, int cap)
     const int n_cwarps = n_cons >> 5;
     const bool producer = (int)threadIdx.x >= n_cons;
     const size_t SB = stage_bytes<Real, RULE>(cap);
-    const int64_t step = *a.d_step;
+    const int64_t step = current_step(a);
     Real *G[6] = {reinterpret_cast<Real *>(a.x), reinterpret_cast<Real *>(a.y), reinterpret_cast<Real *>(a.z),
                   reinterpret_cast<Real *>(a.vx), reinterpret_cast<Real *>(a.vy), reinterpret_cast<Real *>(a.vz)};
     const int K = a.n_tiles > (int)blockIdx.x ? (a.n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
@@ -996,7 +996,7 @@ __global__ void __maxnreg__((WtRegs<Real, RULE>::n)) k_solvent_wt(StepArgs a, in
     const int nwarps = blockDim.x >> 5;
     const size_t SB = stage_bytes<Real, RULE>(cap);
     unsigned char *wsm = smem + (size_t)warp * WT_STAGES * SB;
-    const int64_t step = *a.d_step;
+    const int64_t step = current_step(a);
     // the global arrays are read from the kernel parameters where lane 0 needs them
     auto garr = [&](int c) -> Real * {
         void *p = c == 0 ? a.x : c == 1 ? a.y : c == 2 ? a.z : c == 3 ? a.vx : c == 4 ? a.vy : a.vz;
@@ -1590,7 +1590,7 @@ __global__ void __launch_bounds__(256, 4) k_params32(StepArgs a)
             }
     }
     __syncthreads();   // stile; the words are re-read from shared memory below
-    const int64_t step = *a.d_step;
+    const int64_t step = current_step(a);
 #pragma unroll 1
     for (int k = 0; k < K; ++k) {
         const Tile tl = stile[k];
@@ -1611,7 +1611,7 @@ __global__ void __launch_bounds__(256) k_params(StepArgs a)
 {
     constexpr int NW = NWords<Real, RULE>::n;
     typedef typename SumWord<Real>::type W;
-    const int64_t step = *a.d_step;
+    const int64_t step = current_step(a);
     W *sums = reinterpret_cast<W *>(a.sums);
     W *dbg = reinterpret_cast<W *>(a.dbg_sums);
     const int64_t C = a.n_cells;
@@ -1970,7 +1970,7 @@ __global__ void __launch_bounds__(256) k_sort_rank(StepArgs a, const int32_t *ex
     const Real *X = (const Real *)a.x, *Y = (const Real *)a.y, *Z = (const Real *)a.z;
     const unsigned lane = threadIdx.x & 31u;
     const int units = a.n_tiles * SORT_UNITS;
-    const int64_t step1 = *a.d_step + 1;
+    const int64_t step1 = current_step(a) + 1;
     int last_rep = -1;
     typename ShiftT<Real>::type sh[3] = {};
     for (int w = blockIdx.x; w < units; w += gridDim.x) {   // uniform trip count (warp votes)
@@ -2570,7 +2570,7 @@ __global__ void __launch_bounds__(256) k_order_solvent(StepArgs a, int32_t *coun
                                                        int32_t *cursor, unsigned long long *keys)
 {
     const Real *X = (const Real *)a.x, *Y = (const Real *)a.y, *Z = (const Real *)a.z;
-    const int64_t step = *a.d_step;
+    const int64_t step = current_step(a);
     for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x) {
         const Tile tl = a.tiles[t];
         const DevReplica r = a.reps[tl.rep];

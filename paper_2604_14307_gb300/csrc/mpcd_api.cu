@@ -28,10 +28,16 @@ struct Pending {
     cudaEvent_t a, b;
     double bytes;
 };
+// A sequence of launches that is recorded once and replayed (enqueue_piece).
+enum PieceKind : int { PIECE_HEAD, PIECE_MIDDLE, PIECE_TAIL, PIECE_WHOLE };
+struct Piece {
+    int kind;
+    int64_t steps;      // middle or whole steps
+    bool sort;          // a re-sort after the last of them
+};
 struct GraphEntry {
     cudaGraphExec_t exec;
-    int cur_end;
-    int64_t since_end;
+    int cur_end;        // solvent buffer in use after it
 };
 
 }  // namespace
@@ -103,7 +109,8 @@ struct mpcd_ctx {
     std::map<std::string, KStat> prof;
     std::vector<cudaEvent_t> evpool;
 
-    std::map<std::tuple<int64_t, int, int64_t>, GraphEntry> graphs;
+    std::map<std::tuple<int, int64_t, bool, int>, GraphEntry> graphs;   // (piece, solvent buffer in use before it)
+    int64_t step_off = 0;           // steps enqueued since the device counter last advanced
     cudaStream_t cap_stream = nullptr;
     cudaStream_t io_stream = nullptr;           // host copies that overlap with kernels
     cudaEvent_t io_ev[2] = {nullptr, nullptr};
@@ -261,6 +268,7 @@ StepArgs make_args(const mpcd_ctx *c)
     a.site_cell = c->site_cell;
     a.n_sites = c->Nsite;
     a.d_step = c->d_step;
+    a.step_offset = (int32_t)c->step_off;
     a.d_err = c->d_err;
     a.tile_ctr = c->d_tile_ctr;
     a.site_own = c->slab ? 1 : 0;
@@ -490,7 +498,7 @@ int k_bodies(mpcd_ctx *c, cudaStream_t s, bool impulse = false)
 int k_pre(mpcd_ctx *c, cudaStream_t s, int step_offset = 0)
 {
     StepArgs a = make_args(c);
-    a.step_offset = step_offset;
+    a.step_offset += step_offset;
     double bytes = (double)c->Nsite * (3.0 * c->realsz + 4.0);
     return timed(c, "sites_pre", bytes, s, [&] { launch_sites_pre(a, c->max_sites, s); });
 }
@@ -531,13 +539,19 @@ int k_solvent(mpcd_ctx *c, int flags, cudaStream_t s)
     return timed(c, name, solvent_bytes(c, flags), s, [&] { launch_solvent(a, flags, cfg, s); });
 }
 
-int k_advance(mpcd_ctx *c, cudaStream_t s)
+// n steps are enqueued: the device counter moves on
+int k_advance(mpcd_ctx *c, cudaStream_t s, int64_t n)
 {
     StepArgs a = make_args(c);
-    launch_advance_step(a, s);
-    c->last_key = c->step;
-    c->step += 1;
+    launch_advance_step(a, n, s);
     return MPCD_OK;
+}
+
+// the host's side of it
+void count_steps(mpcd_ctx *c, int64_t n)
+{
+    c->last_key = c->step + n - 1;
+    c->step += n;
 }
 
 static_assert(RN_CAP == MPCD_RNEMD_MAX_CANDIDATES, "candidate capacity of the exchange");
@@ -556,7 +570,7 @@ int k_rnemd(mpcd_ctx *c, cudaStream_t s, int step_offset, int fix)
     g.vtf = (float)g.vt;
     g.max_pairs = r.max_pairs;
     g.period = r.period;
-    g.step_offset = step_offset;
+    g.step_offset = a.step_offset + step_offset;
     g.fix_sums = fix;
     g.hist = c->rn_hist;
     g.count = c->rn_count;
@@ -647,22 +661,80 @@ int k_collide(mpcd_ctx *c, cudaStream_t s)
     return e;
 }
 
-// whole steps in the unpipelined order stream, couple(PRE), collide,
+// one whole step in the unpipelined order stream, couple(PRE), collide,
 // couple(POST) (the +a variants, whose correction needs the cell totals of
 // the rule's velocities before any particle streams on)
-int run_steps_unfused(mpcd_ctx *c, int64_t n, cudaStream_t s)
+int unfused_step(mpcd_ctx *c, cudaStream_t s)
+{
+    int e = k_stream(c, s);
+    if (!e) e = k_pre(c, s);
+    if (!e) e = k_collide(c, s);
+    if (!e) e = k_post(c, s);
+    if (!e) e = k_vacf(c, s);
+    return e;
+}
+
+// Whole steps are software-pipelined: the solvent pass of step k collides (k),
+// streams and bins for step k+1; beside it, on a second stream, run the site
+// POST coupling of step k and the body step and site PRE coupling of step k+1
+// (they need step k's cell parameters and impulse, not its solvent pass; both
+// branches add to the cleared cell sums of step k+1 with integer atomics, so
+// the order between them changes no result).  The branches join before the
+// cell parameters of step k+1.
+int head_step(mpcd_ctx *c, cudaStream_t s)     // before the first collision
+{
+    int e = k_solvent(c, SOLV_STREAM | SOLV_BIN, s);
+    if (!e) e = k_rnemd(c, s, 0, 1);
+    if (!e) e = k_bodies(c, s);
+    if (!e) e = k_pre(c, s);
+    return e;
+}
+
+int middle_step(mpcd_ctx *c, cudaStream_t s)   // step k's collision up to step k+1's
+{
+    int e = k_params(c, s);
+    if (e) return e;
+    CK(c, cudaEventRecord(c->side_ev[0], s));
+    CK(c, cudaStreamWaitEvent(c->side, c->side_ev[0], 0));
+    // the transfer is added by the body step, unless it is sampled in between
+    const bool apart = c->vacf.n_lags > 0;
+    e = k_post(c, c->side, apart);
+    if (!e) e = k_vacf(c, c->side);
+    if (!e) e = k_bodies(c, c->side, !apart);
+    if (!e) e = k_pre(c, c->side, 1);   // of step k+1
+    if (e) return e;
+    CK(c, cudaEventRecord(c->side_ev[1], c->side));
+    if ((e = k_solvent(c, SOLV_COLLIDE | SOLV_STREAM | SOLV_BIN, s))) return e;
+    if ((e = k_rnemd(c, s, 1, 1))) return e;   // before the collision of step k+1
+    CK(c, cudaStreamWaitEvent(s, c->side_ev[1], 0));
+    return MPCD_OK;
+}
+
+int tail_step(mpcd_ctx *c, cudaStream_t s)     // the last step's collision
+{
+    int e = k_params(c, s);
+    if (!e) e = k_post(c, s);
+    if (!e) e = k_vacf(c, s);
+    if (!e) e = k_solvent(c, SOLV_COLLIDE, s);
+    return e;
+}
+
+int enqueue_piece(mpcd_ctx *c, const Piece &p, cudaStream_t s)
 {
     int e = MPCD_OK;
-    for (int64_t k = 0; k < n && !e; ++k) {
-        if ((e = k_stream(c, s))) break;
-        if ((e = k_pre(c, s))) break;
-        if ((e = k_collide(c, s))) break;
-        if ((e = k_post(c, s))) break;
-        if ((e = k_vacf(c, s))) break;
-        if ((e = k_advance(c, s))) break;
-        if (c->prm.sort_period >= 0 && ++c->since_sort >= c->tune.sort_period)
-            if ((e = do_sort(c, 0, s))) break;
-    }
+    const int64_t n = p.kind == PIECE_HEAD ? 0 : (p.kind == PIECE_TAIL ? 1 : p.steps);
+    c->step_off = 0;
+    if (p.kind == PIECE_HEAD) e = head_step(c, s);
+    if (p.kind == PIECE_TAIL) e = tail_step(c, s);
+    if (p.kind == PIECE_MIDDLE || p.kind == PIECE_WHOLE)
+        for (int64_t k = 0; k < n && !e; ++k) {
+            c->step_off = k;
+            e = p.kind == PIECE_MIDDLE ? middle_step(c, s) : unfused_step(c, s);
+        }
+    // the pipelined step has just binned for the next collision
+    if (!e && p.sort) e = do_sort(c, 0, s, p.kind == PIECE_MIDDLE);
+    c->step_off = 0;
+    if (!e && n) e = k_advance(c, s, n);
     if (!e && !c->profiling) {
         cudaError_t ce = cudaGetLastError();
         if (ce != cudaSuccess) return fail(c, MPCD_ERR_CUDA, "kernel launch: %s", cudaGetErrorString(ce));
@@ -670,50 +742,70 @@ int run_steps_unfused(mpcd_ctx *c, int64_t n, cudaStream_t s)
     return e;
 }
 
-// whole steps, software-pipelined: the solvent pass of step k collides (k),
-// streams and bins for step k+1; beside it, on a second stream, run the site
-// POST coupling of step k and the body step and site PRE coupling of step k+1
-// (they need step k's cell parameters and impulse, not its solvent pass; both
-// branches add to the cleared cell sums of step k+1 with integer atomics, so
-// the order between them changes no result).  The branches join before the
-// cell parameters of step k+1.
-int run_steps(mpcd_ctx *c, int64_t n, cudaStream_t s)
+// The pieces of n whole steps: a head, n - 1 middle steps and a tail (n whole
+// steps for the unpipelined variants), with a re-sort wherever the count since
+// the last one reaches the period.  `recorded`: cut so that few different
+// pieces serve every n and every phase of the re-sorts - a whole period ending
+// in its re-sort, one step with a re-sort, and powers of two without.
+// (A graph per step count and phase was recorded anew in nearly every call: the
+// phase moves by n - 1 steps from call to call.  At 5000 particles that was
+// 4.2 of the 9.5 ms of a 100-step call.)
+std::vector<Piece> plan_steps(mpcd_ctx *c, int64_t n, bool recorded)
 {
-    if (n <= 0) return MPCD_OK;
-    if (c->prm.angular) return run_steps_unfused(c, n, s);
-    int e = k_solvent(c, SOLV_STREAM | SOLV_BIN, s);
-    if (!e) e = k_rnemd(c, s, 0, 1);
-    if (!e) e = k_bodies(c, s);
-    if (!e) e = k_pre(c, s);
-    for (int64_t k = 0; k < n && !e; ++k) {
-        if ((e = k_params(c, s))) break;
-        if (k == n - 1) {
-            if ((e = k_post(c, s))) break;
-            if ((e = k_vacf(c, s))) break;
-            if ((e = k_solvent(c, SOLV_COLLIDE, s))) break;
+    constexpr int64_t MOST = 32;   // steps of a recorded piece without a re-sort
+    std::vector<Piece> out;
+    const bool fused = !c->prm.angular, sorts = c->prm.sort_period >= 0;
+    const int kind = fused ? PIECE_MIDDLE : PIECE_WHOLE;
+    const int64_t period = c->tune.sort_period;
+    if (fused) out.push_back(Piece{PIECE_HEAD, 0, false});
+    for (int64_t left = fused ? n - 1 : n; left > 0;) {
+        const int64_t due = sorts ? std::max<int64_t>(1, period - c->since_sort) : left + 1;
+        const int64_t m = std::min(left, due);
+        const bool sort = m == due;
+        if (!recorded || (sort && m == period && period <= 2 * MOST)) {
+            out.push_back(Piece{kind, m, sort});
         } else {
-            CK(c, cudaEventRecord(c->side_ev[0], s));
-            CK(c, cudaStreamWaitEvent(c->side, c->side_ev[0], 0));
-            // the transfer is added by the body step, unless it is sampled in between
-            const bool apart = c->vacf.n_lags > 0;
-            if ((e = k_post(c, c->side, apart))) break;
-            if ((e = k_vacf(c, c->side))) break;
-            if ((e = k_bodies(c, c->side, !apart))) break;
-            if ((e = k_pre(c, c->side, 1))) break;   // step k+1, before the counter advances
-            CK(c, cudaEventRecord(c->side_ev[1], c->side));
-            if ((e = k_solvent(c, SOLV_COLLIDE | SOLV_STREAM | SOLV_BIN, s))) break;
-            if ((e = k_rnemd(c, s, 1, 1))) break;   // before the collision of step k+1
-            CK(c, cudaStreamWaitEvent(s, c->side_ev[1], 0));
-            if (c->prm.sort_period >= 0 && ++c->since_sort >= c->tune.sort_period)
-                if ((e = do_sort(c, 0, s, true))) break;
+            int64_t plain = m - (sort ? 1 : 0);
+            for (int64_t b = MOST; b >= 1; b /= 2)
+                for (; plain >= b; plain -= b) out.push_back(Piece{kind, b, false});
+            if (sort) out.push_back(Piece{kind, 1, true});
         }
-        if ((e = k_advance(c, s))) break;
+        c->since_sort = sort ? 0 : c->since_sort + m;
+        left -= m;
     }
-    if (!e && !c->profiling) {
-        cudaError_t ce = cudaGetLastError();
-        if (ce != cudaSuccess) return fail(c, MPCD_ERR_CUDA, "kernel launch: %s", cudaGetErrorString(ce));
+    if (fused) out.push_back(Piece{PIECE_TAIL, 0, false});
+    return out;
+}
+
+// launch a piece as a CUDA graph, recording it first if it is new
+int replay_piece(mpcd_ctx *c, const Piece &p, cudaStream_t s)
+{
+    const auto key = std::make_tuple(p.kind, p.steps, p.sort, c->cur);
+    auto it = c->graphs.find(key);
+    if (it == c->graphs.end()) {
+        const int cur0 = c->cur;
+        const int64_t since0 = c->since_sort;
+        CK(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
+        int e = enqueue_piece(c, p, c->cap_stream);
+        cudaGraph_t g = nullptr;
+        cudaError_t ce = cudaStreamEndCapture(c->cap_stream, &g);
+        GraphEntry ge{};
+        ge.cur_end = c->cur;
+        c->cur = cur0;
+        c->since_sort = since0;
+        if (e) {
+            if (g) cudaGraphDestroy(g);
+            return e;
+        }
+        if (ce != cudaSuccess) return fail(c, MPCD_ERR_CUDA, "graph capture: %s", cudaGetErrorString(ce));
+        ce = cudaGraphInstantiate(&ge.exec, g, 0);
+        cudaGraphDestroy(g);
+        if (ce != cudaSuccess) return fail(c, MPCD_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(ce));
+        it = c->graphs.emplace(key, ge).first;
     }
-    return e;
+    CK(c, cudaGraphLaunch(it->second.exec, s));
+    c->cur = it->second.cur_end;
+    return MPCD_OK;
 }
 
 int check_device_error(mpcd_ctx *c, cudaStream_t s)
@@ -1138,7 +1230,6 @@ int mpcd_set_state(mpcd_ctx *c, const mpcd_host_state *h, void *stream)
         for (int k = 0; k < 3; ++k) b.Lm[k] = h->Lm[3 * i + k];
     }
     const size_t n3 = (size_t)c->Ns * 3;
-    clear_graphs(c);
     char *stg = (char *)c->staging;
     c->cur = 0;
     StepArgs a = make_args(c);
@@ -1274,7 +1365,8 @@ int mpcd_couple(mpcd_ctx *c, int32_t phase, void *stream)
     cudaStream_t s = (cudaStream_t)stream;
     int e = phase == MPCD_PRE ? k_pre(c, s) : k_post(c, s);
     if (!e && phase == MPCD_POST) e = k_vacf(c, s);
-    if (!e && phase == MPCD_POST) e = k_advance(c, s);
+    if (!e && phase == MPCD_POST) e = k_advance(c, s, 1);
+    if (!e && phase == MPCD_POST) count_steps(c, 1);
     if (!e) CK(c, cudaGetLastError());
     return e;
 }
@@ -1297,38 +1389,14 @@ int mpcd_step(mpcd_ctx *c, int64_t nsteps, void *stream)
     if (nsteps == 0) return MPCD_OK;
     CK(c, cudaSetDevice(c->device));
     cudaStream_t s = (cudaStream_t)stream;
-    if (c->profiling || nsteps < 2) return run_steps(c, nsteps, s);
-    auto key = std::make_tuple(nsteps, c->cur, c->since_sort);
-    auto it = c->graphs.find(key);
-    if (it == c->graphs.end()) {
-        const int cur0 = c->cur;
-        const int64_t since0 = c->since_sort, step0 = c->step, key0 = c->last_key;
-        CK(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-        int e = run_steps(c, nsteps, c->cap_stream);
-        cudaGraph_t g = nullptr;
-        cudaError_t ce = cudaStreamEndCapture(c->cap_stream, &g);
-        if (e) {
-            if (g) cudaGraphDestroy(g);
-            return e;
-        }
-        if (ce != cudaSuccess) return fail(c, MPCD_ERR_CUDA, "graph capture: %s", cudaGetErrorString(ce));
-        GraphEntry ge{};
-        ce = cudaGraphInstantiate(&ge.exec, g, 0);
-        cudaGraphDestroy(g);
-        if (ce != cudaSuccess) return fail(c, MPCD_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(ce));
-        ge.cur_end = c->cur;
-        ge.since_end = c->since_sort;
-        c->cur = cur0;
-        c->since_sort = since0;
-        c->step = step0;
-        c->last_key = key0;
-        it = c->graphs.emplace(key, ge).first;
+    const bool recorded = !c->profiling && nsteps > 1;
+    for (const Piece &p : plan_steps(c, nsteps, recorded)) {
+        const int64_t since = c->since_sort;   // the count after the last piece
+        const int e = recorded ? replay_piece(c, p, s) : enqueue_piece(c, p, s);
+        if (e) return e;
+        c->since_sort = since;
     }
-    CK(c, cudaGraphLaunch(it->second.exec, s));
-    c->cur = it->second.cur_end;
-    c->since_sort = it->second.since_end;
-    c->last_key = c->step + nsteps - 1;
-    c->step += nsteps;
+    count_steps(c, nsteps);
     return MPCD_OK;
 }
 
@@ -1662,7 +1730,8 @@ int mpcd_apply_impulse(mpcd_ctx *c, const double *dPL, void *stream)
         launch_body_apply(a, c->d_dpl, s);
     }
     int e = k_vacf(c, s);
-    if (!e) e = k_advance(c, s);
+    if (!e) e = k_advance(c, s, 1);
+    if (!e) count_steps(c, 1);
     if (!e) CK(c, cudaGetLastError());
     return e;
 }

@@ -136,8 +136,7 @@ struct StepArgs {
     float ahf[3];                   // the same rounded to float (P32)
     double fext[3];                 // constant force on every body at its centre of mass
     const int64_t *d_step;          // completed steps (device)
-    int32_t step_offset;            // added to *d_step by the site PRE pass (1 when it runs
-                                    // for the next step before the counter advances)
+    int32_t step_offset;            // the step a launch works on is *d_step + step_offset
     int *d_err;
     int *tile_ctr;                  // tile counter of the staged solvent pass (null: round robin)
     // slab of a decomposed box: only the sites with z in [site_zlo, site_zhi)
@@ -148,6 +147,11 @@ struct StepArgs {
     const void *ang_params;         // [n_cells] AngParams records
     int4 *ang_shift;                // [n_rep] grid shift of the current collision
 };
+
+// The device counter holds the completed steps when a sequence of steps was
+// enqueued; each launch carries its distance from there, so the counter
+// advances once per sequence and no step waits for a launch of its own.
+__device__ __forceinline__ int64_t current_step(const StepArgs &a) { return *a.d_step + a.step_offset; }
 
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11), GPU/host implementation.
@@ -511,7 +515,7 @@ void launch_body_md(const StepArgs &a, bool impulse, cudaStream_t s);
 void launch_body_force(const StepArgs &a, int kick, cudaStream_t s);
 void launch_sites_pre(const StepArgs &a, int max_sites, cudaStream_t s);
 void launch_sites_post(const StepArgs &a, int max_sites, cudaStream_t s);
-void launch_advance_step(const StepArgs &a, cudaStream_t s);
+void launch_advance_step(const StepArgs &a, int64_t n, cudaStream_t s);
 void launch_body_diag(const StepArgs &a, double *acc, cudaStream_t s);
 void launch_body_impulse(const StepArgs &a, cudaStream_t s);
 cudaError_t configure_body_kernels(int max_sites, int precision);
