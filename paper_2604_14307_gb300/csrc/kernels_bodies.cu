@@ -34,6 +34,46 @@
 
 namespace mpcd {
 
+// The kernels of the body chain (POST, body step, forces, PRE) follow one
+// another on one stream and are short: each may start while the one before it
+// still runs (programmatic dependent launch), and does up to chain_wait() what
+// needs nothing of it - for PRE the thermal draws of all sites.  A kernel lets
+// the next one start with chain_next(); the next one's chain_wait() returns
+// when all of it has completed, and since every kernel of the chain waits,
+// when everything before it has.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+static void launch(void (*kernel)(P...), bool chained, unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                   A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = chained ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);   // the caller reads the launch status
+}
+// Not beside the passes that already fill what an early kernel would take: the
+// MPCD-AT solvent pass (issue slots, registers: 221 bodies 59.3 us per step,
+// 62.6 chained) and the FP64 forms (FP64 pipes: 113 bodies 310 and 319).  FP32
+// SRD gains the launch gaps and the draws: one body 30.1 -> 27.5, 191 bodies
+// unpipelined 310 -> 302, 453 bodies 102 -> 99-102.
+static bool chain_pays(const StepArgs &a) { return a.precision == 1 && a.rule == 0; }
+
+template <typename... P, typename... A>
+static void launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                           const StepArgs &a, A... args)
+{
+    launch(kernel, chain_pays(a), grid, block, smem, s, a, args...);
+}
+
 // a slab of a decomposed box owns the sites whose stored z lies in its range
 // (bounds are integers: the comparison is exact in either precision)
 template <typename Real>
@@ -223,8 +263,14 @@ __global__ void __launch_bounds__(64) k_body_md(StepArgs a)
     const DevReplica &r = a.reps[o->rep];
     const double dt = a.dt;
     int bad = 0;
+    chain_next();
+    if (!IMPULSE) chain_wait();
+    // with IMPULSE the pass before is POST, which writes only the partial sums
     double q = o->q[c], P = o->P[k], L = o->Lm[k], R = o->R[k];
+    LaneRot Q = lane_rot(q, c);
+    const double kickT = lane_torque_kick(q, Q, o->T[k], 0.5 * dt, c);
     if (IMPULSE) {
+        chain_wait();
         const Real *in = reinterpret_cast<const Real *>(a.partial) + (int64_t)i * SITE_WARPS * 6;
         double sP = 0.0, sL = 0.0;
         for (int w = 0; w < SITE_WARPS; ++w) {
@@ -234,10 +280,9 @@ __global__ void __launch_bounds__(64) k_body_md(StepArgs a)
         P += sP;
         L += sL;
     }
-    LaneRot Q = lane_rot(q, c);
     double p = lane_L_to_p(q, Q, L, c);
     P += 0.5 * dt * o->F[k];
-    p += lane_torque_kick(q, Q, o->T[k], 0.5 * dt, c);
+    p += kickT;
     const double d = dt * div_by(P, sh.M, sh.rM);
     const double D = o->D[k] + d;
     R = wrapd(R + d, (double)r.L[k], bad);
@@ -292,11 +337,11 @@ static void body_md(const StepArgs &a, bool impulse, cudaStream_t s)
 {
     const unsigned grid = (unsigned)((a.n_bodies + 15) / 16);   // 64 threads, four lanes per body
     if (a.lone_bodies) {
-        if (impulse) k_body_md<Real, true, true><<<grid, 64, 0, s>>>(a);
-        else k_body_md<Real, false, true><<<grid, 64, 0, s>>>(a);
+        if (impulse) launch_chained(k_body_md<Real, true, true>, grid, 64, 0, s, a);
+        else launch_chained(k_body_md<Real, false, true>, grid, 64, 0, s, a);
     } else {
-        if (impulse) k_body_md<Real, true, false><<<grid, 64, 0, s>>>(a);
-        else k_body_md<Real, false, false><<<grid, 64, 0, s>>>(a);
+        if (impulse) launch_chained(k_body_md<Real, true, false>, grid, 64, 0, s, a);
+        else launch_chained(k_body_md<Real, false, false>, grid, 64, 0, s, a);
     }
 }
 
@@ -319,6 +364,8 @@ __global__ void __launch_bounds__(128) k_body_centres(StepArgs a)
     if (i >= a.n_bodies) return;
     const DevBody &b = a.bodies[i];
     const DevShape &sh = a.shapes[b.shape];
+    chain_next();
+    chain_wait();
     double Q[9];
     rotmat(b.q, Q);
     for (int c = threadIdx.x & 31; c < sh.n_cent; c += 32) {
@@ -386,6 +433,8 @@ __device__ __forceinline__ bool may_interact(const StepArgs &a, const float4 &pi
 // candidate neighbours of each body within the bounding spheres + cutoff + skin
 __global__ void k_nlist_build(StepArgs a)
 {
+    chain_next();
+    chain_wait();
     if (!*a.nl_dirty) return;
     const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
@@ -431,6 +480,8 @@ __global__ void __launch_bounds__(128) k_body_force(StepArgs a, int kick)
     const DevBody &bi = a.bodies[i];
     const DevShape &si = a.shapes[bi.shape];
     const DevReplica r = a.reps[bi.rep];
+    chain_wait();
+    chain_next();
     const float4 pi = a.bpos[i];
     const float cut = (float)(0.5 * (si.wca_d + a.max_wca_d) - 1.0 + 1.122462048309373);
     int n;
@@ -535,6 +586,8 @@ __global__ void __launch_bounds__(32 * WARP_BODIES) k_body_force_warp(StepArgs a
     const DevBody &bi = a.bodies[i];
     const DevShape &si = a.shapes[bi.shape];
     const DevReplica r = a.reps[bi.rep];
+    chain_wait();
+    chain_next();
     double F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
     auto pair = [&](const Real (&dR)[3], const DevBody &bj, const DevShape &sj, int ca, int cc) {
         Real ci[3], cj[3], f[3];
@@ -601,20 +654,20 @@ void launch_body_force(const StepArgs &a, int kick, cudaStream_t s)
     if (kick && a.lone_bodies) return;   // finished by k_body_md
     const unsigned warps = (unsigned)((a.n_bodies + WARP_BODIES - 1) / WARP_BODIES);
     if (!kick) k_body_pos<<<(a.n_bodies + 127) / 128, 128, 0, s>>>(a);
-    if (!kick || a.max_cent > 2) k_body_centres<<<warps, 32 * WARP_BODIES, 0, s>>>(a);
+    if (!kick || a.max_cent > 2) launch_chained(k_body_centres, warps, 32 * WARP_BODIES, 0, s, a);
     if (a.max_cent <= 2) {   // spheres, dumbbells: eight lanes per body
         const unsigned grid = (unsigned)((a.n_bodies + 15) / 16);
         if (a.precision == 1) {
-            if (a.max_cent <= 1) k_body_force<float, 1><<<grid, 128, 0, s>>>(a, kick);
-            else k_body_force<float, 2><<<grid, 128, 0, s>>>(a, kick);
+            if (a.max_cent <= 1) launch_chained(k_body_force<float, 1>, grid, 128, 0, s, a, kick);
+            else launch_chained(k_body_force<float, 2>, grid, 128, 0, s, a, kick);
         } else {
-            if (a.max_cent <= 1) k_body_force<double, 1><<<grid, 128, 0, s>>>(a, kick);
-            else k_body_force<double, 2><<<grid, 128, 0, s>>>(a, kick);
+            if (a.max_cent <= 1) launch_chained(k_body_force<double, 1>, grid, 128, 0, s, a, kick);
+            else launch_chained(k_body_force<double, 2>, grid, 128, 0, s, a, kick);
         }
     } else {                 // many centres: one warp per body
-        k_nlist_build<<<warps, 32 * WARP_BODIES, 0, s>>>(a);
-        if (a.precision == 1) k_body_force_warp<float><<<warps, 32 * WARP_BODIES, 0, s>>>(a, kick);
-        else k_body_force_warp<double><<<warps, 32 * WARP_BODIES, 0, s>>>(a, kick);
+        launch_chained(k_nlist_build, warps, 32 * WARP_BODIES, 0, s, a);
+        if (a.precision == 1) launch_chained(k_body_force_warp<float>, warps, 32 * WARP_BODIES, 0, s, a, kick);
+        else launch_chained(k_body_force_warp<double>, warps, 32 * WARP_BODIES, 0, s, a, kick);
     }
 }
 
@@ -669,7 +722,7 @@ __device__ __forceinline__ int cell_axis(double x, int S, int L)
 // Site geometry of the two forms.  P32: d = Qf bf in float (three products,
 // two adds), r = fl32(R) + d; P64: d = Q b in double.  Both wrapped into [0, L).
 template <typename Real> struct Pose {
-    Real Q[9], R[3], V[3], W[3];
+    Real Q[9], R[3];
 };
 __device__ __forceinline__ void site_geom(const StepArgs &a, int64_t t, const Pose<float> &P, const DevReplica &r,
                                           float d[3], float x[3], int &bad)
@@ -693,26 +746,72 @@ __device__ __forceinline__ const float *pose_ptr(const StepArgs &a, int b, float
 __device__ __forceinline__ const double *pose_ptr(const StepArgs &a, int b, double) { return a.pose64 + (int64_t)b * POSE_W; }
 
 template <typename Real> __device__ __forceinline__ Real site_mass(const StepArgs &a, int64_t t);
-template <> __device__ __forceinline__ float site_mass<float>(const StepArgs &a, int64_t t) { return a.tmf[t]; }
+template <> __device__ __forceinline__ float site_mass<float>(const StepArgs &a, int64_t) { return a.m_site_f; }
 template <> __device__ __forceinline__ double site_mass<double>(const StepArgs &a, int64_t t) { return a.tm[t]; }
+// sqrt(kT / m) of a site, formed once on the host (both operations round
+// correctly there and here; per site they cost 23 FP64 instructions)
+template <typename Real> __device__ __forceinline__ Real site_scale(const StepArgs &a, int64_t t);
+template <> __device__ __forceinline__ float site_scale<float>(const StepArgs &a, int64_t) { return a.site_sc_f; }
+template <> __device__ __forceinline__ double site_scale<double>(const StepArgs &a, int64_t t) { return a.tsc[t]; }
+template <typename Real> __device__ __forceinline__ Real cos_alpha(const StepArgs &a);
+template <> __device__ __forceinline__ float cos_alpha<float>(const StepArgs &a) { return a.cos_af; }
+template <> __device__ __forceinline__ double cos_alpha<double>(const StepArgs &a) { return a.cos_a; }
+template <typename Real> __device__ __forceinline__ Real sin_alpha(const StepArgs &a);
+template <> __device__ __forceinline__ float sin_alpha<float>(const StepArgs &a) { return a.sin_af; }
+template <> __device__ __forceinline__ double sin_alpha<double>(const StepArgs &a) { return a.sin_a; }
 
-// sum six per-thread values over the CTA in the form's precision (thread 0 gets it)
-template <typename Real>
-__device__ void block_sum6(Real (&v)[6], Real (*scratch)[6], Real *out)
+// The sites' sums in the form's precision have one order, whatever the CTA:
+// SITE_THREADS running sums, the j-th over the sites j, j + SITE_THREADS, ... in
+// turn, then a shuffle tree over each 32 of them, then the SITE_WARPS results.
+// With K lanes for each running sum (a CTA of K x SITE_THREADS threads) a lane
+// takes every K-th of its sites, and the terms of the K lanes are added in site
+// order on all of them, so K changes the latency but no bit of the result.
+// Lane layout: 32 / K sums per warp, lane = part * (32 / K) + sum.
+template <int K> struct SiteLane {
+    static constexpr int SUMS = 32 / K;
+    int j, part;
+    __device__ SiteLane()
+    {
+        const int lane = threadIdx.x & 31;
+        part = lane / SUMS;
+        j = (int)(threadIdx.x >> 5) * SUMS + lane % SUMS;
+    }
+    // the s-th site of this lane
+    __device__ int site(int s) const { return j + SITE_THREADS * (K * s + part); }
+    // acc += the parts' terms in site order (zero for a part past the last site)
+    template <typename Real> __device__ void add(Real (&acc)[6], const Real (&t)[6]) const
+    {
+#pragma unroll
+        for (int p = 0; p < K; ++p)
+#pragma unroll
+            for (int k = 0; k < 6; ++k)
+                acc[k] += K == 1 ? t[k] : __shfl_sync(0xffffffffu, t[k], p * SUMS + (int)(threadIdx.x & 31) % SUMS);
+    }
+};
+
+// the shuffle trees: out[w][k] = the sum of component k over the running sums
+// 32 w .. 32 w + 31 (shared memory; a CTA barrier must follow before it is read)
+template <typename Real, int K>
+__device__ __forceinline__ void site_trees(const SiteLane<K> &sl, Real (&acc)[6], Real (*out)[6])
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int k = 0; k < 6; ++k)
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    if (lane == 0)
-        for (int k = 0; k < 6; ++k) scratch[wid][k] = v[k];
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 6; ++k) {
-            Real s = 0;
-            for (int w = 0; w < SITE_WARPS; ++w) s += scratch[w][k];
-            out[k] = s;
+    if constexpr (K == 1) {
+        for (int k = 0; k < 6; ++k)
+            for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_down_sync(0xffffffffu, acc[k], o);
+        if (lane == 0)
+            for (int k = 0; k < 6; ++k) out[wid][k] = acc[k];
+    } else {
+        __shared__ Real sum[6][SITE_THREADS];
+        if (sl.part == 0)
+            for (int k = 0; k < 6; ++k) sum[k][sl.j] = acc[k];
+        __syncthreads();
+        for (int e = wid; e < 6 * SITE_WARPS; e += K * SITE_WARPS) {
+            const int k = e / SITE_WARPS, w = e % SITE_WARPS;
+            Real v = sum[k][32 * w + lane];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0) out[w][k] = v;
         }
-    __syncthreads();
+    }
 }
 
 // FP64 form: the sites' contributions to the double sum arrays
@@ -746,118 +845,161 @@ template <> __device__ __forceinline__ void load_cell<double>(const StepArgs &a,
 // body quantities already reduced to it).
 // FP32 site kernels are held to 64 registers (8 CTAs of 128 threads per SM)
 // so that they fit beside the solvent pass they overlap with.
+// The draws and cells of a thread's sites wait in registers (N of them) for the
+// sums they go into; in shared memory they left room for one CTA beside the
+// three of the staged solvent pass (N = 0: shapes of more sites, in shared
+// memory).  K lanes per running sum shorten the pass when there are few bodies.
 template <typename Real> struct SiteMinBlocks { static constexpr int n = sizeof(Real) == 4 ? 8 : 1; };
+template <typename Real, int K> struct SiteBlocks {
+    static constexpr int n = SiteMinBlocks<Real>::n >= K ? SiteMinBlocks<Real>::n / K : 1;
+};
 
-template <typename Real>
-__global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_sites_pre(StepArgs a)
+template <typename Real, int K, int N>
+__global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_sites_pre(StepArgs a)
 {
     extern __shared__ unsigned char smem_raw[];
-    Real *vt = reinterpret_cast<Real *>(smem_raw);          // [n_sites][3] thermal draws
-    __shared__ Real sPose[POSE_W], sVt[3], sWt[3], sred[6];
+    Real *svt = reinterpret_cast<Real *>(smem_raw);          // N = 0: [n_sites][3] thermal draws
+    __shared__ Real sPose[POSE_W], sdV[3], sdW[3];
     __shared__ Real scratch[SITE_WARPS][6];
     __shared__ int sS[3];
     const DevBody &B = a.bodies[blockIdx.x];
     const int shape = B.shape, rep = B.rep;
     const int64_t site_begin = B.site_begin;
-    const DevShape sh = a.shapes[shape];
+    const DevShape &sh = a.shapes[shape];
     const DevReplica r = a.reps[rep];
     const int64_t step = current_step(a);
+    const int n = sh.n_sites;
+    const SiteLane<K> sl;
+    const int passes = N > 0 ? N : (n + K * SITE_THREADS - 1) / (K * SITE_THREADS);
+    constexpr int NR = N > 0 ? N : 1;
+    Real vt[NR][3];
+    int cells[NR];
+    int bad = 0;
+    Real acc[6] = {0, 0, 0, 0, 0, 0};
+    auto draw_site = [&](int s) {   // the s-th site of the lane: thermal draw
+        const int j = sl.site(s);
+        Real w[3] = {0, 0, 0};
+        if (j < n && !a.naive) {
+            normals3(draw(r, step, (uint32_t)(r.site_id_base + (site_begin + j - r.site_begin)), TAG_SITE, 0u), w);
+            const Real sc = site_scale<Real>(a, sh.site_begin + j);
+            for (int k = 0; k < 3; ++k) w[k] = sc * w[k];
+        }
+        for (int k = 0; k < 3; ++k) {
+            if (N > 0) vt[N > 0 ? s : 0][k] = w[k];
+            else if (j < n) svt[3 * j + k] = w[k];
+        }
+    };
+    if constexpr (N > 0) {
+#pragma unroll
+        for (int s = 0; s < N; ++s) draw_site(s);
+    } else {
+        for (int s = 0; s < passes; ++s) draw_site(s);
+    }
+    if (threadIdx.x == 32) grid_shift(r, step, sS);
+    chain_wait();
     // the force pass of this pose is done: its neighbour lists are fresh
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.nl_dirty = 0;
     if (threadIdx.x < POSE_W) sPose[threadIdx.x] = pose_ptr(a, blockIdx.x, Real(0))[threadIdx.x];
-    if (threadIdx.x == 0) grid_shift(r, step, sS);
     __syncthreads();
     Pose<Real> P;
     for (int k = 0; k < 9; ++k) P.Q[k] = sPose[k];
-    for (int k = 0; k < 3; ++k) { P.R[k] = sPose[9 + k]; P.V[k] = sPose[12 + k]; P.W[k] = sPose[15 + k]; }
-    const Real kT = (Real)a.kT;
-    const int n = sh.n_sites;
-    int bad = 0;
-    Real acc[6] = {0, 0, 0, 0, 0, 0};
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const int64_t t = sh.site_begin + j, g = site_begin + j;
-        Real d[3], x[3];
-        site_geom(a, t, P, r, d, x, bad);
-        const int c = cell_axis(x[0], sS[0], r.L[0]) +
-                      r.L[0] * (cell_axis(x[1], sS[1], r.L[1]) + r.L[1] * cell_axis(x[2], sS[2], r.L[2]));
-        a.site_cell[g] = c;
-        if (!a.naive) {
-            const Real m = site_mass<Real>(a, t);
-            Real nn[3];
-            normals3(draw(r, step, (uint32_t)(r.site_id_base + (g - r.site_begin)), TAG_SITE, 0u), nn);
-            const Real sc = sqrt(kT / m);
-            const Real w[3] = {sc * nn[0], sc * nn[1], sc * nn[2]};
-            for (int k = 0; k < 3; ++k) vt[3 * j + k] = w[k];
-            const Real p[3] = {m * w[0], m * w[1], m * w[2]};
-            acc[0] += p[0]; acc[1] += p[1]; acc[2] += p[2];
-            acc[3] += d[1] * p[2] - d[2] * p[1];
-            acc[4] += d[2] * p[0] - d[0] * p[2];
-            acc[5] += d[0] * p[1] - d[1] * p[0];
+    for (int k = 0; k < 3; ++k) P.R[k] = sPose[9 + k];
+    auto sum_site = [&](int s) {    // cell, terms of the body's sums
+        const int j = sl.site(s);
+        Real t[6] = {0, 0, 0, 0, 0, 0};
+        int c = 0;
+        if (j < n) {
+            const int64_t ts = sh.site_begin + j, g = site_begin + j;
+            Real d[3], x[3];
+            site_geom(a, ts, P, r, d, x, bad);
+            c = cell_axis(x[0], sS[0], r.L[0]) +
+                r.L[0] * (cell_axis(x[1], sS[1], r.L[1]) + r.L[1] * cell_axis(x[2], sS[2], r.L[2]));
+            a.site_cell[g] = c;
+            if (!a.naive) {
+                const Real m = site_mass<Real>(a, ts);
+                for (int k = 0; k < 3; ++k) t[k] = m * (N > 0 ? vt[N > 0 ? s : 0][k] : svt[3 * j + k]);
+                t[3] = d[1] * t[2] - d[2] * t[1];
+                t[4] = d[2] * t[0] - d[0] * t[2];
+                t[5] = d[0] * t[1] - d[1] * t[0];
+            }
         }
+        cells[N > 0 ? s : 0] = c;
+        sl.add(acc, t);
+    };
+    if constexpr (N > 0) {
+#pragma unroll
+        for (int s = 0; s < N; ++s) sum_site(s);
+    } else {
+        for (int s = 0; s < passes; ++s) sum_site(s);
     }
-    block_sum6<Real>(acc, scratch, sred);
-    if (threadIdx.x == 0) {
-        if (a.naive) {
-            for (int k = 0; k < 3; ++k) { sVt[k] = 0; sWt[k] = 0; }
-        } else {
+    site_trees<Real, K>(sl, acc, scratch);
+    __syncthreads();
+    if (threadIdx.x < 32) {   // component k on lane k
+        const int k = threadIdx.x < 3 ? threadIdx.x : 0;
+        Real sp = 0, sL = 0, Vt = 0, Wt = 0;
+        for (int w = 0; w < SITE_WARPS; ++w) {
+            sp += scratch[w][k];
+            sL += scratch[w][3 + k];
+        }
+        if (!a.naive) {
             // V~ = sum m v~ / M, omega~ = Q Ihat^-1 Q^T L~
-            Real lb[3], wb[3];
-            for (int k = 0; k < 3; ++k) sVt[k] = sred[k] / (Real)sh.M;
-            for (int k = 0; k < 3; ++k)
-                lb[k] = (P.Q[k] * sred[3] + P.Q[3 + k] * sred[4]) + P.Q[6 + k] * sred[5];
-            for (int k = 0; k < 3; ++k) wb[k] = sh.Ihat[k] > 0.0 ? lb[k] / (Real)sh.Ihat[k] : Real(0);
-            for (int k = 0; k < 3; ++k)
-                sWt[k] = (P.Q[3 * k] * wb[0] + P.Q[3 * k + 1] * wb[1]) + P.Q[3 * k + 2] * wb[2];
+            Vt = sp / (Real)sh.M;
+            const Real L0 = __shfl_sync(0xffffffffu, sL, 0), L1 = __shfl_sync(0xffffffffu, sL, 1);
+            const Real L2 = __shfl_sync(0xffffffffu, sL, 2);
+            const Real lb = (sPose[k] * L0 + sPose[3 + k] * L1) + sPose[6 + k] * L2;
+            const Real wb = sh.Ihat[k] > 0.0 ? lb / (Real)sh.Ihat[k] : Real(0);
+            const Real w0 = __shfl_sync(0xffffffffu, wb, 0), w1 = __shfl_sync(0xffffffffu, wb, 1);
+            const Real w2 = __shfl_sync(0xffffffffu, wb, 2);
+            Wt = (sPose[3 * k] * w0 + sPose[3 * k + 1] * w1) + sPose[3 * k + 2] * w2;
+        }
+        if (threadIdx.x < 3) {
+            sdV[k] = sPose[12 + k] - Vt;
+            sdW[k] = sPose[15 + k] - Wt;
         }
     }
     __syncthreads();
-    const Real dV[3] = {P.V[0] - sVt[0], P.V[1] - sVt[1], P.V[2] - sVt[2]};
-    const Real dW[3] = {P.W[0] - sWt[0], P.W[1] - sWt[1], P.W[2] - sWt[2]};
+    const Real dV[3] = {sdV[0], sdV[1], sdV[2]}, dW[3] = {sdW[0], sdW[1], sdW[2]};
     Real *SV = reinterpret_cast<Real *>(a.site_v);
     const int64_t NS = a.n_sites;
-    // uniform trip count: every lane reaches the warp-wide record flush
-    for (int j0 = 0; j0 < n; j0 += blockDim.x) {
-        const int j = j0 + threadIdx.x;
-        const bool valid = j < n;
-        Real v[3] = {0, 0, 0}, xi[3] = {0, 0, 0}, m = Real(0);
-        int cell = 0;
-        bool own = true;   // a slab bins only the sites in its z range
-        if (valid) {
-            const int64_t t = sh.site_begin + j, g = site_begin + j;
-            Real d[3], x[3];
-            site_geom(a, t, P, r, d, x, bad);
-            own = site_owned(a, x[2]);
-            v[0] = dV[0] + (dW[1] * d[2] - dW[2] * d[1]);
-            v[1] = dV[1] + (dW[2] * d[0] - dW[0] * d[2]);
-            v[2] = dV[2] + (dW[0] * d[1] - dW[1] * d[0]);
-            if (!a.naive)
-                for (int k = 0; k < 3; ++k) v[k] += vt[3 * j + k];
-            for (int k = 0; k < 3; ++k) SV[k * NS + g] = v[k];
-            m = site_mass<Real>(a, t);
-            if (a.rule == 1) {
-                normals3(draw(r, step, (uint32_t)(r.site_id_base + (g - r.site_begin)), TAG_AT, 0u), xi);
-                const Real sc = sqrt(kT / m);
-                xi[0] *= sc; xi[1] *= sc; xi[2] *= sc;
-            }
-            cell = r.cell_base + a.site_cell[g];
+    auto bin_site = [&](int s) {    // Eq. 7 velocity, cell sums
+        const int j = sl.site(s);
+        if (j >= n) return;
+        const int64_t ts = sh.site_begin + j, g = site_begin + j;
+        Real d[3], x[3], v[3], xi[3] = {0, 0, 0};
+        site_geom(a, ts, P, r, d, x, bad);
+        v[0] = dV[0] + (dW[1] * d[2] - dW[2] * d[1]);
+        v[1] = dV[1] + (dW[2] * d[0] - dW[0] * d[2]);
+        v[2] = dV[2] + (dW[0] * d[1] - dW[1] * d[0]);
+        if (!a.naive)
+            for (int k = 0; k < 3; ++k) v[k] += N > 0 ? vt[N > 0 ? s : 0][k] : svt[3 * j + k];
+        for (int k = 0; k < 3; ++k) SV[k * NS + g] = v[k];
+        const Real m = site_mass<Real>(a, ts);
+        if (a.rule == 1) {
+            normals3(draw(r, step, (uint32_t)(r.site_id_base + (g - r.site_begin)), TAG_AT, 0u), xi);
+            const Real sc = site_scale<Real>(a, ts);
+            xi[0] *= sc; xi[1] *= sc; xi[2] *= sc;
         }
-        if (valid && own) {
-            if constexpr (sizeof(Real) == 4) {
-                long long w[MAX_WORDS32];
-                unsigned long long *S = reinterpret_cast<unsigned long long *>(a.sums);
-                if (a.rule == 0) {
-                    record_terms<0>(m, v[0], v[1], v[2], xi, true, w);
-                    for (int k = 0; k < Words32<0>::n; ++k)
-                        atomicAdd(S + k * a.n_cells + cell, (unsigned long long)w[k]);
-                } else {
-                    record_terms<1>(m, v[0], v[1], v[2], xi, true, w);
-                    for (int k = 0; k < Words32<1>::n; ++k)
-                        atomicAdd(S + k * a.n_cells + cell, (unsigned long long)w[k]);
-                }
+        const int cell = r.cell_base + (N > 0 ? cells[N > 0 ? s : 0] : a.site_cell[g]);
+        if (!site_owned(a, x[2])) return;   // a slab bins only the sites in its z range
+        if constexpr (sizeof(Real) == 4) {
+            long long w[MAX_WORDS32];
+            unsigned long long *S = reinterpret_cast<unsigned long long *>(a.sums);
+            if (a.rule == 0) {
+                record_terms<0>(m, v[0], v[1], v[2], xi, true, w);
+                for (int k = 0; k < Words32<0>::n; ++k) atomicAdd(S + k * a.n_cells + cell, (unsigned long long)w[k]);
             } else {
-                add_sums64(a, cell, m, v, xi);
+                record_terms<1>(m, v[0], v[1], v[2], xi, true, w);
+                for (int k = 0; k < Words32<1>::n; ++k) atomicAdd(S + k * a.n_cells + cell, (unsigned long long)w[k]);
             }
+        } else {
+            add_sums64(a, cell, m, v, xi);
         }
+    };
+    if constexpr (N > 0) {
+#pragma unroll
+        for (int s = 0; s < N; ++s) bin_site(s);
+    } else {
+        for (int s = 0; s < passes; ++s) bin_site(s);
     }
     if (bad) atomicOr(a.d_err, ERR_POSITION);
 }
@@ -867,12 +1009,12 @@ __global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_sites_
 // transferred to the body (Eqs. 3-4); k_body_impulse adds them in FP64.
 // the collision rule for one site: v -> vn with the parameters p of its cell
 template <typename Real>
-__device__ __forceinline__ void site_rule(const StepArgs &a, const DevReplica &r, int64_t step, int64_t g,
-                                          const Real (&v)[3], const Real (&p)[8], Real m, Real (&vn)[3])
+__device__ __forceinline__ void site_rule(const StepArgs &a, const DevReplica &r, int64_t step, int64_t g, int64_t t,
+                                          const Real (&v)[3], const Real (&p)[8], Real (&vn)[3])
 {
     vn[0] = v[0]; vn[1] = v[1]; vn[2] = v[2];
     if (p[3] >= Real(0)) {
-        const Real kT = (Real)a.kT, ca = (Real)a.cos_a, sa = (Real)a.sin_a;
+        const Real ca = cos_alpha<Real>(a), sa = sin_alpha<Real>(a);
         if (a.rule == 0) {
             const Real w[3] = {v[0] - p[0], v[1] - p[1], v[2] - p[2]};
             const Real nd = p[4] * w[0] + p[5] * w[1] + p[6] * w[2];
@@ -885,7 +1027,7 @@ __device__ __forceinline__ void site_rule(const StepArgs &a, const DevReplica &r
         } else {
             Real xi[3];
             normals3(draw(r, step, (uint32_t)(r.site_id_base + (g - r.site_begin)), TAG_AT, 0u), xi);
-            const Real sc = sqrt(kT / m);
+            const Real sc = site_scale<Real>(a, t);
             for (int k = 0; k < 3; ++k) vn[k] = p[k] + sc * xi[k] - p[4 + k];
         }
     }
@@ -902,55 +1044,66 @@ __device__ __forceinline__ void site_lattice_q(const Real (&x)[3], int4 S, int (
 
 // POST coupling; ANG: with the +a correction of the site's cell applied to the
 // rule's velocity before the momentum change is taken
-template <typename Real, bool ANG>
-__global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_sites_post(StepArgs a)
+template <typename Real, bool ANG, int K>
+__global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_sites_post(StepArgs a)
 {
     __shared__ Real sPose[POSE_W];
+    __shared__ Real scratch[SITE_WARPS][6];
     const DevBody &B = a.bodies[blockIdx.x];
     const int64_t site_begin = B.site_begin;
-    const DevShape sh = a.shapes[B.shape];
+    const DevShape &sh = a.shapes[B.shape];
     const DevReplica r = a.reps[B.rep];
     const int64_t step = current_step(a);
+    chain_next();
     if (threadIdx.x < POSE_W) sPose[threadIdx.x] = pose_ptr(a, blockIdx.x, Real(0))[threadIdx.x];
     __syncthreads();
     Pose<Real> P;
     for (int k = 0; k < 9; ++k) P.Q[k] = sPose[k];
-    for (int k = 0; k < 3; ++k) { P.R[k] = sPose[9 + k]; P.V[k] = 0; P.W[k] = 0; }
+    for (int k = 0; k < 3; ++k) P.R[k] = sPose[9 + k];
     const Real *SV = reinterpret_cast<const Real *>(a.site_v);
     const int64_t NS = a.n_sites;
+    const int n = sh.n_sites;
+    const SiteLane<K> sl;
     int bad = 0;
     Real acc[6] = {0, 0, 0, 0, 0, 0};
-    for (int j = threadIdx.x; j < sh.n_sites; j += blockDim.x) {
-        const int64_t t = sh.site_begin + j, g = site_begin + j;
-        Real d[3], x[3];
-        site_geom(a, t, P, r, d, x, bad);
-        const Real v[3] = {SV[g], SV[NS + g], SV[2 * NS + g]};
-        Real vn[3];
-        Real p[8];
-        const int64_t cell = (int64_t)r.cell_base + a.site_cell[g];
-        load_cell<Real>(a, cell, p);
-        const Real m = site_mass<Real>(a, t);
-        site_rule<Real>(a, r, step, g, v, p, m, vn);
-        if constexpr (ANG) {
-            const Real xs[3] = {x[0], x[1], x[2]};
-            int Q[3];
-            site_lattice_q(xs, a.ang_shift[B.rep], Q);
-            ang_correct(reinterpret_cast<const AngParams<Real> *>(a.ang_params)[cell], Q, vn);
+    // uniform trip count: the lanes of a running sum exchange their terms
+    for (int s = 0; K * SITE_THREADS * s < n; ++s) {
+        const int j = sl.site(s);
+        Real dt6[6] = {0, 0, 0, 0, 0, 0};
+        if (j < n) {
+            const int64_t t = sh.site_begin + j, g = site_begin + j;
+            const int64_t cell = (int64_t)r.cell_base + a.site_cell[g];
+            const Real v[3] = {SV[g], SV[NS + g], SV[2 * NS + g]};
+            Real d[3], x[3];
+            site_geom(a, t, P, r, d, x, bad);
+            Real vn[3];
+            Real p[8];
+            load_cell<Real>(a, cell, p);
+            const Real m = site_mass<Real>(a, t);
+            site_rule<Real>(a, r, step, g, t, v, p, vn);
+            if constexpr (ANG) {
+                const Real xs[3] = {x[0], x[1], x[2]};
+                int Q[3];
+                site_lattice_q(xs, a.ang_shift[B.rep], Q);
+                ang_correct(reinterpret_cast<const AngParams<Real> *>(a.ang_params)[cell], Q, vn);
+            }
+            if (site_owned(a, x[2])) {   // a slab transfers only its own sites
+                const Real dp[3] = {m * (vn[0] - v[0]), m * (vn[1] - v[1]), m * (vn[2] - v[2])};
+                dt6[0] = dp[0];
+                dt6[1] = dp[1];
+                dt6[2] = dp[2];
+                dt6[3] = d[1] * dp[2] - d[2] * dp[1];
+                dt6[4] = d[2] * dp[0] - d[0] * dp[2];
+                dt6[5] = d[0] * dp[1] - d[1] * dp[0];
+            }
         }
-        const bool own = site_owned(a, x[2]);   // a slab transfers only its own sites
-        const Real dp[3] = {own ? m * (vn[0] - v[0]) : Real(0), own ? m * (vn[1] - v[1]) : Real(0),
-                            own ? m * (vn[2] - v[2]) : Real(0)};
-        acc[0] += dp[0]; acc[1] += dp[1]; acc[2] += dp[2];
-        acc[3] += d[1] * dp[2] - d[2] * dp[1];
-        acc[4] += d[2] * dp[0] - d[0] * dp[2];
-        acc[5] += d[0] * dp[1] - d[1] * dp[0];
+        sl.add(acc, dt6);
     }
-    for (int k = 0; k < 6; ++k)
-        for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_down_sync(0xffffffffu, acc[k], o);
-    if ((threadIdx.x & 31) == 0) {
-        Real *out = reinterpret_cast<Real *>(a.partial) + ((int64_t)blockIdx.x * SITE_WARPS + (threadIdx.x >> 5)) * 6;
-        for (int k = 0; k < 6; ++k) out[k] = acc[k];
-    }
+    site_trees<Real, K>(sl, acc, scratch);
+    __syncthreads();
+    if (threadIdx.x < SITE_WARPS * 6)
+        (reinterpret_cast<Real *>(a.partial) + (int64_t)blockIdx.x * SITE_WARPS * 6)[threadIdx.x] =
+            scratch[threadIdx.x / 6][threadIdx.x % 6];
     if (bad) atomicOr(a.d_err, ERR_POSITION);
 }
 
@@ -971,34 +1124,72 @@ __global__ void k_body_impulse(StepArgs a)
     }
 }
 
+// Two lanes per running sum up to eight bodies per SM, one beyond: with few
+// bodies the passes are as long as one CTA takes (221 bodies of 642 sites: PRE
+// 18.5 -> 14.7, POST 13.8 -> 9.9 us; 1120 bodies of up to 2000: a step 552 ->
+// 542), with many the wider CTA finds less room beside the solvent pass (8952
+// bodies: a step 1766 us with one lane, 1783 with two).
+static int site_lanes(const StepArgs &a, int num_sms) { return a.n_bodies <= 8 * num_sms ? 2 : 1; }
+
+template <typename Real, int K>
+static void sites_pre(const StepArgs &a, int max_sites, bool chained, cudaStream_t s)
+{
+    constexpr int block = K * SITE_THREADS, FEW = 2 / K, MANY = 6 / K;   // 256 or 768 sites in registers
+    if (max_sites <= FEW * block)
+        launch(k_sites_pre<Real, K, FEW>, chained, a.n_bodies, block, 0, s, a);
+    else if (max_sites <= MANY * block)
+        launch(k_sites_pre<Real, K, MANY>, chained, a.n_bodies, block, 0, s, a);
+    else
+        launch(k_sites_pre<Real, K, 0>, chained, a.n_bodies, block, (size_t)max_sites * 3 * sizeof(Real), s, a);
+}
+
 cudaError_t configure_body_kernels(int max_sites, int precision)
 {
-    size_t bytes = (size_t)max_sites * 3 * (precision == 1 ? sizeof(float) : sizeof(double));
+    const int bytes = max_sites * 3 * (int)(precision == 1 ? sizeof(float) : sizeof(double));
     if (bytes <= 48 * 1024) return cudaSuccess;
-    if (precision == 1)
-        return cudaFuncSetAttribute(k_sites_pre<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    return cudaFuncSetAttribute(k_sites_pre<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    const auto opt_in = [&](auto *f) {
+        return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    cudaError_t e;
+    if (precision == 1) {
+        e = opt_in(k_sites_pre<float, 1, 0>);
+        return e != cudaSuccess ? e : opt_in(k_sites_pre<float, 2, 0>);
+    }
+    e = opt_in(k_sites_pre<double, 1, 0>);
+    return e != cudaSuccess ? e : opt_in(k_sites_pre<double, 2, 0>);
 }
 
-void launch_sites_pre(const StepArgs &a, int max_sites, cudaStream_t s)
+void launch_sites_pre(const StepArgs &a, int max_sites, int num_sms, bool chained, cudaStream_t s)
 {
     if (a.n_bodies == 0) return;
-    if (a.precision == 1)
-        k_sites_pre<float><<<a.n_bodies, SITE_THREADS, (size_t)max_sites * 3 * sizeof(float), s>>>(a);
-    else
-        k_sites_pre<double><<<a.n_bodies, SITE_THREADS, (size_t)max_sites * 3 * sizeof(double), s>>>(a);
-}
-
-void launch_sites_post(const StepArgs &a, int, cudaStream_t s)
-{
-    if (a.n_bodies == 0) return;
-    const bool ang = a.ang_params != nullptr;
+    const bool two = site_lanes(a, num_sms) == 2;
+    chained = chained && chain_pays(a);
     if (a.precision == 1) {
-        if (ang) k_sites_post<float, true><<<a.n_bodies, SITE_THREADS, 0, s>>>(a);
-        else k_sites_post<float, false><<<a.n_bodies, SITE_THREADS, 0, s>>>(a);
+        if (two) sites_pre<float, 2>(a, max_sites, chained, s);
+        else sites_pre<float, 1>(a, max_sites, chained, s);
     } else {
-        if (ang) k_sites_post<double, true><<<a.n_bodies, SITE_THREADS, 0, s>>>(a);
-        else k_sites_post<double, false><<<a.n_bodies, SITE_THREADS, 0, s>>>(a);
+        if (two) sites_pre<double, 2>(a, max_sites, chained, s);
+        else sites_pre<double, 1>(a, max_sites, chained, s);
+    }
+}
+
+template <typename Real, bool ANG>
+static void sites_post(const StepArgs &a, bool two, cudaStream_t s)
+{
+    if (two) k_sites_post<Real, ANG, 2><<<a.n_bodies, 2 * SITE_THREADS, 0, s>>>(a);
+    else k_sites_post<Real, ANG, 1><<<a.n_bodies, SITE_THREADS, 0, s>>>(a);
+}
+
+void launch_sites_post(const StepArgs &a, int num_sms, cudaStream_t s)
+{
+    if (a.n_bodies == 0) return;
+    const bool two = site_lanes(a, num_sms) == 2, ang = a.ang_params != nullptr;
+    if (a.precision == 1) {
+        if (ang) sites_post<float, true>(a, two, s);
+        else sites_post<float, false>(a, two, s);
+    } else {
+        if (ang) sites_post<double, true>(a, two, s);
+        else sites_post<double, false>(a, two, s);
     }
 }
 
@@ -1026,7 +1217,7 @@ __global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_ang_si
     __syncthreads();
     Pose<Real> P;
     for (int k = 0; k < 9; ++k) P.Q[k] = sPose[k];
-    for (int k = 0; k < 3; ++k) { P.R[k] = sPose[9 + k]; P.V[k] = 0; P.W[k] = 0; }
+    for (int k = 0; k < 3; ++k) P.R[k] = sPose[9 + k];
     const Real *SV = reinterpret_cast<const Real *>(a.site_v);
     const int64_t NS = a.n_sites;
     int bad = 0;
@@ -1041,7 +1232,7 @@ __global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_ang_si
         if (!PRE) {
             Real p[8];
             load_cell<Real>(a, cell, p);
-            site_rule<Real>(a, r, step, g, v, p, m, u);
+            site_rule<Real>(a, r, step, g, t, v, p, u);
         }
         const Real xs[3] = {x[0], x[1], x[2]};
         int Qi[3];

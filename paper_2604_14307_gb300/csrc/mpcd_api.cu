@@ -82,7 +82,8 @@ struct mpcd_ctx {
     int64_t n_cent_bodies = 0;                  // WCA centres over all bodies
     int max_cent = 0;                           // most centres of any shape
     bool lone_bodies = true;                    // no replica has more than one body
-    float *d_tbf = nullptr, *d_tmf = nullptr;
+    double *d_tsc = nullptr;
+    float *d_tbf = nullptr;
     void *sol[2][6] = {};
     uint32_t *tag[2] = {nullptr, nullptr};
     int cur = 0;
@@ -257,7 +258,8 @@ StepArgs make_args(const mpcd_ctx *c)
     a.tb = c->d_tb;
     a.tbf = c->d_tbf;
     a.tm = c->d_tm;
-    a.tmf = c->d_tmf;
+    a.tsc = c->d_tsc;
+    a.site_sc_f = c->m_site > 0.0 ? std::sqrt(a.kTf / a.m_site_f) : 0.0f;
     a.tcent = c->d_tcent;
     a.max_wca_d = c->max_wca_d;
     a.max_cent = c->max_cent;
@@ -495,12 +497,12 @@ int k_bodies(mpcd_ctx *c, cudaStream_t s, bool impulse = false)
     return timed(c, "body_force", 0, s, [&] { launch_body_force(a, 1, s); });
 }
 
-int k_pre(mpcd_ctx *c, cudaStream_t s, int step_offset = 0)
+int k_pre(mpcd_ctx *c, cudaStream_t s, bool chained, int step_offset = 0)
 {
     StepArgs a = make_args(c);
     a.step_offset += step_offset;
     double bytes = (double)c->Nsite * (3.0 * c->realsz + 4.0);
-    return timed(c, "sites_pre", bytes, s, [&] { launch_sites_pre(a, c->max_sites, s); });
+    return timed(c, "sites_pre", bytes, s, [&] { launch_sites_pre(a, c->max_sites, c->num_sms, chained, s); });
 }
 
 int k_params(mpcd_ctx *c, cudaStream_t s)
@@ -514,7 +516,7 @@ int k_post(mpcd_ctx *c, cudaStream_t s, bool impulse = true)
 {
     StepArgs a = make_args(c);
     double bytes = (double)c->Nsite * (3.0 * c->realsz + 4.0);
-    int e = timed(c, "sites_post", bytes, s, [&] { launch_sites_post(a, c->max_sites, s); });
+    int e = timed(c, "sites_post", bytes, s, [&] { launch_sites_post(a, c->num_sms, s); });
     if (e || !impulse) return e;
     return timed(c, "body_impulse", 0, s, [&] { launch_body_impulse(a, s); });
 }
@@ -667,7 +669,7 @@ int k_collide(mpcd_ctx *c, cudaStream_t s)
 int unfused_step(mpcd_ctx *c, cudaStream_t s)
 {
     int e = k_stream(c, s);
-    if (!e) e = k_pre(c, s);
+    if (!e) e = k_pre(c, s, true);
     if (!e) e = k_collide(c, s);
     if (!e) e = k_post(c, s);
     if (!e) e = k_vacf(c, s);
@@ -686,7 +688,7 @@ int head_step(mpcd_ctx *c, cudaStream_t s)     // before the first collision
     int e = k_solvent(c, SOLV_STREAM | SOLV_BIN, s);
     if (!e) e = k_rnemd(c, s, 0, 1);
     if (!e) e = k_bodies(c, s);
-    if (!e) e = k_pre(c, s);
+    if (!e) e = k_pre(c, s, true);
     return e;
 }
 
@@ -701,7 +703,7 @@ int middle_step(mpcd_ctx *c, cudaStream_t s)   // step k's collision up to step 
     e = k_post(c, c->side, apart);
     if (!e) e = k_vacf(c, c->side);
     if (!e) e = k_bodies(c, c->side, !apart);
-    if (!e) e = k_pre(c, c->side, 1);   // of step k+1
+    if (!e) e = k_pre(c, c->side, true, 1);   // of step k+1
     if (e) return e;
     CK(c, cudaEventRecord(c->side_ev[1], c->side));
     if ((e = k_solvent(c, SOLV_COLLIDE | SOLV_STREAM | SOLV_BIN, s))) return e;
@@ -1042,7 +1044,7 @@ int mpcd_create(const mpcd_params *params, int32_t n_shapes, const mpcd_shape_de
     ok &= (c->d_tb = (double *)A(std::max<size_t>(1, tb.size()) * 8)) != nullptr;
     ok &= (c->d_tbf = (float *)A(std::max<size_t>(1, tb.size()) * 4)) != nullptr;
     ok &= (c->d_tm = (double *)A(std::max<size_t>(1, tm.size()) * 8)) != nullptr;
-    ok &= (c->d_tmf = (float *)A(std::max<size_t>(1, tm.size()) * 4)) != nullptr;
+    ok &= (c->d_tsc = (double *)A(std::max<size_t>(1, tm.size()) * 8)) != nullptr;
     ok &= (c->d_tcent = (double *)A(std::max<size_t>(1, tcent.size()) * 8)) != nullptr;
     {
         int64_t nc = 0;
@@ -1074,7 +1076,9 @@ int mpcd_create(const mpcd_params *params, int32_t n_shapes, const mpcd_shape_de
         mpcd_destroy(c);
         return MPCD_ERR_OOM;
     }
-    std::vector<float> tbf(tb.begin(), tb.end()), tmf(tm.begin(), tm.end());
+    std::vector<float> tbf(tb.begin(), tb.end());
+    std::vector<double> tsc;
+    for (double m : tm) tsc.push_back(std::sqrt(p.kT / m));
     std::vector<DevBody> hb(std::max<int64_t>(1, c->B));
     {
         int64_t site = 0, cent = 0, bi = 0;
@@ -1102,7 +1106,7 @@ int mpcd_create(const mpcd_params *params, int32_t n_shapes, const mpcd_shape_de
     H2D(c->d_tb, tb.data(), tb.size() * 8);
     H2D(c->d_tbf, tbf.data(), tbf.size() * 4);
     H2D(c->d_tm, tm.data(), tm.size() * 8);
-    H2D(c->d_tmf, tmf.data(), tmf.size() * 4);
+    H2D(c->d_tsc, tsc.data(), tsc.size() * 8);
     H2D(c->d_tcent, tcent.data(), tcent.size() * 8);
     for (int b = 0; b < 2; ++b) {
         for (int k = 0; k < 6; ++k)
@@ -1363,7 +1367,7 @@ int mpcd_couple(mpcd_ctx *c, int32_t phase, void *stream)
     if (phase != MPCD_PRE && phase != MPCD_POST) return MPCD_ERR_ARG;
     CK(c, cudaSetDevice(c->device));
     cudaStream_t s = (cudaStream_t)stream;
-    int e = phase == MPCD_PRE ? k_pre(c, s) : k_post(c, s);
+    int e = phase == MPCD_PRE ? k_pre(c, s, false) : k_post(c, s);
     if (!e && phase == MPCD_POST) e = k_vacf(c, s);
     if (!e && phase == MPCD_POST) e = k_advance(c, s, 1);
     if (!e && phase == MPCD_POST) count_steps(c, 1);
@@ -1700,7 +1704,7 @@ int mpcd_couple_post_partial(mpcd_ctx *c, double *dPL, void *stream)
     if (c->B == 0) return MPCD_OK;
     StepArgs a = make_args(c);
     int e = timed(c, "sites_post", (double)c->Nsite * (3.0 * c->realsz + 4.0), s,
-                  [&] { launch_sites_post(a, c->max_sites, s); });
+                  [&] { launch_sites_post(a, c->num_sms, s); });
     if (e) return e;
     double *dpl = c->d_dpl;
     if (!dpl) {   // a context that is not a slab: allocated on first use

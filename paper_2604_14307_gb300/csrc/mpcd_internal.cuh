@@ -121,7 +121,8 @@ struct StepArgs {
     const double *tb;               // template offsets [sites][3]
     const float *tbf;               // the same rounded to float
     const double *tm;               // template masses
-    const float *tmf;
+    const double *tsc;              // sqrt(kT / m) of every template site
+    float site_sc_f;                // the same of the uniform site mass, formed in float (P32)
     const double *tcent;            // WCA centres [centres][3]
     double max_wca_d;               // largest centre diameter of any shape
     int32_t max_cent;               // most WCA centres of any shape
@@ -513,8 +514,10 @@ void launch_body_apply(const StepArgs &a, const double *dpl, cudaStream_t s);
 // impulse: with the transfer's sums (launch_body_impulse) added first
 void launch_body_md(const StepArgs &a, bool impulse, cudaStream_t s);
 void launch_body_force(const StepArgs &a, int kick, cudaStream_t s);
-void launch_sites_pre(const StepArgs &a, int max_sites, cudaStream_t s);
-void launch_sites_post(const StepArgs &a, int max_sites, cudaStream_t s);
+// chained: the launch before it on the stream is the body step's (it may start
+// before that has completed; it reads the step counter, which must be settled)
+void launch_sites_pre(const StepArgs &a, int max_sites, int num_sms, bool chained, cudaStream_t s);
+void launch_sites_post(const StepArgs &a, int num_sms, cudaStream_t s);
 void launch_advance_step(const StepArgs &a, int64_t n, cudaStream_t s);
 void launch_body_diag(const StepArgs &a, double *acc, cudaStream_t s);
 void launch_body_impulse(const StepArgs &a, cudaStream_t s);

@@ -95,3 +95,42 @@ def test_overflowing_candidate_lists(B, precision):
     q = I.random_quaternions(rng, len(R))
     prm = I.Params(precision=precision, seed=6)
     check(B, I.build_system(prm, [small, big], [(15, 15, 15)], 0.5, [[0] * 360 + [1]], "overflow", R_q=[(R, q)]), 5)
+
+
+@pytest.mark.parametrize("precision", [I.P64, I.P32])
+@pytest.mark.parametrize("sites", [3, 127, 128, 129, 256, 257, 640, 642, 768, 769, 1030])
+def test_site_passes_at_their_edges(B, sites, precision):
+    """One step with a shell of `sites` sites: the PRE and POST passes hold up to
+    256 or 768 sites in registers and the rest in shared memory, in sums of 128
+    lanes.  The bars are those of the parity tests (the site sums of the FP32 form
+    are taken in FP32 by the device alone)."""
+    rng = np.random.default_rng(sites)
+    d = rng.standard_normal((sites, 3))
+    b = 2.0 * d / np.linalg.norm(d, axis=1, keepdims=True)
+    b -= b.mean(0)
+    _, ax = np.linalg.eigh(b.T @ b)                   # principal axes
+    sh = I.Shape(b=b @ ax, m=np.full(sites, 5.0), centres=np.zeros((1, 3)), wca_d=4.0)
+    R = np.array([[3.0, 4.0, 5.0], [9.0, 10.0, 4.0]])
+    prm = I.Params(precision=precision, thermostat=1, seed=sites)
+    system = I.build_system(prm, [sh], [(13, 13, 13)], 5.0, [[0, 0]], "edges", R_q=[(R, I.random_quaternions(rng, 2))])
+    st = I.initial_state(system, 1)
+    osys = O.OracleSystem(system)
+    ost = O.OracleState(osys, st)
+    sim = B.Simulation(system)
+    sim.set_debug(True)
+    sim.set_state(st)
+    sim.stream()
+    O.stream(osys, ost)
+    sim.couple(B.MPCD_PRE)
+    sim.collide()
+    dbg = sim.debug_cells()
+    sim.couple(B.MPCD_POST)
+    tr = O.collide(osys, ost)
+    g = sim.get_state()
+    sim.close()
+    tol = TOL[precision]
+    assert np.array_equal(dbg["site_cell"], tr["cell_site"])
+    assert (np.abs(dbg["site_v"] - tr["site_v"]) / (np.abs(tr["site_v"]) + np.sqrt(1 / 5.0))).max() <= tol
+    sP, sL = np.sqrt(sh.m.sum()), np.sqrt(I.shape_inertia_diag(sh).max())
+    assert (np.abs(g.P - ost.P) / (np.abs(ost.P) + sP)).max() <= tol
+    assert (np.abs(g.Lm - ost.Lm) / (np.abs(ost.Lm) + sL)).max() <= tol
