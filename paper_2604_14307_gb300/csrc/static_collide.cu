@@ -1,10 +1,9 @@
 // mpcd_collide_solvent_static: one solvent collision (Sec. II.A) of a single
-// periodic box whose scratch - cell sums, collision parameters, the work-tile
-// tables, the step counter and the error word - lives in one statically
-// reserved device array of this translation unit, so the call allocates no
-// device memory.  The binning, parameter and collision kernels are the
-// library's own (kernels_solvent.cu); only their scratch pointers differ from
-// a context's.
+// periodic box whose scratch - cell sums, collision parameters, barrier counters
+// and the error word - lives in one statically reserved device array of this
+// translation unit, so the call allocates no device memory.  The collision is
+// one kernel (k_collide_box in kernels_solvent.cu) built from the parts of a
+// context's passes.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -19,22 +18,15 @@ namespace {
 
 constexpr int64_t MAX_CELLS = MPCD_STATIC_MAX_CELLS;
 constexpr int64_t MAX_SOLVENT = MPCD_STATIC_MAX_SOLVENT;
-constexpr int64_t TILE = 2048;                 // particles per work tile (a multiple of 4)
-constexpr int64_t CELL_TILE = 256;             // cells per parameter tile (one CTA each)
-constexpr int64_t MAX_TILES = MAX_SOLVENT / TILE;
-constexpr int64_t MAX_CTILES = MAX_CELLS / CELL_TILE;
-constexpr int MAX_WORDS = MAX_WORDS32;         // P32 cell words: 4 (SRD) or 6 (AT)
 
-// byte offsets inside the scratch array (each 256-byte aligned)
+// byte offsets inside the scratch array (each 256-byte aligned); the barrier
+// counters lie before the cell sums, so that one memset clears both
 constexpr size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
-constexpr size_t OFF_SUMS = 0;
-constexpr size_t OFF_PARAMS = OFF_SUMS + align256(sizeof(long long) * MAX_WORDS * MAX_CELLS);
-constexpr size_t OFF_TILES = OFF_PARAMS + align256(32 * MAX_CELLS);
-constexpr size_t OFF_CTILES = OFF_TILES + align256(sizeof(Tile) * MAX_TILES);
-constexpr size_t OFF_REP = OFF_CTILES + align256(sizeof(Tile) * MAX_CTILES);
-constexpr size_t OFF_STEP = OFF_REP + align256(sizeof(DevReplica));
-constexpr size_t OFF_ERR = OFF_STEP + 256;
-constexpr size_t SCRATCH_BYTES = OFF_ERR + 256;
+constexpr size_t OFF_ERR = 0;
+constexpr size_t OFF_COUNT = OFF_ERR + 256;
+constexpr size_t OFF_SUMS = OFF_COUNT + 256;
+constexpr size_t OFF_PARAMS = OFF_SUMS + align256(sizeof(long long) * MAX_WORDS32 * MAX_CELLS);
+constexpr size_t SCRATCH_BYTES = OFF_PARAMS + align256(32 * MAX_CELLS);
 
 }  // namespace
 
@@ -50,31 +42,6 @@ struct DeviceSetup {
 constexpr int MAX_DEVICES = 64;
 std::mutex g_setup_mutex;
 DeviceSetup g_setup[MAX_DEVICES];
-
-// Per-call initialisation of the scratch: replica record, regular tile
-// tables, step counter, cleared error word and zeroed cell sums (the binning
-// pass accumulates into them).
-__global__ void k_static_setup(unsigned char *base, DevReplica rep, int64_t n_solvent, int64_t n_cells,
-                               int n_words, int64_t step)
-{
-    long long *sums = reinterpret_cast<long long *>(base + OFF_SUMS);
-    Tile *tiles = reinterpret_cast<Tile *>(base + OFF_TILES);
-    Tile *ctiles = reinterpret_cast<Tile *>(base + OFF_CTILES);
-    const int64_t n_tiles = (n_solvent + TILE - 1) / TILE;
-    const int64_t n_ctiles = (n_cells + CELL_TILE - 1) / CELL_TILE;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (int64_t i = t0; i < (int64_t)n_words * n_cells; i += stride) sums[i] = 0;
-    for (int64_t t = t0; t < n_tiles; t += stride)
-        tiles[t] = Tile{0, 0, t * TILE, min((t + 1) * TILE, n_solvent)};
-    for (int64_t t = t0; t < n_ctiles; t += stride)
-        ctiles[t] = Tile{0, 0, t * CELL_TILE, min((t + 1) * CELL_TILE, n_cells)};
-    if (t0 == 0) {
-        *reinterpret_cast<DevReplica *>(base + OFF_REP) = rep;
-        *reinterpret_cast<int64_t *>(base + OFF_STEP) = step;
-        *reinterpret_cast<int *>(base + OFF_ERR) = 0;
-    }
-}
 
 int reject(char *msg, size_t len, const char *text)
 {
@@ -147,7 +114,6 @@ extern "C" int mpcd_collide_solvent_static(const mpcd_params *p, const int32_t L
         su = g_setup[dev];
     }
 
-    const int nw = p->rule == MPCD_SRD ? Words32<0>::n : Words32<1>::n;
     DevReplica rep{};
     rep.L[0] = L[0]; rep.L[1] = L[1]; rep.L[2] = L[2];
     rep.cell_base = 0;
@@ -159,13 +125,6 @@ extern "C" int mpcd_collide_solvent_static(const mpcd_params *p, const int32_t L
     rep.row_begin = 0;
     rep.key0 = (uint32_t)p->seed;
     rep.key1 = (uint32_t)(p->seed >> 32);   // replica 0: seed_hi ^ 0
-
-    cudaStream_t s = (cudaStream_t)stream;
-    const int64_t n_tiles = (n + TILE - 1) / TILE;
-    const int64_t n_ctiles = (cells + CELL_TILE - 1) / CELL_TILE;
-    const int64_t setup_work = std::max<int64_t>((int64_t)nw * cells, n_tiles);
-    const int setup_grid = (int)std::min<int64_t>((setup_work + 255) / 256, (int64_t)su.num_sms * 4);
-    k_static_setup<<<setup_grid, 256, 0, s>>>(su.base, rep, n, cells, nw, step);
 
     StepArgs a{};
     a.precision = MPCD_P32;
@@ -186,12 +145,6 @@ extern "C" int mpcd_collide_solvent_static(const mpcd_params *p, const int32_t L
     a.qm_solvent = (long long)std::llrint((double)a.m_solvent_f * 16777216.0);
     a.m_site_f = 0.0f;
     a.qm_site = 0;
-    a.reps = reinterpret_cast<const DevReplica *>(su.base + OFF_REP);
-    a.n_rep = 1;
-    a.tiles = reinterpret_cast<const Tile *>(su.base + OFF_TILES);
-    a.n_tiles = (int32_t)n_tiles;
-    a.ctiles = reinterpret_cast<const Tile *>(su.base + OFF_CTILES);
-    a.n_ctiles = (int32_t)n_ctiles;
     a.x = const_cast<float *>(x);
     a.y = const_cast<float *>(y);
     a.z = const_cast<float *>(z);
@@ -199,22 +152,16 @@ extern "C" int mpcd_collide_solvent_static(const mpcd_params *p, const int32_t L
     a.vy = vy;
     a.vz = vz;
     a.tag = const_cast<uint32_t *>(tag);
-    a.sums = su.base + OFF_SUMS;
     a.params = su.base + OFF_PARAMS;
-    a.dbg_sums = nullptr;
     a.n_cells = cells;
-    a.nw = nw;
-    a.d_step = reinterpret_cast<const int64_t *>(su.base + OFF_STEP);
-    a.d_err = reinterpret_cast<int *>(su.base + OFF_ERR);
-
-    // direct (unstaged) passes: bin at the step's shift, per-cell parameters,
-    // then the collision of every particle (the order of mpcd_collide)
-    const LaunchCfg cfg{256, (int)std::max<int64_t>(1, std::min<int64_t>(n_tiles, (int64_t)su.num_sms * 4)), 0,
-                        (int)TILE};
-    launch_solvent(a, SOLV_BIN, cfg, s);
-    launch_params(a, 0, s);
-    launch_solvent(a, SOLV_COLLIDE, cfg, s);
-    const cudaError_t e = cudaGetLastError();
+    BoxScratch sc{};
+    sc.err = reinterpret_cast<int *>(su.base + OFF_ERR);
+    sc.count = reinterpret_cast<unsigned *>(su.base + OFF_COUNT);
+    sc.quad = reinterpret_cast<long long *>(su.base + OFF_SUMS);
+    sc.pair = sc.quad + 4 * cells;
+    cudaError_t e = launch_collide_box(a, rep, n, step, sc, su.num_sms, (cudaStream_t)stream);
+    const cudaError_t last = cudaGetLastError();
+    if (e == cudaSuccess) e = last;
     if (e != cudaSuccess) {
         if (msg && msg_len) snprintf(msg, msg_len, "launch failed: %s", cudaGetErrorString(e));
         return MPCD_ERR_CUDA;
