@@ -48,7 +48,7 @@ namespace {
 // X = floor(x 2^20) of the binning rule, as in the plain passes (box edges
 // below 2048 cells keep it within int32)
 __device__ __forceinline__ int lattice_X(float x) { return __float2int_rd(x * 1048576.0f); }
-__device__ __forceinline__ int lattice_X(double x) { return __double2int_rd(x * 1048576.0); }
+__device__ __forceinline__ int lattice_X(double x) { return lattice_floor(x); }
 
 __device__ __forceinline__ int axis_cell(int X, int S, int L)
 {

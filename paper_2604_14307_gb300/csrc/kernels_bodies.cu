@@ -103,13 +103,6 @@ __device__ __forceinline__ void mtv(const double Q[9], const double x[3], double
     for (int a = 0; a < 3; ++a) o[a] = (Q[a] * x[0] + Q[3 + a] * x[1]) + Q[6 + a] * x[2];
 }
 
-__device__ __forceinline__ double wrapd(double y, double L, int &bad)
-{
-    if (y >= L) y = y - L;
-    else if (y < 0.0) { y = y + L; if (y >= L) y = 0.0; }
-    bad |= !(y >= 0.0 && y < L);
-    return y;
-}
 __device__ __forceinline__ float wrapf(float y, float L, int &bad)
 {
     if (y >= L) y = y - L;
@@ -134,17 +127,6 @@ __device__ __forceinline__ float lane4(float v, int c) { return __shfl_sync(0xff
 __device__ __forceinline__ double flip(double v, bool neg)   // -v if neg, exactly
 {
     return __hiloint2double(__double2hiint(v) ^ (neg ? 0x80000000 : 0), __double2loint(v));
-}
-
-// a / b with rb = RN(1 / b): Markstein's correction (IBM J. Res. Dev. 34, 111
-// (1990)) applied twice.  The first makes the quotient faithful, the second
-// rounds it correctly, so the result is that of the IEEE division (no overflow
-// or underflow in between), in 5 instructions of 64 cycles instead of about 11.
-__device__ __forceinline__ double div_by(double a, double b, double rb)
-{
-    double q = a * rb;
-    q = fma(fma(-b, q, a), rb, q);
-    return fma(fma(-b, q, a), rb, q);
 }
 
 // component c of the quaternion product (quat_mul); a, b: lane c's component
@@ -285,7 +267,7 @@ __global__ void __launch_bounds__(64) k_body_md(StepArgs a)
     p += kickT;
     const double d = dt * div_by(P, sh.M, sh.rM);
     const double D = o->D[k] + d;
-    R = wrapd(R + d, (double)r.L[k], bad);
+    R = wrap_box(R + d, (double)r.L[k], bad);
 #pragma unroll 1
     for (int e = 0; e < 5; ++e) {   // axes 3, 2, 1, 2, 3
         const int ax = e < 3 ? 3 - e : e - 1;
@@ -678,7 +660,6 @@ __device__ __forceinline__ float u01f(uint32_t x)
 {
     return __fmaf_rn(__uint2float_rn(x), 2.3283064365386962890625e-10f, 1.16415321826934814453125e-10f);
 }
-__device__ __forceinline__ double u01d(uint32_t x) { return ((double)x + 0.5) * 2.3283064365386962890625e-10; }
 // -2 ln u, accurate near u = 1 through the exact complement 1 - u
 __device__ __forceinline__ float neg2log(uint32_t x)
 {
@@ -696,11 +677,10 @@ __device__ __forceinline__ void normals3(uint4 w, float n[3])
 }
 __device__ __forceinline__ void normals3(uint4 w, double n[3])
 {
-    const double two_pi = 6.283185307179586476925286766559;
     double r1 = sqrt(-2.0 * log(u01d(w.x))), r2 = sqrt(-2.0 * log(u01d(w.z)));
     double s1, c1;
-    sincos(two_pi * u01d(w.y), &s1, &c1);
-    n[0] = r1 * c1; n[1] = r1 * s1; n[2] = r2 * cos(two_pi * u01d(w.w));
+    sincospi(2.0 * u01d(w.y), &s1, &c1);
+    n[0] = r1 * c1; n[1] = r1 * s1; n[2] = r2 * cospi(2.0 * u01d(w.w));
 }
 __device__ __forceinline__ int cell_axis(float x, int S, int L)
 {
@@ -712,7 +692,7 @@ __device__ __forceinline__ int cell_axis(float x, int S, int L)
 }
 __device__ __forceinline__ int cell_axis(double x, int S, int L)
 {
-    int c = (__double2int_rd(x * 1048576.0) - S) >> 20;
+    int c = (lattice_floor(x) - S) >> 20;
     c += (c < 0) ? L : 0;
     c -= (c >= L) ? L : 0;
     return ((unsigned)c < (unsigned)L) ? c : 0;   // only a non-finite position gets here; it is flagged
@@ -740,7 +720,7 @@ __device__ __forceinline__ void site_geom(const StepArgs &a, int64_t t, const Po
                                           double d[3], double x[3], int &bad)
 {
     mv(P.Q, a.tb + 3 * t, d);
-    for (int k = 0; k < 3; ++k) x[k] = wrapd(P.R[k] + d[k], (double)r.L[k], bad);
+    for (int k = 0; k < 3; ++k) x[k] = wrap_box(P.R[k] + d[k], (double)r.L[k], bad);
 }
 __device__ __forceinline__ const float *pose_ptr(const StepArgs &a, int b, float) { return a.pose32 + (int64_t)b * POSE_W; }
 __device__ __forceinline__ const double *pose_ptr(const StepArgs &a, int b, double) { return a.pose64 + (int64_t)b * POSE_W; }
@@ -872,8 +852,10 @@ __global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_si
     const SiteLane<K> sl;
     const int passes = N > 0 ? N : (n + K * SITE_THREADS - 1) / (K * SITE_THREADS);
     constexpr int NR = N > 0 ? N : 1;
-    Real vt[NR][3];
+    constexpr bool KEEP = sizeof(Real) == 8 && N > 0;   // FP64: the offsets too (formed again in FP32)
+    Real vt[NR][3], off[NR][3];
     int cells[NR];
+    bool own[NR];
     int bad = 0;
     Real acc[6] = {0, 0, 0, 0, 0, 0};
     auto draw_site = [&](int s) {   // the s-th site of the lane: thermal draw
@@ -915,6 +897,10 @@ __global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_si
             c = cell_axis(x[0], sS[0], r.L[0]) +
                 r.L[0] * (cell_axis(x[1], sS[1], r.L[1]) + r.L[1] * cell_axis(x[2], sS[2], r.L[2]));
             a.site_cell[g] = c;
+            if (KEEP) {
+                for (int k = 0; k < 3; ++k) off[N > 0 ? s : 0][k] = d[k];
+                own[N > 0 ? s : 0] = site_owned(a, x[2]);
+            }
             if (!a.naive) {
                 const Real m = site_mass<Real>(a, ts);
                 for (int k = 0; k < 3; ++k) t[k] = m * (N > 0 ? vt[N > 0 ? s : 0][k] : svt[3 * j + k]);
@@ -965,8 +951,16 @@ __global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_si
         const int j = sl.site(s);
         if (j >= n) return;
         const int64_t ts = sh.site_begin + j, g = site_begin + j;
-        Real d[3], x[3], v[3], xi[3] = {0, 0, 0};
-        site_geom(a, ts, P, r, d, x, bad);
+        Real d[3], v[3], xi[3] = {0, 0, 0};
+        bool mine;   // a slab bins only the sites in its z range
+        if (KEEP) {
+            for (int k = 0; k < 3; ++k) d[k] = off[N > 0 ? s : 0][k];
+            mine = own[N > 0 ? s : 0];
+        } else {
+            Real x[3];
+            site_geom(a, ts, P, r, d, x, bad);
+            mine = site_owned(a, x[2]);
+        }
         v[0] = dV[0] + (dW[1] * d[2] - dW[2] * d[1]);
         v[1] = dV[1] + (dW[2] * d[0] - dW[0] * d[2]);
         v[2] = dV[2] + (dW[0] * d[1] - dW[1] * d[0]);
@@ -980,7 +974,7 @@ __global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_si
             xi[0] *= sc; xi[1] *= sc; xi[2] *= sc;
         }
         const int cell = r.cell_base + (N > 0 ? cells[N > 0 ? s : 0] : a.site_cell[g]);
-        if (!site_owned(a, x[2])) return;   // a slab bins only the sites in its z range
+        if (!mine) return;
         if constexpr (sizeof(Real) == 4) {
             long long w[MAX_WORDS32];
             unsigned long long *S = reinterpret_cast<unsigned long long *>(a.sums);

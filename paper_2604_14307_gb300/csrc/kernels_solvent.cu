@@ -38,10 +38,6 @@ __device__ __forceinline__ float u01f(uint32_t x)
 {
     return __fmaf_rn(__uint2float_rn(x), 2.3283064365386962890625e-10f, 1.16415321826934814453125e-10f);
 }
-__device__ __forceinline__ double u01d(uint32_t x)
-{
-    return ((double)x + 0.5) * 2.3283064365386962890625e-10;     // (x + 1/2) 2^-32
-}
 
 // -2 ln u for u = (x + 1/2) 2^-32 with full relative precision also near u = 1,
 // where 1 - u = (~x + 1/2) 2^-32 is formed exactly from the integer complement
@@ -64,14 +60,13 @@ __device__ __forceinline__ void normals3(uint4 w, float n[3])
 }
 __device__ __forceinline__ void normals3(uint4 w, double n[3])
 {
-    const double two_pi = 6.283185307179586476925286766559;
     double r1 = sqrt(-2.0 * log(u01d(w.x)));
     double r2 = sqrt(-2.0 * log(u01d(w.z)));
     double s1, c1;
-    sincos(two_pi * u01d(w.y), &s1, &c1);
+    sincospi(2.0 * u01d(w.y), &s1, &c1);
     n[0] = r1 * c1;
     n[1] = r1 * s1;
-    n[2] = r2 * cos(two_pi * u01d(w.w));
+    n[2] = r2 * cospi(2.0 * u01d(w.w));
 }
 
 // binning rule: X = floor(x 2^20), cell = floor((X - S) / 2^20) mod L
@@ -85,7 +80,7 @@ __device__ __forceinline__ int cell_axis(float x, int S, int L)
 }
 __device__ __forceinline__ int cell_axis(double x, int S, int L)
 {
-    int c = (__double2int_rd(x * 1048576.0) - S) >> 20;
+    int c = (lattice_floor(x) - S) >> 20;
     c += (c < 0) ? L : 0;
     c -= (c >= L) ? L : 0;
     return ((unsigned)c < (unsigned)L) ? c : 0;   // only a non-finite position gets here; it is flagged
@@ -128,11 +123,7 @@ __device__ __forceinline__ float drift(float x, float v, float dt, float L, int 
 }
 __device__ __forceinline__ double drift(double x, double v, double dt, double L, int &bad)
 {
-    double y = __dadd_rn(x, __dmul_rn(v, dt));
-    if (y >= L) y = __dsub_rn(y, L);
-    else if (y < 0.0) { y = __dadd_rn(y, L); if (y >= L) y = 0.0; }
-    bad |= !(y >= 0.0 && y < L);
-    return y;
+    return wrap_box(__dadd_rn(x, __dmul_rn(v, dt)), L, bad);
 }
 // Streaming under a constant force (the solvent's share of the balancing
 // force of the sedimentation protocol): v += a dt/2, x += v dt, v += a dt/2,
@@ -1375,18 +1366,30 @@ __device__ float gamma_half_dof(const DevReplica &r, int64_t step, uint32_t lc, 
 }
 __device__ double gamma_half_dof(const DevReplica &r, int64_t step, uint32_t lc, int n_dof, double)
 {
-    int nE = n_dof / 2;
+    // one logarithm for up to 16 uniforms u = (2 x + 1) 2^-33: the product of
+    // the odd integers stays below 2^528, and a relative error of 15 roundings
+    // in it is as much in the sum as 16 rounded logarithms bring (34 FP64
+    // instructions each; a cell beside colloid sites takes about 30)
+    constexpr int MOST = 16;
+    const int nE = n_dof / 2;
     double g = 0.0;
-    uint4 w = make_uint4(0, 0, 0, 0);
-    for (int i = 0; i < nE; ++i) {
-        if ((i & 3) == 0) w = draw(r, step, lc, TAG_THERMO, (uint32_t)(i >> 2));
-        uint32_t x = (i & 3) == 0 ? w.x : (i & 3) == 1 ? w.y : (i & 3) == 2 ? w.z : w.w;
-        g += -log(u01d(x));
+    for (int i = 0; i < nE;) {
+        double prod = 1.0;
+        const int k = min(MOST, nE - i);
+        for (int e = 0; e < k; e += 4) {
+            const uint4 w = draw(r, step, lc, TAG_THERMO, (uint32_t)((i + e) >> 2));
+            prod *= odd_of(w.x);
+            if (e + 1 < k) prod *= odd_of(w.y);
+            if (e + 2 < k) prod *= odd_of(w.z);
+            if (e + 3 < k) prod *= odd_of(w.w);
+        }
+        g -= log(prod * __hiloint2double((1023 - 33 * k) << 20, 0));
+        i += k;
     }
-    if (n_dof & 1) {
-        w = draw(r, step, lc, TAG_THERMO_ODD, 0u);
-        double z = sqrt(-2.0 * log(u01d(w.x))) * cos(6.283185307179586476925286766559 * u01d(w.y));
-        g += 0.5 * z * z;
+    if (n_dof & 1) {   // z^2 / 2 = -ln u1 cos^2(2 pi u2)
+        const uint4 w = draw(r, step, lc, TAG_THERMO_ODD, 0u);
+        const double cs = cospi(2.0 * u01d(w.y));
+        g -= log(u01d(w.x)) * (cs * cs);
     }
     return g;
 }
@@ -1440,14 +1443,15 @@ __device__ double gamma_mt(const DevReplica &r, int64_t step, uint32_t lc, int n
         const uint4 w = draw(r, step, lc, TAG_THERMO_MT, k);
         const double rr = sqrt(-2.0 * log(u01d(w.x)));
         double sn, cs;
-        sincos(6.283185307179586476925286766559 * u01d(w.y), &sn, &cs);
+        sincospi(2.0 * u01d(w.y), &sn, &cs);
         const double xs[2] = {rr * cs, rr * sn};
         const uint32_t us[2] = {w.z, w.w};
         for (int j = 0; j < 2; ++j) {
             const double x = xs[j], t = 1.0 + c * x;
             if (t <= 0.0) continue;
-            const double v = t * t * t;
-            if (log(u01d(us[j])) < 0.5 * x * x + d - d * v + d * log(v)) return d * v;
+            const double v = t * t * t, x2 = x * x, u = u01d(us[j]);
+            if (u < 1.0 - 0.0331 * (x2 * x2)) return d * v;   // the squeeze, as in the FP32 form
+            if (log(u) < 0.5 * x * x + d - d * v + d * log(v)) return d * v;
         }
     }
     return d;
@@ -1639,7 +1643,8 @@ __global__ void __launch_bounds__(256) k_params(StepArgs a)
             }
             Real rec[8] = {0, 0, 0, Real(-1), 0, 0, 0, 0};
             if (n >= 2) {
-                Real u[3] = {p[0] / M, p[1] / M, p[2] / M};
+                const Real iM = Real(1) / M;
+                Real u[3] = {div_by(p[0], M, iM), div_by(p[1], M, iM), div_by(p[2], M, iM)};
                 rec[0] = u[0]; rec[1] = u[1]; rec[2] = u[2];
                 const uint32_t lc = (uint32_t)(c - r.cell_base);
                 if (RULE == 0) {
@@ -1650,13 +1655,13 @@ __global__ void __launch_bounds__(256) k_params(StepArgs a)
                         zz = (Real)(2.0 * u01d(wa.x) - 1.0);
                         rho = (Real)sqrt(1.0 - (double)zz * (double)zz);
                         double s_, c_;
-                        sincos(6.283185307179586476925286766559 * u01d(wa.y), &s_, &c_);
+                        sincospi(2.0 * u01d(wa.y), &s_, &c_);
                         sp = (Real)s_; cp = (Real)c_;
                     }
                     rec[4] = rho * cp; rec[5] = rho * sp; rec[6] = zz;
                     Real kappa = Real(1);
                     if (a.thermostat) {
-                        Real erel = Real(0.5) * (s2 - (p[0] * p[0] + p[1] * p[1] + p[2] * p[2]) / M);
+                        Real erel = Real(0.5) * (s2 - div_by(p[0] * p[0] + p[1] * p[1] + p[2] * p[2], M, iM));
                         Real g = a.thermostat == 2 ? gamma_mt(r, step, lc, 3 * (n - 1), Real(0))
                                                    : gamma_half_dof(r, step, lc, 3 * (n - 1), Real(0));
                         kappa = erel > Real(0) ? sqrt(kT * g / erel) : Real(1);
@@ -1664,7 +1669,7 @@ __global__ void __launch_bounds__(256) k_params(StepArgs a)
                     rec[3] = kappa;
                 } else {
                     rec[3] = Real(1);
-                    rec[4] = xi[0] / M; rec[5] = xi[1] / M; rec[6] = xi[2] / M;
+                    for (int k = 0; k < 3; ++k) rec[4 + k] = div_by(xi[k], M, iM);
                 }
             }
             if (sizeof(Real) == 4) {

@@ -435,29 +435,25 @@ bool staged_fits(const mpcd_ctx *c, int tile, int mode, int block)
 // cut the tiles short keep the ring.  Otherwise FP32 takes a ring per warp of
 // 128-particle tiles; MPCD-AT beside colloids with 384 threads, because 512 of
 // its 128 registers fill the SM and the site/body chain then waits for the
-// whole pass (0.6 M particles, 221 bodies: 144 and 65 us per step).  FP64 takes
-// the warp-specialised pass with the largest tile whose ring fits, else direct
-// loads.
+// whole pass (0.6 M particles, 221 bodies: 144 and 65 us per step).  FP64 keeps
+// its own pipe full in any form; a ring per warp in 256 threads leaves the most
+// room beside it (warp-specialised with 1024-particle tiles against it: 0.3 M
+// particles with 113 bodies 184 and 167 us per step, 10 M 1990 and 1737), MPCD-AT
+// with its 160 registers and more takes direct loads (540 and 328).
 void default_tuning(mpcd_ctx *c)
 {
     const int period = c->tune.sort_period;
     const bool p32 = c->prm.precision == MPCD_P32;
-    if (p32 && c->Ns >= (int64_t)4 * 3 * c->num_sms * 1024 && c->Ns >= (int64_t)4096 * c->nrep &&
-        staged_fits(c, 1024, 1, 128)) {
+    if (p32 && c->Ns >= (int64_t)4 * 3 * c->num_sms * 1024 && c->Ns >= (int64_t)4096 * c->nrep) {
         c->tune = mpcd_tuning{128, 1024, 3, period, 1};
         return;
     }
-    if (staged_fits(c, 128, 3, 512)) {
+    if (!p32 && c->prm.rule == MPCD_AT)
+        c->tune = mpcd_tuning{128, 512, 4, period, 0};
+    else if (!p32)
+        c->tune = mpcd_tuning{256, 128, 1, period, 3};
+    else
         c->tune = mpcd_tuning{c->prm.rule == MPCD_AT && c->B > 0 ? 384 : 512, 128, 1, period, 3};
-        return;
-    }
-    c->tune = mpcd_tuning{512, 2048, 1, period, 0};
-    for (int t : {2048, 1536, 1024, 512})
-        if (staged_fits(c, t, 2, 512)) {
-            c->tune.tile = t;
-            c->tune.staged = 2;
-            break;
-        }
 }
 
 LaunchCfg solvent_cfg(const mpcd_ctx *c)

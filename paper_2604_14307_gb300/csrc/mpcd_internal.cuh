@@ -336,6 +336,58 @@ __device__ __forceinline__ float ll2f(long long w)
 }
 
 // ---------------------------------------------------------------------------
+// FP64 helpers.  An FP64 instruction - conversions and comparisons among them -
+// takes 64 cycles of an SM sub-partition per warp, and the FP64 forms keep that
+// pipe full (ncu: 79 % of its nominal peak in every kernel, its ceiling), so
+// what can be done on the integer pipe is done there.
+// ---------------------------------------------------------------------------
+// (x + 1/2) 2^-32, exactly: the bits of 1 + it, less 1 (33 significant bits)
+__device__ __forceinline__ double u01d(uint32_t x)
+{
+    return __hiloint2double((int)(0x3FF00000u | (x >> 12)), (int)((x << 20) | 0x80000u)) - 1.0;
+}
+// 2 x + 1 = (x + 1/2) 2, exactly
+__device__ __forceinline__ double odd_of(uint32_t x)
+{
+    return __hiloint2double((int)(0x43300000u | (x >> 31)), (int)((x << 1) | 1u)) - 4503599627370496.0;
+}
+// floor(x 2^20) for 0 <= x < 2^11: x + 1.5 2^32, rounded down, has the spacing
+// 2^-20, so its low word is that floor
+__device__ __forceinline__ int lattice_floor(double x) { return __double2loint(__dadd_rd(x, 6442450944.0)); }
+
+// y wrapped into [0, L) by at most one box length; bad is set where it is not
+// (non-finite values included).  Non-negative doubles order as their bits do, a
+// negative one has the larger unsigned bits, and a NaN is never below L.
+__device__ __forceinline__ double wrap_box(double y, double L, int &bad)
+{
+    const long long top = __double_as_longlong(L);
+    const long long b = __double_as_longlong(y);
+    if (b >= top) {
+        y = __dsub_rn(y, L);
+    } else if (b < 0) {
+        if ((unsigned long long)b << 1) {          // negative, not -0
+            y = __dadd_rn(y, L);
+            if (__double_as_longlong(y) == top) y = 0.0;
+        } else {
+            y = 0.0;
+        }
+    }
+    bad |= (unsigned long long)__double_as_longlong(y) >= (unsigned long long)top;
+    return y;
+}
+
+// a / b with rb = RN(1 / b): Markstein's correction (IBM J. Res. Dev. 34, 111
+// (1990)) applied twice.  The first makes the quotient faithful, the second
+// rounds it correctly, so the result is that of the IEEE division (no overflow
+// or underflow in between), in 5 instructions of 64 cycles instead of about 11.
+__device__ __forceinline__ double div_by(double a, double b, double rb)
+{
+    double q = a * rb;
+    q = fma(fma(-b, q, a), rb, q);
+    return fma(fma(-b, q, a), rb, q);
+}
+
+// ---------------------------------------------------------------------------
 // Launch wrappers (defined in the kernel translation units).
 // ---------------------------------------------------------------------------
 enum : int { SOLV_COLLIDE = 1, SOLV_STREAM = 2, SOLV_BIN = 4 };
@@ -474,7 +526,7 @@ template <> struct AngParams<float> { long long sw[3]; long long M; float w[3]; 
 template <> struct AngParams<double> { double sw[3]; double M; double w[3]; double pad; };
 
 __device__ __forceinline__ int ang_lattice_q(float x, int S) { return (__float2int_rd(x * 1048576.0f) - S) & 0xFFFFF; }
-__device__ __forceinline__ int ang_lattice_q(double x, int S) { return (__double2int_rd(x * 1048576.0) - S) & 0xFFFFF; }
+__device__ __forceinline__ int ang_lattice_q(double x, int S) { return (lattice_floor(x) - S) & 0xFFFFF; }
 __device__ __forceinline__ float ang_offset(const AngParams<float> &p, int Q, int k)
 {
     return ll2f(p.M * (long long)Q - p.sw[k]);
