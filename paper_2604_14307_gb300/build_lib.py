@@ -39,7 +39,8 @@ def nvcc() -> str:
 
 def _sources():
     srcs = [os.path.join(CSRC, f) for f in UNITS]
-    deps = srcs + [os.path.join(CSRC, "mpcd_internal.cuh"), os.path.join(ROOT, "include", "mpcd.h")]
+    deps = srcs + [os.path.join(CSRC, "mpcd_internal.cuh"),
+                   os.path.join(CSRC, "solvent_device.cuh"), os.path.join(ROOT, "include", "mpcd.h")]
     return srcs, deps
 
 

@@ -14,18 +14,21 @@
 // mod 2^20 is the member's offset inside its shifted cell in units of 2^-20,
 // an integer, which makes the geometric sums exact.
 //
-// Passes around the plain collision of a step (all keyed on the same step):
-//   k_ang_shift       the grid shift of every replica (once per collision)
-//   k_ang_sums<PRE>   solvent, before the rule: count, sum Q, sum Q_a Q_b,
-//                     + sum Q x P, + sum P (the sites add theirs from the
-//                     thermalised velocities, kernels_bodies.cu)
-//   k_ang_sums<POST>  after the rule: - sum Q x P*, - sum P* (sites likewise)
+// Passes of a step (all keyed on the same step):
+//   k_ang_collide     solvent: the rule, and the cell words: count, sum Q,
+//                     sum Q_a Q_b, sum Q x (P - P*), sum (P - P*) (the sites'
+//                     words in kernels_bodies.cu, beside it)
 //   k_ang_params      per cell: centre of mass, Pi and the angular-momentum
 //                     change in FP64, w by the adjugate of Pi (least-norm form
 //                     for collinear members); clears the words
-//   k_ang_apply       solvent: v = v* + w' x (M Q - sum mu Q), w' = w / (M 2^20);
-//                     the site POST coupling applies the same to the sites
-//                     before it transfers their momentum change to the body
+//   k_ang_stream      solvent: v = v* + w' x (M Q - sum mu Q), w' = w / (M 2^20),
+//                     then streams and bins for the next step (k_ang_apply: the
+//                     correction alone); the site POST coupling applies the
+//                     same to the sites before it transfers their momentum
+//                     change to the body
+// so that the particles are read and written twice in a step.  (Binning, sums
+// before the rule, rule, sums after it, correction and streaming were six
+// passes: 1.08 M particles with 191 bodies 300 us per step.)
 // Word layout and record: AW_* and AngParams in mpcd_internal.cuh.  The
 // geometric sums are kept per species (solvent, sites) and exact; masses enter
 // in the per-cell solve (P32: mu = round(m 2^24), the quantised masses of the
@@ -39,7 +42,7 @@
 // sums FP64 atomics.
 #include <algorithm>
 
-#include "mpcd_internal.cuh"
+#include "solvent_device.cuh"
 
 namespace mpcd {
 
@@ -61,20 +64,6 @@ __device__ __forceinline__ int axis_cell(int X, int S, int L)
 // momentum term P of one particle: the P32 fixed-point value or the FP64 product
 __device__ __forceinline__ long long mom_term(float m, float v) { return q20(__fmul_rn(m, v)); }
 __device__ __forceinline__ double mom_term(double m, double v) { return m * v; }
-
-template <typename Real> __device__ __forceinline__ Real solvent_mass(const StepArgs &a);
-template <> __device__ __forceinline__ float solvent_mass<float>(const StepArgs &a) { return a.m_solvent_f; }
-template <> __device__ __forceinline__ double solvent_mass<double>(const StepArgs &a) { return a.m_solvent; }
-
-// per-replica grid shift of the collision, computed once per collision
-__global__ void k_ang_shift(StepArgs a, int4 *shifts)
-{
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= a.n_rep) return;
-    int32_t S[3];
-    grid_shift(a.reps[r], current_step(a), S);
-    shifts[r] = make_int4(S[0], S[1], S[2], 0);
-}
 
 __device__ __forceinline__ void ld4v(const float *p, float (&o)[4])
 {
@@ -99,7 +88,7 @@ __device__ __forceinline__ void st4v(double *p, const double (&o)[4])
 // cell and lattice offset Q of each of a thread's 4 particles
 template <typename Real>
 __device__ __forceinline__ void cells4(const Real (&x)[4], const Real (&y)[4], const Real (&z)[4], int4 S,
-                                       const DevReplica &r, int64_t (&c)[4], int (&Q)[4][3])
+                                       const DevReplica &r, int (&c)[4], int (&Q)[4][3])
 {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -111,85 +100,115 @@ __device__ __forceinline__ void cells4(const Real (&x)[4], const Real (&y)[4], c
             cc[k] = axis_cell(X[k], Sk[k], r.L[k]);
             Q[j][k] = (X[k] - Sk[k]) & 0xFFFFF;
         }
-        c[j] = r.cell_base + cc[0] + (int64_t)r.L[0] * (cc[1] + (int64_t)r.L[1] * cc[2]);
+        c[j] = r.cell_base + cc[0] + r.L[0] * (cc[1] + r.L[1] * cc[2]);   // below 2^31 cells
     }
 }
 
-// One warp per tile; each lane takes 4 consecutive particles (128-bit loads;
-// tiles start on multiples of 8 slots, and the slots past a replica's last
-// particle are allocated padding), merges runs of equal cells in registers and
-// issues one atomic per word and run.  PRE adds the solvent's 16 terms, POST
-// subtracts the rule's new momentum terms.
-template <typename Real, bool PRE>
-__global__ void __launch_bounds__(256) k_ang_sums(StepArgs a)
+// The rule and the cell words.  One warp per tile; each lane takes 4 consecutive
+// particles (128-bit loads; tiles start on multiples of 8 slots, and the slots
+// past a replica's last particle are allocated padding) and merges runs of equal
+// cells in registers.  The 16 words of a cell are one 128-byte line, and the
+// pass is bound by the sectors its L2 reductions touch: the runs that end at a
+// slot go through shared memory, and sixteen lanes add the words of one (4 sectors
+// a run; word arrays n_cells long touched about 10).
+constexpr int ANG_ROW = AW_SOLVENT + 1;   // a lane's row of words, padded against bank conflicts
+
+template <typename Real, int RULE>
+__global__ void __launch_bounds__(256) k_ang_collide(StepArgs a)
 {
     typedef typename AngWord<Real>::type W;
-    W *w = reinterpret_cast<W *>(a.ang_words);
-    const int4 *shifts = a.ang_shift;
-    const int64_t C = a.n_cells;
-    const Real m = solvent_mass<Real>(a);
+    __shared__ W rows[8][32 * ANG_ROW];
+    W *words = reinterpret_cast<W *>(a.ang_words);
+    const int64_t step = current_step(a);
+    const Real m = Consts<Real>::m(a), ca = Consts<Real>::ca(a), sa = Consts<Real>::sa(a);
+    const Real sc = sqrt(Consts<Real>::kT(a) / m);
     const Real *X = reinterpret_cast<const Real *>(a.x), *Y = reinterpret_cast<const Real *>(a.y);
-    const Real *Z = reinterpret_cast<const Real *>(a.z), *VX = reinterpret_cast<const Real *>(a.vx);
-    const Real *VY = reinterpret_cast<const Real *>(a.vy), *VZ = reinterpret_cast<const Real *>(a.vz);
+    const Real *Z = reinterpret_cast<const Real *>(a.z);
+    Real *VX = reinterpret_cast<Real *>(a.vx), *VY = reinterpret_cast<Real *>(a.vy);
+    Real *VZ = reinterpret_cast<Real *>(a.vz);
     const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+    W *row = rows[threadIdx.x >> 5];
+    int4 S = make_int4(0, 0, 0, 0);
+    int last_rep = -1;
     for (int t = blockIdx.x * warps + (threadIdx.x >> 5); t < a.n_tiles; t += gridDim.x * warps) {
         const Tile tl = a.tiles[t];
         const DevReplica r = a.reps[tl.rep];
-        const int4 S = shifts[tl.rep];
-        for (int64_t i = tl.begin + 4 * lane; i < tl.end; i += 128) {
-            const int nv = (int)min((int64_t)4, tl.end - i);
-            Real x[4], y[4], z[4], vx[4], vy[4], vz[4];
-            ld4v(X + i, x); ld4v(Y + i, y); ld4v(Z + i, z);
-            ld4v(VX + i, vx); ld4v(VY + i, vy); ld4v(VZ + i, vz);
-            int64_t c[4];
+        if (tl.rep != last_rep) {
+            int32_t s3[3];
+            grid_shift(r, step, s3);
+            S = make_int4(s3[0], s3[1], s3[2], 0);
+            last_rep = tl.rep;
+        }
+        for (int64_t i0 = tl.begin; i0 < tl.end; i0 += 128) {   // uniform: the lanes add each other's runs
+            const int64_t i = i0 + 4 * lane;
+            const int nv = (int)max((int64_t)0, min((int64_t)4, tl.end - i));
+            Real x[4] = {}, y[4] = {}, z[4] = {}, vx[4] = {}, vy[4] = {}, vz[4] = {};
+            uint32_t tg[4] = {0, 0, 0, 0};
+            if (nv > 0) {
+                ld4v(X + i, x); ld4v(Y + i, y); ld4v(Z + i, z);
+                ld4v(VX + i, vx); ld4v(VY + i, vy); ld4v(VZ + i, vz);
+                if (RULE == 1) {
+                    const uint4 t4 = *reinterpret_cast<const uint4 *>(a.tag + i);
+                    tg[0] = t4.x; tg[1] = t4.y; tg[2] = t4.z; tg[3] = t4.w;
+                }
+            }
+            int c[4];
             int Q[4][3];
             cells4(x, y, z, S, r, c, Q);
-            W P[4][3];
+            CellParams<Real> p[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) p[j] = get_params<Real>(a.params, j < nv ? c[j] : r.cell_base);
+            W D[4][3];   // P - P*
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                P[j][0] = mom_term(m, vx[j]); P[j][1] = mom_term(m, vy[j]); P[j][2] = mom_term(m, vz[j]);
-            }
-            bool join[4], head[4];   // join[j]: particle j+1 is in j's cell
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                join[j] = j + 1 < nv && c[j + 1] == c[j];
-                head[j] = j < nv && (j == 0 || c[j] != c[j - 1]);
-            }
-            // the solvent's words: count, sum Q, sum Q_a Q_b (PRE only), then
-            // the momentum words; k indexes the 16 terms, wk the word
-#pragma unroll
-            for (int k = PRE ? 0 : 10; k < 16; ++k) {
-                const int wk = k == 0 ? AW_COUNT : k < 4 ? AW_SQ + k - 1 : k < 10 ? AW_QQ + k - 4
-                                                        : k < 13 ? AW_L + k - 10 : AW_P + k - 13;
-                W v[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const W q0 = (W)Q[j][0], q1 = (W)Q[j][1], q2 = (W)Q[j][2];
-                    W e;
-                    switch (k) {
-                    case 0: e = (W)1; break;
-                    case 1: e = q0; break;
-                    case 2: e = q1; break;
-                    case 3: e = q2; break;
-                    case 4: e = q0 * q0; break;
-                    case 5: e = q1 * q1; break;
-                    case 6: e = q2 * q2; break;
-                    case 7: e = q0 * q1; break;
-                    case 8: e = q0 * q2; break;
-                    case 9: e = q1 * q2; break;
-                    case 10: e = q1 * P[j][2] - q2 * P[j][1]; break;
-                    case 11: e = q2 * P[j][0] - q0 * P[j][2]; break;
-                    case 12: e = q0 * P[j][1] - q1 * P[j][0]; break;
-                    default: e = P[j][k - 13]; break;
-                    }
-                    v[j] = PRE ? e : -e;
+                const W P0 = mom_term(m, vx[j]), P1 = mom_term(m, vy[j]), P2 = mom_term(m, vz[j]);
+                const bool on = j < nv && p[j].kappa >= Real(0);
+                Real rx = vx[j], ry = vy[j], rz = vz[j];
+                if (RULE == 0) {
+                    srd_rotate<Real>(p[j], ca, sa, rx, ry, rz);
+                } else {
+                    Real nn[3];
+                    normals3(draw(r, step, tg[j], TAG_AT, 0u), nn);
+                    rx = p[j].ux + sc * nn[0] - p[j].ax;
+                    ry = p[j].uy + sc * nn[1] - p[j].ay;
+                    rz = p[j].uz + sc * nn[2] - p[j].az;
                 }
+                vx[j] = on ? rx : vx[j];
+                vy[j] = on ? ry : vy[j];
+                vz[j] = on ? rz : vz[j];
+                D[j][0] = P0 - mom_term(m, vx[j]);
+                D[j][1] = P1 - mom_term(m, vy[j]);
+                D[j][2] = P2 - mom_term(m, vz[j]);
+            }
+            if (nv > 0) { st4v(VX + i, vx); st4v(VY + i, vy); st4v(VZ + i, vz); }
+            W acc[AW_SOLVENT];
 #pragma unroll
-                for (int j = 2; j >= 0; --j)
-                    if (join[j]) v[j] += v[j + 1];
+            for (int j = 0; j < 4; ++j) {
+                const W q0 = (W)Q[j][0], q1 = (W)Q[j][1], q2 = (W)Q[j][2];
+                const W e[AW_SOLVENT] = {(W)1, q0, q1, q2, q0 * q0, q1 * q1, q2 * q2, q0 * q1, q0 * q2, q1 * q2,
+                                         q1 * D[j][2] - q2 * D[j][1], q2 * D[j][0] - q0 * D[j][2],
+                                         q0 * D[j][1] - q1 * D[j][0], D[j][0], D[j][1], D[j][2]};
+                const bool more = j > 0 && j < nv && c[j] == c[j > 0 ? j - 1 : 0];
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (head[j]) ang_red(w + wk * C + c[j], v[j]);
+                for (int k = 0; k < AW_SOLVENT; ++k) acc[k] = more ? acc[k] + e[k] : e[k];
+                const bool end = j < nv && (j + 1 >= nv || c[j < 3 ? j + 1 : 3] != c[j]);
+                unsigned left = __ballot_sync(0xffffffffu, end);
+                if (!left) continue;
+                __syncwarp();
+                if (end)
+#pragma unroll
+                    for (int k = 0; k < AW_SOLVENT; ++k) row[lane * ANG_ROW + k] = acc[k];
+                __syncwarp();
+                while (left) {   // two runs at a time, one per half warp
+                    const int r0 = __ffs(left) - 1;
+                    left &= left - 1;
+                    const int r1 = left ? __ffs(left) - 1 : -1;
+                    left &= left - 1;
+                    const int src = lane < 16 ? r0 : r1;
+                    const int cell = __shfl_sync(0xffffffffu, c[j], max(src, 0));
+                    if (src >= 0)
+                        ang_red(words + (int64_t)AW_SOLVENT * cell + (lane & 15), row[src * ANG_ROW + (lane & 15)]);
+                }
             }
         }
     }
@@ -198,22 +217,28 @@ __global__ void __launch_bounds__(256) k_ang_sums(StepArgs a)
 // record of one cell from its words.  mu_s, mu_b: the solvent and site mass
 // in the units of the form (P32: round(m 2^24), P64: m); pscale: the unit of
 // the P terms (P32: 2^-20, P64: 1); mscale: the unit of mu (P32: 2^-24, P64: 1).
+// FP64 instructions bound the solve: the sites' words enter only where a cell has
+// sites, and the two forms of the solution share one division.
 template <typename Real, typename W>
-__device__ void cell_record(const W (&wd)[ANG_WORDS], double mu_s, double mu_b, double pscale, double mscale,
+__device__ void cell_record(const W (&wd)[AW_SOLVENT], const W *wb, double mu_s, double mu_b, double unit,
                             AngParams<Real> &o)
 {
     const long long cnt = (long long)wd[AW_COUNT];
-    const double ns = (double)(cnt & 0xFFF), nb = (double)((cnt >> 12) & 0x3FF);
-    const double M = ns * mu_s + nb * mu_b;     // exact (integers below 2^53 in P32)
+    const int n_s = (int)(cnt & 0xFFF), n_b = (int)((cnt >> 12) & 0x3FF);
+    const bool sites = n_b > 0;
+    double M = (double)n_s * mu_s;
+    if (sites) M += (double)n_b * mu_b;         // exact (integers below 2^53 in P32)
     double sw[3];
     for (int k = 0; k < 3; ++k) {
         if constexpr (sizeof(Real) == 4) {
             // exact in int64: mu Q sums below M 2^20
-            const long long v = (long long)mu_s * (long long)wd[AW_SQ + k] + (long long)mu_b * (long long)wd[AW_SQB + k];
+            long long v = (long long)mu_s * (long long)wd[AW_SQ + k];
+            if (sites) v += (long long)mu_b * (long long)wb[AW_SQB + k];
             o.sw[k] = v;
             sw[k] = (double)v;
         } else {
-            sw[k] = mu_s * (double)wd[AW_SQ + k] + mu_b * (double)wd[AW_SQB + k];
+            sw[k] = mu_s * (double)wd[AW_SQ + k];
+            if (sites) sw[k] += mu_b * (double)wb[AW_SQB + k];
             o.sw[k] = sw[k];
         }
         o.w[k] = (Real)0;
@@ -221,14 +246,17 @@ __device__ void cell_record(const W (&wd)[ANG_WORDS], double mu_s, double mu_b, 
     if constexpr (sizeof(Real) == 4) o.M = (long long)M;
     else o.M = M;
     o.pad = (Real)0;
-    if (ns + nb < 2.0) return;
+    if (n_s + n_b < 2) return;
     const double iM = 1.0 / M;
     const double Qc[3] = {sw[0] * iM, sw[1] * iM, sw[2] * iM};
     // mass-weighted lattice covariance about the centre of mass
     double Cm[3][3];
     const int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};
+#pragma unroll
     for (int q = 0; q < 6; ++q) {
-        const double v = mu_s * (double)wd[AW_QQ + q] + mu_b * (double)wd[AW_QQB + q] - sw[ia[q]] * Qc[ib[q]];
+        double v = mu_s * (double)wd[AW_QQ + q];
+        if (sites) v = mu_s * (double)wd[AW_QQ + q] + mu_b * (double)wb[AW_QQB + q];
+        v = v - sw[ia[q]] * Qc[ib[q]];
         Cm[ia[q]][ib[q]] = Cm[ib[q]][ia[q]] = v;
     }
     const double tr = Cm[0][0] + Cm[1][1] + Cm[2][2];
@@ -244,25 +272,38 @@ __device__ void cell_record(const W (&wd)[ANG_WORDS], double mu_s, double mu_b, 
     const double c00 = a11 * a22 - a12 * a12, c01 = a02 * a12 - a01 * a22, c02 = a01 * a12 - a02 * a11;
     const double c11 = a00 * a22 - a02 * a02, c12 = a01 * a02 - a00 * a12, c22 = a00 * a11 - a01 * a01;
     const double det = a00 * c00 + a01 * c01 + a02 * c02;
+    // collinear members: C = tr(C) d d^T, G = tr(C) (I - d d^T); least-norm x
+    // = (dL - d (d.dL)) / tr(C) with d d^T = C / tr(C)
+    const bool full = det > 1e-12 * tr * tr * tr;
+    const double inv = 1.0 / (full ? det : tr);
     double x[3];
-    if (det > 1e-12 * tr * tr * tr) {
-        const double inv = 1.0 / det;
+    if (full) {
         x[0] = (c00 * dL[0] + c01 * dL[1] + c02 * dL[2]) * inv;
         x[1] = (c01 * dL[0] + c11 * dL[1] + c12 * dL[2]) * inv;
         x[2] = (c02 * dL[0] + c12 * dL[1] + c22 * dL[2]) * inv;
     } else {
-        // collinear members: C = tr(C) d d^T, G = tr(C) (I - d d^T); least-norm x
-        // = (dL - d (d.dL)) / tr(C) with d d^T = C / tr(C)
-        const double it = 1.0 / tr;
         for (int i = 0; i < 3; ++i) {
             const double CdL = Cm[i][0] * dL[0] + Cm[i][1] * dL[1] + Cm[i][2] * dL[2];
-            x[i] = (dL[i] - CdL * it) * it;
+            x[i] = (dL[i] - CdL * inv) * inv;
         }
     }
-    // Pi w = dL_phys with Pi = mscale 2^-40 G and dL_phys = 2^-20 pscale dL;
-    // the record keeps w' = w / (M 2^20)
-    const double s = pscale / (mscale * M);
+    // Pi w = dL_phys with Pi = mscale 2^-40 G and dL_phys = 2^-20 pscale dL; the
+    // record keeps w' = w / (M 2^20); unit = pscale / mscale, a power of two
+    const double s = unit * iM;
     for (int k = 0; k < 3; ++k) o.w[k] = (Real)(x[k] * s);
+}
+
+// sixteen bytes of a cell's words at a time: the line of a cell is a thread's own
+template <typename W, int N>
+__device__ __forceinline__ void take_words(W *p, W (&o)[N])
+{
+    longlong2 *q = reinterpret_cast<longlong2 *>(p);
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) {
+        const longlong2 v = q[k];
+        reinterpret_cast<longlong2 *>(o)[k] = v;
+        q[k] = make_longlong2(0, 0);   // also 0.0 in the FP64 form
+    }
 }
 
 template <typename Real>
@@ -272,43 +313,71 @@ __global__ void __launch_bounds__(256) k_ang_params(StepArgs a)
     W *w = reinterpret_cast<W *>(a.ang_words);
     AngParams<Real> *params = reinterpret_cast<AngParams<Real> *>(const_cast<void *>(a.ang_params));
     const int64_t C = a.n_cells;
+    W *wsites = w + (int64_t)AW_SOLVENT * C;
     const bool p32 = sizeof(Real) == 4;
     const double mu_s = p32 ? (double)a.qm_solvent : a.m_solvent;
     const double mu_b = p32 ? (double)a.qm_site : a.m_site;
-    const double pscale = p32 ? 0x1p-20 : 1.0, mscale = p32 ? 0x1p-24 : 1.0;
+    const double unit = p32 ? 16.0 : 1.0;   // P terms 2^-20 or 1 over mu 2^-24 or 1
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < C; c += (int64_t)gridDim.x * blockDim.x) {
-        W wd[ANG_WORDS];
+        alignas(16) W wd[AW_SOLVENT];
+        W wb[AW_SITES];
+        take_words(w + AW_SOLVENT * c, wd);
+        if ((((long long)wd[AW_COUNT]) >> 12) & 0x3FF) {
 #pragma unroll
-        for (int k = 0; k < ANG_WORDS; ++k) {
-            wd[k] = w[k * C + c];
-            w[k * C + c] = (W)0;
+            for (int k = 0; k < AW_SITES; ++k) {
+                wb[k] = wsites[AW_SITES * c + k];
+                wsites[AW_SITES * c + k] = (W)0;
+            }
         }
         AngParams<Real> o;
-        cell_record<Real>(wd, mu_s, mu_b, pscale, mscale, o);
+        cell_record<Real>(wd, wb, mu_s, mu_b, unit, o);
         params[c] = o;
     }
 }
 
-template <typename Real>
+// The correction; STREAM: then the drift and the binning for the next collision
+// (the arithmetic of the plain passes, in the layout of k_ang_collide).
+template <typename Real, int RULE, bool STREAM>
 __global__ void __launch_bounds__(256) k_ang_apply(StepArgs a)
 {
     const AngParams<Real> *params = reinterpret_cast<const AngParams<Real> *>(a.ang_params);
-    const int4 *shifts = a.ang_shift;
-    const Real *X = reinterpret_cast<const Real *>(a.x), *Y = reinterpret_cast<const Real *>(a.y);
-    const Real *Z = reinterpret_cast<const Real *>(a.z);
+    typedef typename SumWord<Real>::type SW;
+    SW *sums = reinterpret_cast<SW *>(a.sums);
+    const int64_t step = current_step(a);
+    const Real m = Consts<Real>::m(a), dt = Consts<Real>::dt(a);
+    const Real sc = sqrt(Consts<Real>::kT(a) / m);
+    Real *X = reinterpret_cast<Real *>(a.x), *Y = reinterpret_cast<Real *>(a.y), *Z = reinterpret_cast<Real *>(a.z);
     Real *VX = reinterpret_cast<Real *>(a.vx), *VY = reinterpret_cast<Real *>(a.vy);
     Real *VZ = reinterpret_cast<Real *>(a.vz);
     const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+    int4 S = make_int4(0, 0, 0, 0);
+    typename ShiftT<Real>::type sF[3] = {};
+    int last_rep = -1, bad = 0;
     for (int t = blockIdx.x * warps + (threadIdx.x >> 5); t < a.n_tiles; t += gridDim.x * warps) {
         const Tile tl = a.tiles[t];
         const DevReplica r = a.reps[tl.rep];
-        const int4 S = shifts[tl.rep];
+        if (tl.rep != last_rep) {
+            int32_t s3[3];
+            grid_shift(r, step, s3);
+            S = make_int4(s3[0], s3[1], s3[2], 0);
+            if (STREAM) {
+                grid_shift(r, step + 1, s3);
+                for (int k = 0; k < 3; ++k) sF[k] = shift_as(s3[k], typename ShiftT<Real>::type());
+            }
+            last_rep = tl.rep;
+        }
+        const Real L[3] = {(Real)r.L[0], (Real)r.L[1], (Real)r.L[2]};
         for (int64_t i = tl.begin + 4 * lane; i < tl.end; i += 128) {
             const int nv = (int)min((int64_t)4, tl.end - i);
             Real x[4], y[4], z[4], vx[4], vy[4], vz[4];
             ld4v(X + i, x); ld4v(Y + i, y); ld4v(Z + i, z);
             ld4v(VX + i, vx); ld4v(VY + i, vy); ld4v(VZ + i, vz);
-            int64_t c[4];
+            uint32_t tg[4] = {0, 0, 0, 0};
+            if (STREAM && RULE == 1) {
+                const uint4 t4 = *reinterpret_cast<const uint4 *>(a.tag + i);
+                tg[0] = t4.x; tg[1] = t4.y; tg[2] = t4.z; tg[3] = t4.w;
+            }
+            int c[4];
             int Q[4][3];
             cells4(x, y, z, S, r, c, Q);
 #pragma unroll
@@ -317,16 +386,31 @@ __global__ void __launch_bounds__(256) k_ang_apply(StepArgs a)
                 Real v[3] = {vx[j], vy[j], vz[j]};
                 ang_correct(params[c[j]], Q[j], v);
                 vx[j] = v[0]; vy[j] = v[1]; vz[j] = v[2];
+                if (STREAM) {
+                    if (a.accel) {
+                        vx[j] = kick(vx[j], Consts<Real>::ah(a, 0));
+                        vy[j] = kick(vy[j], Consts<Real>::ah(a, 1));
+                        vz[j] = kick(vz[j], Consts<Real>::ah(a, 2));
+                    }
+                    x[j] = drift(x[j], vx[j], dt, L[0], bad);
+                    y[j] = drift(y[j], vy[j], dt, L[1], bad);
+                    z[j] = drift(z[j], vz[j], dt, L[2], bad);
+                    if (a.accel) {
+                        vx[j] = kick(vx[j], Consts<Real>::ah(a, 0));
+                        vy[j] = kick(vy[j], Consts<Real>::ah(a, 1));
+                        vz[j] = kick(vz[j], Consts<Real>::ah(a, 2));
+                    }
+                }
             }
-            if (nv == 4) {
-                st4v(VX + i, vx); st4v(VY + i, vy); st4v(VZ + i, vz);
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (j < nv) { VX[i + j] = vx[j]; VY[i + j] = vy[j]; VZ[i + j] = vz[j]; }
+            if (STREAM) {
+                bin4<Real, RULE, true>(a, x, y, z, vx, vy, vz, tg, nv, sF, r.L[0], r.L[1], r.L[2], r.cell_base, r, step,
+                                       m, sc, sums, a.n_cells);
+                st4v(X + i, x); st4v(Y + i, y); st4v(Z + i, z);
             }
+            st4v(VX + i, vx); st4v(VY + i, vy); st4v(VZ + i, vz);
         }
     }
+    if (bad) atomicOr(a.d_err, ERR_POSITION);
 }
 
 }  // namespace
@@ -337,35 +421,30 @@ size_t angular_param_bytes(int precision)
     return precision == 1 ? sizeof(AngParams<float>) : sizeof(AngParams<double>);
 }
 
+template <typename Real, int RULE>
+static void angular_phase(const StepArgs &a, int phase, int num_sms, cudaStream_t s)
+{
+    const int grid_p = (int)std::max<int64_t>(1, std::min<int64_t>((a.n_cells + 255) / 256, (int64_t)num_sms * 16));
+    const int grid_t = std::max(1, std::min((a.n_tiles + 7) / 8, num_sms * 8));   // 8 warps, one tile each
+    if (phase != ANG_PARAMS && a.n_tiles == 0) return;
+    switch (phase) {
+    case ANG_COLLIDE: k_ang_collide<Real, RULE><<<grid_t, 256, 0, s>>>(a); break;
+    case ANG_PARAMS: k_ang_params<Real><<<grid_p, 256, 0, s>>>(a); break;
+    case ANG_APPLY: k_ang_apply<Real, 0, false><<<grid_t, 256, 0, s>>>(a); break;
+    case ANG_STREAM: k_ang_apply<Real, RULE, true><<<grid_t, 256, 0, s>>>(a); break;
+    default: break;
+    }
+}
+
 void launch_angular(const StepArgs &a, int phase, int num_sms, cudaStream_t s)
 {
     if (a.n_cells == 0) return;
-    const int grid_p = std::max(1, num_sms * 16);
-    const int grid_t = (int)std::max(1, std::min((a.n_tiles + 7) / 8, num_sms * 8));   // 8 warps, one tile each
-    const bool p32 = a.precision == 1;
-    switch (phase) {
-    case ANG_PRE:
-        k_ang_shift<<<(a.n_rep + 127) / 128, 128, 0, s>>>(a, a.ang_shift);
-        if (a.n_tiles == 0) return;
-        if (p32) k_ang_sums<float, true><<<grid_t, 256, 0, s>>>(a);
-        else k_ang_sums<double, true><<<grid_t, 256, 0, s>>>(a);
-        break;
-    case ANG_POST:
-        if (a.n_tiles == 0) return;
-        if (p32) k_ang_sums<float, false><<<grid_t, 256, 0, s>>>(a);
-        else k_ang_sums<double, false><<<grid_t, 256, 0, s>>>(a);
-        break;
-    case ANG_PARAMS:
-        if (p32) k_ang_params<float><<<grid_p, 256, 0, s>>>(a);
-        else k_ang_params<double><<<grid_p, 256, 0, s>>>(a);
-        break;
-    case ANG_APPLY:
-        if (a.n_tiles == 0) return;
-        if (p32) k_ang_apply<float><<<grid_t, 256, 0, s>>>(a);
-        else k_ang_apply<double><<<grid_t, 256, 0, s>>>(a);
-        break;
-    default:
-        break;
+    if (a.precision == 1) {
+        if (a.rule == 0) angular_phase<float, 0>(a, phase, num_sms, s);
+        else angular_phase<float, 1>(a, phase, num_sms, s);
+    } else {
+        if (a.rule == 0) angular_phase<double, 0>(a, phase, num_sms, s);
+        else angular_phase<double, 1>(a, phase, num_sms, s);
     }
 }
 

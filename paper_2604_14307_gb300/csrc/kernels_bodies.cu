@@ -25,9 +25,9 @@
 //               the next step recomputes them from P and L.  The ANG instance
 //               (angular-momentum-conserving variants) adds the cell's
 //               rigid-rotation correction to the rule's velocity first.
-// k_ang_sites   the sites' terms of the +a cell words: before the rule from
-//               the thermalised velocities, after it from the rule's
-//               velocities (recomputed with the POST coupling's arithmetic).
+// k_ang_sites   the sites' terms of the +a cell words, from the thermalised
+//               and the rule's velocities (the latter recomputed with the POST
+//               coupling's arithmetic).
 // This file is compiled without fused multiply-add so that the FP64 body and
 // site-position arithmetic rounds the same way as the oracle.
 #include "mpcd_internal.cuh"
@@ -1029,11 +1029,9 @@ __device__ __forceinline__ void site_rule(const StepArgs &a, const DevReplica &r
 
 // lattice offset of a stored site position inside its shifted cell (+a variants)
 template <typename Real>
-__device__ __forceinline__ void site_lattice_q(const Real (&x)[3], int4 S, int (&Q)[3])
+__device__ __forceinline__ void site_lattice_q(const Real (&x)[3], const int (&S)[3], int (&Q)[3])
 {
-    Q[0] = ang_lattice_q(x[0], S.x);
-    Q[1] = ang_lattice_q(x[1], S.y);
-    Q[2] = ang_lattice_q(x[2], S.z);
+    for (int k = 0; k < 3; ++k) Q[k] = ang_lattice_q(x[k], S[k]);
 }
 
 // POST coupling; ANG: with the +a correction of the site's cell applied to the
@@ -1043,12 +1041,14 @@ __global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_si
 {
     __shared__ Real sPose[POSE_W];
     __shared__ Real scratch[SITE_WARPS][6];
+    __shared__ int sS[3];   // ANG: grid shift
     const DevBody &B = a.bodies[blockIdx.x];
     const int64_t site_begin = B.site_begin;
     const DevShape &sh = a.shapes[B.shape];
     const DevReplica r = a.reps[B.rep];
     const int64_t step = current_step(a);
     chain_next();
+    if (ANG && threadIdx.x == 32) grid_shift(r, step, sS);
     if (threadIdx.x < POSE_W) sPose[threadIdx.x] = pose_ptr(a, blockIdx.x, Real(0))[threadIdx.x];
     __syncthreads();
     Pose<Real> P;
@@ -1078,7 +1078,7 @@ __global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_si
             if constexpr (ANG) {
                 const Real xs[3] = {x[0], x[1], x[2]};
                 int Q[3];
-                site_lattice_q(xs, a.ang_shift[B.rep], Q);
+                site_lattice_q(xs, sS, Q);
                 ang_correct(reinterpret_cast<const AngParams<Real> *>(a.ang_params)[cell], Q, vn);
             }
             if (site_owned(a, x[2])) {   // a slab transfers only its own sites
@@ -1187,27 +1187,30 @@ void launch_sites_post(const StepArgs &a, int num_sms, cudaStream_t s)
     }
 }
 
-// +a variants: the sites' contributions to the angular words of their cells,
-// one CTA per body.  PRE: count, sum Q, sum Q_a Q_b, + Q x P, + P from the
-// thermalised velocities of Eq. 7; POST: - Q x P*, - P* from the rule's
-// velocities (recomputed with the same arithmetic as the POST coupling).
+// +a variants: the sites' contributions to the angular words of their cells, one
+// CTA per body: count, sum Q, sum Q_a Q_b, Q x (P - P*) and P - P* with P from
+// the thermalised velocities of Eq. 7 and P* from the rule's (recomputed with
+// the same arithmetic as the POST coupling).
 __device__ __forceinline__ long long site_mom_term(float m, float v) { return q20(__fmul_rn(m, v)); }
 __device__ __forceinline__ double site_mom_term(double m, double v) { return m * v; }
 
-template <typename Real, bool PRE>
+constexpr int ANG_SITE_CTAS = 2;   // CTAs per body (the order of the integer sums is free)
+
+template <typename Real>
 __global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_ang_sites(StepArgs a)
 {
     typedef typename AngWord<Real>::type W;
     __shared__ Real sPose[POSE_W];
-    const DevBody &B = a.bodies[blockIdx.x];
+    __shared__ int sS[3];
+    const DevBody &B = a.bodies[blockIdx.x / ANG_SITE_CTAS];
+    const int part = blockIdx.x % ANG_SITE_CTAS;
     const int64_t site_begin = B.site_begin;
-    const DevShape sh = a.shapes[B.shape];
+    const DevShape &sh = a.shapes[B.shape];
     const DevReplica r = a.reps[B.rep];
     const int64_t step = current_step(a);
-    const int4 S = a.ang_shift[B.rep];
-    W *w = reinterpret_cast<W *>(a.ang_words);
-    const int64_t C = a.n_cells;
-    if (threadIdx.x < POSE_W) sPose[threadIdx.x] = pose_ptr(a, blockIdx.x, Real(0))[threadIdx.x];
+    W *words = reinterpret_cast<W *>(a.ang_words);
+    if (threadIdx.x < POSE_W) sPose[threadIdx.x] = pose_ptr(a, blockIdx.x / ANG_SITE_CTAS, Real(0))[threadIdx.x];
+    if (threadIdx.x == 32) grid_shift(r, step, sS);
     __syncthreads();
     Pose<Real> P;
     for (int k = 0; k < 9; ++k) P.Q[k] = sPose[k];
@@ -1215,55 +1218,45 @@ __global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_ang_si
     const Real *SV = reinterpret_cast<const Real *>(a.site_v);
     const int64_t NS = a.n_sites;
     int bad = 0;
-    for (int j = threadIdx.x; j < sh.n_sites; j += blockDim.x) {
+    for (int j = part * SITE_THREADS + threadIdx.x; j < sh.n_sites; j += ANG_SITE_CTAS * SITE_THREADS) {
         const int64_t t = sh.site_begin + j, g = site_begin + j;
+        const int64_t cell = (int64_t)r.cell_base + a.site_cell[g];
         Real d[3], x[3];
         site_geom(a, t, P, r, d, x, bad);
         const Real v[3] = {SV[g], SV[NS + g], SV[2 * NS + g]};
-        const int64_t cell = (int64_t)r.cell_base + a.site_cell[g];
         const Real m = site_mass<Real>(a, t);
-        Real u[3] = {v[0], v[1], v[2]};
-        if (!PRE) {
-            Real p[8];
-            load_cell<Real>(a, cell, p);
-            site_rule<Real>(a, r, step, g, t, v, p, u);
-        }
+        Real u[3], p[8];
+        load_cell<Real>(a, cell, p);
+        site_rule<Real>(a, r, step, g, t, v, p, u);
         const Real xs[3] = {x[0], x[1], x[2]};
         int Qi[3];
-        site_lattice_q(xs, S, Qi);
+        site_lattice_q(xs, sS, Qi);
         const W q[3] = {(W)Qi[0], (W)Qi[1], (W)Qi[2]};
-        const W Pm[3] = {(W)site_mom_term(m, u[0]), (W)site_mom_term(m, u[1]), (W)site_mom_term(m, u[2])};
-        const W L[3] = {q[1] * Pm[2] - q[2] * Pm[1], q[2] * Pm[0] - q[0] * Pm[2], q[0] * Pm[1] - q[1] * Pm[0]};
-        const W sg = PRE ? (W)1 : (W)-1;
-        if (PRE) {
-            ang_red(w + AW_COUNT * C + cell, (W)4096);
-            for (int k = 0; k < 3; ++k) ang_red(w + (AW_SQB + k) * C + cell, q[k]);
-            ang_red(w + (AW_QQB + 0) * C + cell, q[0] * q[0]);
-            ang_red(w + (AW_QQB + 1) * C + cell, q[1] * q[1]);
-            ang_red(w + (AW_QQB + 2) * C + cell, q[2] * q[2]);
-            ang_red(w + (AW_QQB + 3) * C + cell, q[0] * q[1]);
-            ang_red(w + (AW_QQB + 4) * C + cell, q[0] * q[2]);
-            ang_red(w + (AW_QQB + 5) * C + cell, q[1] * q[2]);
-        }
-        for (int k = 0; k < 3; ++k) {
-            ang_red(w + (AW_L + k) * C + cell, sg * L[k]);
-            ang_red(w + (AW_P + k) * C + cell, sg * Pm[k]);
-        }
+        W D[3];
+        for (int k = 0; k < 3; ++k) D[k] = (W)site_mom_term(m, v[k]) - (W)site_mom_term(m, u[k]);
+        W *w = words + AW_SOLVENT * cell, *ws = words + AW_SOLVENT * a.n_cells + AW_SITES * cell;
+        ang_red(w + AW_COUNT, (W)4096);
+        ang_red(w + AW_L, q[1] * D[2] - q[2] * D[1]);
+        ang_red(w + AW_L + 1, q[2] * D[0] - q[0] * D[2]);
+        ang_red(w + AW_L + 2, q[0] * D[1] - q[1] * D[0]);
+        for (int k = 0; k < 3; ++k) ang_red(w + AW_P + k, D[k]);
+        for (int k = 0; k < 3; ++k) ang_red(ws + AW_SQB + k, q[k]);
+        ang_red(ws + AW_QQB + 0, q[0] * q[0]);
+        ang_red(ws + AW_QQB + 1, q[1] * q[1]);
+        ang_red(ws + AW_QQB + 2, q[2] * q[2]);
+        ang_red(ws + AW_QQB + 3, q[0] * q[1]);
+        ang_red(ws + AW_QQB + 4, q[0] * q[2]);
+        ang_red(ws + AW_QQB + 5, q[1] * q[2]);
     }
     if (bad) atomicOr(a.d_err, ERR_POSITION);
 }
 
-void launch_angular_sites(const StepArgs &a, int phase, cudaStream_t s)
+void launch_angular_sites(const StepArgs &a, cudaStream_t s)
 {
     if (a.n_bodies == 0) return;
-    const bool p32 = a.precision == 1;
-    if (phase == ANG_PRE) {
-        if (p32) k_ang_sites<float, true><<<a.n_bodies, SITE_THREADS, 0, s>>>(a);
-        else k_ang_sites<double, true><<<a.n_bodies, SITE_THREADS, 0, s>>>(a);
-    } else if (phase == ANG_POST) {
-        if (p32) k_ang_sites<float, false><<<a.n_bodies, SITE_THREADS, 0, s>>>(a);
-        else k_ang_sites<double, false><<<a.n_bodies, SITE_THREADS, 0, s>>>(a);
-    }
+    const unsigned grid = (unsigned)a.n_bodies * ANG_SITE_CTAS;
+    if (a.precision == 1) k_ang_sites<float><<<grid, SITE_THREADS, 0, s>>>(a);
+    else k_ang_sites<double><<<grid, SITE_THREADS, 0, s>>>(a);
 }
 
 void launch_body_impulse(const StepArgs &a, cudaStream_t s)

@@ -29,10 +29,10 @@ struct Pending {
     double bytes;
 };
 // A sequence of launches that is recorded once and replayed (enqueue_piece).
-enum PieceKind : int { PIECE_HEAD, PIECE_MIDDLE, PIECE_TAIL, PIECE_WHOLE };
+enum PieceKind : int { PIECE_HEAD, PIECE_MIDDLE, PIECE_TAIL };
 struct Piece {
     int kind;
-    int64_t steps;      // middle or whole steps
+    int64_t steps;      // middle steps
     bool sort;          // a re-sort after the last of them
 };
 struct GraphEntry {
@@ -127,9 +127,8 @@ struct mpcd_ctx {
     int32_t *rn_ncand = nullptr;
     double *rn_tot = nullptr;                   // [0] momentum, [1] pairs (as long long)
     double *d_profile = nullptr;                // [2][PROFILE bins] velocity-profile sums
-    void *ang_words = nullptr;                  // [ANG_WORDS][C] angular-momentum sums (+a variants)
+    void *ang_words = nullptr;                  // [C][ANG_WORDS] angular-momentum sums (+a variants)
     void *ang_params = nullptr;                 // [C] AngParams records of the +a correction
-    int4 *ang_shift = nullptr;                  // [nrep] grid shift of the current collision
     double f_ext[3] = {0.0, 0.0, 0.0};          // constant force on every body (one replica)
     VacfArgs vacf{};                            // velocity autocorrelations (n_lags 0: off)
     // slab of a decomposed box (mpcd_create_slab): the active solvent count is
@@ -224,7 +223,6 @@ StepArgs make_args(const mpcd_ctx *c)
     a.m_site = c->m_site;
     a.ang_words = c->ang_words;
     a.ang_params = c->ang_params;
-    a.ang_shift = c->ang_shift;
     a.qm_site = (long long)std::llrint((double)a.m_site_f * 16777216.0);
     a.reps = c->d_reps;
     a.n_rep = c->nrep;
@@ -621,54 +619,42 @@ int do_sort(mpcd_ctx *c, int canonical, cudaStream_t s, bool from_words = false)
     return MPCD_OK;
 }
 
-// one pass of the +a correction (kernels_angular.cu; the sites' sums in
-// kernels_bodies.cu)
+// one pass of the +a variants (kernels_angular.cu)
 int k_ang(mpcd_ctx *c, int phase, cudaStream_t s)
 {
-    static const char *names[] = {"angular_pre", "angular_post", "angular_params", "angular_apply"};
-    // algorithmic bytes: the solvent arrays each pass reads (and writes), the
-    // cell words written or read once, the per-cell records
+    static const char *names[] = {"angular_collide", "angular_params", "angular_apply", "angular_stream"};
+    // algorithmic bytes: the solvent arrays each pass reads and writes, the cell
+    // words written or read once, the per-cell records
     const double N = (double)c->Ns, C = (double)c->C, r = c->realsz;
-    const double rec = (double)angular_param_bytes(c->prm.precision);
-    const double bytes[] = {N * 6 * r + C * 16 * 8, N * 6 * r + C * 6 * 8,
-                            C * (2.0 * ANG_WORDS * 8 + rec), N * 9 * r + C * rec};
+    const double rec = (double)angular_param_bytes(c->prm.precision), at = c->prm.rule == MPCD_AT ? 4 * N : 0;
+    const double words = c->B > 0 ? ANG_WORDS : AW_SOLVENT;
+    const double bytes[] = {N * 9 * r + C * (c->param_bytes + AW_SOLVENT * 8.0) + at, C * (2.0 * words * 8 + rec),
+                            N * 9 * r + C * rec, N * 12 * r + C * (rec + c->nw * 8.0) + at};
     StepArgs a = make_args(c);
-    int e = timed(c, names[phase], bytes[phase], s, [&] { launch_angular(a, phase, c->num_sms, s); });
-    if (!e && c->B > 0 && (phase == ANG_PRE || phase == ANG_POST)) {
-        const double sb = (double)c->Nsite * (3.0 * r + 4.0);
-        e = timed(c, phase == ANG_PRE ? "angular_sites_pre" : "angular_sites_post", sb, s,
-                  [&] { launch_angular_sites(a, phase, s); });
-    }
-    return e;
+    return timed(c, names[phase], bytes[phase], s, [&] { launch_angular(a, phase, c->num_sms, s); });
+}
+
+int k_ang_sites(mpcd_ctx *c, cudaStream_t s)
+{
+    if (c->B == 0) return MPCD_OK;
+    StepArgs a = make_args(c);
+    const double bytes = (double)c->Nsite * (3.0 * c->realsz + 4.0);
+    return timed(c, "angular_sites", bytes, s, [&] { launch_angular_sites(a, s); });
 }
 
 // the unpipelined collision of the solvent at the current step (a2, a5-a7):
-// exchange, binning, cell parameters, rule; with the +a variant the angular
-// sums are taken before and after the rule and the correction applied
+// exchange, binning, cell parameters, rule; with the +a variant the rule's pass
+// takes the angular words and the correction follows
 int k_collide(mpcd_ctx *c, cudaStream_t s)
 {
-    const bool ang = c->prm.angular != 0;
     int e = k_rnemd(c, s, 0, 0);
     if (!e) e = k_solvent(c, SOLV_BIN, s);
-    if (!e && ang) e = k_ang(c, ANG_PRE, s);
     if (!e) e = k_params(c, s);
-    if (!e) e = k_solvent(c, SOLV_COLLIDE, s);
-    if (!e && ang) e = k_ang(c, ANG_POST, s);
-    if (!e && ang) e = k_ang(c, ANG_PARAMS, s);
-    if (!e && ang) e = k_ang(c, ANG_APPLY, s);
-    return e;
-}
-
-// one whole step in the unpipelined order stream, couple(PRE), collide,
-// couple(POST) (the +a variants, whose correction needs the cell totals of
-// the rule's velocities before any particle streams on)
-int unfused_step(mpcd_ctx *c, cudaStream_t s)
-{
-    int e = k_stream(c, s);
-    if (!e) e = k_pre(c, s, true);
-    if (!e) e = k_collide(c, s);
-    if (!e) e = k_post(c, s);
-    if (!e) e = k_vacf(c, s);
+    if (!c->prm.angular) return e ? e : k_solvent(c, SOLV_COLLIDE, s);
+    if (!e) e = k_ang_sites(c, s);
+    if (!e) e = k_ang(c, ANG_COLLIDE, s);
+    if (!e) e = k_ang(c, ANG_PARAMS, s);
+    if (!e) e = k_ang(c, ANG_APPLY, s);
     return e;
 }
 
@@ -678,7 +664,36 @@ int unfused_step(mpcd_ctx *c, cudaStream_t s)
 // (they need step k's cell parameters and impulse, not its solvent pass; both
 // branches add to the cleared cell sums of step k+1 with integer atomics, so
 // the order between them changes no result).  The branches join before the
-// cell parameters of step k+1.
+// cell parameters of step k+1.  The +a variants need the cell totals of the
+// rule's velocities before any particle streams on: their solvent branch is the
+// rule's pass, the per-cell solve, and a pass that corrects, streams and bins;
+// the sites' words are added beside the first, the chain runs beside the last.
+int fork_side(mpcd_ctx *c, cudaStream_t s)
+{
+    CK(c, cudaEventRecord(c->side_ev[0], s));
+    CK(c, cudaStreamWaitEvent(c->side, c->side_ev[0], 0));
+    return MPCD_OK;
+}
+int join_side(mpcd_ctx *c, cudaStream_t s)
+{
+    CK(c, cudaEventRecord(c->side_ev[1], c->side));
+    CK(c, cudaStreamWaitEvent(s, c->side_ev[1], 0));
+    return MPCD_OK;
+}
+
+// cell parameters, and with the +a variants the rule's pass and the solve
+int params_step(mpcd_ctx *c, cudaStream_t s)
+{
+    int e = k_params(c, s);
+    if (e || !c->prm.angular) return e;
+    if ((e = fork_side(c, s))) return e;
+    e = k_ang_sites(c, c->side);
+    if (!e) e = k_ang(c, ANG_COLLIDE, s);
+    if (!e) e = join_side(c, s);
+    if (!e) e = k_ang(c, ANG_PARAMS, s);
+    return e;
+}
+
 int head_step(mpcd_ctx *c, cudaStream_t s)     // before the first collision
 {
     int e = k_solvent(c, SOLV_STREAM | SOLV_BIN, s);
@@ -690,10 +705,9 @@ int head_step(mpcd_ctx *c, cudaStream_t s)     // before the first collision
 
 int middle_step(mpcd_ctx *c, cudaStream_t s)   // step k's collision up to step k+1's
 {
-    int e = k_params(c, s);
+    int e = params_step(c, s);
+    if (!e) e = fork_side(c, s);
     if (e) return e;
-    CK(c, cudaEventRecord(c->side_ev[0], s));
-    CK(c, cudaStreamWaitEvent(c->side, c->side_ev[0], 0));
     // the transfer is added by the body step, unless it is sampled in between
     const bool apart = c->vacf.n_lags > 0;
     e = k_post(c, c->side, apart);
@@ -701,19 +715,18 @@ int middle_step(mpcd_ctx *c, cudaStream_t s)   // step k's collision up to step 
     if (!e) e = k_bodies(c, c->side, !apart);
     if (!e) e = k_pre(c, c->side, true, 1);   // of step k+1
     if (e) return e;
-    CK(c, cudaEventRecord(c->side_ev[1], c->side));
-    if ((e = k_solvent(c, SOLV_COLLIDE | SOLV_STREAM | SOLV_BIN, s))) return e;
-    if ((e = k_rnemd(c, s, 1, 1))) return e;   // before the collision of step k+1
-    CK(c, cudaStreamWaitEvent(s, c->side_ev[1], 0));
-    return MPCD_OK;
+    e = c->prm.angular ? k_ang(c, ANG_STREAM, s) : k_solvent(c, SOLV_COLLIDE | SOLV_STREAM | SOLV_BIN, s);
+    if (!e) e = k_rnemd(c, s, 1, 1);   // before the collision of step k+1
+    if (!e) e = join_side(c, s);
+    return e;
 }
 
 int tail_step(mpcd_ctx *c, cudaStream_t s)     // the last step's collision
 {
-    int e = k_params(c, s);
+    int e = params_step(c, s);
     if (!e) e = k_post(c, s);
     if (!e) e = k_vacf(c, s);
-    if (!e) e = k_solvent(c, SOLV_COLLIDE, s);
+    if (!e) e = c->prm.angular ? k_ang(c, ANG_APPLY, s) : k_solvent(c, SOLV_COLLIDE, s);
     return e;
 }
 
@@ -724,13 +737,13 @@ int enqueue_piece(mpcd_ctx *c, const Piece &p, cudaStream_t s)
     c->step_off = 0;
     if (p.kind == PIECE_HEAD) e = head_step(c, s);
     if (p.kind == PIECE_TAIL) e = tail_step(c, s);
-    if (p.kind == PIECE_MIDDLE || p.kind == PIECE_WHOLE)
+    if (p.kind == PIECE_MIDDLE)
         for (int64_t k = 0; k < n && !e; ++k) {
             c->step_off = k;
-            e = p.kind == PIECE_MIDDLE ? middle_step(c, s) : unfused_step(c, s);
+            e = middle_step(c, s);
         }
-    // the pipelined step has just binned for the next collision
-    if (!e && p.sort) e = do_sort(c, 0, s, p.kind == PIECE_MIDDLE);
+    // the step has just binned for the next collision
+    if (!e && p.sort) e = do_sort(c, 0, s, true);
     c->step_off = 0;
     if (!e && n) e = k_advance(c, s, n);
     if (!e && !c->profiling) {
@@ -740,9 +753,8 @@ int enqueue_piece(mpcd_ctx *c, const Piece &p, cudaStream_t s)
     return e;
 }
 
-// The pieces of n whole steps: a head, n - 1 middle steps and a tail (n whole
-// steps for the unpipelined variants), with a re-sort wherever the count since
-// the last one reaches the period.  `recorded`: cut so that few different
+// The pieces of n whole steps: a head, n - 1 middle steps and a tail, with a
+// re-sort wherever the count since the last one reaches the period.  `recorded`: cut so that few different
 // pieces serve every n and every phase of the re-sorts - a whole period ending
 // in its re-sort, one step with a re-sort, and powers of two without.
 // (A graph per step count and phase was recorded anew in nearly every call: the
@@ -752,11 +764,11 @@ std::vector<Piece> plan_steps(mpcd_ctx *c, int64_t n, bool recorded)
 {
     constexpr int64_t MOST = 32;   // steps of a recorded piece without a re-sort
     std::vector<Piece> out;
-    const bool fused = !c->prm.angular, sorts = c->prm.sort_period >= 0;
-    const int kind = fused ? PIECE_MIDDLE : PIECE_WHOLE;
+    const bool sorts = c->prm.sort_period >= 0;
+    const int kind = PIECE_MIDDLE;
     const int64_t period = c->tune.sort_period;
-    if (fused) out.push_back(Piece{PIECE_HEAD, 0, false});
-    for (int64_t left = fused ? n - 1 : n; left > 0;) {
+    out.push_back(Piece{PIECE_HEAD, 0, false});
+    for (int64_t left = n - 1; left > 0;) {
         const int64_t due = sorts ? std::max<int64_t>(1, period - c->since_sort) : left + 1;
         const int64_t m = std::min(left, due);
         const bool sort = m == due;
@@ -771,7 +783,7 @@ std::vector<Piece> plan_steps(mpcd_ctx *c, int64_t n, bool recorded)
         c->since_sort = sort ? 0 : c->since_sort + m;
         left -= m;
     }
-    if (fused) out.push_back(Piece{PIECE_TAIL, 0, false});
+    out.push_back(Piece{PIECE_TAIL, 0, false});
     return out;
 }
 
@@ -1066,7 +1078,6 @@ int mpcd_create(const mpcd_params *params, int32_t n_shapes, const mpcd_shape_de
     if (p.angular) {
         ok &= (c->ang_words = A((size_t)c->C * ANG_WORDS * 8)) != nullptr;
         ok &= (c->ang_params = A((size_t)c->C * angular_param_bytes(p.precision))) != nullptr;
-        ok &= (c->ang_shift = (int4 *)A((size_t)c->nrep * sizeof(int4))) != nullptr;
     }
     if (!ok) {
         mpcd_destroy(c);

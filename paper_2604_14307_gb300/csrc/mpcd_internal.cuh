@@ -21,8 +21,7 @@
 //             lists and candidates; the velocity-profile sums; the per-body
 //             autocorrelation rings and sums.
 //   +a        (angular-momentum-conserving variants only) ANG_WORDS more words
-//             per cell, one AngParams record per cell, one grid shift per
-//             replica.
+//             and one AngParams record per cell.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -144,9 +143,8 @@ struct StepArgs {
     // are binned and transfer their momentum here (site_own = 0: every site)
     int32_t site_own, site_zlo, site_zhi;
     // angular-momentum-conserving variants (null when off)
-    void *ang_words;                // [ANG_WORDS][n_cells]
+    void *ang_words;                // [n_cells][AW_SOLVENT], then [n_cells][AW_SITES]
     const void *ang_params;         // [n_cells] AngParams records
-    int4 *ang_shift;                // [n_rep] grid shift of the current collision
 };
 
 // The device counter holds the completed steps when a sequence of steps was
@@ -504,18 +502,21 @@ void launch_gather_rows(const StepArgs &a, const uint32_t *vals, const void *rec
 
 // angular-momentum-conserving collision variants (kernels_angular.cu for the
 // solvent and the per-cell solve, kernels_bodies.cu for the sites).
-// Cell words, SoA [ANG_WORDS][n_cells], int64 (P32) or double (P64); Q is a
-// member's integer lattice offset inside its shifted cell (units 2^-20), P its
-// momentum term (P32: round(fl32(m v) 2^20); P64: m v):
+// Cell words, int64 (P32) or double (P64), cell by cell: [n_cells][AW_SOLVENT]
+// (one 128-byte line each), then [n_cells][AW_SITES].  Q is a member's integer
+// lattice offset inside its shifted cell (units 2^-20), P and P* its momentum term
+// before and after the rule (P32: round(fl32(m v) 2^20); P64: m v):
 enum : int { AW_COUNT = 0,      // 1 per solvent particle, 2^12 per site
              AW_SQ = 1,         // 1-3   sum Q of the solvent
-             AW_SQB = 4,        // 4-6   sum Q of the sites
-             AW_QQ = 7,         // 7-12  sum Q_a Q_b of the solvent (xx, yy, zz, xy, xz, yz)
-             AW_QQB = 13,       // 13-18 the same of the sites
-             AW_L = 19,         // 19-21 sum Q x (P - P*)
-             AW_P = 22,         // 22-24 sum (P - P*)
-             ANG_WORDS = 25 };
-enum : int { ANG_PRE = 0, ANG_POST = 1, ANG_PARAMS = 2, ANG_APPLY = 3 };
+             AW_QQ = 4,         // 4-9   sum Q_a Q_b of the solvent (xx, yy, zz, xy, xz, yz)
+             AW_L = 10,         // 10-12 sum Q x (P - P*), solvent and sites
+             AW_P = 13,         // 13-15 sum (P - P*), solvent and sites
+             AW_SOLVENT = 16,
+             AW_SQB = 0,        // 0-2   sum Q of the sites
+             AW_QQB = 3,        // 3-8   sum Q_a Q_b of the sites
+             AW_SITES = 9,
+             ANG_WORDS = AW_SOLVENT + AW_SITES };
+enum : int { ANG_COLLIDE = 0, ANG_PARAMS = 1, ANG_APPLY = 2, ANG_STREAM = 3 };
 
 // Per-cell record of the correction: the mass-weighted lattice sums sw = sum mu Q,
 // the cell mass M = sum mu (mu = round(m 2^24) in P32, m in P64) and
@@ -554,11 +555,11 @@ template <> struct AngWord<float> { typedef long long type; };
 template <> struct AngWord<double> { typedef double type; };
 
 size_t angular_param_bytes(int precision);
-// solvent phases and the per-cell solve; ANG_PRE also writes a.ang_shift
+// solvent phases and the per-cell solve
 void launch_angular(const StepArgs &a, int phase, int num_sms, cudaStream_t s);
-// the sites' sums (ANG_PRE: thermalised velocities; ANG_POST: the rule's velocities);
-// the correction itself is applied by the site POST coupling when a.ang_params is set
-void launch_angular_sites(const StepArgs &a, int phase, cudaStream_t s);
+// the sites' words (between the cell parameters and the per-cell solve); the
+// correction itself is applied by the site POST coupling when a.ang_params is set
+void launch_angular_sites(const StepArgs &a, cudaStream_t s);
 
 // spatial domain decomposition into slabs (kernels_slab.cu); a.tiles are the
 // fixed 2048-particle io tiles over the active particles
