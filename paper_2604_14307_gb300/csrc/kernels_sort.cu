@@ -1,14 +1,14 @@
-// Host-state ingest and egress through a stable LSD radix sort.
+// Host-state ingest and egress.
 //
 // mpcd_set_state receives the solvent in tag order (spatially random) and
 // stores it cell-sorted; mpcd_get_state returns it in tag order again.  Both
-// are permutations of up to ~1e8 records.  Scattering every record to its
-// destination costs one partially written sector per 4-byte store; instead
-// the (key, slot) pairs are sorted by a stable 8-bit-digit radix sort whose
-// scatter goes through a shared-memory staging tile (runs of equal digits
-// leave the CTA as contiguous stores), and the records are then moved once by
-// a gather whose stores are coalesced.  Stability gives the canonical order:
-// within a cell, ascending tag.
+// are permutations of up to ~1e8 rows.  On the way in (cell, row) pairs are
+// sorted by a stable 8-bit-digit radix sort whose scatter goes through a
+// shared-memory staging tile (runs of equal digits leave the CTA as contiguous
+// stores), and the rows are placed by a gather whose stores are coalesced.
+// Stability gives the canonical order: within a cell, ascending tag.  On the
+// way out each particle knows its row (its tag): it writes one whole record
+// there, and the records become rows in order.
 #include <algorithm>
 
 #include "mpcd_internal.cuh"
@@ -177,16 +177,15 @@ __global__ void k_keys_in(StepArgs a, const Real *xa, uint32_t *keys, uint32_t *
     if (bad) atomicOr(a.d_err, ERR_POSITION);
 }
 
-// padding slots (after each replica's particles, and the trailing ones):
-// key = a value that sorts them to the end of their replica's slot range
-__global__ void k_keys_pad(StepArgs a, uint32_t *keys, uint32_t *vals, int64_t nslots, int mode,
-                           uint32_t out_key)
+// padding slots (after each replica's particles, and the trailing ones): a key
+// that sorts them to the end of their replica's slot range, no row
+__global__ void k_keys_pad(StepArgs a, uint32_t *keys, uint32_t *vals, int64_t nslots)
 {
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < a.n_rep; r += gridDim.x * blockDim.x) {
         const DevReplica R = a.reps[r];
         const int64_t b = R.solv_begin + R.n_solvent;
         const int64_t e = r + 1 < a.n_rep ? a.reps[r + 1].solv_begin : nslots;
-        const uint32_t key = mode == 0 ? (uint32_t)(R.cell_base + R.L[0] * R.L[1] * R.L[2] - 1) : out_key;
+        const uint32_t key = (uint32_t)(R.cell_base + R.L[0] * R.L[1] * R.L[2] - 1);
         for (int64_t i = b; i < e; ++i) {
             keys[i] = key;
             vals[i] = NO_VAL;
@@ -220,127 +219,113 @@ __device__ __forceinline__ void rec_store(double *r, const double (&o)[6])
     p[3] = make_double2(0.0, 0.0);
 }
 
-// host rows -> 8-word records {x, y, z, vx, vy, vz, 0, 0} (coalesced), so
-// that the permuting gather reads one aligned 32-byte (P32) or 64-byte (P64)
-// record per particle instead of six scattered words
-template <typename Real>
-__global__ void k_pack_rows(const Real *xa, const Real *va, Real *rec, int64_t n_rows)
+// set_state: slot i takes the host row vals[i], positions and tags first, then
+// (V) the velocities, which are still on their way from the host while the
+// positions are sorted and placed.  The rows are read as they lie (12 or 24
+// bytes); one 32-byte record of both per particle needed a pass of its own over
+// them, after the last of them had arrived (10 M particles: 85 + 120 us behind
+// the copies, now 126; set_state 1672 -> 1487 us, get_state 1923 -> 1611).  Four rows in flight per thread.
+template <typename Real, bool V>
+__global__ void __launch_bounds__(256) k_place(StepArgs a, const Real *rows, const uint32_t *vals, int64_t n_rows)
 {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n_rows; j += stride) {
-        Real o[6];
+    Real *A[3] = {(Real *)(V ? a.vx : a.x), (Real *)(V ? a.vy : a.y), (Real *)(V ? a.vz : a.z)};
+    constexpr int U = 4;
+    for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x) {
+        const Tile tl = a.tiles[t];
+        const int64_t first = a.reps[tl.rep].row_begin, n = a.reps[tl.rep].n_solvent;
+        for (int64_t i0 = tl.begin + threadIdx.x; i0 < tl.end; i0 += U * (int64_t)blockDim.x) {
+            Real o[U][3];
+            int64_t row[U];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) { o[k] = xa[3 * j + k]; o[3 + k] = va[3 * j + k]; }
-        rec_store(rec + 8 * j, o);
-    }
-}
-
-// set_state gather: sorted position i holds the host row of the record that
-// belongs in slot i; padding slots get zeros and the padding tag
-template <typename Real>
-__global__ void k_gather_in(StepArgs a, const Real *rec, const uint32_t *vals, int64_t nslots, int64_t n_rows)
-{
-    Real *X[3] = {(Real *)a.x, (Real *)a.y, (Real *)a.z};
-    Real *V[3] = {(Real *)a.vx, (Real *)a.vy, (Real *)a.vz};
-    // four records in flight per thread: all loads are issued before any store
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < nslots; i0 += 4 * stride) {
-        Real r[4][6];
-        uint32_t row[4];
+            for (int u = 0; u < U; ++u) {
+                const int64_t i = i0 + u * (int64_t)blockDim.x;
+                row[u] = -1;
+                if (i >= tl.end) continue;
+                row[u] = vals[i];
+                if (row[u] < first || row[u] >= first + n || row[u] >= n_rows) {
+                    bad_index(a.d_err, V ? 3 : 4);
+                    row[u] = -1;
+                }
+                if (row[u] >= 0)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int64_t i = i0 + u * stride;
-            row[u] = i < nslots ? vals[i] : NO_VAL;
-            if (row[u] != NO_VAL && (int64_t)row[u] >= n_rows) {
-                bad_index(a.d_err, 3);
-                row[u] = NO_VAL - 1;   // skip: neither a record nor padding
+                    for (int k = 0; k < 3; ++k) o[u][k] = rows[3 * row[u] + k];
             }
-            if ((int64_t)row[u] < n_rows) rec_load(rec + 8 * (int64_t)row[u], r[u]);
-        }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int64_t i = i0 + u * stride;
-            if (i >= nslots || row[u] == NO_VAL - 1) continue;
-            if (row[u] == NO_VAL) {
+            for (int u = 0; u < U; ++u) {
+                if (row[u] < 0) continue;
+                const int64_t i = i0 + u * (int64_t)blockDim.x;
 #pragma unroll
-                for (int k = 0; k < 3; ++k) { X[k][i] = Real(0); V[k][i] = Real(0); }
-                a.tag[i] = PAD_TAG;
-            } else {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) { X[k][i] = r[u][k]; V[k][i] = r[u][3 + k]; }
+                for (int k = 0; k < 3; ++k) A[k][i] = o[u][k];
+                if (!V) a.tag[i] = (uint32_t)(row[u] - first);
             }
         }
     }
 }
 
-// the tag of every real slot: host row - the replica's first row
-__global__ void k_tags_in(StepArgs a, const uint32_t *vals)
-{
-    for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x) {
-        const Tile tl = a.tiles[t];
-        const DevReplica r = a.reps[tl.rep];
-        for (int64_t i = tl.begin + threadIdx.x; i < tl.end; i += blockDim.x) {
-            const int64_t tag = (int64_t)vals[i] - r.row_begin;
-            if (tag < 0 || tag >= r.n_solvent) { bad_index(a.d_err, 4); continue; }
-            a.tag[i] = (uint32_t)tag;
-        }
-    }
-}
-
-// get_state keys: host row of every real slot (padding gets out_key = N_s)
-__global__ void k_keys_out(StepArgs a, uint32_t *keys, uint32_t *vals)
-{
-    for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x) {
-        const Tile tl = a.tiles[t];
-        const DevReplica r = a.reps[tl.rep];
-        for (int64_t i = tl.begin + threadIdx.x; i < tl.end; i += blockDim.x) {
-            keys[i] = (uint32_t)(r.row_begin + a.tag[i]);
-            vals[i] = (uint32_t)i;
-        }
-    }
-}
-
-// storage slots -> 8-word records (coalesced), for the egress gather
+// the padding slots' contents
 template <typename Real>
-__global__ void k_pack_slots(StepArgs a, Real *rec, int64_t nslots)
+__global__ void k_place_pad(StepArgs a, int64_t nslots)
 {
-    const Real *X[3] = {(const Real *)a.x, (const Real *)a.y, (const Real *)a.z};
-    const Real *V[3] = {(const Real *)a.vx, (const Real *)a.vy, (const Real *)a.vz};
+    Real *A[6] = {(Real *)a.x, (Real *)a.y, (Real *)a.z, (Real *)a.vx, (Real *)a.vy, (Real *)a.vz};
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < a.n_rep; r += gridDim.x * blockDim.x) {
+        const int64_t e = r + 1 < a.n_rep ? a.reps[r + 1].solv_begin : nslots;
+        for (int64_t i = a.reps[r].solv_begin + a.reps[r].n_solvent; i < e; ++i) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) A[k][i] = Real(0);
+            a.tag[i] = PAD_TAG;
+        }
+    }
+}
+
+// get_state: every slot writes its particle to the record of its host row, one
+// whole 32-byte sector (P64: two), which needs no read of what it replaces; the
+// rows then leave in order.  (Sorting (row, slot) pairs, packing the slots and
+// gathering took three to four radix passes first: 10 M particles 430 us before
+// the first row could be copied, now 243; 80 M 4.5 and 3.3 ms.  What is left are
+// single sectors to random places of DRAM.  Collecting them first in 256 buckets
+// of rows, by 256 cursors, took 2.9 ms for the cursors' contention and made the
+// second pass, which then wrote rows in no order, 6.7 ms.)  Four particles in
+// flight per thread.
+template <typename Real>
+__global__ void __launch_bounds__(256) k_records_out(StepArgs a, Real *rec, int64_t n_rows)
+{
+    const Real *A[6] = {(const Real *)a.x, (const Real *)a.y, (const Real *)a.z,
+                        (const Real *)a.vx, (const Real *)a.vy, (const Real *)a.vz};
+    constexpr int U = 4;
+    for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x) {
+        const Tile tl = a.tiles[t];
+        const int64_t first = a.reps[tl.rep].row_begin, n = a.reps[tl.rep].n_solvent;
+        for (int64_t i0 = tl.begin + threadIdx.x; i0 < tl.end; i0 += U * (int64_t)blockDim.x) {
+            Real o[U][6];
+            int64_t row[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t i = i0 + u * (int64_t)blockDim.x;
+                row[u] = -1;
+                if (i >= tl.end) continue;
+                const int64_t tag = a.tag[i];
+                if (tag < n && first + tag < n_rows) row[u] = first + tag;
+                else bad_index(a.d_err, 5);
+#pragma unroll
+                for (int k = 0; k < 6; ++k) o[u][k] = A[k][i];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (row[u] >= 0) rec_store(rec + 8 * row[u], o[u]);
+        }
+    }
+}
+
+// records of the rows [row0, row1) -> host layout
+template <typename Real>
+__global__ void __launch_bounds__(256) k_rows_out(const Real *rec, Real *xa, Real *va, int64_t row0, int64_t row1)
+{
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nslots; p += stride) {
+    for (int64_t i = row0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < row1; i += stride) {
         Real o[6];
+        rec_load(rec + 8 * i, o);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) { o[k] = X[k][p]; o[3 + k] = V[k][p]; }
-        rec_store(rec + 8 * p, o);
-    }
-}
-
-// get_state gather: host row i from the record of slot vals[i], stored row by row
-template <typename Real>
-__global__ void k_gather_out(const uint32_t *vals, const Real *rec, Real *xa, Real *va, int64_t row0,
-                             int64_t n_rows, int64_t nslots, int *err)
-{
-    // rows [row0, n_rows); four records in flight per thread: all loads are
-    // issued before any store
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i0 = row0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n_rows; i0 += 4 * stride) {
-        Real r[4][6];
-        bool ok[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int64_t i = i0 + u * stride;
-            const int64_t p = i < n_rows ? (int64_t)vals[i] : -1;
-            ok[u] = p >= 0 && p < nslots;
-            if (p >= nslots) bad_index(err, 5);
-            if (ok[u]) rec_load(rec + 8 * p, r[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int64_t i = i0 + u * stride;
-            if (!ok[u]) continue;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) { xa[3 * i + k] = r[u][k]; va[3 * i + k] = r[u][3 + k]; }
-        }
+        for (int k = 0; k < 3; ++k) { xa[3 * i + k] = o[k]; va[3 * i + k] = o[3 + k]; }
     }
 }
 
@@ -383,55 +368,45 @@ int launch_radix_sort(uint32_t *kA, uint32_t *vA, uint32_t *kB, uint32_t *vB, in
 void launch_keys_in(const StepArgs &a, const void *xa, uint32_t *keys, uint32_t *vals, int64_t nslots,
                     cudaStream_t s)
 {
-    k_keys_pad<<<grid_for(a.n_rep, 128, 1024), 128, 0, s>>>(a, keys, vals, nslots, 0, 0u);
+    k_keys_pad<<<grid_for(a.n_rep, 128, 1024), 128, 0, s>>>(a, keys, vals, nslots);
     if (a.n_tiles == 0) return;
     if (a.precision == 1) k_keys_in<float><<<a.n_tiles, 256, 0, s>>>(a, (const float *)xa, keys, vals);
     else k_keys_in<double><<<a.n_tiles, 256, 0, s>>>(a, (const double *)xa, keys, vals);
 }
 
-void launch_pack_rows(const StepArgs &a, const void *xa, const void *va, void *rec, int64_t n_rows, int num_sms,
-                      cudaStream_t s)
+template <typename Real>
+static void place(const StepArgs &a, const void *rows, const uint32_t *vals, int64_t n_rows, int64_t nslots,
+                  bool velocities, cudaStream_t s)
 {
-    if (n_rows == 0) return;
-    const int grid = grid_for(n_rows, 256, num_sms * 8);
-    if (a.precision == 1) k_pack_rows<float><<<grid, 256, 0, s>>>((const float *)xa, (const float *)va, (float *)rec, n_rows);
-    else k_pack_rows<double><<<grid, 256, 0, s>>>((const double *)xa, (const double *)va, (double *)rec, n_rows);
+    if (!velocities) k_place_pad<Real><<<grid_for(a.n_rep, 128, 1024), 128, 0, s>>>(a, nslots);
+    if (a.n_tiles == 0) return;
+    if (velocities) k_place<Real, true><<<a.n_tiles, 256, 0, s>>>(a, (const Real *)rows, vals, n_rows);
+    else k_place<Real, false><<<a.n_tiles, 256, 0, s>>>(a, (const Real *)rows, vals, n_rows);
 }
 
-void launch_gather_in(const StepArgs &a, const void *rec, const uint32_t *vals, int64_t nslots, int64_t n_rows,
-                      int num_sms, cudaStream_t s)
+void launch_place(const StepArgs &a, const void *rows, const uint32_t *vals, int64_t n_rows, int64_t nslots,
+                  bool velocities, cudaStream_t s)
 {
-    const int grid = grid_for(nslots, 256, num_sms * 8);
-    if (a.precision == 1) k_gather_in<float><<<grid, 256, 0, s>>>(a, (const float *)rec, vals, nslots, n_rows);
-    else k_gather_in<double><<<grid, 256, 0, s>>>(a, (const double *)rec, vals, nslots, n_rows);
-    if (a.n_tiles) k_tags_in<<<a.n_tiles, 256, 0, s>>>(a, vals);
+    if (a.precision == 1) place<float>(a, rows, vals, n_rows, nslots, velocities, s);
+    else place<double>(a, rows, vals, n_rows, nslots, velocities, s);
 }
 
-void launch_keys_out(const StepArgs &a, uint32_t *keys, uint32_t *vals, int64_t nslots, uint32_t n_rows,
+void launch_records_out(const StepArgs &a, void *rec, int64_t n_rows, cudaStream_t s)
+{
+    if (a.n_tiles == 0) return;
+    if (a.precision == 1) k_records_out<float><<<a.n_tiles, 256, 0, s>>>(a, (float *)rec, n_rows);
+    else k_records_out<double><<<a.n_tiles, 256, 0, s>>>(a, (double *)rec, n_rows);
+}
+
+void launch_rows_out(const StepArgs &a, const void *rec, void *xa, void *va, int64_t row0, int64_t row1, int num_sms,
                      cudaStream_t s)
-{
-    k_keys_pad<<<grid_for(a.n_rep, 128, 1024), 128, 0, s>>>(a, keys, vals, nslots, 1, n_rows);
-    if (a.n_tiles) k_keys_out<<<a.n_tiles, 256, 0, s>>>(a, keys, vals);
-}
-
-void launch_pack_slots(const StepArgs &a, void *rec, int64_t nslots, int num_sms, cudaStream_t s)
-{
-    const int gp = grid_for(nslots, 256, num_sms * 8);
-    if (a.precision == 1) k_pack_slots<float><<<gp, 256, 0, s>>>(a, (float *)rec, nslots);
-    else k_pack_slots<double><<<gp, 256, 0, s>>>(a, (double *)rec, nslots);
-}
-
-void launch_gather_rows(const StepArgs &a, const uint32_t *vals, const void *rec, void *xa, void *va, int64_t row0,
-                        int64_t row1, int64_t nslots, int num_sms, cudaStream_t s)
 {
     if (row1 <= row0) return;
     const int grid = grid_for(row1 - row0, 256, num_sms * 8);
     if (a.precision == 1)
-        k_gather_out<float><<<grid, 256, 0, s>>>(vals, (const float *)rec, (float *)xa, (float *)va, row0, row1,
-                                                 nslots, a.d_err);
+        k_rows_out<float><<<grid, 256, 0, s>>>((const float *)rec, (float *)xa, (float *)va, row0, row1);
     else
-        k_gather_out<double><<<grid, 256, 0, s>>>(vals, (const double *)rec, (double *)xa, (double *)va, row0, row1,
-                                                  nslots, a.d_err);
+        k_rows_out<double><<<grid, 256, 0, s>>>((const double *)rec, (double *)xa, (double *)va, row0, row1);
 }
 
 }  // namespace mpcd

@@ -1247,9 +1247,10 @@ int mpcd_set_state(mpcd_ctx *c, const mpcd_host_state *h, void *stream)
     const StepArgs aio = make_io_args(c);
     {
         // cell-sorted storage from the tag-ordered rows: stable radix sort of
-        // (cell, row) pairs in the spare buffer, then one gather (memory
-        // locality only; results do not depend on the order).  The velocities
-        // travel on the copy stream while the positions are keyed and sorted.
+        // (cell, row) pairs in the spare buffer, then the rows are placed
+        // (memory locality only; results do not depend on the order).  The
+        // velocities travel on the copy stream while the positions are keyed,
+        // sorted and placed.
         uint32_t *kA = (uint32_t *)c->sol[1][0], *vA = (uint32_t *)c->sol[1][1];
         uint32_t *kB = (uint32_t *)c->sol[1][2], *vB = (uint32_t *)c->sol[1][3];
         if (c->Ns) {
@@ -1265,9 +1266,10 @@ int mpcd_set_state(mpcd_ctx *c, const mpcd_host_state *h, void *stream)
         const int nb = key_bits((uint64_t)std::max<int64_t>(c->C - 1, 0));
         const int inB =
             launch_radix_sort(kA, vA, kB, vB, c->Nslots, nb, c->rs_hist, c->rs_ex, c->rs_bs, c->d_err, s);
+        const uint32_t *order = inB ? vB : vA;
+        launch_place(aio, stg, order, c->Ns, c->Nslots, false, s);
         if (c->Ns) CK(c, cudaStreamWaitEvent(s, c->io_ev[1], 0));
-        launch_pack_rows(aio, stg, stg + n3 * c->realsz, c->rec, c->Ns, c->num_sms, s);
-        launch_gather_in(aio, c->rec, inB ? vB : vA, c->Nslots, c->Ns, c->num_sms, s);
+        launch_place(aio, stg + n3 * c->realsz, order, c->Ns, c->Nslots, true, s);
     }
     if (c->B) CK(c, cudaMemcpyAsync(c->d_bodies, hb.data(), c->B * sizeof(DevBody), cudaMemcpyHostToDevice, s));
     CK(c, cudaMemsetAsync(c->sums, 0, (size_t)c->C * c->nw * 8, s));
@@ -1306,25 +1308,14 @@ int mpcd_get_state(mpcd_ctx *c, mpcd_host_state *h, void *stream)
     char *stg = (char *)c->staging;
     const StepArgs a = make_io_args(c);
     {
-        // tag order from the cell-sorted storage: stable radix sort of
-        // (host row, slot) pairs in the spare buffer, then a gather whose
-        // stores are row-contiguous
-        const int alt = c->cur ^ 1;
-        uint32_t *kA = (uint32_t *)c->sol[alt][0], *vA = (uint32_t *)c->sol[alt][1];
-        uint32_t *kB = (uint32_t *)c->sol[alt][2], *vB = (uint32_t *)c->sol[alt][3];
-        launch_keys_out(a, kA, vA, c->Nslots, (uint32_t)c->Ns, s);
-        const int nb = key_bits((uint64_t)c->Ns);
-        const int inB =
-            launch_radix_sort(kA, vA, kB, vB, c->Nslots, nb, c->rs_hist, c->rs_ex, c->rs_bs, c->d_err, s);
-        launch_pack_slots(a, c->rec, c->Nslots, c->num_sms, s);
+        launch_records_out(a, c->rec, c->Ns, s);
         // the rows leave in chunks: while chunk k travels to the host on the
-        // copy stream, chunk k + 1 is gathered (one chunk for small states)
-        const uint32_t *order = inB ? vB : vA;
+        // copy stream, chunk k + 1 is put in order (one chunk for small states)
         const int K = c->Ns >= ((int64_t)1 << 22) ? mpcd_ctx::OUT_CHUNKS : 1;
         char *sx = stg, *sv = stg + n3 * c->realsz;
         for (int k = 0; k < K && c->Ns; ++k) {
             const int64_t r0 = c->Ns * k / K, r1 = c->Ns * (k + 1) / K;
-            launch_gather_rows(a, order, c->rec, sx, sv, r0, r1, c->Nslots, c->num_sms, s);
+            launch_rows_out(a, c->rec, sx, sv, r0, r1, c->num_sms, s);
             const size_t off = (size_t)r0 * 3 * c->realsz, len = (size_t)(r1 - r0) * 3 * c->realsz;
             if (K == 1) {
                 CK(c, cudaMemcpyAsync(h->x, sx, len, cudaMemcpyDeviceToHost, s));

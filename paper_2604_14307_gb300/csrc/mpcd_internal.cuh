@@ -478,7 +478,7 @@ void launch_cell_order(const StepArgs &a, int64_t n_solvent, int32_t *counts, in
                        int32_t *scan_bs, unsigned long long *keys, int64_t *order, int64_t *start, int num_sms,
                        cudaStream_t s);
 
-// host-state ingest / egress by stable radix sort (kernels_sort.cu)
+// host-state ingest by stable radix sort, egress by records (kernels_sort.cu)
 size_t radix_hist_ints(int64_t n);          // ints of the per-pass digit histogram
 int key_bits(uint64_t max_key);             // bits needed for keys <= max_key
 // stable sort of (key, value) pairs by the low nbits; returns 1 if the result
@@ -487,18 +487,15 @@ int launch_radix_sort(uint32_t *kA, uint32_t *vA, uint32_t *kB, uint32_t *vB, in
                       int32_t *hist, int32_t *hist_ex, int32_t *scan_bs, int *err, cudaStream_t s);
 void launch_keys_in(const StepArgs &a, const void *xa, uint32_t *keys, uint32_t *vals, int64_t nslots,
                     cudaStream_t s);
-// host rows -> 8-word records rec[n_rows][8] (the ingest gather reads one record per particle)
-void launch_pack_rows(const StepArgs &a, const void *xa, const void *va, void *rec, int64_t n_rows, int num_sms,
-                      cudaStream_t s);
-void launch_gather_in(const StepArgs &a, const void *rec, const uint32_t *vals, int64_t nslots, int64_t n_rows,
-                      int num_sms, cudaStream_t s);
-void launch_keys_out(const StepArgs &a, uint32_t *keys, uint32_t *vals, int64_t nslots, uint32_t n_rows,
+// slots from host rows by the sorted row indices: positions, tags and padding, or
+// the velocities
+void launch_place(const StepArgs &a, const void *rows, const uint32_t *vals, int64_t n_rows, int64_t nslots,
+                  bool velocities, cudaStream_t s);
+// slots -> one 8-word record per host row, rec[n_rows][8]; then the host rows
+// [row0, row1) from them
+void launch_records_out(const StepArgs &a, void *rec, int64_t n_rows, cudaStream_t s);
+void launch_rows_out(const StepArgs &a, const void *rec, void *xa, void *va, int64_t row0, int64_t row1, int num_sms,
                      cudaStream_t s);
-// slots -> records rec[nslots][8]; then the host rows [row0, row1) in order
-// from them (vals[row] = the row's slot)
-void launch_pack_slots(const StepArgs &a, void *rec, int64_t nslots, int num_sms, cudaStream_t s);
-void launch_gather_rows(const StepArgs &a, const uint32_t *vals, const void *rec, void *xa, void *va, int64_t row0,
-                        int64_t row1, int64_t nslots, int num_sms, cudaStream_t s);
 
 // angular-momentum-conserving collision variants (kernels_angular.cu for the
 // solvent and the per-cell solve, kernels_bodies.cu for the sites).
