@@ -155,6 +155,8 @@ __global__ void __launch_bounds__(256) k_ang_collide(StepArgs a)
             int c[4];
             int Q[4][3];
             cells4(x, y, z, S, r, c, Q);
+            Real nn[4][3];
+            if (RULE == 1) at_normals4(a, r, step, tg, nv, i, nn);
             CellParams<Real> p[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) p[j] = get_params<Real>(a.params, j < nv ? c[j] : r.cell_base);
@@ -167,11 +169,9 @@ __global__ void __launch_bounds__(256) k_ang_collide(StepArgs a)
                 if (RULE == 0) {
                     srd_rotate<Real>(p[j], ca, sa, rx, ry, rz);
                 } else {
-                    Real nn[3];
-                    normals3(draw(r, step, tg[j], TAG_AT, 0u), nn);
-                    rx = p[j].ux + sc * nn[0] - p[j].ax;
-                    ry = p[j].uy + sc * nn[1] - p[j].ay;
-                    rz = p[j].uz + sc * nn[2] - p[j].az;
+                    rx = p[j].ux + sc * nn[j][0] - p[j].ax;
+                    ry = p[j].uy + sc * nn[j][1] - p[j].ay;
+                    rz = p[j].uz + sc * nn[j][2] - p[j].az;
                 }
                 vx[j] = on ? rx : vx[j];
                 vy[j] = on ? ry : vy[j];
@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(256) k_ang_apply(StepArgs a)
             }
             if (STREAM) {
                 bin4<Real, RULE, true>(a, x, y, z, vx, vy, vz, tg, nv, sF, r.L[0], r.L[1], r.L[2], r.cell_base, r, step,
-                                       m, sc, sums, a.n_cells);
+                                       m, sc, sums, a.n_cells, i);
                 st4v(X + i, x); st4v(Y + i, y); st4v(Z + i, z);
             }
             st4v(VX + i, vx); st4v(VY + i, vy); st4v(VZ + i, vz);

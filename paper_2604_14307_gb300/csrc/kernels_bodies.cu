@@ -971,7 +971,11 @@ __global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_si
         if (a.rule == 1) {
             normals3(draw(r, step, (uint32_t)(r.site_id_base + (g - r.site_begin)), TAG_AT, 0u), xi);
             const Real sc = site_scale<Real>(a, ts);
-            xi[0] *= sc; xi[1] *= sc; xi[2] *= sc;
+            Real *XI = reinterpret_cast<Real *>(a.site_xi);
+            for (int k = 0; k < 3; ++k) {
+                xi[k] *= sc;
+                XI[k * NS + g] = xi[k];
+            }
         }
         const int cell = r.cell_base + (N > 0 ? cells[N > 0 ? s : 0] : a.site_cell[g]);
         if (!mine) return;
@@ -1003,8 +1007,8 @@ __global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_si
 // transferred to the body (Eqs. 3-4); k_body_impulse adds them in FP64.
 // the collision rule for one site: v -> vn with the parameters p of its cell
 template <typename Real>
-__device__ __forceinline__ void site_rule(const StepArgs &a, const DevReplica &r, int64_t step, int64_t g, int64_t t,
-                                          const Real (&v)[3], const Real (&p)[8], Real (&vn)[3])
+__device__ __forceinline__ void site_rule(const StepArgs &a, int64_t g, const Real (&v)[3], const Real (&p)[8],
+                                          Real (&vn)[3])
 {
     vn[0] = v[0]; vn[1] = v[1]; vn[2] = v[2];
     if (p[3] >= Real(0)) {
@@ -1019,10 +1023,8 @@ __device__ __forceinline__ void site_rule(const StepArgs &a, const DevReplica &r
             vn[1] = p[1] + p[3] * (w[1] * ca + cy * sa + p[5] * tt);
             vn[2] = p[2] + p[3] * (w[2] * ca + cz * sa + p[6] * tt);
         } else {
-            Real xi[3];
-            normals3(draw(r, step, (uint32_t)(r.site_id_base + (g - r.site_begin)), TAG_AT, 0u), xi);
-            const Real sc = site_scale<Real>(a, t);
-            for (int k = 0; k < 3; ++k) vn[k] = p[k] + sc * xi[k] - p[4 + k];
+            const Real *XI = reinterpret_cast<const Real *>(a.site_xi);   // the draws of the PRE pass
+            for (int k = 0; k < 3; ++k) vn[k] = p[k] + XI[k * a.n_sites + g] - p[4 + k];
         }
     }
 }
@@ -1074,7 +1076,7 @@ __global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_si
             Real p[8];
             load_cell<Real>(a, cell, p);
             const Real m = site_mass<Real>(a, t);
-            site_rule<Real>(a, r, step, g, t, v, p, vn);
+            site_rule<Real>(a, g, v, p, vn);
             if constexpr (ANG) {
                 const Real xs[3] = {x[0], x[1], x[2]};
                 int Q[3];
@@ -1227,7 +1229,7 @@ __global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_ang_si
         const Real m = site_mass<Real>(a, t);
         Real u[3], p[8];
         load_cell<Real>(a, cell, p);
-        site_rule<Real>(a, r, step, g, t, v, p, u);
+        site_rule<Real>(a, g, v, p, u);
         const Real xs[3] = {x[0], x[1], x[2]};
         int Qi[3];
         site_lattice_q(xs, sS, Qi);

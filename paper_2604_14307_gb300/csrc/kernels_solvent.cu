@@ -91,6 +91,8 @@ __global__ void __launch_bounds__(512) k_solvent(StepArgs a)
                 uint4 t4 = __ldcs(reinterpret_cast<const uint4 *>(a.tag + i));
                 tg[0] = t4.x; tg[1] = t4.y; tg[2] = t4.z; tg[3] = t4.w;
             }
+            Real nn[4][3];
+            if (COLLIDE && RULE == 1) at_normals4(a, rr, step, tg, nv, i, nn);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 if (j >= nv) break;
@@ -102,11 +104,9 @@ __global__ void __launch_bounds__(512) k_solvent(StepArgs a)
                         if (RULE == 0) {
                             srd_rotate<Real>(p, ca, sa, vx[j], vy[j], vz[j]);
                         } else {
-                            Real n[3];
-                            normals3(draw(rr, step, tg[j], TAG_AT, 0u), n);
-                            vx[j] = p.ux + sc * n[0] - p.ax;
-                            vy[j] = p.uy + sc * n[1] - p.ay;
-                            vz[j] = p.uz + sc * n[2] - p.az;
+                            vx[j] = p.ux + sc * nn[j][0] - p.ax;
+                            vy[j] = p.uy + sc * nn[j][1] - p.ay;
+                            vz[j] = p.uz + sc * nn[j][2] - p.az;
                         }
                     }
                 }
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(512) k_solvent(StepArgs a)
                 }
             }
             if (BIN) bin4<Real, RULE, COLLIDE>(a, x, y, z, vx, vy, vz, tg, nv, sF + 3, L0, L1, L2, base, rr, step,
-                                                m, sc, sums, C);
+                                                m, sc, sums, C, i);
             if (STREAM) { st4(X + i, x); st4(Y + i, y); st4(Z + i, z); }
             if (COLLIDE || (STREAM && a.accel)) { st4(VX + i, vx); st4(VY + i, vy); st4(VZ + i, vz); }
         }
@@ -395,13 +395,7 @@ __global__ void __maxnreg__((StRegs<Real, RULE>::n)) k_solvent_staged(StepArgs a
                     p[j] = get_params<Real>(a.params, c);
                 }
                 Real nn[4][3];
-                if (RULE == 1) {
-                    // the four particles' Philox blocks are independent: draw
-                    // them all (a lane past the tile end draws for id 0), so
-                    // that their dependent rounds interleave
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) normals3(draw(rr, step, tg[j], TAG_AT, 0u), nn[j]);
-                }
+                if (RULE == 1) at_normals4(a, rr, step, tg, nv, mt.beg + i, nn);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     // the rule is applied to every slot and kept where it
@@ -441,7 +435,7 @@ __global__ void __maxnreg__((StRegs<Real, RULE>::n)) k_solvent_staged(StepArgs a
                     }
             }
             if (BIN) bin4<Real, RULE, COLLIDE>(a, x, y, z, vx, vy, vz, tg, nv, sF + 3, L0, L1, L2, base, rr, step,
-                                                m, sc, sums, C);
+                                                m, sc, sums, C, mt.beg + i);
             if (nv > 0) {
                 if (STREAM) { sst4(S[0] + i, x); sst4(S[1] + i, y); sst4(S[2] + i, z); }
                 if (COLLIDE || (STREAM && a.accel)) { sst4(S[3] + i, vx); sst4(S[4] + i, vy); sst4(S[5] + i, vz); }
@@ -619,13 +613,7 @@ __global__ void __launch_bounds__(544) k_solvent_ws(StepArgs a, int cap)
                     p[j] = get_params<Real>(a.params, c);
                 }
                 Real nn[4][3];
-                if (RULE == 1) {
-                    // the four particles' Philox blocks are independent: draw
-                    // them all (a lane past the tile end draws for id 0), so
-                    // that their dependent rounds interleave
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) normals3(draw(rr, step, tg[j], TAG_AT, 0u), nn[j]);
-                }
+                if (RULE == 1) at_normals4(a, rr, step, tg, nv, mt.beg + i, nn);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     // the rule is applied to every slot and kept where it
@@ -665,7 +653,7 @@ __global__ void __launch_bounds__(544) k_solvent_ws(StepArgs a, int cap)
                     }
             }
             if (BIN) bin4<Real, RULE, COLLIDE>(a, x, y, z, vx, vy, vz, tg, nv, sF + 3, L0, L1, L2, base, rr, step,
-                                                m, sc, sums, C);
+                                                m, sc, sums, C, mt.beg + i);
             if (nv > 0) {
                 if (STREAM) { sst4(S[0] + i, x); sst4(S[1] + i, y); sst4(S[2] + i, z); }
                 if (COLLIDE || (STREAM && a.accel)) { sst4(S[3] + i, vx); sst4(S[4] + i, vy); sst4(S[5] + i, vz); }
@@ -841,13 +829,7 @@ __global__ void __maxnreg__((WtRegs<Real, RULE>::n)) k_solvent_wt(StepArgs a, in
                     p[j] = get_params<Real>(a.params, c);
                 }
                 Real nn[4][3];
-                if (RULE == 1) {
-                    // the four particles' Philox blocks are independent: draw
-                    // them all (a lane past the tile end draws for id 0), so
-                    // that their dependent rounds interleave
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) normals3(draw(rr, step, tg[j], TAG_AT, 0u), nn[j]);
-                }
+                if (RULE == 1) at_normals4(a, rr, step, tg, nv, mt.beg + i, nn);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     // the rule is applied to every slot and kept where it
@@ -887,7 +869,7 @@ __global__ void __maxnreg__((WtRegs<Real, RULE>::n)) k_solvent_wt(StepArgs a, in
                     }
             }
             if (BIN) bin4<Real, RULE, COLLIDE>(a, x, y, z, vx, vy, vz, tg, nv, sF + 3, L0, L1, L2, base, rr, step,
-                                                m, sc, sums, C);
+                                                m, sc, sums, C, mt.beg + i);
             if (nv > 0) {
                 if (STREAM) { sst4(S[0] + i, x); sst4(S[1] + i, y); sst4(S[2] + i, z); }
                 if (COLLIDE || (STREAM && a.accel)) { sst4(S[3] + i, vx); sst4(S[4] + i, vy); sst4(S[5] + i, vz); }

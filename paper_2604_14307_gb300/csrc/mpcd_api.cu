@@ -90,6 +90,12 @@ struct mpcd_ctx {
     void *sums = nullptr, *params = nullptr, *dbg_sums = nullptr;
     bool debug = false;
     void *site_v = nullptr;
+    void *site_xi = nullptr;        // MPCD-AT: [3][n_sites] scaled normals of the sites
+    // MPCD-AT: the normals drawn by the last binning, slot by slot, for the
+    // collision of step noise_step, while noise_ok (the slots keep their order)
+    void *noise[3] = {};
+    bool noise_ok = false;
+    int64_t noise_step = 0;
     int32_t *site_cell = nullptr;
     int64_t *d_step = nullptr;
     int *d_err = nullptr;
@@ -110,7 +116,8 @@ struct mpcd_ctx {
     std::map<std::string, KStat> prof;
     std::vector<cudaEvent_t> evpool;
 
-    std::map<std::tuple<int, int64_t, bool, int>, GraphEntry> graphs;   // (piece, solvent buffer in use before it)
+    // (piece, solvent buffer in use before it, whether its first collision finds its normals)
+    std::map<std::tuple<int, int64_t, bool, int, bool>, GraphEntry> graphs;
     int64_t step_off = 0;           // steps enqueued since the device counter last advanced
     cudaStream_t cap_stream = nullptr;
     cudaStream_t io_stream = nullptr;           // host copies that overlap with kernels
@@ -265,6 +272,8 @@ StepArgs make_args(const mpcd_ctx *c)
     a.cent64 = c->d_cent64;
     a.cent32 = c->d_cent32;
     a.site_v = c->site_v;
+    a.site_xi = c->site_xi;
+    for (int k = 0; k < 3; ++k) a.noise[k] = c->noise[k];
     a.site_cell = c->site_cell;
     a.n_sites = c->Nsite;
     a.d_step = c->d_step;
@@ -339,6 +348,7 @@ int slab_set_count(mpcd_ctx *c, int64_t n)
 {
     c->reps[0].n_solvent = n;
     c->Ns = n;
+    c->noise_ok = false;
     CK(c, cudaMemcpy(c->d_reps, c->reps.data(), c->reps.size() * sizeof(DevReplica), cudaMemcpyHostToDevice));
     build_tiles(c);
     int e = upload_tiles(c);
@@ -428,22 +438,28 @@ bool staged_fits(const mpcd_ctx *c, int tile, int mode, int block)
 // FP32, at least four 1024-particle tiles for each of three CTAs per SM: the
 // staged pass, whose work counter evens out the SMs that the site/body chain
 // shares (us per step, per-warp ring against staged: 80 M particles 1940 and
-// 1794, 17 M in 512 boxes 450 and 398, 17 M of solvent alone 504 and 462, 9 M
-// MPCD-AT 736 and 559, 2.6 M 110 and 104; 0.6 M MPCD-AT 65 and 69).  Boxes that
-// cut the tiles short keep the ring.  Otherwise FP32 takes a ring per warp of
-// 128-particle tiles; MPCD-AT beside colloids with 384 threads, because 512 of
+// 1794, 17 M in 512 boxes 450 and 398, 17 M of solvent alone 504 and 462, 2.6 M
+// 110 and 104; 0.6 M MPCD-AT 65 and 69).  SRD takes 3 CTAs of 128 threads.
+// MPCD-AT gains more from warps (2 x 256 against them: 34 M 1192 and 1456, 17 M in
+// 512 boxes 646 and 750, 17 M alone 692 and 790), unless the chain is as long as
+// the pass: shapes of many centres, whose forces take a warp per body, get the
+// registers that 3 x 128 threads leave (9 M, 1120 bodies: 496 and 608).  Boxes
+// that cut the tiles short keep the ring.  Otherwise FP32 takes a ring per warp
+// of 128-particle tiles; MPCD-AT beside colloids with 384 threads, because 512 of
 // its 128 registers fill the SM and the site/body chain then waits for the
-// whole pass (0.6 M particles, 221 bodies: 144 and 65 us per step).  FP64 keeps
+// whole pass (0.6 M particles, 221 bodies: 135 and 56 us per step).  FP64 keeps
 // its own pipe full in any form; a ring per warp in 256 threads leaves the most
 // room beside it (warp-specialised with 1024-particle tiles against it: 0.3 M
 // particles with 113 bodies 184 and 167 us per step, 10 M 1990 and 1737), MPCD-AT
-// with its 160 registers and more takes direct loads (540 and 328).
+// with its 128 registers and spills takes direct loads (295 and 241).
 void default_tuning(mpcd_ctx *c)
 {
     const int period = c->tune.sort_period;
     const bool p32 = c->prm.precision == MPCD_P32;
     if (p32 && c->Ns >= (int64_t)4 * 3 * c->num_sms * 1024 && c->Ns >= (int64_t)4096 * c->nrep) {
-        c->tune = mpcd_tuning{128, 1024, 3, period, 1};
+        c->tune = c->prm.rule == MPCD_SRD ? mpcd_tuning{128, 1024, 3, period, 1}
+                  : c->max_cent > 2       ? mpcd_tuning{128, 512, 3, period, 1}
+                                          : mpcd_tuning{256, 1024, 2, period, 1};
         return;
     }
     if (!p32 && c->prm.rule == MPCD_AT)
@@ -523,9 +539,23 @@ int k_vacf(mpcd_ctx *c, cudaStream_t s)
     return timed(c, "vacf", 0, s, [&] { launch_vacf_sample(a, c->vacf, s); });
 }
 
+// the step that a launch works on
+int64_t step_now(const mpcd_ctx *c) { return c->step + c->step_off; }
+
+bool noise_fits(const mpcd_ctx *c) { return c->noise_ok && c->noise_step == step_now(c); }
+
+// a pass has binned for the collision of `step` (and kept its normals)
+void noise_kept(mpcd_ctx *c, int64_t step)
+{
+    c->noise_ok = c->noise[0] != nullptr;
+    c->noise_step = step;
+}
+
 int k_solvent(mpcd_ctx *c, int flags, cudaStream_t s)
 {
     StepArgs a = make_args(c);
+    a.noise_in = noise_fits(c) ? 1 : 0;
+    if (flags & SOLV_BIN) noise_kept(c, step_now(c) + (flags & SOLV_COLLIDE ? 1 : 0));
     LaunchCfg cfg = solvent_cfg(c);
     const char *name = flags == (SOLV_COLLIDE | SOLV_STREAM | SOLV_BIN) ? "solvent_fused"
                        : flags == SOLV_COLLIDE                          ? "solvent_collide"
@@ -616,6 +646,7 @@ int do_sort(mpcd_ctx *c, int canonical, cudaStream_t s, bool from_words = false)
     if (e) return e;
     c->cur = nxt;
     c->since_sort = 0;
+    c->noise_ok = false;
     return MPCD_OK;
 }
 
@@ -631,6 +662,8 @@ int k_ang(mpcd_ctx *c, int phase, cudaStream_t s)
     const double bytes[] = {N * 9 * r + C * (c->param_bytes + AW_SOLVENT * 8.0) + at, C * (2.0 * words * 8 + rec),
                             N * 9 * r + C * rec, N * 12 * r + C * (rec + c->nw * 8.0) + at};
     StepArgs a = make_args(c);
+    a.noise_in = noise_fits(c) ? 1 : 0;
+    if (phase == ANG_STREAM) noise_kept(c, step_now(c) + 1);
     return timed(c, names[phase], bytes[phase], s, [&] { launch_angular(a, phase, c->num_sms, s); });
 }
 
@@ -730,10 +763,15 @@ int tail_step(mpcd_ctx *c, cudaStream_t s)     // the last step's collision
     return e;
 }
 
+int64_t piece_steps(const Piece &p)   // steps that the piece completes
+{
+    return p.kind == PIECE_HEAD ? 0 : (p.kind == PIECE_TAIL ? 1 : p.steps);
+}
+
 int enqueue_piece(mpcd_ctx *c, const Piece &p, cudaStream_t s)
 {
     int e = MPCD_OK;
-    const int64_t n = p.kind == PIECE_HEAD ? 0 : (p.kind == PIECE_TAIL ? 1 : p.steps);
+    const int64_t n = piece_steps(p);
     c->step_off = 0;
     if (p.kind == PIECE_HEAD) e = head_step(c, s);
     if (p.kind == PIECE_TAIL) e = tail_step(c, s);
@@ -790,11 +828,12 @@ std::vector<Piece> plan_steps(mpcd_ctx *c, int64_t n, bool recorded)
 // launch a piece as a CUDA graph, recording it first if it is new
 int replay_piece(mpcd_ctx *c, const Piece &p, cudaStream_t s)
 {
-    const auto key = std::make_tuple(p.kind, p.steps, p.sort, c->cur);
+    const auto key = std::make_tuple(p.kind, p.steps, p.sort, c->cur, noise_fits(c));
     auto it = c->graphs.find(key);
     if (it == c->graphs.end()) {
         const int cur0 = c->cur;
-        const int64_t since0 = c->since_sort;
+        const int64_t since0 = c->since_sort, nstep0 = c->noise_step;
+        const bool noise0 = c->noise_ok;
         CK(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
         int e = enqueue_piece(c, p, c->cap_stream);
         cudaGraph_t g = nullptr;
@@ -803,6 +842,8 @@ int replay_piece(mpcd_ctx *c, const Piece &p, cudaStream_t s)
         ge.cur_end = c->cur;
         c->cur = cur0;
         c->since_sort = since0;
+        c->noise_ok = noise0;
+        c->noise_step = nstep0;
         if (e) {
             if (g) cudaGraphDestroy(g);
             return e;
@@ -1061,6 +1102,10 @@ int mpcd_create(const mpcd_params *params, int32_t n_shapes, const mpcd_shape_de
         ok &= (c->d_cent32 = (float4 *)A((size_t)std::max<int64_t>(1, nc) * sizeof(float4))) != nullptr;
     }
     ok &= (c->site_v = A(std::max<int64_t>(1, c->Nsite) * 3 * c->realsz)) != nullptr;
+    if (p.rule == MPCD_AT) {
+        ok &= (c->site_xi = A(std::max<int64_t>(1, c->Nsite) * 3 * c->realsz)) != nullptr;
+        for (int k = 0; k < 3; ++k) ok &= (c->noise[k] = A(c->Nslots * c->realsz)) != nullptr;
+    }
     ok &= (c->site_cell = (int32_t *)A(std::max<int64_t>(1, c->Nsite) * 4)) != nullptr;
     ok &= (c->d_step = (int64_t *)A(8)) != nullptr;
     ok &= (c->d_err = (int *)A(8)) != nullptr;
@@ -1292,6 +1337,7 @@ int mpcd_set_state(mpcd_ctx *c, const mpcd_host_state *h, void *stream)
     c->step = h->step;
     c->since_sort = 0;
     c->last_key = -1;
+    c->noise_ok = false;
     c->have_state = true;
     return MPCD_OK;
 }
@@ -1397,8 +1443,11 @@ int mpcd_step(mpcd_ctx *c, int64_t nsteps, void *stream)
         const int e = recorded ? replay_piece(c, p, s) : enqueue_piece(c, p, s);
         if (e) return e;
         c->since_sort = since;
+        // what the piece leaves, recorded now or before
+        if (const int64_t n = piece_steps(p)) count_steps(c, n);
+        noise_kept(c, c->step);
+        if (p.kind == PIECE_TAIL || p.sort) c->noise_ok = false;
     }
-    count_steps(c, nsteps);
     return MPCD_OK;
 }
 
@@ -2054,6 +2103,7 @@ int mpcd_autotune(mpcd_ctx *c, int32_t steps_per_trial, void *stream)
         c->step = step0;
         c->since_sort = since0;
         c->last_key = key0;
+        c->noise_ok = false;
         return MPCD_OK;
     };
     mpcd_tuning best = c->tune;

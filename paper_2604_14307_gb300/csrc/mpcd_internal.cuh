@@ -104,6 +104,8 @@ struct StepArgs {
     void *sums;                     // [nw][n_cells]
     void *params;                   // [n_cells] records
     void *dbg_sums;                 // copy of the sums when debugging, else null
+    void *noise[3];                 // MPCD-AT: normals of every slot, kept from the binning to the collision (null: not)
+    int32_t noise_in;               // they are those of this collision, in the present slot order
     int64_t n_cells;
     int32_t nw;
     DevBody *bodies;
@@ -129,6 +131,7 @@ struct StepArgs {
     double *cent64;                 // per body centre: Q c in the space frame [n][3] (this step's pose)
     float4 *cent32;                 // the same rounded to float
     void *site_v;                   // [3][n_sites] SoA
+    void *site_xi;                  // [3][n_sites] MPCD-AT: the sites' scaled normals (PRE to POST)
     int32_t *site_cell;             // replica-local cell of each site
     int64_t n_sites;
     int32_t accel;                  // constant-force streaming of the solvent (below)
