@@ -193,36 +193,46 @@ __device__ __forceinline__ void lane_rotor(double &q, double &p, int k, double h
     p = cs * p + sn * Pp;
 }
 
-// Forces done: external force, stored F and T, the second half kick (kick)
-// and the pose record the site kernels read.  Component c of every vector on
-// lane c; store: this lane writes (lane 3 and repeated lanes do not).
-__device__ __forceinline__ void lane_force_finish(const StepArgs &a, int64_t i, const DevShape &sh, double q, double R,
-                                                  double P, double L, double F, double T, int kick, int c, bool store)
+// Forces done: external force, stored F and T, the second half kick (kick) and
+// the pose record the site kernels read, in two parts that share nothing, so
+// that different warps can take them.  Component c of every vector on lane c;
+// store: this lane writes (lane 3 and repeated lanes do not).
+__device__ __forceinline__ void lane_finish_linear(const StepArgs &a, int64_t i, const DevShape &sh, double R, double P,
+                                                   double F, int kick, int k, bool store)
+{
+    F += a.fext[k];   // external force at the centre of mass (no torque)
+    if (kick) P = P + 0.5 * a.dt * F;
+    const double V = div_by(P, sh.M, sh.rM);
+    if (!store) return;
+    DevBody *o = a.bodies + i;
+    o->F[k] = F;
+    if (kick) o->P[k] = P;
+    double *p64 = a.pose64 + i * POSE_W;
+    float *p32 = a.pose32 + i * POSE_W;
+    p64[9 + k] = R; p32[9 + k] = (float)R;
+    p64[12 + k] = V; p32[12 + k] = (float)V;
+}
+__device__ __forceinline__ void lane_finish_angular(const StepArgs &a, int64_t i, const DevShape &sh, double q, double L,
+                                                    double T, int kick, int c, bool store)
 {
     const int k = c == 3 ? 0 : c;
-    F += a.fext[k];   // external force at the centre of mass (no torque)
     const LaneRot Q = lane_rot(q, c);
-    DevBody *o = a.bodies + i;
     if (kick) {
         double p = lane_L_to_p(q, Q, L, c);
-        P = P + 0.5 * a.dt * F;
         p += lane_torque_kick(q, Q, T, 0.5 * a.dt, c);
         L = lane_mv(Q, lane_p_to_Lb(q, p, c));
     }
-    // pose: Q, R, V = P/M, omega = Q Ihat^-1 Q^T L (Eq. 5)
-    const double V = div_by(P, sh.M, sh.rM);
+    // omega = Q Ihat^-1 Q^T L (Eq. 5)
     const double Lb = lane_mtv(Q, L);
     const double wb = sh.Ihat[k] > 0.0 ? div_by(Lb, sh.Ihat[k], sh.rI[k]) : 0.0;
     const double W = lane_mv(Q, wb);
     if (!store) return;
-    o->F[k] = F;
+    DevBody *o = a.bodies + i;
     o->T[k] = T;
-    if (kick) { o->P[k] = P; o->Lm[k] = L; }
+    if (kick) o->Lm[k] = L;
     double *p64 = a.pose64 + i * POSE_W;
     float *p32 = a.pose32 + i * POSE_W;
     for (int m = 0; m < 3; ++m) { p64[3 * k + m] = Q.r[m]; p32[3 * k + m] = (float)Q.r[m]; }
-    p64[9 + k] = R; p32[9 + k] = (float)R;
-    p64[12 + k] = V; p32[12 + k] = (float)V;
     p64[15 + k] = W; p32[15 + k] = (float)W;
 }
 
@@ -232,10 +242,13 @@ __device__ __forceinline__ void lane_force_finish(const StepArgs &a, int64_t i, 
 // LONE: every replica has one body at most, so no force acts between bodies and
 // the force pass is finished here.  Also writes the space-frame WCA centres of
 // shapes with one or two of them.
+// Two warps take eight bodies: one their rotation, one their translation.
+constexpr int MD_BODIES = 8;
 template <typename Real, bool IMPULSE, bool LONE>
 __global__ void __launch_bounds__(64) k_body_md(StepArgs a)
 {
-    const int g = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 2);
+    const int g = (int)(blockIdx.x * MD_BODIES + ((threadIdx.x & 31) >> 2));
+    const bool linear = threadIdx.x >= 32;
     const int c = threadIdx.x & 3, k = c == 3 ? 0 : c;
     const bool valid = g < a.n_bodies;
     const int i = valid ? g : a.n_bodies - 1;   // every lane takes part in the shuffles
@@ -244,30 +257,57 @@ __global__ void __launch_bounds__(64) k_body_md(StepArgs a)
     const DevShape &sh = a.shapes[o->shape];
     const DevReplica &r = a.reps[o->rep];
     const double dt = a.dt;
-    int bad = 0;
+    // component k (3 + k) of the transfer, with IMPULSE
+    const Real *in = reinterpret_cast<const Real *>(a.partial) + (int64_t)i * SITE_WARPS * 6 + (linear ? k : 3 + k);
+    auto transfer = [&]() {
+        double s = 0.0;
+        for (int w = 0; w < SITE_WARPS; ++w) s += (double)in[w * 6];
+        return s;
+    };
     chain_next();
     if (!IMPULSE) chain_wait();
     // with IMPULSE the pass before is POST, which writes only the partial sums
-    double q = o->q[c], P = o->P[k], L = o->Lm[k], R = o->R[k];
+    if (linear) {
+        int bad = 0;
+        double P = o->P[k], R = o->R[k];
+        const double kickF = 0.5 * dt * o->F[k], D0 = o->D[k];
+        const float4 p0 = a.bpos_build[i];
+        const float h = 0.5f * r.L[k], bound = (float)sh.bound;
+        if (IMPULSE) {
+            chain_wait();
+            P += transfer();
+        }
+        P += kickF;
+        const double d = dt * div_by(P, sh.M, sh.rM);
+        const double D = D0 + d;
+        R = wrap_box(R + d, (double)r.L[k], bad);
+        if (store) { o->R[k] = R; o->D[k] = D; }
+        if (store && !LONE) o->P[k] = P;
+        // neighbour lists stay valid while every body is within half the skin of
+        // its position at the last build
+        const float Rf = (float)R;
+        float dx = Rf - (k == 0 ? p0.x : (k == 1 ? p0.y : p0.z));
+        dx = dx > h ? dx - r.L[k] : (dx < -h ? dx + r.L[k] : dx);
+        const float x2 = dx * dx;
+        const float d2 = ((0.0f + lane4(x2, 0)) + lane4(x2, 1)) + lane4(x2, 2);
+        const float4 at = make_float4(lane4(Rf, 0), lane4(Rf, 1), lane4(Rf, 2), bound);
+        if (valid && c == 3) {
+            a.bpos[i] = at;
+            if (!LONE && d2 > 0.25f * NLIST_SKIN * NLIST_SKIN) atomicOr(a.nl_dirty, 1);
+        }
+        if (store && bad) atomicOr(a.d_err, ERR_POSITION);
+        if (LONE) lane_finish_linear(a, i, sh, R, P, 0.0, 1, k, store);
+        return;
+    }
+    double q = o->q[c], L = o->Lm[k];
     LaneRot Q = lane_rot(q, c);
     const double kickT = lane_torque_kick(q, Q, o->T[k], 0.5 * dt, c);
     if (IMPULSE) {
         chain_wait();
-        const Real *in = reinterpret_cast<const Real *>(a.partial) + (int64_t)i * SITE_WARPS * 6;
-        double sP = 0.0, sL = 0.0;
-        for (int w = 0; w < SITE_WARPS; ++w) {
-            sP += (double)in[w * 6 + k];
-            sL += (double)in[w * 6 + 3 + k];
-        }
-        P += sP;
-        L += sL;
+        L += transfer();
     }
     double p = lane_L_to_p(q, Q, L, c);
-    P += 0.5 * dt * o->F[k];
     p += kickT;
-    const double d = dt * div_by(P, sh.M, sh.rM);
-    const double D = o->D[k] + d;
-    R = wrap_box(R + d, (double)r.L[k], bad);
 #pragma unroll 1
     for (int e = 0; e < 5; ++e) {   // axes 3, 2, 1, 2, 3
         const int ax = e < 3 ? 3 - e : e - 1;
@@ -277,8 +317,7 @@ __global__ void __launch_bounds__(64) k_body_md(StepArgs a)
     q /= sqrt(((lane4(qq, 0) + lane4(qq, 1)) + lane4(qq, 2)) + lane4(qq, 3));
     Q = lane_rot(q, c);
     L = lane_mv(Q, lane_p_to_Lb(q, p, c));
-    if (store) { o->R[k] = R; o->D[k] = D; }
-    if (store && !LONE) { o->P[k] = P; o->Lm[k] = L; }
+    if (store && !LONE) o->Lm[k] = L;
     if (valid) o->q[c] = q;
     if (a.max_cent <= 2)
         for (int e = 0; e < sh.n_cent; ++e) {
@@ -289,21 +328,7 @@ __global__ void __launch_bounds__(64) k_body_md(StepArgs a)
                 reinterpret_cast<float *>(a.cent32 + o->cent_begin + e)[k] = (float)x;
             }
         }
-    // neighbour lists stay valid while every body is within half the skin of
-    // its position at the last build
-    const float Rf = (float)R, h = 0.5f * r.L[k];
-    const float4 p0 = a.bpos_build[i];
-    float dx = Rf - (k == 0 ? p0.x : (k == 1 ? p0.y : p0.z));
-    dx = dx > h ? dx - r.L[k] : (dx < -h ? dx + r.L[k] : dx);
-    const float x2 = dx * dx;
-    const float d2 = ((0.0f + lane4(x2, 0)) + lane4(x2, 1)) + lane4(x2, 2);
-    const float4 at = make_float4(lane4(Rf, 0), lane4(Rf, 1), lane4(Rf, 2), (float)sh.bound);
-    if (valid && c == 3) {
-        a.bpos[i] = at;
-        if (!LONE && d2 > 0.25f * NLIST_SKIN * NLIST_SKIN) atomicOr(a.nl_dirty, 1);
-    }
-    if (store && bad) atomicOr(a.d_err, ERR_POSITION);
-    if (LONE) lane_force_finish(a, i, sh, q, R, P, L, 0.0, 0.0, 1, c, store);
+    if (LONE) lane_finish_angular(a, i, sh, q, L, 0.0, 1, c, store);
 }
 
 __global__ void k_body_pos(StepArgs a)
@@ -317,7 +342,7 @@ __global__ void k_body_pos(StepArgs a)
 template <typename Real>
 static void body_md(const StepArgs &a, bool impulse, cudaStream_t s)
 {
-    const unsigned grid = (unsigned)((a.n_bodies + 15) / 16);   // 64 threads, four lanes per body
+    const unsigned grid = (unsigned)((a.n_bodies + MD_BODIES - 1) / MD_BODIES);
     if (a.lone_bodies) {
         if (impulse) launch_chained(k_body_md<Real, true, true>, grid, 64, 0, s, a);
         else launch_chained(k_body_md<Real, false, true>, grid, 64, 0, s, a);
@@ -453,21 +478,25 @@ template <typename Real, int MAXC>
 __global__ void __launch_bounds__(128) k_body_force(StepArgs a, int kick)
 {
     constexpr int NP = MAXC * MAXC;
+    __shared__ double sF[16][3], sT[16][3];   // the CTA's 16 bodies
     const unsigned full = 0xffffffffu;
     const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
     const int sub = threadIdx.x & 7, gsh = threadIdx.x & 24;   // lane of the body, its first lane in the warp
-    const int c = sub & 3, k = c == 3 ? 0 : c, k1 = k == 2 ? 0 : k + 1, k2 = k == 0 ? 2 : k - 1;
+    const int k = (sub & 3) == 3 ? 0 : sub & 3, k1 = k == 2 ? 0 : k + 1, k2 = k == 0 ? 2 : k - 1;
     const bool valid = g < a.n_bodies;
     const int64_t i = valid ? g : a.n_bodies - 1;   // every lane takes part in the votes and shuffles
     const DevBody &bi = a.bodies[i];
     const DevShape &si = a.shapes[bi.shape];
     const DevReplica r = a.reps[bi.rep];
+    const float cut = (float)(0.5 * (si.wca_d + a.max_wca_d) - 1.0 + 1.122462048309373);
     chain_wait();
     chain_next();
+    // (loads that do not wait for one another)
+    const int dirty = *a.nl_dirty;
     const float4 pi = a.bpos[i];
-    const float cut = (float)(0.5 * (si.wca_d + a.max_wca_d) - 1.0 + 1.122462048309373);
-    int n;
-    if (*a.nl_dirty) {
+    const int32_t near0 = a.nlist[i * NLIST_MAX + sub];   // the first candidates, if the list holds
+    int n = a.ncount[i];
+    if (dirty) {
         // candidates within the bounding spheres + cutoff + skin, ascending
         const float reach = cut + NLIST_SKIN + 1e-2f;
         n = 0;
@@ -492,8 +521,6 @@ __global__ void __launch_bounds__(128) k_body_force(StepArgs a, int kick)
             a.bpos_build[i] = pi;
         }
         __syncwarp();   // the list is read by the body's other lanes
-    } else {
-        n = a.ncount[i];
     }
     const bool listed = n >= 0 && n <= NLIST_MAX;
     const int64_t total = !valid ? 0 : (listed ? n : r.body_end - r.body_begin);
@@ -503,7 +530,7 @@ __global__ void __launch_bounds__(128) k_body_force(StepArgs a, int kick)
         bool on = e < total;
         int64_t j = i;
         if (on) {
-            j = listed ? (int64_t)a.nlist[i * NLIST_MAX + e] : r.body_begin + e;
+            j = !listed ? r.body_begin + e : (e0 == 0 && !dirty ? near0 : a.nlist[i * NLIST_MAX + e]);
             on = j >= r.body_begin && j < r.body_end;
             if (!listed) on = on && j != i && may_interact(a, pi, a.bpos[j], r, cut + 1e-2f);
         }
@@ -547,7 +574,21 @@ __global__ void __launch_bounds__(128) k_body_force(StepArgs a, int kick)
             some &= some - 1;
         }
     }
-    lane_force_finish(a, i, si, bi.q[c], bi.R[k], bi.P[k], bi.Lm[k], F, T, kick, c, valid && sub < 3);
+    if (sub < 3) {
+        sF[threadIdx.x >> 3][k] = F;
+        sT[threadIdx.x >> 3][k] = T;
+    }
+    __syncthreads();
+    // four lanes per body: two warps for the angular part, two for the linear one
+    const int m = (threadIdx.x & 63) >> 2, cm = threadIdx.x & 3, km = cm == 3 ? 0 : cm;
+    const int64_t gm = (int64_t)blockIdx.x * 16 + m, im = min(gm, (int64_t)a.n_bodies - 1);
+    const DevBody &bm = a.bodies[im];
+    const DevShape &sm = a.shapes[bm.shape];
+    const bool store = gm < a.n_bodies && cm < 3;
+    if (threadIdx.x < 64)
+        lane_finish_angular(a, im, sm, bm.q[cm], bm.Lm[km], sT[m][km], kick, cm, store);
+    else
+        lane_finish_linear(a, im, sm, bm.R[km], bm.P[km], sF[m][km], kick, km, store);
 }
 
 // One warp per body (shapes with many centres, e.g. rods): the lanes take the
@@ -626,7 +667,8 @@ __global__ void __launch_bounds__(32 * WARP_BODIES) k_body_force_warp(StepArgs a
         const double f = __shfl_sync(0xffffffffu, F[m], 0), t = __shfl_sync(0xffffffffu, T[m], 0);
         if (m == k) { Fk = f; Tk = t; }
     }
-    lane_force_finish(a, i, si, bi.q[c], bi.R[k], bi.P[k], bi.Lm[k], Fk, Tk, kick, c, lane < 3);
+    lane_finish_linear(a, i, si, bi.R[k], bi.P[k], Fk, kick, k, lane < 3);
+    lane_finish_angular(a, i, si, bi.q[c], bi.Lm[k], Tk, kick, c, lane < 3);
     if (i == 0 && lane == 0) *a.nl_dirty = 0;   // the lists used by this step are fresh
 }
 

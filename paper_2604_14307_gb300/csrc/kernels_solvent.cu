@@ -1205,12 +1205,10 @@ __device__ __forceinline__ float ll2f48(long long w)
 }
 
 // FP32 form: cell words -> collision parameters with FP32/integer pipes only.
-// Each CTA takes PARAM_TILES consecutive 256-cell tiles, one cell of each per
-// thread.  The word loads of all of them are issued before any arithmetic (a
+// Each CTA takes K consecutive 256-cell tiles, one cell of each per thread.  The word loads of all of them are issued before any arithmetic (a
 // warp keeps PARAM_TILES x NW loads in flight instead of a chain of dependent
 // loads) and parked in shared memory, so the registers of the arithmetic that
 // follows are not tied up by the parked words.
-constexpr int PARAM_TILES = 2;
 
 template <int RULE>
 __device__ __forceinline__ void params32_cell(const StepArgs &a, const DevReplica &r, int64_t step, int64_t c,
@@ -1259,11 +1257,10 @@ __device__ __forceinline__ void params32_cell(const StepArgs &a, const DevReplic
     o[1] = make_float4(rec[4], rec[5], rec[6], 0.0f);
 }
 
-template <int RULE>
+template <int RULE, int K>
 __global__ void __launch_bounds__(256, 4) k_params32(StepArgs a)
 {
     constexpr int NW = Words32<RULE>::n;
-    constexpr int K = PARAM_TILES;
     __shared__ long long sw[K][NW][256];
     __shared__ Tile stile[K];
     long long *sums = reinterpret_cast<long long *>(a.sums);
@@ -1401,14 +1398,25 @@ __global__ void __launch_bounds__(256) k_params(StepArgs a)
     if (err) atomicOr(a.d_err, ERR_CELL);
 }
 
-void launch_params(const StepArgs &a, int, cudaStream_t s)
+constexpr int PARAM_ONE = 16;   // 256-cell tiles per SM
+
+void launch_params(const StepArgs &a, int num_sms, cudaStream_t s)
 {
     if (a.n_ctiles == 0) return;
     const int grid = a.n_ctiles;   // one 256-cell tile per CTA, one cell per thread
     if (a.precision == 1) {
-        const int grid32 = (a.n_ctiles + PARAM_TILES - 1) / PARAM_TILES;
-        if (a.rule == 0) k_params32<0><<<grid32, 256, 0, s>>>(a);
-        else k_params32<1><<<grid32, 256, 0, s>>>(a);
+        // one tile per CTA while the device takes them in a few rounds of four CTAs
+        // per SM: a second cell per thread only makes a round longer (54 tiles: a
+        // step 19.3 -> 16.9 us, 432: 29.5 -> 27.4, 2001: 102 -> 100); two beyond,
+        // whose loads overlap the arithmetic (13500 tiles: 90 us, 96 with one)
+        if (a.n_ctiles <= PARAM_ONE * num_sms) {
+            if (a.rule == 0) k_params32<0, 1><<<grid, 256, 0, s>>>(a);
+            else k_params32<1, 1><<<grid, 256, 0, s>>>(a);
+        } else {
+            const int grid2 = (a.n_ctiles + 1) / 2;
+            if (a.rule == 0) k_params32<0, 2><<<grid2, 256, 0, s>>>(a);
+            else k_params32<1, 2><<<grid2, 256, 0, s>>>(a);
+        }
     } else {
         if (a.rule == 0) k_params<double, 0><<<grid, 256, 0, s>>>(a);
         else k_params<double, 1><<<grid, 256, 0, s>>>(a);

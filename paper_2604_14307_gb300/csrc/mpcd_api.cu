@@ -519,7 +519,7 @@ int k_params(mpcd_ctx *c, cudaStream_t s)
 {
     StepArgs a = make_args(c);
     double bytes = (double)c->C * (2.0 * c->nw * 8.0 + c->param_bytes);
-    return timed(c, "cell_params", bytes, s, [&] { launch_params(a, c->num_sms * 8, s); });
+    return timed(c, "cell_params", bytes, s, [&] { launch_params(a, c->num_sms, s); });
 }
 
 int k_post(mpcd_ctx *c, cudaStream_t s, bool impulse = true)

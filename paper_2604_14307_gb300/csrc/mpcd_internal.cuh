@@ -402,7 +402,7 @@ struct LaunchCfg {
 
 // solvent pass (kernels_solvent.cu)
 void launch_solvent(const StepArgs &a, int flags, LaunchCfg cfg, cudaStream_t s);
-void launch_params(const StepArgs &a, int grid, cudaStream_t s);
+void launch_params(const StepArgs &a, int num_sms, cudaStream_t s);
 // one collision of a single box on the caller's SoA arrays (a.x .. a.vz, a.tag;
 // n a multiple of 4; a.params holds the cells' records), enqueued as one kernel
 struct BoxScratch {
