@@ -591,18 +591,26 @@ __global__ void __launch_bounds__(128) k_body_force(StepArgs a, int kick)
         lane_finish_linear(a, im, sm, bm.R[km], bm.P[km], sF[m][km], kick, km, store);
 }
 
-// One warp per body (shapes with many centres, e.g. rods): the lanes take the
-// (neighbour, centre, centre) triples of the body's candidates in turn, each
-// lane summing its triples in order, and a fixed shuffle tree adds the lanes,
-// so the result depends only on the candidate list.  R_i - R_j is formed once
-// per candidate and kept in shared memory (formed for every triple, its FP64
-// subtractions and conversions were most of the pass: 200 us against 147 for
-// 1120 bodies of up to 19 centres).
+// One warp per body (shapes with many centres, e.g. rods): triple t = ((candidate
+// e) n_centres + own centre) max_centres + its centre belongs to lane t mod 32,
+// each lane sums its triples in order, and a fixed shuffle tree adds the lanes,
+// so the result depends only on the candidate list.  A row of triples (candidate,
+// own centre) is left out when the own centre is further from the candidate than
+// its bounding sphere and the cutoff reach, which adds nothing: the lanes test 32
+// rows at a time, and one row at a time is summed (rods see most bodies of a box
+// as candidates, but few of their own centres lie near each).  What belongs to a candidate
+// - R_i - R_j and the mean diameter, formed in FP64, and where its centres lie -
+// is formed once and kept in shared memory: nine FP64 instructions per triple and
+// the loads one behind the other were most of the pass (1120 bodies of up to 19
+// centres: 200 us, 147 with R_i - R_j kept, 95 with all, 40 with rows left out).
 constexpr int WARP_BODIES = 4;   // bodies (warps) per CTA
 template <typename Real>
 __global__ void __launch_bounds__(32 * WARP_BODIES) k_body_force_warp(StepArgs a, int kick)
 {
-    __shared__ Real sdR[WARP_BODIES][NLIST_MAX][3];
+    __shared__ Real sdR[WARP_BODIES][NLIST_MAX][3], sdij[WARP_BODIES][NLIST_MAX];
+    __shared__ int64_t scent[WARP_BODIES][NLIST_MAX];
+    __shared__ float sreach[WARP_BODIES][NLIST_MAX];   // squared, of a row
+    __shared__ int sncent[WARP_BODIES][NLIST_MAX];
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (i >= a.n_bodies) return;   // uniform over the warp
@@ -612,11 +620,12 @@ __global__ void __launch_bounds__(32 * WARP_BODIES) k_body_force_warp(StepArgs a
     chain_wait();
     chain_next();
     double F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
-    auto pair = [&](const Real (&dR)[3], const DevBody &bj, const DevShape &sj, int ca, int cc) {
+    const int64_t cent_i = bi.cent_begin;
+    auto pair = [&](const Real (&dR)[3], Real dij, int64_t cent_j, int ca, int cc) {
         Real ci[3], cj[3], f[3];
-        CentreOf<Real>::get(a, bi.cent_begin + ca, ci);
-        CentreOf<Real>::get(a, bj.cent_begin + cc, cj);
-        if (!centre_force<Real>(Real(0.5 * (si.wca_d + sj.wca_d)), dR, ci, cj, r, f)) return;
+        CentreOf<Real>::get(a, cent_i + ca, ci);
+        CentreOf<Real>::get(a, cent_j + cc, cj);
+        if (!centre_force<Real>(dij, dR, ci, cj, r, f)) return;
         for (int k = 0; k < 3; ++k) F[k] += (double)f[k];
         T[0] += (double)ci[1] * (double)f[2] - (double)ci[2] * (double)f[1];
         T[1] += (double)ci[2] * (double)f[0] - (double)ci[0] * (double)f[2];
@@ -628,17 +637,40 @@ __global__ void __launch_bounds__(32 * WARP_BODIES) k_body_force_warp(StepArgs a
         for (int e = lane; e < n; e += 32) {
             const int64_t j = a.nlist[i * NLIST_MAX + e];
             const bool on = j >= r.body_begin && j < r.body_end;
-            for (int k = 0; k < 3; ++k) sdR[wid][e][k] = on ? (Real)(bi.R[k] - a.bodies[j].R[k]) : Real(0);
+            const DevBody &bj = a.bodies[on ? j : i];
+            const DevShape &sj = a.shapes[bj.shape];
+            for (int k = 0; k < 3; ++k) sdR[wid][e][k] = (Real)(bi.R[k] - bj.R[k]);
+            sdij[wid][e] = Real(0.5 * (si.wca_d + sj.wca_d));
+            scent[wid][e] = bj.cent_begin;
+            sncent[wid][e] = on ? sj.n_cent : 0;
+            const float reach = (float)(sj.bound + 0.5 * (si.wca_d + sj.wca_d) - 1.0 + 1.122462048309373) + 1e-2f;
+            sreach[wid][e] = on ? reach * reach : -1.0f;
         }
         __syncwarp();
-        const int per = nci * maxc;
-        for (int t = lane; t < n * per; t += 32) {
-            const int e = t / per, rem = t - e * per, ca = rem / maxc, cc = rem - ca * maxc;
-            const int64_t j = a.nlist[i * NLIST_MAX + e];
-            if (j < r.body_begin || j >= r.body_end) continue;
-            const DevBody &bj = a.bodies[j];
-            const DevShape &sj = a.shapes[bj.shape];
-            if (cc < sj.n_cent) pair(sdR[wid][e], bj, sj, ca, cc);
+        const float L[3] = {(float)r.L[0], (float)r.L[1], (float)r.L[2]};
+        for (int r0 = 0; r0 < n * nci; r0 += 32) {
+            const int row = r0 + lane, e = row / nci, ca = row - e * nci;
+            bool near = row < n * nci;
+            if (near) {
+                Real ci[3];
+                CentreOf<Real>::get(a, cent_i + ca, ci);
+                float d2 = 0.0f;
+                for (int k = 0; k < 3; ++k) {   // the nearest image: no image of the pair is closer
+                    float d = (float)sdR[wid][e][k] + (float)ci[k];
+                    d -= L[k] * rintf(d / L[k]);
+                    d2 += d * d;
+                }
+                near = d2 <= sreach[wid][e];
+            }
+            for (unsigned left = __ballot_sync(0xffffffffu, near); left; left &= left - 1) {
+                const int src = __ffs(left) - 1;
+                const int en = __shfl_sync(0xffffffffu, e, src), cn = __shfl_sync(0xffffffffu, ca, src);
+                const unsigned t0 = (unsigned)(r0 + src) * (unsigned)maxc;   // its low bits name the lanes
+                for (int c0 = 0; c0 < maxc; c0 += 32) {
+                    const int cc = c0 + (int)(((unsigned)lane - t0 - (unsigned)c0) & 31u);
+                    if (cc < sncent[wid][en]) pair(sdR[wid][en], sdij[wid][en], scent[wid][en], cn, cc);
+                }
+            }
         }
     } else {
         // the list overflowed: every body of the replica, prefiltered
@@ -650,8 +682,9 @@ __global__ void __launch_bounds__(32 * WARP_BODIES) k_body_force_warp(StepArgs a
             const DevShape &sj = a.shapes[bj.shape];
             Real dR[3];
             for (int k = 0; k < 3; ++k) dR[k] = (Real)(bi.R[k] - bj.R[k]);
+            const Real dij = Real(0.5 * (si.wca_d + sj.wca_d));
             for (int ca = 0; ca < nci; ++ca)
-                for (int cc = 0; cc < sj.n_cent; ++cc) pair(dR, bj, sj, ca, cc);
+                for (int cc = 0; cc < sj.n_cent; ++cc) pair(dR, dij, bj.cent_begin, ca, cc);
         }
     }
 #pragma unroll

@@ -134,3 +134,15 @@ def test_site_passes_at_their_edges(B, sites, precision):
     sP, sL = np.sqrt(sh.m.sum()), np.sqrt(I.shape_inertia_diag(sh).max())
     assert (np.abs(g.P - ost.P) / (np.abs(ost.P) + sP)).max() <= tol
     assert (np.abs(g.Lm - ost.Lm) / (np.abs(ost.Lm) + sL)).max() <= tol
+
+
+@pytest.mark.parametrize("precision", [I.P64, I.P32])
+@pytest.mark.parametrize("length", [5.0, 9.0, 13.0])
+def test_rods_crossing_the_box(B, length, precision):
+    """Rods in a box little longer than they are, packed at every angle and through
+    its faces: the rows of centre pairs that are left out are those out of reach."""
+    rng = np.random.default_rng(int(length))
+    sh = I.spherocylinder_shape(2.4, length, 1.5, 5.0, cap_level=1)
+    R, q, placed = I.rsa_place(rng, (14, 14, 14), [sh], [0] * 60, gap=0.0, max_attempts=300)
+    prm = I.Params(precision=precision, seed=int(length))
+    check(B, I.build_system(prm, [sh], [(14, 14, 14)], 0.5, [placed], "rods", R_q=[(R, q)]), 2)
