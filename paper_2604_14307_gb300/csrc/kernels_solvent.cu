@@ -2177,6 +2177,8 @@ __device__ __forceinline__ bool rn_due(const StepArgs &a, const RnemdArgs &g)
 // global list through contended atomics)
 constexpr int RN_SBUF = 512;
 
+constexpr int RN_TODO = 512;   // marks that a CTA reads at once
+
 template <typename Real>
 __global__ void __launch_bounds__(512) k_rnemd_scan(StepArgs a, RnemdArgs g)
 {
@@ -2191,13 +2193,10 @@ __global__ void __launch_bounds__(512) k_rnemd_scan(StepArgs a, RnemdArgs g)
     const Real *Y = (const Real *)a.y, *VX = (const Real *)a.vx;
     const int64_t beg = r.solv_begin, n = r.n_solvent;
     int bad = 0;
-    auto visit = [&](int64_t i, Real y) {
-        const int sl = rn_slab(g, y);
-        if (sl < 0) return;
-        const Real k = rn_key(g, VX[beg + i], sl);
+    auto member = [&](int64_t i, Real vx, uint32_t tag, int sl, int pos) {   // pos: its place in the CTA's list
+        const Real k = rn_key(g, vx, sl);
         atomicAdd(&sh[sl * RN_BUCKETS + rn_bucket((float)k)], 1);
-        const RnEntry e{rn_bits(k), a.tag[beg + i], (uint32_t)i};
-        const int pos = atomicAdd(&scount[sl], 1);
+        const RnEntry e{rn_bits(k), tag, (uint32_t)i};
         if (pos < RN_SBUF) {
             sbuf[sl][pos] = e;
         } else {   // a crowded CTA: straight to the global list
@@ -2206,11 +2205,71 @@ __global__ void __launch_bounds__(512) k_rnemd_scan(StepArgs a, RnemdArgs g)
             else bad = 1;
         }
     };
+    auto visit = [&](int64_t i, Real y) {
+        const int sl = rn_slab(g, y);
+        if (sl >= 0) member(i, VX[beg + i], a.tag[beg + i], sl, atomicAdd(&scount[sl], 1));
+    };
     // four consecutive particles per vector load of y (the replica's first
     // slot is a multiple of 8), RN_LOADS loads in flight per thread: the pass
     // is bound by how many bytes are in flight
     constexpr int RN_LOADS = 4;
-    const int64_t n4 = n & ~(int64_t)3;
+    if (g.mark) {
+        // the CTA's share of the marks is read at once, then it takes its marked
+        // blocks of 1024 slots, four at a time (a few per cent of the blocks, which
+        // lie together: neighbours go to different CTAs).  17 M particles, slabs of
+        // 1/240 of the box: 29 us for all of y, 18 this way, a chain of latencies now;
+        // a block for one warp, 32 members in a row per lane, took 41.
+        __shared__ int todo[RN_TODO], n_todo;
+        const int lane = threadIdx.x & 31;
+        const int64_t end = beg + n, blocks = (end + RN_MARK - 1) / RN_MARK;
+        for (int64_t b0 = blockIdx.x; b0 < blocks; b0 += (int64_t)RN_TODO * gridDim.x) {
+            if (threadIdx.x == 0) n_todo = 0;
+            __syncthreads();
+            for (int t = threadIdx.x; t < RN_TODO; t += blockDim.x) {
+                const int64_t b = b0 + (int64_t)t * gridDim.x;
+                if (b < blocks && g.mark[b]) {
+                    todo[atomicAdd(&n_todo, 1)] = (int)b;
+                    g.mark[b] = 0;
+                }
+            }
+            __syncthreads();
+            constexpr int U = 8;   // particles of a thread in flight: four blocks
+            for (int q = 0; q < n_todo; q += U * 512 / RN_MARK) {
+                int64_t i[U];
+                int sl[U];
+                Real y[U], vx[U];
+                uint32_t tag[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int qu = q + u * 512 / RN_MARK;
+                    i[u] = qu < n_todo ? (int64_t)todo[qu] * RN_MARK + (u * 512) % RN_MARK + threadIdx.x : -1;
+                    y[u] = i[u] >= beg && i[u] < end ? Y[i[u]] : Real(-1);   // below every slab
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    sl[u] = rn_slab(g, y[u]);
+                    vx[u] = sl[u] >= 0 ? VX[i[u]] : Real(0);
+                    tag[u] = sl[u] >= 0 ? a.tag[i[u]] : 0u;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {   // one atomic per warp and slab for the places
+                    int pos = 0;
+#pragma unroll
+                    for (int l = 0; l < 2; ++l) {
+                        const unsigned m = __ballot_sync(0xffffffffu, sl[u] == l);
+                        if (!m) continue;
+                        int base = 0;
+                        if (lane == __ffs(m) - 1) base = atomicAdd(&scount[l], __popc(m));
+                        base = __shfl_sync(0xffffffffu, base, __ffs(m) - 1);
+                        if (sl[u] == l) pos = base + __popc(m & ((1u << lane) - 1u));
+                    }
+                    if (sl[u] >= 0) member(i[u] - beg, vx[u], tag[u], sl[u], pos);
+                }
+            }
+            __syncthreads();
+        }
+    }
+    const int64_t n4 = g.mark ? 0 : n & ~(int64_t)3;
     const int64_t stride = 4 * (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); i < n4; i += RN_LOADS * stride) {
         Real y[RN_LOADS][4];
@@ -2223,7 +2282,7 @@ __global__ void __launch_bounds__(512) k_rnemd_scan(StepArgs a, RnemdArgs g)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) visit(i + u * stride + j, y[u][j]);
     }
-    if (blockIdx.x == 0 && threadIdx.x < n - n4) visit(n4 + threadIdx.x, Y[beg + n4 + threadIdx.x]);
+    if (!g.mark && blockIdx.x == 0 && threadIdx.x < n - n4) visit(n4 + threadIdx.x, Y[beg + n4 + threadIdx.x]);
     __syncthreads();
     if (threadIdx.x < 2) {
         const int m = min(scount[threadIdx.x], RN_SBUF);
@@ -2331,6 +2390,8 @@ __global__ void __launch_bounds__(512) k_rnemd_filter(StepArgs a, RnemdArgs g)
     }
 }
 
+constexpr int RN_RANKED = 1024;   // longest lists sorted by ranks (at most RN_CAP / 2)
+
 template <typename Real, int RULE>
 __global__ void __launch_bounds__(1024) k_rnemd_select(StepArgs a, RnemdArgs g)
 {
@@ -2351,14 +2412,33 @@ __global__ void __launch_bounds__(1024) k_rnemd_select(StepArgs a, RnemdArgs g)
     } else {
         int P = 2;
         while (P < nA || P < nB) P <<= 1;
-        const RnEntry pad{~0ull, ~0u, 0u};
-        for (int t = threadIdx.x; t < P; t += blockDim.x) {
-            if (t >= nA) E[t] = pad;
-            if (t >= nB) E[RN_CAP + t] = pad;
+        if (P <= RN_RANKED) {
+            // few candidates: an entry's place is the number of entries before it (all
+            // differ); the sorted lists go behind the unsorted ones (100 pairs: the kernel
+            // took 19 us with the barriers of the bitonic sort, 15 with ranks)
+            __syncthreads();
+            for (int t = threadIdx.x; t < 2 * P; t += blockDim.x) {
+                const int l = t >= P ? 1 : 0, u = t - l * P, n = l ? nB : nA;
+                if (u >= n) continue;
+                const RnEntry *src = E + l * RN_CAP;
+                const RnEntry e = src[u];
+                int at = 0;
+                for (int v = 0; v < n; ++v) at += rn_less(src[v], e) ? 1 : 0;
+                E[l * RN_CAP + RN_CAP / 2 + at] = e;
+            }
+            E += RN_CAP / 2;
+            __syncthreads();
         }
-        __syncthreads();
+        const RnEntry pad{~0ull, ~0u, 0u};
+        if (P > RN_RANKED) {
+            for (int t = threadIdx.x; t < P; t += blockDim.x) {
+                if (t >= nA) E[t] = pad;
+                if (t >= nB) E[RN_CAP + t] = pad;
+            }
+            __syncthreads();
+        }
         // bitonic sort of both lists, ascending by (key, id)
-        for (int k = 2; k <= P; k <<= 1)
+        for (int k = P > RN_RANKED ? 2 : P + 1; k <= P; k <<= 1)
             for (int j = k >> 1; j > 0; j >>= 1) {
                 for (int t = threadIdx.x; t < 2 * P; t += blockDim.x) {
                     const int l = t >= P ? 1 : 0, u = t - l * P, v = u ^ j;
@@ -2384,16 +2464,18 @@ __global__ void __launch_bounds__(1024) k_rnemd_select(StepArgs a, RnemdArgs g)
         for (int i = threadIdx.x; i < np; i += blockDim.x) {
             const int64_t ia = r.solv_begin + E[i].idx, ib = r.solv_begin + E[RN_CAP + i].idx;
             const Real va = VX[ia], vb = VX[ib];
+            const Real xa[3] = {X[ia], Y[ia], Z[ia]}, xb[3] = {X[ib], Y[ib], Z[ib]};   // all loads before any store
+            const Real ya = VY[ia], za = VZ[ia], yb = VY[ib], zb = VZ[ib];
             VX[ia] = vb;
             VX[ib] = va;
             dp += (double)Consts<Real>::m(a) * ((double)va - (double)vb);
             if (g.fix_sums) {
-                const int ca = r.cell_base + cell_axis(X[ia], S[0], r.L[0]) +
-                               r.L[0] * (cell_axis(Y[ia], S[1], r.L[1]) + r.L[1] * cell_axis(Z[ia], S[2], r.L[2]));
-                const int cb = r.cell_base + cell_axis(X[ib], S[0], r.L[0]) +
-                               r.L[0] * (cell_axis(Y[ib], S[1], r.L[1]) + r.L[1] * cell_axis(Z[ib], S[2], r.L[2]));
-                rn_fix<RULE>(a, ca, va, vb, VY[ia], VZ[ia]);
-                rn_fix<RULE>(a, cb, vb, va, VY[ib], VZ[ib]);
+                const int ca = r.cell_base + cell_axis(xa[0], S[0], r.L[0]) +
+                               r.L[0] * (cell_axis(xa[1], S[1], r.L[1]) + r.L[1] * cell_axis(xa[2], S[2], r.L[2]));
+                const int cb = r.cell_base + cell_axis(xb[0], S[0], r.L[0]) +
+                               r.L[0] * (cell_axis(xb[1], S[1], r.L[1]) + r.L[1] * cell_axis(xb[2], S[2], r.L[2]));
+                rn_fix<RULE>(a, ca, va, vb, ya, za);
+                rn_fix<RULE>(a, cb, vb, va, yb, zb);
             }
         }
         // deterministic block sum of the exchanged momentum

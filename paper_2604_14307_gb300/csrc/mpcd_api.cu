@@ -130,6 +130,7 @@ struct mpcd_ctx {
     // reverse non-equilibrium exchange (allocated on first use)
     mpcd_rnemd rn{};
     int32_t *rn_hist = nullptr, *rn_count = nullptr;
+    uint8_t *rn_mark = nullptr;                 // blocks of slots that hold slab members
     RnEntry *rn_list = nullptr, *rn_cand = nullptr;
     int32_t *rn_ncand = nullptr;
     double *rn_tot = nullptr;                   // [0] momentum, [1] pairs (as long long)
@@ -274,6 +275,14 @@ StepArgs make_args(const mpcd_ctx *c)
     a.site_v = c->site_v;
     a.site_xi = c->site_xi;
     for (int k = 0; k < 3; ++k) a.noise[k] = c->noise[k];
+    if (c->rn.enabled) {
+        a.slab_mark = c->rn_mark;
+        const double y[4] = {c->rn.y_a, c->rn.y_a + c->rn.width, c->rn.y_b, c->rn.y_b + c->rn.width};
+        for (int k = 0; k < 4; ++k) {
+            a.rn_y[k] = y[k];
+            a.rn_yf[k] = (float)y[k];
+        }
+    }
     a.site_cell = c->site_cell;
     a.n_sites = c->Nsite;
     a.d_step = c->d_step;
@@ -598,6 +607,7 @@ int k_rnemd(mpcd_ctx *c, cudaStream_t s, int step_offset, int fix)
     g.period = r.period;
     g.step_offset = a.step_offset + step_offset;
     g.fix_sums = fix;
+    g.mark = fix ? c->rn_mark : nullptr;   // the pass that has just binned marked the slabs' blocks
     g.hist = c->rn_hist;
     g.count = c->rn_count;
     g.list = c->rn_list;
@@ -1909,7 +1919,8 @@ int mpcd_set_rnemd(mpcd_ctx *c, const mpcd_rnemd *cfg)
             c->rn_ncand = (int32_t *)dalloc(c, 2 * sizeof(int32_t));
             c->rn_cand = (RnEntry *)dalloc(c, (size_t)2 * RN_CAP * sizeof(RnEntry));
             c->rn_tot = (double *)dalloc(c, 2 * sizeof(double));
-            if (!c->rn_hist || !c->rn_count || !c->rn_list || !c->rn_ncand || !c->rn_cand || !c->rn_tot)
+            c->rn_mark = (uint8_t *)dalloc(c, (size_t)(c->Nslots / RN_MARK + 1));
+            if (!c->rn_hist || !c->rn_count || !c->rn_list || !c->rn_ncand || !c->rn_cand || !c->rn_tot || !c->rn_mark)
                 return fail(c, MPCD_ERR_OOM, "exchange buffers");
         }
         CK(c, cudaDeviceSynchronize());   // no step in flight uses the buffers
@@ -1917,6 +1928,7 @@ int mpcd_set_rnemd(mpcd_ctx *c, const mpcd_rnemd *cfg)
         CK(c, cudaMemset(c->rn_count, 0, 2 * sizeof(int32_t)));
         CK(c, cudaMemset(c->rn_ncand, 0, 2 * sizeof(int32_t)));
         CK(c, cudaMemset(c->rn_tot, 0, 2 * sizeof(double)));
+        CK(c, cudaMemset(c->rn_mark, 0, (size_t)(c->Nslots / RN_MARK + 1)));
     }
     c->rn = *cfg;
     clear_graphs(c);   // captured steps include (or omit) the exchange

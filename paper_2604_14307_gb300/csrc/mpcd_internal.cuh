@@ -104,6 +104,9 @@ struct StepArgs {
     void *sums;                     // [nw][n_cells]
     void *params;                   // [n_cells] records
     void *dbg_sums;                 // copy of the sums when debugging, else null
+    uint8_t *slab_mark;             // per 1024 slots: holds a particle of an exchange slab (null: no exchange)
+    float rn_yf[4];                 // the slabs [0], [1] and [2], [3] in y (P32 decisions)
+    double rn_y[4];                 // the same in double (P64 decisions)
     void *noise[3];                 // MPCD-AT: normals of every slot, kept from the binning to the collision (null: not)
     int32_t noise_in;               // they are those of this collision, in the present slot order
     int64_t n_cells;
@@ -445,7 +448,9 @@ struct RnEntry {
     unsigned long long key;          // bits of the non-negative rank key (float or double)
     uint32_t tag, idx;               // particle id, slot - solv_begin
 };
+constexpr int RN_MARK = 1024;      // slots per mark
 struct RnemdArgs {
+    uint8_t *mark;                       // scan the marked blocks of slots only and clear the marks (null: all)
     float ya0f, ya1f, yb0f, yb1f, vtf;   // slab bounds and target (P32 decisions)
     double ya0, ya1, yb0, yb1, vt;       // the same in double (P64 decisions)
     int32_t max_pairs, period;

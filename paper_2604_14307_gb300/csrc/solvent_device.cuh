@@ -244,6 +244,16 @@ __device__ __forceinline__ void at_normals4(const StepArgs &a, const DevReplica 
     }
 }
 
+// y in one of the exchange slabs (the test of the exchange itself)
+__device__ __forceinline__ bool in_slab(const StepArgs &a, float y)
+{
+    return (y >= a.rn_yf[0] && y < a.rn_yf[1]) || (y >= a.rn_yf[2] && y < a.rn_yf[3]);
+}
+__device__ __forceinline__ bool in_slab(const StepArgs &a, double y)
+{
+    return (y >= a.rn_y[0] && y < a.rn_y[1]) || (y >= a.rn_y[2] && y < a.rn_y[3]);
+}
+
 // Binning of a thread's 4 consecutive particles: cell under the shift S,
 // per-particle fixed-point (P32) or double (P64) terms, runs of equal cells
 // merged in registers, then one atomic per word and run.
@@ -256,6 +266,12 @@ __device__ __forceinline__ void bin4(const StepArgs &a, const Real (&x)[4], cons
 {
     int cc[4];
     Real xi[4][3];
+    if (a.slab_mark) {   // the exchange reads the marked blocks of slots only
+        bool in = false;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) in = in || (j < nv && in_slab(a, y[j]));
+        if (in) a.slab_mark[slot / RN_MARK] = 1;
+    }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         cc[j] = base + cell_bin(x[j], S[0], L0) + L0 * (cell_bin(y[j], S[1], L1) + L1 * cell_bin(z[j], S[2], L2));
