@@ -206,6 +206,13 @@ void *dalloc(mpcd_ctx *c, size_t bytes)
     }
     return p;
 }
+// The same at a 32-byte boundary, for records read by 256-bit loads: a caller's
+// allocator may give less.
+void *dalloc32(mpcd_ctx *c, size_t bytes)
+{
+    const uintptr_t p = (uintptr_t)dalloc(c, bytes + 32);
+    return (void *)((p + 31) & ~(uintptr_t)31);
+}
 
 StepArgs make_args(const mpcd_ctx *c)
 {
@@ -1088,7 +1095,7 @@ int mpcd_create(const mpcd_params *params, int32_t n_shapes, const mpcd_shape_de
         ok &= (c->tag[b] = (uint32_t *)A(c->Nslots * sizeof(uint32_t))) != nullptr;
     }
     ok &= (c->sums = A((size_t)c->C * c->nw * 8)) != nullptr;
-    ok &= (c->params = A((size_t)c->C * c->param_bytes)) != nullptr;
+    ok &= (c->params = dalloc32(c, (size_t)c->C * c->param_bytes)) != nullptr;
     ok &= (c->d_reps = (DevReplica *)A(c->reps.size() * sizeof(DevReplica))) != nullptr;
     ok &= (c->d_shapes = (DevShape *)A(std::max<size_t>(1, c->shapes.size()) * sizeof(DevShape))) != nullptr;
     ok &= (c->d_bodies = (DevBody *)A(std::max<int64_t>(1, c->B) * sizeof(DevBody))) != nullptr;
