@@ -104,7 +104,18 @@ __device__ __forceinline__ void cells4(const Real (&x)[4], const Real (&y)[4], c
     }
 }
 
-// The rule and the cell words.  One warp per tile; each lane takes 4 consecutive
+// Work of the solvent passes: a warp takes ANG_UNIT particles of a tile, so that
+// a box of few tiles still fills the chip, and ANG_CTAS CTAs of 256 threads share
+// an SM (80 registers a thread instead of 104 to 144: both passes wait for gathers
+// and reductions, and MPCD-AT+a had one CTA an SM in k_ang_apply).  60^3 cells, 1.08 M
+// particles: SRD+a 186 -> 178 us a step (k_ang_collide 58 -> 51), MPCD-AT+a 235
+// -> 207; 110^3, 6.7 M: 1098 -> 1033 and 1467 -> 1237 (k_ang_apply 694 -> 458).
+// With 64 registers 180 and 208, 1008 and 1222.  The FP64 form is bound by its
+// FP64 instructions: 128 registers (40^3 cells: 234 and 319 us; 80: 253 and 353).
+constexpr int ANG_UNIT = 256;
+template <typename Real> constexpr int ANG_CTAS = sizeof(Real) == 4 ? 3 : 2;
+
+// The rule and the cell words.  Each lane takes 4 consecutive
 // particles (128-bit loads; tiles start on multiples of 8 slots, and the slots
 // past a replica's last particle are allocated padding) and merges runs of equal
 // cells in registers.  The 16 words of a cell are one 128-byte line, and the
@@ -114,7 +125,7 @@ __device__ __forceinline__ void cells4(const Real (&x)[4], const Real (&y)[4], c
 constexpr int ANG_ROW = AW_SOLVENT + 1;   // a lane's row of words, padded against bank conflicts
 
 template <typename Real, int RULE>
-__global__ void __launch_bounds__(256) k_ang_collide(StepArgs a)
+__global__ void __launch_bounds__(256, ANG_CTAS<Real>) k_ang_collide(StepArgs a, int subs)
 {
     typedef typename AngWord<Real>::type W;
     __shared__ W rows[8][32 * ANG_ROW];
@@ -130,8 +141,10 @@ __global__ void __launch_bounds__(256) k_ang_collide(StepArgs a)
     W *row = rows[threadIdx.x >> 5];
     int4 S = make_int4(0, 0, 0, 0);
     int last_rep = -1;
-    for (int t = blockIdx.x * warps + (threadIdx.x >> 5); t < a.n_tiles; t += gridDim.x * warps) {
-        const Tile tl = a.tiles[t];
+    for (int u = blockIdx.x * warps + (threadIdx.x >> 5); u < a.n_tiles * subs; u += gridDim.x * warps) {
+        Tile tl = a.tiles[u / subs];
+        tl.begin += (int64_t)(u % subs) * ANG_UNIT;
+        tl.end = min(tl.end, tl.begin + ANG_UNIT);
         const DevReplica r = a.reps[tl.rep];
         if (tl.rep != last_rep) {
             int32_t s3[3];
@@ -338,7 +351,7 @@ __global__ void __launch_bounds__(256) k_ang_params(StepArgs a)
 // The correction; STREAM: then the drift and the binning for the next collision
 // (the arithmetic of the plain passes, in the layout of k_ang_collide).
 template <typename Real, int RULE, bool STREAM>
-__global__ void __launch_bounds__(256) k_ang_apply(StepArgs a)
+__global__ void __launch_bounds__(256, ANG_CTAS<Real>) k_ang_apply(StepArgs a, int subs)
 {
     const AngParams<Real> *params = reinterpret_cast<const AngParams<Real> *>(a.ang_params);
     typedef typename SumWord<Real>::type SW;
@@ -353,8 +366,10 @@ __global__ void __launch_bounds__(256) k_ang_apply(StepArgs a)
     int4 S = make_int4(0, 0, 0, 0);
     typename ShiftT<Real>::type sF[3] = {};
     int last_rep = -1, bad = 0;
-    for (int t = blockIdx.x * warps + (threadIdx.x >> 5); t < a.n_tiles; t += gridDim.x * warps) {
-        const Tile tl = a.tiles[t];
+    for (int u = blockIdx.x * warps + (threadIdx.x >> 5); u < a.n_tiles * subs; u += gridDim.x * warps) {
+        Tile tl = a.tiles[u / subs];
+        tl.begin += (int64_t)(u % subs) * ANG_UNIT;
+        tl.end = min(tl.end, tl.begin + ANG_UNIT);
         const DevReplica r = a.reps[tl.rep];
         if (tl.rep != last_rep) {
             int32_t s3[3];
@@ -422,29 +437,30 @@ size_t angular_param_bytes(int precision)
 }
 
 template <typename Real, int RULE>
-static void angular_phase(const StepArgs &a, int phase, int num_sms, cudaStream_t s)
+static void angular_phase(const StepArgs &a, int phase, int tile, int num_sms, cudaStream_t s)
 {
     const int grid_p = (int)std::max<int64_t>(1, std::min<int64_t>((a.n_cells + 255) / 256, (int64_t)num_sms * 16));
-    const int grid_t = std::max(1, std::min((a.n_tiles + 7) / 8, num_sms * 8));   // 8 warps, one tile each
+    const int subs = (tile + ANG_UNIT - 1) / ANG_UNIT;
+    const int grid_t = std::max(1, std::min((a.n_tiles * subs + 7) / 8, num_sms * 8));   // 8 warps, one unit each
     if (phase != ANG_PARAMS && a.n_tiles == 0) return;
     switch (phase) {
-    case ANG_COLLIDE: k_ang_collide<Real, RULE><<<grid_t, 256, 0, s>>>(a); break;
+    case ANG_COLLIDE: k_ang_collide<Real, RULE><<<grid_t, 256, 0, s>>>(a, subs); break;
     case ANG_PARAMS: k_ang_params<Real><<<grid_p, 256, 0, s>>>(a); break;
-    case ANG_APPLY: k_ang_apply<Real, 0, false><<<grid_t, 256, 0, s>>>(a); break;
-    case ANG_STREAM: k_ang_apply<Real, RULE, true><<<grid_t, 256, 0, s>>>(a); break;
+    case ANG_APPLY: k_ang_apply<Real, 0, false><<<grid_t, 256, 0, s>>>(a, subs); break;
+    case ANG_STREAM: k_ang_apply<Real, RULE, true><<<grid_t, 256, 0, s>>>(a, subs); break;
     default: break;
     }
 }
 
-void launch_angular(const StepArgs &a, int phase, int num_sms, cudaStream_t s)
+void launch_angular(const StepArgs &a, int phase, int tile, int num_sms, cudaStream_t s)
 {
     if (a.n_cells == 0) return;
     if (a.precision == 1) {
-        if (a.rule == 0) angular_phase<float, 0>(a, phase, num_sms, s);
-        else angular_phase<float, 1>(a, phase, num_sms, s);
+        if (a.rule == 0) angular_phase<float, 0>(a, phase, tile, num_sms, s);
+        else angular_phase<float, 1>(a, phase, tile, num_sms, s);
     } else {
-        if (a.rule == 0) angular_phase<double, 0>(a, phase, num_sms, s);
-        else angular_phase<double, 1>(a, phase, num_sms, s);
+        if (a.rule == 0) angular_phase<double, 0>(a, phase, tile, num_sms, s);
+        else angular_phase<double, 1>(a, phase, tile, num_sms, s);
     }
 }
 

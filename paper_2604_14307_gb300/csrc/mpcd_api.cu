@@ -681,7 +681,7 @@ int k_ang(mpcd_ctx *c, int phase, cudaStream_t s)
     StepArgs a = make_args(c);
     a.noise_in = noise_fits(c) ? 1 : 0;
     if (phase == ANG_STREAM) noise_kept(c, step_now(c) + 1);
-    return timed(c, names[phase], bytes[phase], s, [&] { launch_angular(a, phase, c->num_sms, s); });
+    return timed(c, names[phase], bytes[phase], s, [&] { launch_angular(a, phase, c->tune.tile, c->num_sms, s); });
 }
 
 int k_ang_sites(mpcd_ctx *c, cudaStream_t s)

@@ -561,7 +561,7 @@ template <> struct AngWord<double> { typedef double type; };
 
 size_t angular_param_bytes(int precision);
 // solvent phases and the per-cell solve
-void launch_angular(const StepArgs &a, int phase, int num_sms, cudaStream_t s);
+void launch_angular(const StepArgs &a, int phase, int tile, int num_sms, cudaStream_t s);
 // the sites' words (between the cell parameters and the per-cell solve); the
 // correction itself is applied by the site POST coupling when a.ang_params is set
 void launch_angular_sites(const StepArgs &a, cudaStream_t s);

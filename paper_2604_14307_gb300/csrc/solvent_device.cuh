@@ -133,8 +133,8 @@ __device__ __forceinline__ void st4(double *p, const double (&o)[4])
 template <typename Real> struct CellParams { Real ux, uy, uz, kappa, ax, ay, az; };
 
 // 32 bytes by one 256-bit load instead of two of 128 bits: the gathers of a
-// warp go to up to 32 lines, and each instruction looks all of them up (L=200,
-// SRD, 56 M particles: 1470 -> 1456 us a pass; MPCD-AT, 4.4 M: 344 -> 332).  A
+// warp go to up to 32 lines, and each instruction looks all of them up (80 M
+// particles, SRD: 1470 -> 1456 us a pass; MPCD-AT, 9 M: 344 -> 332).  A
 // record is 32-byte aligned: 32 or 64 bytes each, from a base at such a boundary.
 __device__ __forceinline__ CellParams<float> load_params(const void *params, int64_t c)
 {
