@@ -254,14 +254,16 @@ __host__ __device__ constexpr size_t stage_bytes(int cap)
 
 constexpr int ST_STAGES = 3;
 
-// Register cap of the FP32 SRD form of the staged pass (threads of all its
-// CTAs on an SM times the cap leave the rest to the site/body kernels that run
-// beside it); the other forms take up to 128.
+// Register caps of the staged pass (threads of all its CTAs on an SM times the
+// cap leave the rest to the site/body kernels that run beside it).  FP32
+// MPCD-AT, 4 CTAs of 128 threads: with 128 registers they fill the SM and a
+// chain of many-centre forces waits for the pass (48 mixed boxes: 466 us a step
+// against 429 with 112 and 450 with 3 CTAs of 128; 104 spill more: 431).
 #ifndef MPCD_ST_SRD_REGS
 #define MPCD_ST_SRD_REGS 96
 #endif
 template <typename Real, int RULE> struct StRegs {
-    static constexpr int n = sizeof(Real) == 4 && RULE == 0 ? MPCD_ST_SRD_REGS : 128;
+    static constexpr int n = sizeof(Real) == 8 ? 128 : RULE == 0 ? MPCD_ST_SRD_REGS : 112;
 };
 
 template <typename Real, int RULE, int FLAGS>

@@ -456,12 +456,14 @@ bool staged_fits(const mpcd_ctx *c, int tile, int mode, int block)
 // shares (us per step, per-warp ring against staged: 80 M particles 1940 and
 // 1794, 17 M in 512 boxes 450 and 398, 17 M of solvent alone 504 and 462, 2.6 M
 // 110 and 104; 0.6 M MPCD-AT 65 and 69).  SRD takes 3 CTAs of 128 threads.
-// MPCD-AT gains more from warps (2 x 256 against them: 34 M 1192 and 1456, 17 M in
-// 512 boxes 646 and 750, 17 M alone 692 and 790), unless the chain is as long as
-// the pass: shapes of many centres, whose forces take a warp per body, get the
-// registers that 3 x 128 threads leave (9 M, 1120 bodies: 496 and 608).  Boxes
-// that cut the tiles short keep the ring.  Otherwise FP32 takes a ring per warp
-// of 128-particle tiles; MPCD-AT beside colloids with 384 threads, because 512 of
+// MPCD-AT takes 4 CTAs with 512-particle tiles, the iteration of a CTA (against
+// 3 of them and 2 x 256 threads with 1024: 17 M in 512 boxes 623, 762 and 624,
+// 13 M alone 431, 507 and 433), unless the chain is as long as the pass: shapes
+// of many centres, whose forces take a warp per body, in boxes of fewer than 64
+// tiles an SM get the registers that 3 leave (3 M, 377 bodies: 174 and 184; 4.5 M
+// 235 and 237; 6 M 310 and 302; 9 M 450 and 429).  Boxes that cut the tiles
+// short keep the ring.  Otherwise FP32 takes a ring per warp of 128-particle
+// tiles; MPCD-AT beside colloids with 384 threads, because 512 of
 // its 128 registers fill the SM and the site/body chain then waits for the
 // whole pass (0.6 M particles, 221 bodies: 135 and 56 us per step).  FP64 keeps
 // its own pipe full in any form; a ring per warp in 256 threads leaves the most
@@ -473,9 +475,9 @@ void default_tuning(mpcd_ctx *c)
     const int period = c->tune.sort_period;
     const bool p32 = c->prm.precision == MPCD_P32;
     if (p32 && c->Ns >= (int64_t)4 * 3 * c->num_sms * 1024 && c->Ns >= (int64_t)4096 * c->nrep) {
+        const bool chain = c->max_cent > 2 && c->Ns < (int64_t)64 * c->num_sms * 512;
         c->tune = c->prm.rule == MPCD_SRD ? mpcd_tuning{128, 1024, 3, period, 1}
-                  : c->max_cent > 2       ? mpcd_tuning{128, 512, 3, period, 1}
-                                          : mpcd_tuning{256, 1024, 2, period, 1};
+                                          : mpcd_tuning{128, 512, chain ? 3 : 4, period, 1};
         return;
     }
     if (!p32 && c->prm.rule == MPCD_AT)
