@@ -269,8 +269,8 @@ def rnemd_protocol(Bd, I, stream, hbm, steps: int = 20):
     120 cells of pure solvent at 5 particles per cell (17.28M particles, P32,
     SRD + cell thermostat), exchanging up to 100 pairs between the slabs at
     y = 0 and y = 120 every step.  Reports the exchange kernels' time (CUDA
-    events inside mpcd_step), their algorithmic bytes (two passes reading y and
-    v_x of every particle) against the HBM peak, the step time with and without
+    events inside mpcd_step), their algorithmic bytes (y and v_x of the slab
+    members and their list) against the HBM peak, the step time with and without
     the exchange, and the oracle's time for one exchange on the same state."""
     import torch
     import oracle as O
@@ -306,7 +306,8 @@ def rnemd_protocol(Bd, I, stream, hbm, steps: int = 20):
     pk = prof["rnemd"]
     ms_x = pk["total_ms"] / max(pk["launches"], 1)
     n_slab = 2 * L[0] * L[2] * 5
-    alg = 4.0 * n + n_slab * (4.0 + 16.0 + 16.0)   # the candidates (a few hundred entries) are not counted
+    # one mark per 1024 slots from the solvent pass; the candidates (a few hundred entries) are not counted
+    alg = n / 1024 + n_slab * (4.0 + 4.0 + 16.0 + 16.0)
     osys = O.OracleSystem(system)
     ost = O.OracleState(osys, st, compute_forces=False)
     t0 = time.perf_counter()
@@ -317,8 +318,8 @@ def rnemd_protocol(Bd, I, stream, hbm, steps: int = 20):
             "ms_per_exchange": ms_x, "launches_per_exchange": 3,
             "roofline": {"bound": "hbm", "achieved": alg / (ms_x / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
                          "frac": alg / (ms_x / 1e3) / 1e9 / hbm, "bytes_per_exchange": alg,
-                         "bytes_note": ("y of every particle (4 B); v_x of the slab members, their 16-B list "
-                                        "entries written and read back (36 B per member)")},
+                         "bytes_note": ("the marks of the blocks of slots that hold slab members; y and v_x of the "
+                                        "members, their 16-B list entries written and read back (40 B per member)")},
             "ms_per_step_without": base, "ms_per_step_with": with_x,
             "pairs_per_exchange": npairs / (2 * steps + 3),
             "cpu_baseline": {"value": 1.0 / t_cpu, "unit": "exchanges/s", "cores": 1, "kind": "oracle",
@@ -357,16 +358,17 @@ def run_reference(a, ws, rank):
 
 def place_timed_call(step_call, steps: int, period: int) -> int:
     """Run `step_call` (one mpcd_step(steps) call) from the state right after a
-    re-sort until the next call replays a recorded graph and holds its share of
-    re-sorts; returns that share.
+    re-sort until the next call replays recorded pieces only and holds its share
+    of re-sorts; returns that share.
 
-    mpcd_step(n) replays a CUDA graph keyed by (n, solvent buffer parity,
-    passes since the last re-sort); a call of n steps runs n - 1 fused passes,
-    each counting towards the next re-sort, so from `since` it re-sorts
-    (since + n - 1) // period times (each flips the parity) and ends at
-    (since + n - 1) % period.  First every key of the replay cycle is recorded;
-    then, since the call right after the re-sort would hold none, the phase is
-    moved within the cycle until the call holds ceil((n - 1) / period)."""
+    mpcd_step(n) replays its steps in pieces (CUDA graphs) between re-sorts, cut
+    by the passes since the last one and recorded per solvent buffer; a call of
+    n steps runs n - 1 fused passes, each counting towards the next re-sort, so
+    from `since` it re-sorts (since + n - 1) // period times (each flips the
+    buffer) and ends at (since + n - 1) % period.  First every (since, buffer)
+    of the cycle is run once, which records every piece it needs; then, since
+    the call right after the re-sort would hold none, the phase is moved within
+    the cycle until the call holds ceil((n - 1) / period)."""
     since, par, seen = 0, 0, set()
 
     def advance():
@@ -454,8 +456,8 @@ def main():
     else:
         tuning = sim.tuning() if a.no_tune else sim.autotune(steps_per_trial=10)
     sim.step(a.warmup)
-    # every graph of the replay cycle is recorded and the timed call placed so
-    # that it replays graphs and holds its share of re-sorts
+    # every piece of the replay cycle is recorded and the timed call placed so
+    # that it replays them only and holds its share of re-sorts
     sim.sort()
     period = max(1, int(tuning["sort_period"]))
     resorts = place_timed_call(lambda: sim.step(a.steps), a.steps, period)
@@ -513,7 +515,9 @@ def main():
             "bytes_per_launch": pk["bytes_per_launch"], "ms_per_launch": per_launch_ms,
             "share_of_step": pk["total_ms"] / ms_prof,
             "measured_in": "profiled pass (kernel-by-kernel launches with CUDA events, same step count)"}
-    launches = a.steps + sum(v["launches"] * (6 if k == "sort" else 1) for k, v in prof.items())
+    # the kernels of the timed scopes (the step counter, one launch per piece, is left out)
+    launches = sum(v["launches"] * (6 if k == "sort" else 1) for k, v in prof.items()
+                   if system.n_bodies or not k.startswith(("body_", "sites_")))
     # whole-step effective bandwidth: algorithmic bytes of every kernel / step time
     step_bytes = sum(v["bytes_per_launch"] * v["launches"] for v in prof.values()) / a.steps
     hbm_eff = {"bytes_per_update": step_bytes / n_upd, "gbs": step_bytes / (ms / a.steps / 1e3) / 1e9}

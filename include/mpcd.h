@@ -91,7 +91,7 @@ typedef struct {
                              collinear members).  Colloid sites take part like
                              solvent; their corrected velocities enter the
                              transfer to the body.  Needs one site mass for all
-                             shapes (MPCD_ERR_ARG otherwise); steps run unfused.
+                             shapes (MPCD_ERR_ARG otherwise).
                              0: off */
 } mpcd_params;
 
@@ -357,7 +357,7 @@ int mpcd_reset_profile(mpcd_ctx *ctx);
  * one sample after every `every`-th step (every sample is a time origin).
  * mpcd_set_vacf(ctx, n_lags, every) clears the sums and starts sampling from the
  * current step; n_lags = 0 stops it.  It synchronises the device.  FP64 on the
- * device, one thread per body, after the POST coupling of each sampled step.
+ * device, one lag per lane, after the POST coupling of each sampled step.
  * mpcd_get_vacf copies the sums, [n_bodies][n_lags] each, and the number of
  * origins summed per lag, [n_lags] (divide to get the averages); any pointer
  * may be NULL; it synchronises the stream and returns MPCD_ERR_ARG while
@@ -439,7 +439,7 @@ int mpcd_velocity_profile(mpcd_ctx *ctx, int32_t bin_axis, int32_t vel_axis, int
  * autotuner times candidate configurations on the current state (which it
  * restores afterwards) and keeps the fastest: each candidate runs
  * mpcd_step(steps_per_trial) twice from that state, the first run recording its
- * CUDA graph, the second, timed, replaying it; the trials leave the exchange
+ * CUDA graphs, the second, timed, replaying them; the trials leave the exchange
  * totals and the autocorrelation sums as they were.  set_tuning fixes one directly.
  * Any field <= 0 keeps its current value. */
 typedef struct {

@@ -682,9 +682,10 @@ constexpr int WT_STAGES = 3, WT_MAX_WARPS = 16;
 // registers leave 24 K of the SM's 64 K registers to the site/body kernels
 // that run beside this pass on the second stream (a cap of 96 left room for
 // one of their CTAs per SM, none without a cap; 72 and below spill in the
-// loop).  The AT form draws two Philox normals per particle and is latency-
-// bound on their rounds: it gains more from registers (ILP) than from the
-// overlap (L=200: 2.40 ms with 128, 2.69 with 112, 3.01 with 96).
+// loop).  The AT form draws a Philox block and three
+// normals per particle and is latency-bound on its rounds: it gains more from
+// registers (ILP) than from the overlap (0.6 M particles, 221 bodies, 384
+// threads: 55 us a step with 128, 56 with 112, 61 with 96).
 #ifndef MPCD_WT_SRD_REGS
 #define MPCD_WT_SRD_REGS 80
 #endif
@@ -1207,10 +1208,11 @@ __device__ __forceinline__ float ll2f48(long long w)
 }
 
 // FP32 form: cell words -> collision parameters with FP32/integer pipes only.
-// Each CTA takes K consecutive 256-cell tiles, one cell of each per thread.  The word loads of all of them are issued before any arithmetic (a
-// warp keeps PARAM_TILES x NW loads in flight instead of a chain of dependent
-// loads) and parked in shared memory, so the registers of the arithmetic that
-// follows are not tied up by the parked words.
+// Each CTA takes K consecutive 256-cell tiles, one cell of each per thread.  The
+// word loads of all of them are issued before any arithmetic (a warp keeps K x NW
+// loads in flight instead of a chain of dependent loads) and parked in shared
+// memory, so the registers of the arithmetic that follows are not tied up by the
+// parked words.
 
 template <int RULE>
 __device__ __forceinline__ void params32_cell(const StepArgs &a, const DevReplica &r, int64_t step, int64_t c,
@@ -1332,7 +1334,6 @@ __global__ void __launch_bounds__(256) k_params(StepArgs a)
     W *dbg = reinterpret_cast<W *>(a.dbg_sums);
     const int64_t C = a.n_cells;
     const Real kT = Consts<Real>::kT(a);
-    int err = 0;
     for (int t = blockIdx.x; t < a.n_ctiles; t += gridDim.x) {
         const Tile tl = a.ctiles[t];
         const DevReplica r = a.reps[tl.rep];
@@ -1384,20 +1385,13 @@ __global__ void __launch_bounds__(256) k_params(StepArgs a)
                     for (int k = 0; k < 3; ++k) rec[4 + k] = div_by(xi[k], M, iM);
                 }
             }
-            if (sizeof(Real) == 4) {
-                float4 *o = reinterpret_cast<float4 *>(a.params) + 2 * c;
-                o[0] = make_float4((float)rec[0], (float)rec[1], (float)rec[2], (float)rec[3]);
-                o[1] = make_float4((float)rec[4], (float)rec[5], (float)rec[6], 0.0f);
-            } else {
-                double2 *o = reinterpret_cast<double2 *>(a.params) + 4 * c;
-                o[0] = make_double2(rec[0], rec[1]);
-                o[1] = make_double2(rec[2], rec[3]);
-                o[2] = make_double2(rec[4], rec[5]);
-                o[3] = make_double2(rec[6], 0.0);
-            }
+            double2 *o = reinterpret_cast<double2 *>(a.params) + 4 * c;
+            o[0] = make_double2(rec[0], rec[1]);
+            o[1] = make_double2(rec[2], rec[3]);
+            o[2] = make_double2(rec[4], rec[5]);
+            o[3] = make_double2(rec[6], 0.0);
         }
     }
-    if (err) atomicOr(a.d_err, ERR_CELL);
 }
 
 constexpr int PARAM_ONE = 16;   // 256-cell tiles per SM
@@ -1643,64 +1637,6 @@ cudaError_t launch_collide_box(const StepArgs &a, const DevReplica &r, int64_t n
     return a.rule == 0 ? collide_box<0>(a, r, n, step, sc, num_sms, s) : collide_box<1>(a, r, n, step, sc, num_sms, s);
 }
 
-// ------------------------------------------------- layout transforms (I/O)
-// host rows (tag order) -> SoA slots; positions outside [0, L) set ERR_POSITION
-template <typename Real>
-__global__ void k_aos_to_soa(StepArgs a, const Real *xa, const Real *va)
-{
-    Real *X[3] = {(Real *)a.x, (Real *)a.y, (Real *)a.z};
-    Real *V[3] = {(Real *)a.vx, (Real *)a.vy, (Real *)a.vz};
-    int bad = 0;
-    for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x) {
-        const Tile tl = a.tiles[t];
-        const DevReplica r = a.reps[tl.rep];
-        for (int64_t i = tl.begin + threadIdx.x; i < tl.end; i += blockDim.x) {
-            int64_t tag = i - r.solv_begin, row = r.row_begin + tag;
-            for (int k = 0; k < 3; ++k) {
-                Real x = xa[3 * row + k];
-                bad |= !(x >= Real(0) && x < (Real)r.L[k]);
-                X[k][i] = x;
-                V[k][i] = va[3 * row + k];
-            }
-            a.tag[i] = (uint32_t)tag;
-        }
-    }
-    if (bad) atomicOr(a.d_err, ERR_POSITION);
-}
-
-template <typename Real>
-__global__ void k_soa_to_aos(StepArgs a, Real *xa, Real *va)
-{
-    const Real *X[3] = {(const Real *)a.x, (const Real *)a.y, (const Real *)a.z};
-    const Real *V[3] = {(const Real *)a.vx, (const Real *)a.vy, (const Real *)a.vz};
-    for (int t = blockIdx.x; t < a.n_tiles; t += gridDim.x) {
-        const Tile tl = a.tiles[t];
-        const DevReplica r = a.reps[tl.rep];
-        for (int64_t i = tl.begin + threadIdx.x; i < tl.end; i += blockDim.x) {
-            uint32_t tag = a.tag[i];
-            if (tag == PAD_TAG || (int64_t)tag >= r.n_solvent) continue;
-            int64_t row = r.row_begin + tag;
-            for (int k = 0; k < 3; ++k) {
-                xa[3 * row + k] = X[k][i];
-                va[3 * row + k] = V[k][i];
-            }
-        }
-    }
-}
-
-void launch_aos_to_soa(const StepArgs &a, const void *xaos, const void *vaos, cudaStream_t s)
-{
-    if (a.n_tiles == 0) return;
-    if (a.precision == 1) k_aos_to_soa<float><<<a.n_tiles, 256, 0, s>>>(a, (const float *)xaos, (const float *)vaos);
-    else k_aos_to_soa<double><<<a.n_tiles, 256, 0, s>>>(a, (const double *)xaos, (const double *)vaos);
-}
-
-void launch_soa_to_aos(const StepArgs &a, void *xaos, void *vaos, const int64_t *, cudaStream_t s)
-{
-    if (a.n_tiles == 0) return;
-    if (a.precision == 1) k_soa_to_aos<float><<<a.n_tiles, 256, 0, s>>>(a, (float *)xaos, (float *)vaos);
-    else k_soa_to_aos<double><<<a.n_tiles, 256, 0, s>>>(a, (double *)xaos, (double *)vaos);
-}
 
 // ---------------------------------------------------- FP64 diagnostics
 template <typename Real>

@@ -7,21 +7,26 @@
 //             solv_begin a multiple of 8; padding slots carry tag 0xFFFFFFFF.
 //   cells     `sums`:   NW word arrays of n_cells entries (SoA: the lanes of a
 //                       warp handle neighbouring cells, so their atomics share
-//                       sectors): int64 fixed point for P32 (3 words SRD, 4 AT),
+//                       sectors): int64 fixed point for P32 (4 words SRD, 6 AT),
 //                       double for P64.  Zero between collisions.
 //             `params`: one record per cell (32 B for P32, 64 B for P64):
 //                       u, kappa (< 0 marks a cell that does not collide),
-//                       and the SRD axis or the AT mean noise.
+//                       and the SRD axis or the AT mean noise; at a 32-byte
+//                       boundary (256-bit loads).
+//   noise     (MPCD-AT) the normals that the binning drew for the collision it
+//             is for, one array per component, by solvent slot.
 //   bodies    one FP64 record per body (R, q, P, L, F, T, unwrapped
 //             displacement D); the space-frame offsets of every WCA centre
 //             (FP64 and float copies), recomputed once per pose.
 //   sites     thermalised velocity (3 x Real SoA) and cell of every site,
-//             written by the PRE coupling and read by the POST coupling.
+//             written by the PRE coupling and read by the POST coupling; with
+//             MPCD-AT the normals of their collision too.
 //   protocols (allocated on first use) the exchange's key histogram, member
-//             lists and candidates; the velocity-profile sums; the per-body
-//             autocorrelation rings and sums.
-//   +a        (angular-momentum-conserving variants only) ANG_WORDS more words
-//             and one AngParams record per cell.
+//             lists, candidates and a mark per RN_MARK slots; the velocity-
+//             profile sums; the per-body autocorrelation rings and sums.
+//   +a        (angular-momentum-conserving variants only) 16 solvent words and
+//             9 site words per cell, cell by cell (a cell's 16 are one 128-byte
+//             line in P32), and one AngParams record per cell.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -420,9 +425,6 @@ cudaError_t launch_collide_box(const StepArgs &a, const DevReplica &r, int64_t n
                                int num_sms, cudaStream_t s);
 size_t solvent_stage_bytes(int precision, int rule, int cap);
 size_t solvent_smem_bytes(int precision, int rule, int cap, int block);  // dynamic smem of the staged pass
-void launch_aos_to_soa(const StepArgs &a, const void *xaos, const void *vaos, cudaStream_t s);
-void launch_soa_to_aos(const StepArgs &a, void *xaos, void *vaos, const int64_t *out_off,
-                       cudaStream_t s);
 void launch_solvent_diag(const StepArgs &a, double *acc, cudaStream_t s);
 // re-sort (kernels_solvent.cu)
 void launch_sort_count(const StepArgs &a, int32_t *counts, int num_sms, cudaStream_t s);

@@ -198,10 +198,8 @@ __device__ __forceinline__ void srd_rotate(const CellParams<Real> &p, Real ca, R
     vz = p.uz + p.kappa * (wz * ca + cz * sa + p.az * t);
 }
 
-// word count of the cell sums
+// word count of the cell sums (FP64 form; Words32: the FP32 form's)
 template <typename Real, int RULE> struct NWords;
-template <> struct NWords<float, 0> { static constexpr int n = 3; };
-template <> struct NWords<float, 1> { static constexpr int n = 4; };
 template <> struct NWords<double, 0> { static constexpr int n = 6; };
 template <> struct NWords<double, 1> { static constexpr int n = 8; };
 template <typename Real> struct SumWord { typedef double type; };
