@@ -227,58 +227,59 @@ __global__ void __launch_bounds__(256, ANG_CTAS<Real>) k_ang_collide(StepArgs a,
     }
 }
 
+__device__ __forceinline__ double word_double(long long v) { return i64_double(v); }
+__device__ __forceinline__ double word_double(double v) { return v; }
+
 // record of one cell from its words.  mu_s, mu_b: the solvent and site mass
-// in the units of the form (P32: round(m 2^24), P64: m); pscale: the unit of
-// the P terms (P32: 2^-20, P64: 1); mscale: the unit of mu (P32: 2^-24, P64: 1).
-// FP64 instructions bound the solve: the sites' words enter only where a cell has
-// sites, and the two forms of the solution share one division.
-template <typename Real, typename W>
-__device__ void cell_record(const W (&wd)[AW_SOLVENT], const W *wb, double mu_s, double mu_b, double unit,
+// in the units of the form (P32: round(m 2^24), P64: m); unit: the P terms' (P32:
+// 2^-20, P64: 1) over the mass's (P32: 2^-24, P64: 1).
+// FP64 instructions, 64 cycles each, bound the solve: the sites' words enter
+// only where a cell has sites, the two forms of the solution share one
+// division, and conversions, comparisons and roundings to float go to the
+// integer pipe with the same results (216,000 cells: 65.5 -> 57.8 us; with the
+// small CTAs below 55).
+template <typename Real, typename W, typename MU>
+__device__ void cell_record(const W (&wd)[AW_SOLVENT], const W *wb, MU mu_s, MU mu_b, double unit,
                             AngParams<Real> &o)
 {
     const long long cnt = (long long)wd[AW_COUNT];
     const int n_s = (int)(cnt & 0xFFF), n_b = (int)((cnt >> 12) & 0x3FF);
     const bool sites = n_b > 0;
-    double M = (double)n_s * mu_s;
-    if (sites) M += (double)n_b * mu_b;         // exact (integers below 2^53 in P32)
+    const double ms = word_double(mu_s), mb = sites ? word_double(mu_b) : 0.0;
+    o.M = (MU)n_s * mu_s;
+    if (sites) o.M += (MU)n_b * mu_b;
     double sw[3];
     for (int k = 0; k < 3; ++k) {
-        if constexpr (sizeof(Real) == 4) {
-            // exact in int64: mu Q sums below M 2^20
-            long long v = (long long)mu_s * (long long)wd[AW_SQ + k];
-            if (sites) v += (long long)mu_b * (long long)wb[AW_SQB + k];
-            o.sw[k] = v;
-            sw[k] = (double)v;
-        } else {
-            sw[k] = mu_s * (double)wd[AW_SQ + k];
-            if (sites) sw[k] += mu_b * (double)wb[AW_SQB + k];
-            o.sw[k] = sw[k];
-        }
+        // P32: exact in int64 (mu Q sums below M 2^20)
+        MU v = mu_s * (MU)wd[AW_SQ + k];
+        if (sites) v += mu_b * (MU)wb[AW_SQB + k];
+        o.sw[k] = v;
+        sw[k] = word_double(v);
         o.w[k] = (Real)0;
     }
-    if constexpr (sizeof(Real) == 4) o.M = (long long)M;
-    else o.M = M;
+    const double M = word_double(o.M);
     o.pad = (Real)0;
     if (n_s + n_b < 2) return;
-    const double iM = 1.0 / M;
+    const double iM = recip(M);
     const double Qc[3] = {sw[0] * iM, sw[1] * iM, sw[2] * iM};
     // mass-weighted lattice covariance about the centre of mass
     double Cm[3][3];
     const int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
     for (int q = 0; q < 6; ++q) {
-        double v = mu_s * (double)wd[AW_QQ + q];
-        if (sites) v = mu_s * (double)wd[AW_QQ + q] + mu_b * (double)wb[AW_QQB + q];
+        double v = ms * word_double(wd[AW_QQ + q]);
+        if (sites) v = ms * word_double(wd[AW_QQ + q]) + mb * word_double(wb[AW_QQB + q]);
         v = v - sw[ia[q]] * Qc[ib[q]];
         Cm[ia[q]][ib[q]] = Cm[ib[q]][ia[q]] = v;
     }
     const double tr = Cm[0][0] + Cm[1][1] + Cm[2][2];
-    if (!(tr > 0.0)) return;                  // every member on one lattice point
+    // every member on one lattice point: tr is not above 0
+    if ((unsigned long long)__double_as_longlong(tr) - 1 >= 0x7FF0000000000000ull) return;
     // angular-momentum change about the centre (units 2^-20 pscale)
-    const double dP[3] = {(double)wd[AW_P], (double)wd[AW_P + 1], (double)wd[AW_P + 2]};
-    const double dL[3] = {(double)wd[AW_L] - (Qc[1] * dP[2] - Qc[2] * dP[1]),
-                          (double)wd[AW_L + 1] - (Qc[2] * dP[0] - Qc[0] * dP[2]),
-                          (double)wd[AW_L + 2] - (Qc[0] * dP[1] - Qc[1] * dP[0])};
+    const double dP[3] = {word_double(wd[AW_P]), word_double(wd[AW_P + 1]), word_double(wd[AW_P + 2])};
+    const double dL[3] = {word_double(wd[AW_L]) - (Qc[1] * dP[2] - Qc[2] * dP[1]),
+                          word_double(wd[AW_L + 1]) - (Qc[2] * dP[0] - Qc[0] * dP[2]),
+                          word_double(wd[AW_L + 2]) - (Qc[0] * dP[1] - Qc[1] * dP[0])};
     // G = tr(C) I - C = Pi / (mscale 2^-40); solve G x = dL by its adjugate
     const double a00 = tr - Cm[0][0], a11 = tr - Cm[1][1], a22 = tr - Cm[2][2];
     const double a01 = -Cm[0][1], a02 = -Cm[0][2], a12 = -Cm[1][2];
@@ -287,8 +288,9 @@ __device__ void cell_record(const W (&wd)[AW_SOLVENT], const W *wb, double mu_s,
     const double det = a00 * c00 + a01 * c01 + a02 * c02;
     // collinear members: C = tr(C) d d^T, G = tr(C) (I - d d^T); least-norm x
     // = (dL - d (d.dL)) / tr(C) with d d^T = C / tr(C)
-    const bool full = det > 1e-12 * tr * tr * tr;
-    const double inv = 1.0 / (full ? det : tr);
+    // (the right side is positive: the bits order as the values do)
+    const bool full = __double_as_longlong(det) > __double_as_longlong(1e-12 * tr * tr * tr);
+    const double inv = recip(full ? det : tr);
     double x[3];
     if (full) {
         x[0] = (c00 * dL[0] + c01 * dL[1] + c02 * dL[2]) * inv;
@@ -303,7 +305,10 @@ __device__ void cell_record(const W (&wd)[AW_SOLVENT], const W *wb, double mu_s,
     // Pi w = dL_phys with Pi = mscale 2^-40 G and dL_phys = 2^-20 pscale dL; the
     // record keeps w' = w / (M 2^20); unit = pscale / mscale, a power of two
     const double s = unit * iM;
-    for (int k = 0; k < 3; ++k) o.w[k] = (Real)(x[k] * s);
+    for (int k = 0; k < 3; ++k) {
+        if constexpr (sizeof(Real) == 4) o.w[k] = double_float(x[k] * s);
+        else o.w[k] = x[k] * s;
+    }
 }
 
 // sixteen bytes of a cell's words at a time: the line of a cell is a thread's own
@@ -319,8 +324,11 @@ __device__ __forceinline__ void take_words(W *p, W (&o)[N])
     }
 }
 
+// Small CTAs: every SM's FP64 pipe is full, so the cells are spread evenly (64
+// threads against 256: 24^3 cells 16.9 -> 12.9 us, 60^3 57.8 -> 55, 110^3 276 -> 262).
+constexpr int ANG_CELLS = 64;
 template <typename Real>
-__global__ void __launch_bounds__(256) k_ang_params(StepArgs a)
+__global__ void __launch_bounds__(ANG_CELLS) k_ang_params(StepArgs a)
 {
     typedef typename AngWord<Real>::type W;
     W *w = reinterpret_cast<W *>(a.ang_words);
@@ -328,8 +336,8 @@ __global__ void __launch_bounds__(256) k_ang_params(StepArgs a)
     const int64_t C = a.n_cells;
     W *wsites = w + (int64_t)AW_SOLVENT * C;
     const bool p32 = sizeof(Real) == 4;
-    const double mu_s = p32 ? (double)a.qm_solvent : a.m_solvent;
-    const double mu_b = p32 ? (double)a.qm_site : a.m_site;
+    typedef decltype(AngParams<Real>::M) MU;
+    const MU mu_s = p32 ? (MU)a.qm_solvent : (MU)a.m_solvent, mu_b = p32 ? (MU)a.qm_site : (MU)a.m_site;
     const double unit = p32 ? 16.0 : 1.0;   // P terms 2^-20 or 1 over mu 2^-24 or 1
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < C; c += (int64_t)gridDim.x * blockDim.x) {
         alignas(16) W wd[AW_SOLVENT];
@@ -439,13 +447,13 @@ size_t angular_param_bytes(int precision)
 template <typename Real, int RULE>
 static void angular_phase(const StepArgs &a, int phase, int tile, int num_sms, cudaStream_t s)
 {
-    const int grid_p = (int)std::max<int64_t>(1, std::min<int64_t>((a.n_cells + 255) / 256, (int64_t)num_sms * 16));
+    const int grid_p = (int)std::max<int64_t>(1, std::min<int64_t>((a.n_cells + ANG_CELLS - 1) / ANG_CELLS, (int64_t)num_sms * 64));
     const int subs = (tile + ANG_UNIT - 1) / ANG_UNIT;
     const int grid_t = std::max(1, std::min((a.n_tiles * subs + 7) / 8, num_sms * 8));   // 8 warps, one unit each
     if (phase != ANG_PARAMS && a.n_tiles == 0) return;
     switch (phase) {
     case ANG_COLLIDE: k_ang_collide<Real, RULE><<<grid_t, 256, 0, s>>>(a, subs); break;
-    case ANG_PARAMS: k_ang_params<Real><<<grid_p, 256, 0, s>>>(a); break;
+    case ANG_PARAMS: k_ang_params<Real><<<grid_p, ANG_CELLS, 0, s>>>(a); break;
     case ANG_APPLY: k_ang_apply<Real, 0, false><<<grid_t, 256, 0, s>>>(a, subs); break;
     case ANG_STREAM: k_ang_apply<Real, RULE, true><<<grid_t, 256, 0, s>>>(a, subs); break;
     default: break;
