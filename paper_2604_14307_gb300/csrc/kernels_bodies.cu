@@ -178,14 +178,16 @@ __device__ __forceinline__ double lane_torque_kick(double q, const LaneRot &Q, d
 {
     return 2.0 * h * lane_qmul(q, lane_vec_to_quat(lane_mtv(Q, T), c), c);
 }
-// free rotation about body axis k (rotor); Ih its moment, r4 = RN(1 / (4 Ih))
+// free rotation about body axis k (rotor); Ih its moment, r4 = RN(1 / (4 Ih)).
+// No rotation about an axis without a moment: that is one body's matter, and the
+// warp holds eight of any shape, so every lane takes part in the shuffles first.
 __device__ __forceinline__ void lane_rotor(double &q, double &p, int k, double h, double Ih, double r4, int c)
 {
-    if (Ih == 0.0) return;   // the same for all lanes of the body
     const bool neg = k == 1 ? (c == 0 || c == 3) : (k == 2 ? c < 2 : (c == 0 || c == 2));
     const double Pq = flip(lane4(q, c ^ k), neg), Pp = flip(lane4(p, c ^ k), neg);
     const double t = p * Pq;
     const double dot = ((lane4(t, 0) + lane4(t, 1)) + lane4(t, 2)) + lane4(t, 3);
+    if (Ih == 0.0) return;
     const double zeta = div_by(dot, 4.0 * Ih, r4);
     double sn, cs;
     sincos(zeta * h, &sn, &cs);
