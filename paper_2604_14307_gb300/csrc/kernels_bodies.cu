@@ -1197,6 +1197,8 @@ __global__ void k_body_impulse(StepArgs a)
     }
 }
 
+constexpr int SITES_KEPT = 6 * SITE_THREADS;   // most sites of a shape whose draws stay in registers
+
 // Two lanes per running sum up to eight bodies per SM, one beyond: with few
 // bodies the passes are as long as one CTA takes (221 bodies of 642 sites: PRE
 // 18.5 -> 14.7, POST 13.8 -> 9.9 us; 1120 bodies of up to 2000: a step 552 ->
@@ -1204,32 +1206,55 @@ __global__ void k_body_impulse(StepArgs a)
 // bodies: a step 1766 us with one lane, 1783 with two).
 static int site_lanes(const StepArgs &a, int num_sms) { return a.n_bodies <= 8 * num_sms ? 2 : 1; }
 
+// Dynamic shared memory that a kernel is allowed (allow_shared_memory).
+template <typename... P>
+static size_t shared_room(void (*kernel)(P...))
+{
+    cudaFuncAttributes at{};
+    return cudaFuncGetAttributes(&at, kernel) == cudaSuccess ? (size_t)at.maxDynamicSharedSizeBytes : 0;
+}
+// All that a CTA can have beside the kernel's own static arrays: the same for every
+// context, so that none lowers what another one needs.
+template <typename... P>
+static cudaError_t allow_shared_memory(void (*kernel)(P...))
+{
+    int dev = 0, most = 0;
+    cudaFuncAttributes at{};
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, kernel);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes);
+}
+
 template <typename Real, int K>
 static void sites_pre(const StepArgs &a, int max_sites, bool chained, cudaStream_t s)
 {
     constexpr int block = K * SITE_THREADS, FEW = 2 / K, MANY = 6 / K;   // 256 or 768 sites in registers
+    static_assert(MANY * block == SITES_KEPT, "");
+    const size_t bytes = (size_t)max_sites * 3 * sizeof(Real);
     if (max_sites <= FEW * block)
         launch(k_sites_pre<Real, K, FEW>, chained, a.n_bodies, block, 0, s, a);
-    else if (max_sites <= MANY * block)
+    else if (max_sites <= SITES_KEPT)
         launch(k_sites_pre<Real, K, MANY>, chained, a.n_bodies, block, 0, s, a);
-    else
-        launch(k_sites_pre<Real, K, 0>, chained, a.n_bodies, block, (size_t)max_sites * 3 * sizeof(Real), s, a);
+    else if (K == 1 || bytes <= shared_room(k_sites_pre<Real, K, 0>))
+        launch(k_sites_pre<Real, K, 0>, chained, a.n_bodies, block, bytes, s, a);
+    else   // the running sums of two lanes (3 or 6 KB) do not fit beside the draws
+        sites_pre<Real, 1>(a, max_sites, chained, s);
 }
 
 cudaError_t configure_body_kernels(int max_sites, int precision)
 {
-    const int bytes = max_sites * 3 * (int)(precision == 1 ? sizeof(float) : sizeof(double));
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    const auto opt_in = [&](auto *f) {
-        return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (max_sites <= SITES_KEPT) return cudaSuccess;
+    const size_t bytes = (size_t)max_sites * 3 * (precision == 1 ? sizeof(float) : sizeof(double));
+    const auto configure = [&](auto *one, auto *two) {
+        cudaError_t e = allow_shared_memory(one);
+        if (e == cudaSuccess) e = allow_shared_memory(two);
+        if (e != cudaSuccess) return e;
+        return bytes <= shared_room(one) ? cudaSuccess : cudaErrorInvalidValue;
     };
-    cudaError_t e;
-    if (precision == 1) {
-        e = opt_in(k_sites_pre<float, 1, 0>);
-        return e != cudaSuccess ? e : opt_in(k_sites_pre<float, 2, 0>);
-    }
-    e = opt_in(k_sites_pre<double, 1, 0>);
-    return e != cudaSuccess ? e : opt_in(k_sites_pre<double, 2, 0>);
+    return precision == 1 ? configure(k_sites_pre<float, 1, 0>, k_sites_pre<float, 2, 0>)
+                          : configure(k_sites_pre<double, 1, 0>, k_sites_pre<double, 2, 0>);
 }
 
 void launch_sites_pre(const StepArgs &a, int max_sites, int num_sms, bool chained, cudaStream_t s)
