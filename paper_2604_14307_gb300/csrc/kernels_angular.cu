@@ -260,7 +260,7 @@ __device__ void cell_record(const W (&wd)[AW_SOLVENT], const W *wb, MU mu_s, MU 
     const double M = word_double(o.M);
     o.pad = (Real)0;
     if (n_s + n_b < 2) return;
-    const double iM = recip(M);
+    const double iM = 1.0 / M;
     const double Qc[3] = {sw[0] * iM, sw[1] * iM, sw[2] * iM};
     // mass-weighted lattice covariance about the centre of mass
     double Cm[3][3];
@@ -290,7 +290,7 @@ __device__ void cell_record(const W (&wd)[AW_SOLVENT], const W *wb, MU mu_s, MU 
     // = (dL - d (d.dL)) / tr(C) with d d^T = C / tr(C)
     // (the right side is positive: the bits order as the values do)
     const bool full = __double_as_longlong(det) > __double_as_longlong(1e-12 * tr * tr * tr);
-    const double inv = recip(full ? det : tr);
+    const double inv = 1.0 / (full ? det : tr);
     double x[3];
     if (full) {
         x[0] = (c00 * dL[0] + c01 * dL[1] + c02 * dL[2]) * inv;

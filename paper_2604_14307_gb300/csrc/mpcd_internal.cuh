@@ -396,20 +396,6 @@ __device__ __forceinline__ double div_by(double a, double b, double rb)
     return fma(fma(-b, q, a), rb, q);
 }
 
-// RN(1 / x): a coarse reciprocal y (relative error e below 2^-19), one cubic step
-// y (1 + e + e^2), then Markstein's rounding correction (the paper above; 1 ulp
-// off at most where x has all significand bits set; equal to the division for
-// 7.8e8 arguments).  5 FP64 instructions instead of about 11; the division where
-// x is not of moderate size.
-__device__ __forceinline__ double recip(double x)
-{
-    if ((uint32_t)(__double2hiint(x) & 0x7FF00000) - 0x02000000u >= 0x7C000000u) return 1.0 / x;   // not 2^+-991
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    y = fma(y, fma(e, e, e), y);
-    return fma(fma(-x, y, 1.0), y, y);
-}
 // (double)v on the integer pipe (exact below 2^53)
 __device__ __forceinline__ double i64_double(long long v)
 {
