@@ -374,12 +374,9 @@ __device__ __forceinline__ double wrap_box(double y, double L, int &bad)
     if (b >= top) {
         y = __dsub_rn(y, L);
     } else if (b < 0) {
-        if ((unsigned long long)b << 1) {          // negative, not -0
-            y = __dadd_rn(y, L);
-            if (__double_as_longlong(y) == top) y = 0.0;
-        } else {
-            y = 0.0;
-        }
+        if (!((unsigned long long)b << 1)) return y;   // -0 stays
+        y = __dadd_rn(y, L);
+        if (__double_as_longlong(y) == top) y = 0.0;
     }
     bad |= (unsigned long long)__double_as_longlong(y) >= (unsigned long long)top;
     return y;
@@ -387,10 +384,14 @@ __device__ __forceinline__ double wrap_box(double y, double L, int &bad)
 
 // a / b with rb = RN(1 / b): Markstein's correction (IBM J. Res. Dev. 34, 111
 // (1990)) applied twice.  The first makes the quotient faithful, the second
-// rounds it correctly, so the result is that of the IEEE division (no overflow
-// or underflow in between), in 5 instructions of 64 cycles instead of about 11.
+// rounds it correctly, so the result is that of the IEEE division, in 5
+// instructions of 64 cycles.  The division itself where a or b is not of
+// moderate size (exponents -400 to 399): there a product could overflow or
+// underflow on the way, a zero would lose its sign, an infinity give NaN.
 __device__ __forceinline__ double div_by(double a, double b, double rb)
 {
+    const uint32_t ea = (uint32_t)__double2hiint(a) & 0x7FF00000u, eb = (uint32_t)__double2hiint(b) & 0x7FF00000u;
+    if (ea - 0x26F00000u >= 0x32000000u || eb - 0x26F00000u >= 0x32000000u) return a / b;
     double q = a * rb;
     q = fma(fma(-b, q, a), rb, q);
     return fma(fma(-b, q, a), rb, q);
