@@ -91,7 +91,8 @@ typedef struct {
                              collinear members).  Colloid sites take part like
                              solvent; their corrected velocities enter the
                              transfer to the body.  Needs one site mass for all
-                             shapes (MPCD_ERR_ARG otherwise).
+                             shapes (MPCD_ERR_ARG otherwise).  P32: the mass of
+                             the members of a cell below 2^18 (not checked).
                              0: off */
 } mpcd_params;
 

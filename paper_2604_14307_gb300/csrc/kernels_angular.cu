@@ -243,7 +243,7 @@ __device__ void cell_record(const W (&wd)[AW_SOLVENT], const W *wb, MU mu_s, MU 
                             AngParams<Real> &o)
 {
     const long long cnt = (long long)wd[AW_COUNT];
-    const int n_s = (int)(cnt & 0xFFF), n_b = (int)((cnt >> 12) & 0x3FF);
+    const int n_s = (int)(cnt & (AW_SITE - 1)), n_b = (int)(cnt / AW_SITE);
     const bool sites = n_b > 0;
     const double ms = word_double(mu_s), mb = sites ? word_double(mu_b) : 0.0;
     o.M = (MU)n_s * mu_s;
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(ANG_CELLS) k_ang_params(StepArgs a)
         alignas(16) W wd[AW_SOLVENT];
         W wb[AW_SITES];
         take_words(w + AW_SOLVENT * c, wd);
-        if ((((long long)wd[AW_COUNT]) >> 12) & 0x3FF) {
+        if ((long long)wd[AW_COUNT] >= AW_SITE) {   // sites have added their words
 #pragma unroll
             for (int k = 0; k < AW_SITES; ++k) {
                 wb[k] = wsites[AW_SITES * c + k];

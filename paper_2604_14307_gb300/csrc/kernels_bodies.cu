@@ -1339,7 +1339,7 @@ __global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_ang_si
         W D[3];
         for (int k = 0; k < 3; ++k) D[k] = (W)site_mom_term(m, v[k]) - (W)site_mom_term(m, u[k]);
         W *w = words + AW_SOLVENT * cell, *ws = words + AW_SOLVENT * a.n_cells + AW_SITES * cell;
-        ang_red(w + AW_COUNT, (W)4096);
+        ang_red(w + AW_COUNT, (W)AW_SITE);
         ang_red(w + AW_L, q[1] * D[2] - q[2] * D[1]);
         ang_red(w + AW_L + 1, q[2] * D[0] - q[0] * D[2]);
         ang_red(w + AW_L + 2, q[0] * D[1] - q[1] * D[0]);

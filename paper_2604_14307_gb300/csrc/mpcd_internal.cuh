@@ -534,7 +534,7 @@ void launch_rows_out(const StepArgs &a, const void *rec, void *xa, void *va, int
 // (one 128-byte line each), then [n_cells][AW_SITES].  Q is a member's integer
 // lattice offset inside its shifted cell (units 2^-20), P and P* its momentum term
 // before and after the rule (P32: round(fl32(m v) 2^20); P64: m v):
-enum : int { AW_COUNT = 0,      // 1 per solvent particle, 2^12 per site
+enum : int { AW_COUNT = 0,      // 1 per solvent particle, AW_SITE per site (65535 of each, as in the plain words)
              AW_SQ = 1,         // 1-3   sum Q of the solvent
              AW_QQ = 4,         // 4-9   sum Q_a Q_b of the solvent (xx, yy, zz, xy, xz, yz)
              AW_L = 10,         // 10-12 sum Q x (P - P*), solvent and sites
@@ -543,7 +543,8 @@ enum : int { AW_COUNT = 0,      // 1 per solvent particle, 2^12 per site
              AW_SQB = 0,        // 0-2   sum Q of the sites
              AW_QQB = 3,        // 3-8   sum Q_a Q_b of the sites
              AW_SITES = 9,
-             ANG_WORDS = AW_SOLVENT + AW_SITES };
+             ANG_WORDS = AW_SOLVENT + AW_SITES,
+             AW_SITE = 1 << 20 };
 enum : int { ANG_COLLIDE = 0, ANG_PARAMS = 1, ANG_APPLY = 2, ANG_STREAM = 3 };
 
 // Per-cell record of the correction: the mass-weighted lattice sums sw = sum mu Q,
