@@ -1048,11 +1048,9 @@ __global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_si
         if (a.rule == 1) {
             normals3(draw(r, step, (uint32_t)(r.site_id_base + (g - r.site_begin)), TAG_AT, 0u), xi);
             const Real sc = site_scale<Real>(a, ts);
-            Real *XI = reinterpret_cast<Real *>(a.site_xi);
-            for (int k = 0; k < 3; ++k) {
-                xi[k] *= sc;
-                XI[k * NS + g] = xi[k];
-            }
+            for (int k = 0; k < 3; ++k) xi[k] *= sc;
+            if (Real *XI = reinterpret_cast<Real *>(a.site_xi))   // kept for POST
+                for (int k = 0; k < 3; ++k) XI[k * NS + g] = xi[k];
         }
         const int cell = r.cell_base + (N > 0 ? cells[N > 0 ? s : 0] : a.site_cell[g]);
         if (!mine) return;
@@ -1082,10 +1080,12 @@ __global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_si
 // POST coupling: site collision and the per-warp partial sums of the
 // momentum dP = sum m (v' - v) and angular momentum dL = sum d x m (v' - v)
 // transferred to the body (Eqs. 3-4); k_body_impulse adds them in FP64.
-// the collision rule for one site: v -> vn with the parameters p of its cell
-template <typename Real>
-__device__ __forceinline__ void site_rule(const StepArgs &a, int64_t g, const Real (&v)[3], const Real (&p)[8],
-                                          Real (&vn)[3])
+// the collision rule for one site: v -> vn with the parameters p of its cell; KEPT: the
+// MPCD-AT draws of the PRE pass are read, else drawn again (the FP64 form with
+// both in one kernel took 158 registers instead of 116)
+template <typename Real, bool KEPT>
+__device__ __forceinline__ void site_rule(const StepArgs &a, const DevReplica &r, int64_t step, int64_t ts, int64_t g,
+                                          const Real (&v)[3], const Real (&p)[8], Real (&vn)[3])
 {
     vn[0] = v[0]; vn[1] = v[1]; vn[2] = v[2];
     if (p[3] >= Real(0)) {
@@ -1100,8 +1100,16 @@ __device__ __forceinline__ void site_rule(const StepArgs &a, int64_t g, const Re
             vn[1] = p[1] + p[3] * (w[1] * ca + cy * sa + p[5] * tt);
             vn[2] = p[2] + p[3] * (w[2] * ca + cz * sa + p[6] * tt);
         } else {
-            const Real *XI = reinterpret_cast<const Real *>(a.site_xi);   // the draws of the PRE pass
-            for (int k = 0; k < 3; ++k) vn[k] = p[k] + XI[k * a.n_sites + g] - p[4 + k];
+            Real xi[3];
+            if constexpr (KEPT) {
+                const Real *XI = reinterpret_cast<const Real *>(a.site_xi);
+                for (int k = 0; k < 3; ++k) xi[k] = XI[k * a.n_sites + g];
+            } else {
+                normals3(draw(r, step, (uint32_t)(r.site_id_base + (g - r.site_begin)), TAG_AT, 0u), xi);
+                const Real sc = site_scale<Real>(a, ts);
+                for (int k = 0; k < 3; ++k) xi[k] *= sc;
+            }
+            for (int k = 0; k < 3; ++k) vn[k] = p[k] + xi[k] - p[4 + k];
         }
     }
 }
@@ -1115,7 +1123,7 @@ __device__ __forceinline__ void site_lattice_q(const Real (&x)[3], const int (&S
 
 // POST coupling; ANG: with the +a correction of the site's cell applied to the
 // rule's velocity before the momentum change is taken
-template <typename Real, bool ANG, int K>
+template <typename Real, bool ANG, bool KEPT, int K>
 __global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_sites_post(StepArgs a)
 {
     __shared__ Real sPose[POSE_W];
@@ -1153,7 +1161,7 @@ __global__ void __launch_bounds__(K * SITE_THREADS, SiteBlocks<Real, K>::n) k_si
             Real p[8];
             load_cell<Real>(a, cell, p);
             const Real m = site_mass<Real>(a, t);
-            site_rule<Real>(a, g, v, p, vn);
+            site_rule<Real, KEPT>(a, r, step, t, g, v, p, vn);
             if constexpr (ANG) {
                 const Real xs[3] = {x[0], x[1], x[2]};
                 int Q[3];
@@ -1271,24 +1279,35 @@ void launch_sites_pre(const StepArgs &a, int max_sites, int num_sms, bool chaine
     }
 }
 
-template <typename Real, bool ANG>
+// the sites' draws of the rule are kept, or there are none
+static bool draws_kept(const StepArgs &a) { return a.rule == 0 || a.site_xi; }
+
+template <typename Real, bool ANG, bool KEPT>
 static void sites_post(const StepArgs &a, bool two, cudaStream_t s)
 {
-    if (two) k_sites_post<Real, ANG, 2><<<a.n_bodies, 2 * SITE_THREADS, 0, s>>>(a);
-    else k_sites_post<Real, ANG, 1><<<a.n_bodies, SITE_THREADS, 0, s>>>(a);
+    if (two) k_sites_post<Real, ANG, KEPT, 2><<<a.n_bodies, 2 * SITE_THREADS, 0, s>>>(a);
+    else k_sites_post<Real, ANG, KEPT, 1><<<a.n_bodies, SITE_THREADS, 0, s>>>(a);
+}
+
+template <typename Real>
+static void sites_post(const StepArgs &a, bool two, cudaStream_t s)
+{
+    const bool ang = a.ang_params != nullptr;
+    if (draws_kept(a)) {
+        if (ang) sites_post<Real, true, true>(a, two, s);
+        else sites_post<Real, false, true>(a, two, s);
+    } else {
+        if (ang) sites_post<Real, true, false>(a, two, s);
+        else sites_post<Real, false, false>(a, two, s);
+    }
 }
 
 void launch_sites_post(const StepArgs &a, int num_sms, cudaStream_t s)
 {
     if (a.n_bodies == 0) return;
-    const bool two = site_lanes(a, num_sms) == 2, ang = a.ang_params != nullptr;
-    if (a.precision == 1) {
-        if (ang) sites_post<float, true>(a, two, s);
-        else sites_post<float, false>(a, two, s);
-    } else {
-        if (ang) sites_post<double, true>(a, two, s);
-        else sites_post<double, false>(a, two, s);
-    }
+    const bool two = site_lanes(a, num_sms) == 2;
+    if (a.precision == 1) sites_post<float>(a, two, s);
+    else sites_post<double>(a, two, s);
 }
 
 // +a variants: the sites' contributions to the angular words of their cells, one
@@ -1300,7 +1319,7 @@ __device__ __forceinline__ double site_mom_term(double m, double v) { return m *
 
 constexpr int ANG_SITE_CTAS = 2;   // CTAs per body (the order of the integer sums is free)
 
-template <typename Real>
+template <typename Real, bool KEPT>
 __global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_ang_sites(StepArgs a)
 {
     typedef typename AngWord<Real>::type W;
@@ -1331,7 +1350,7 @@ __global__ void __launch_bounds__(SITE_THREADS, SiteMinBlocks<Real>::n) k_ang_si
         const Real m = site_mass<Real>(a, t);
         Real u[3], p[8];
         load_cell<Real>(a, cell, p);
-        site_rule<Real>(a, g, v, p, u);
+        site_rule<Real, KEPT>(a, r, step, t, g, v, p, u);
         const Real xs[3] = {x[0], x[1], x[2]};
         int Qi[3];
         site_lattice_q(xs, sS, Qi);
@@ -1359,8 +1378,13 @@ void launch_angular_sites(const StepArgs &a, cudaStream_t s)
 {
     if (a.n_bodies == 0) return;
     const unsigned grid = (unsigned)a.n_bodies * ANG_SITE_CTAS;
-    if (a.precision == 1) k_ang_sites<float><<<grid, SITE_THREADS, 0, s>>>(a);
-    else k_ang_sites<double><<<grid, SITE_THREADS, 0, s>>>(a);
+    if (draws_kept(a)) {
+        if (a.precision == 1) k_ang_sites<float, true><<<grid, SITE_THREADS, 0, s>>>(a);
+        else k_ang_sites<double, true><<<grid, SITE_THREADS, 0, s>>>(a);
+    } else {
+        if (a.precision == 1) k_ang_sites<float, false><<<grid, SITE_THREADS, 0, s>>>(a);
+        else k_ang_sites<double, false><<<grid, SITE_THREADS, 0, s>>>(a);
+    }
 }
 
 void launch_body_impulse(const StepArgs &a, cudaStream_t s)

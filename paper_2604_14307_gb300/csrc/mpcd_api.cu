@@ -90,10 +90,12 @@ struct mpcd_ctx {
     void *sums = nullptr, *params = nullptr, *dbg_sums = nullptr;
     bool debug = false;
     void *site_v = nullptr;
-    void *site_xi = nullptr;        // MPCD-AT: [3][n_sites] scaled normals of the sites
-    // MPCD-AT: the normals drawn by the last binning, slot by slot, for the
-    // collision of step noise_step, while noise_ok (the slots keep their order)
-    void *noise[3] = {};
+    // MPCD-AT: [3][n_sites] scaled normals of the sites, kept from PRE to POST;
+    // null (drawn again) where the device has no memory left for them
+    void *site_xi = nullptr;
+    // MPCD-AT: the normals drawn by the last binning, slot by slot in the spare
+    // solvent buffer (which only a change of the order writes), for the collision
+    // of step noise_step, while noise_ok
     bool noise_ok = false;
     int64_t noise_step = 0;
     int32_t *site_cell = nullptr;
@@ -189,6 +191,8 @@ int fail(mpcd_ctx *c, int st, const char *fmt, ...)
         if ((ctx)->status) return (ctx)->status; \
     } while (0)
 
+void release_site_xi(mpcd_ctx *c);
+
 void *dalloc(mpcd_ctx *c, size_t bytes)
 {
     if (bytes == 0) bytes = 16;
@@ -200,12 +204,29 @@ void *dalloc(mpcd_ctx *c, size_t bytes)
         cudaGetLastError();
         p = nullptr;
     }
+    if (!p && c->site_xi) {   // what the library can do without goes first
+        release_site_xi(c);
+        return dalloc(c, bytes);
+    }
     if (p) {
         c->allocations.push_back(p);
         c->dev_bytes += (int64_t)bytes;
     }
     return p;
 }
+size_t site_xi_bytes(const mpcd_ctx *c) { return (size_t)std::max<int64_t>(1, c->Nsite) * 3 * c->realsz; }
+
+void release_site_xi(mpcd_ctx *c)
+{
+    cudaDeviceSynchronize();   // no step in flight uses it
+    clear_graphs(c);           // captured steps carry its address
+    c->allocations.erase(std::find(c->allocations.begin(), c->allocations.end(), c->site_xi));
+    c->dev_bytes -= (int64_t)((site_xi_bytes(c) + 255) & ~(size_t)255);
+    if (c->use_alloc) c->alloc.free(c->site_xi, c->alloc.user);
+    else cudaFree(c->site_xi);
+    c->site_xi = nullptr;
+}
+
 // The same at a 32-byte boundary, for records read by 256-bit loads: a caller's
 // allocator may give less.
 void *dalloc32(mpcd_ctx *c, size_t bytes)
@@ -281,7 +302,8 @@ StepArgs make_args(const mpcd_ctx *c)
     a.cent32 = c->d_cent32;
     a.site_v = c->site_v;
     a.site_xi = c->site_xi;
-    for (int k = 0; k < 3; ++k) a.noise[k] = c->noise[k];
+    if (p.rule == MPCD_AT)
+        for (int k = 0; k < 3; ++k) a.noise[k] = c->sol[c->cur ^ 1][k];
     if (c->rn.enabled) {
         a.slab_mark = c->rn_mark;
         const double y[4] = {c->rn.y_a, c->rn.y_a + c->rn.width, c->rn.y_b, c->rn.y_b + c->rn.width};
@@ -565,7 +587,7 @@ bool noise_fits(const mpcd_ctx *c) { return c->noise_ok && c->noise_step == step
 // a pass has binned for the collision of `step` (and kept its normals)
 void noise_kept(mpcd_ctx *c, int64_t step)
 {
-    c->noise_ok = c->noise[0] != nullptr;
+    c->noise_ok = c->prm.rule == MPCD_AT;
     c->noise_step = step;
 }
 
@@ -1121,10 +1143,6 @@ int mpcd_create(const mpcd_params *params, int32_t n_shapes, const mpcd_shape_de
         ok &= (c->d_cent32 = (float4 *)A((size_t)std::max<int64_t>(1, nc) * sizeof(float4))) != nullptr;
     }
     ok &= (c->site_v = A(std::max<int64_t>(1, c->Nsite) * 3 * c->realsz)) != nullptr;
-    if (p.rule == MPCD_AT) {
-        ok &= (c->site_xi = A(std::max<int64_t>(1, c->Nsite) * 3 * c->realsz)) != nullptr;
-        for (int k = 0; k < 3; ++k) ok &= (c->noise[k] = A(c->Nslots * c->realsz)) != nullptr;
-    }
     ok &= (c->site_cell = (int32_t *)A(std::max<int64_t>(1, c->Nsite) * 4)) != nullptr;
     ok &= (c->d_step = (int64_t *)A(8)) != nullptr;
     ok &= (c->d_err = (int *)A(8)) != nullptr;
@@ -1226,6 +1244,7 @@ int mpcd_create(const mpcd_params *params, int32_t n_shapes, const mpcd_shape_de
         mpcd_destroy(c);
         return st;
     }
+    if (p.rule == MPCD_AT) c->site_xi = dalloc(c, site_xi_bytes(c));   // last: it may be refused
     *out = c;
     return MPCD_OK;
 }
@@ -1307,6 +1326,7 @@ int mpcd_set_state(mpcd_ctx *c, const mpcd_host_state *h, void *stream)
     const size_t n3 = (size_t)c->Ns * 3;
     char *stg = (char *)c->staging;
     c->cur = 0;
+    c->noise_ok = false;   // the spare buffer is scratch here
     StepArgs a = make_args(c);
     const StepArgs aio = make_io_args(c);
     {
@@ -1356,7 +1376,6 @@ int mpcd_set_state(mpcd_ctx *c, const mpcd_host_state *h, void *stream)
     c->step = h->step;
     c->since_sort = 0;
     c->last_key = -1;
-    c->noise_ok = false;
     c->have_state = true;
     return MPCD_OK;
 }

@@ -14,13 +14,15 @@
 //                       and the SRD axis or the AT mean noise; at a 32-byte
 //                       boundary (256-bit loads).
 //   noise     (MPCD-AT) the normals that the binning drew for the collision it
-//             is for, one array per component, by solvent slot.
+//             is for, one array per component, by solvent slot: three arrays of
+//             the solvent buffer that is not in use (a change of the order, which
+//             writes them, makes the binning's draws void).
 //   bodies    one FP64 record per body (R, q, P, L, F, T, unwrapped
 //             displacement D); the space-frame offsets of every WCA centre
 //             (FP64 and float copies), recomputed once per pose.
 //   sites     thermalised velocity (3 x Real SoA) and cell of every site,
 //             written by the PRE coupling and read by the POST coupling; with
-//             MPCD-AT the normals of their collision too.
+//             MPCD-AT the normals of their collision too (if there is memory).
 //   protocols (allocated on first use) the exchange's key histogram, member
 //             lists, candidates and a mark per RN_MARK slots; the velocity-
 //             profile sums; the per-body autocorrelation rings and sums.
@@ -112,7 +114,7 @@ struct StepArgs {
     uint8_t *slab_mark;             // per 1024 slots: holds a particle of an exchange slab (null: no exchange)
     float rn_yf[4];                 // the slabs [0], [1] and [2], [3] in y (P32 decisions)
     double rn_y[4];                 // the same in double (P64 decisions)
-    void *noise[3];                 // MPCD-AT: normals of every slot, kept from the binning to the collision (null: not)
+    void *noise[3];                 // MPCD-AT: normals of every slot, kept from the binning to the collision
     int32_t noise_in;               // they are those of this collision, in the present slot order
     int64_t n_cells;
     int32_t nw;
@@ -139,7 +141,7 @@ struct StepArgs {
     double *cent64;                 // per body centre: Q c in the space frame [n][3] (this step's pose)
     float4 *cent32;                 // the same rounded to float
     void *site_v;                   // [3][n_sites] SoA
-    void *site_xi;                  // [3][n_sites] MPCD-AT: the sites' scaled normals (PRE to POST)
+    void *site_xi;                  // [3][n_sites] MPCD-AT: the sites' scaled normals (PRE to POST; null: not kept)
     int32_t *site_cell;             // replica-local cell of each site
     int64_t n_sites;
     int32_t accel;                  // constant-force streaming of the solvent (below)

@@ -290,7 +290,7 @@ __device__ __forceinline__ void bin4(const StepArgs &a, const Real (&x)[4], cons
         if (RULE == 1) normals3(draw(rr, step + (COLLIDE ? 1 : 0), tg[j], TAG_AT, 0u), xi[j]);
     }
     if (RULE == 1) {
-        if (a.noise[0] && nv > 0)   // kept for the collision that this binning is for
+        if (nv > 0)   // kept for the collision that this binning is for
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const Real o[4] = {xi[0][k], xi[1][k], xi[2][k], xi[3][k]};
