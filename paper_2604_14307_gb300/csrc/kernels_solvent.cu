@@ -27,6 +27,8 @@
 #include <mutex>
 #include <utility>
 
+#include <cooperative_groups.h>
+
 #include "solvent_device.cuh"
 
 namespace mpcd {
@@ -1436,38 +1438,25 @@ void launch_params(const StepArgs &a, int num_sms, cudaStream_t s)
 // instead of four.  A thread keeps its first four particles (velocity, cell,
 // AT normals) in registers from the binning to the rule.
 //   CLUSTER: one cluster of eight CTAs and its hardware barrier (small boxes);
-//   else a cooperative grid and a counter barrier with a bounded wait.
+//   else a cooperative grid, whose CTAs are all resident or the launch is
+//   refused, and its barrier.  Neither gives up: the call has returned by then,
+//   and there is nobody to tell of a collision done in part.
 // Against four launches (set-up, binning, parameters, rule) over SoA sums, per
 // call: 20992 particles in 4199 cells 26.7 -> 15.2 us (then bound by the caller's
-// host work, 17 us), 640000 MPCD-AT particles in 64000 cells 61.3 -> 36.8 us.
+// host work, 17 us), 640000 MPCD-AT particles in 64000 cells 61.3 -> 32.9 us (36.6
+// with a counter of its own for the barrier).
 constexpr int BOX_CLUSTER = 8;                      // CTAs of the cluster form (portable size)
 constexpr int BOX_CLUSTER_THREADS = 1024, BOX_THREADS = 256;
 constexpr int BOX_PER_SM = 5;                       // 48 registers; 4 left 640000 particles a second round (40.7 us)
 constexpr int BOX_WARP_WORDS = 32 * 5;              // one word row per lane: 4 words and one of padding
 
 template <bool CLUSTER>
-__device__ __forceinline__ bool box_barrier(unsigned *count, int *err)
+__device__ __forceinline__ void box_barrier()
 {
-    if (CLUSTER) {
+    if (CLUSTER)
         asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-        return true;
-    }
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(count, 1u);
-        unsigned seen = 0;
-        uint32_t spins = 0;
-        do {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
-        } while (seen < gridDim.x && ++spins < SPIN_LIMIT);
-        ok = seen >= gridDim.x;
-        if (!ok) atomicOr(err, ERR_TIMEOUT);
-        __threadfence();
-    }
-    __syncthreads();
-    return ok != 0;
+    else
+        cooperative_groups::this_grid().sync();
 }
 
 template <int RULE, bool CLUSTER>
@@ -1512,7 +1501,7 @@ __global__ void __launch_bounds__(CLUSTER ? BOX_CLUSTER_THREADS : BOX_THREADS, C
     };
     const int64_t groups = n / 4;
     if (t0 < groups) load(t0);
-    if (CLUSTER) box_barrier<true>(nullptr, nullptr);   // the sums are cleared
+    if (CLUSTER) box_barrier<true>();   // the sums are cleared
     // uniform trip count over a warp (its lanes add each other's terms)
     const int64_t first = t0 - lane;
     for (int64_t g0 = first; g0 < groups; g0 += T) {
@@ -1551,7 +1540,7 @@ __global__ void __launch_bounds__(CLUSTER ? BOX_CLUSTER_THREADS : BOX_THREADS, C
             }
         }
     }
-    if (!box_barrier<CLUSTER>(sc.count, sc.err)) return;
+    box_barrier<CLUSTER>();
     for (int64_t c = t0; c < C; c += T) {
         long long w[MAX_WORDS32] = {0, 0, 0, 0, 0, 0};
         const longlong2 q0 = __ldcg(reinterpret_cast<const longlong2 *>(sc.quad) + 2 * c);
@@ -1563,7 +1552,7 @@ __global__ void __launch_bounds__(CLUSTER ? BOX_CLUSTER_THREADS : BOX_THREADS, C
         }
         params32_cell<RULE>(a, r, step, c, w);
     }
-    if (!box_barrier<CLUSTER>(sc.count + 1, sc.err)) return;
+    box_barrier<CLUSTER>();
     // the group still in registers first (the last one loaded), then the others
     auto rule = [&](int64_t g) {
         CellParams<float> p[4];
@@ -1625,7 +1614,7 @@ static cudaError_t collide_box(const StepArgs &a, const DevReplica &r, int64_t n
         cfg.blockDim = dim3((unsigned)std::min<int64_t>(BOX_CLUSTER_THREADS, std::max<int64_t>(128, (want + 31) / 32 * 32)));
         return cudaLaunchKernelEx(&cfg, k_collide_box<RULE, true>, a, r, n, step, sc);
     }
-    cudaError_t e = cudaMemsetAsync(sc.count, 0, sc.clear_bytes(RULE, cells), s);
+    cudaError_t e = cudaMemsetAsync(sc.quad, 0, sc.sum_bytes(RULE, cells), s);
     if (e != cudaSuccess) return e;
     at.id = cudaLaunchAttributeCooperative;
     at.val.cooperative = 1;

@@ -437,12 +437,10 @@ void launch_params(const StepArgs &a, int num_sms, cudaStream_t s);
 // one collision of a single box on the caller's SoA arrays (a.x .. a.vz, a.tag;
 // n a multiple of 4; a.params holds the cells' records), enqueued as one kernel
 struct BoxScratch {
-    unsigned *count;        // [2] barrier counters, 256 bytes before quad
-    int *err;
     long long *quad;        // [cells][4] words 0-3
     long long *pair;        // [cells][2] words 4, 5 (MPCD-AT), behind quad
-    // the counters and the sums of a box, which lie in one piece (MPCD-AT: pair = quad + 4 cells)
-    static size_t clear_bytes(int rule, int64_t cells) { return 256 + (size_t)cells * (rule == 0 ? 4 : 6) * 8; }
+    // the sums of a box, which lie in one piece (MPCD-AT: pair = quad + 4 cells)
+    static size_t sum_bytes(int rule, int64_t cells) { return (size_t)cells * (rule == 0 ? 4 : 6) * 8; }
 };
 cudaError_t launch_collide_box(const StepArgs &a, const DevReplica &r, int64_t n, int64_t step, const BoxScratch &sc,
                                int num_sms, cudaStream_t s);

@@ -1,9 +1,8 @@
 // mpcd_collide_solvent_static: one solvent collision (Sec. II.A) of a single
-// periodic box whose scratch - cell sums, collision parameters, barrier counters
-// and the error word - lives in one statically reserved device array of this
-// translation unit, so the call allocates no device memory.  The collision is
-// one kernel (k_collide_box in kernels_solvent.cu) built from the parts of a
-// context's passes.
+// periodic box whose scratch - cell sums and collision parameters - lives in one
+// statically reserved device array of this translation unit, so the call
+// allocates no device memory.  The collision is one kernel (k_collide_box in
+// kernels_solvent.cu) built from the parts of a context's passes.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -19,12 +18,9 @@ namespace {
 constexpr int64_t MAX_CELLS = MPCD_STATIC_MAX_CELLS;
 constexpr int64_t MAX_SOLVENT = MPCD_STATIC_MAX_SOLVENT;
 
-// byte offsets inside the scratch array (each 256-byte aligned); the barrier
-// counters lie before the cell sums, so that one memset clears both
+// byte offsets inside the scratch array (each 256-byte aligned)
 constexpr size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
-constexpr size_t OFF_ERR = 0;
-constexpr size_t OFF_COUNT = OFF_ERR + 256;
-constexpr size_t OFF_SUMS = OFF_COUNT + 256;
+constexpr size_t OFF_SUMS = 0;
 constexpr size_t OFF_PARAMS = OFF_SUMS + align256(sizeof(long long) * MAX_WORDS32 * MAX_CELLS);
 constexpr size_t SCRATCH_BYTES = OFF_PARAMS + align256(32 * MAX_CELLS);
 
@@ -155,8 +151,6 @@ extern "C" int mpcd_collide_solvent_static(const mpcd_params *p, const int32_t L
     a.params = su.base + OFF_PARAMS;
     a.n_cells = cells;
     BoxScratch sc{};
-    sc.err = reinterpret_cast<int *>(su.base + OFF_ERR);
-    sc.count = reinterpret_cast<unsigned *>(su.base + OFF_COUNT);
     sc.quad = reinterpret_cast<long long *>(su.base + OFF_SUMS);
     sc.pair = sc.quad + 4 * cells;
     cudaError_t e = launch_collide_box(a, rep, n, step, sc, su.num_sms, (cudaStream_t)stream);
