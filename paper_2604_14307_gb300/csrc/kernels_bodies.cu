@@ -345,12 +345,16 @@ template <typename Real>
 static void body_md(const StepArgs &a, bool impulse, cudaStream_t s)
 {
     const unsigned grid = (unsigned)((a.n_bodies + MD_BODIES - 1) / MD_BODIES);
+    // Without solvent nothing stands between the step counter's advance and the
+    // first body step of a call, which lets PRE start and read the counter
+    // before anything has waited for it: a full dependency there.
+    const bool chained = chain_pays(a) && (impulse || a.n_tiles > 0);
     if (a.lone_bodies) {
-        if (impulse) launch_chained(k_body_md<Real, true, true>, grid, 64, 0, s, a);
-        else launch_chained(k_body_md<Real, false, true>, grid, 64, 0, s, a);
+        if (impulse) launch(k_body_md<Real, true, true>, chained, grid, 64, 0, s, a);
+        else launch(k_body_md<Real, false, true>, chained, grid, 64, 0, s, a);
     } else {
-        if (impulse) launch_chained(k_body_md<Real, true, false>, grid, 64, 0, s, a);
-        else launch_chained(k_body_md<Real, false, false>, grid, 64, 0, s, a);
+        if (impulse) launch(k_body_md<Real, true, false>, chained, grid, 64, 0, s, a);
+        else launch(k_body_md<Real, false, false>, chained, grid, 64, 0, s, a);
     }
 }
 
