@@ -48,19 +48,6 @@ namespace mpcd {
 
 namespace {
 
-// X = floor(x 2^20) of the binning rule, as in the plain passes (box edges
-// below 2048 cells keep it within int32)
-__device__ __forceinline__ int lattice_X(float x) { return __float2int_rd(x * 1048576.0f); }
-__device__ __forceinline__ int lattice_X(double x) { return lattice_floor(x); }
-
-__device__ __forceinline__ int axis_cell(int X, int S, int L)
-{
-    int c = (X - S) >> 20;
-    c += (c < 0) ? L : 0;
-    c -= (c >= L) ? L : 0;
-    return ((unsigned)c < (unsigned)L) ? c : 0;   // only a non-finite position gets here
-}
-
 // momentum term P of one particle: the P32 fixed-point value or the FP64 product
 __device__ __forceinline__ long long mom_term(float m, float v) { return q20(__fmul_rn(m, v)); }
 __device__ __forceinline__ double mom_term(double m, double v) { return m * v; }

@@ -30,7 +30,7 @@
 //               coupling's arithmetic).
 // This file is compiled without fused multiply-add so that the FP64 body and
 // site-position arithmetic rounds the same way as the oracle.
-#include "mpcd_internal.cuh"
+#include "solvent_device.cuh"
 
 namespace mpcd {
 
@@ -735,51 +735,6 @@ void launch_body_force(const StepArgs &a, int kick, cudaStream_t s)
 }
 
 // ---------------------------------------------------------------- sites
-// (x + 1/2) 2^-32 from all 32 bits, relative error <= 2^-24 (never 0; 1 only
-// when x rounds up to 2^32)
-__device__ __forceinline__ float u01f(uint32_t x)
-{
-    return __fmaf_rn(__uint2float_rn(x), 2.3283064365386962890625e-10f, 1.16415321826934814453125e-10f);
-}
-// -2 ln u, accurate near u = 1 through the exact complement 1 - u
-__device__ __forceinline__ float neg2log(uint32_t x)
-{
-    return (x & 0x80000000u) ? -2.0f * log1pf(-u01f(~x)) : -2.0f * __logf(u01f(x));
-}
-// Box-Muller; the angles are shifted by pi into [-pi, pi) where the fast
-// sine/cosine are accurate: cos(2 pi u) = -cos(2 pi (u - 1/2))
-__device__ __forceinline__ void normals3(uint4 w, float n[3])
-{
-    const float r1 = sqrtf(neg2log(w.x)), r2 = sqrtf(neg2log(w.z));
-    float s1, c1;
-    __sincosf(6.283185307179586f * (u01f(w.y) - 0.5f), &s1, &c1);
-    n[0] = -r1 * c1; n[1] = -r1 * s1;
-    n[2] = -r2 * __cosf(6.283185307179586f * (u01f(w.w) - 0.5f));
-}
-__device__ __forceinline__ void normals3(uint4 w, double n[3])
-{
-    double r1 = sqrt(-2.0 * log(u01d(w.x))), r2 = sqrt(-2.0 * log(u01d(w.z)));
-    double s1, c1;
-    sincospi(2.0 * u01d(w.y), &s1, &c1);
-    n[0] = r1 * c1; n[1] = r1 * s1; n[2] = r2 * cospi(2.0 * u01d(w.w));
-}
-__device__ __forceinline__ int cell_axis(float x, int S, int L)
-{
-    int c = (__float2int_rd(x * 1048576.0f) - S) >> 20;
-    c += (c < 0) ? L : 0;
-    c -= (c >= L) ? L : 0;
-    return ((unsigned)c < (unsigned)L) ? c : 0;   // only a non-finite position gets here; it is flagged
-
-}
-__device__ __forceinline__ int cell_axis(double x, int S, int L)
-{
-    int c = (lattice_floor(x) - S) >> 20;
-    c += (c < 0) ? L : 0;
-    c -= (c >= L) ? L : 0;
-    return ((unsigned)c < (unsigned)L) ? c : 0;   // only a non-finite position gets here; it is flagged
-
-}
-
 // Site geometry of the two forms.  P32: d = Qf bf in float (three products,
 // two adds), r = fl32(R) + d; P64: d = Q b in double.  Both wrapped into [0, L).
 template <typename Real> struct Pose {

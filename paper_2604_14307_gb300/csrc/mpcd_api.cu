@@ -833,18 +833,17 @@ int enqueue_piece(mpcd_ctx *c, const Piece &p, cudaStream_t s)
 }
 
 // The pieces of n whole steps: a head, n - 1 middle steps and a tail, with a
-// re-sort wherever the count since the last one reaches the period.  `recorded`: cut so that few different
-// pieces serve every n and every phase of the re-sorts - a whole period ending
-// in its re-sort, one step with a re-sort, and powers of two without.
-// (A graph per step count and phase was recorded anew in nearly every call: the
-// phase moves by n - 1 steps from call to call.  At 5000 particles that was
-// 4.2 of the 9.5 ms of a 100-step call.)
+// re-sort wherever the count since the last one reaches the period.  `recorded`:
+// cut so that few different pieces serve every n and every phase of the re-sorts -
+// a whole period ending in its re-sort, one step with a re-sort, and powers of two
+// without.  (A graph per step count and phase was recorded anew in nearly every
+// call: the phase moves by n - 1 steps from call to call.  At 5000 particles that
+// was 4.2 of the 9.5 ms of a 100-step call.)
 std::vector<Piece> plan_steps(mpcd_ctx *c, int64_t n, bool recorded)
 {
     constexpr int64_t MOST = 32;   // steps of a recorded piece without a re-sort
     std::vector<Piece> out;
     const bool sorts = c->prm.sort_period >= 0;
-    const int kind = PIECE_MIDDLE;
     const int64_t period = c->tune.sort_period;
     out.push_back(Piece{PIECE_HEAD, 0, false});
     for (int64_t left = n - 1; left > 0;) {
@@ -852,12 +851,12 @@ std::vector<Piece> plan_steps(mpcd_ctx *c, int64_t n, bool recorded)
         const int64_t m = std::min(left, due);
         const bool sort = m == due;
         if (!recorded || (sort && m == period && period <= 2 * MOST)) {
-            out.push_back(Piece{kind, m, sort});
+            out.push_back(Piece{PIECE_MIDDLE, m, sort});
         } else {
             int64_t plain = m - (sort ? 1 : 0);
             for (int64_t b = MOST; b >= 1; b /= 2)
-                for (; plain >= b; plain -= b) out.push_back(Piece{kind, b, false});
-            if (sort) out.push_back(Piece{kind, 1, true});
+                for (; plain >= b; plain -= b) out.push_back(Piece{PIECE_MIDDLE, b, false});
+            if (sort) out.push_back(Piece{PIECE_MIDDLE, 1, true});
         }
         c->since_sort = sort ? 0 : c->since_sort + m;
         left -= m;

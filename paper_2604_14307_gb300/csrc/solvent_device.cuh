@@ -1,7 +1,8 @@
 // Device functions of the solvent passes (Sec. II.A of arXiv 2604.14307): draws,
 // binning, streaming, cell records, the SRD rule and the run-merged binning of a
 // thread's four particles.  Shared by the passes of kernels_solvent.cu and of the
-// angular-momentum-conserving variants (kernels_angular.cu).
+// angular-momentum-conserving variants (kernels_angular.cu); the draws and the binning
+// rule also by the sites (kernels_bodies.cu).
 #pragma once
 
 #include "mpcd_internal.cuh"
@@ -45,22 +46,20 @@ __device__ __forceinline__ void normals3(uint4 w, double n[3])
     n[2] = r2 * cospi(2.0 * u01d(w.w));
 }
 
-// binning rule: X = floor(x 2^20), cell = floor((X - S) / 2^20) mod L
-__device__ __forceinline__ int cell_axis(float x, int S, int L)
+// binning rule: X = floor(x 2^20) (box edges below 2048 cells keep it within int32),
+// cell = floor((X - S) / 2^20) mod L
+__device__ __forceinline__ int lattice_X(float x) { return __float2int_rd(x * 1048576.0f); }
+__device__ __forceinline__ int lattice_X(double x) { return lattice_floor(x); }
+__device__ __forceinline__ int axis_cell(int X, int S, int L)
 {
-    int c = (__float2int_rd(x * 1048576.0f) - S) >> 20;
+    int c = (X - S) >> 20;
     c += (c < 0) ? L : 0;
     c -= (c >= L) ? L : 0;
     return ((unsigned)c < (unsigned)L) ? c : 0;   // only a non-finite position gets here; it is flagged
-
 }
-__device__ __forceinline__ int cell_axis(double x, int S, int L)
+template <typename Real> __device__ __forceinline__ int cell_axis(Real x, int S, int L)
 {
-    int c = (lattice_floor(x) - S) >> 20;
-    c += (c < 0) ? L : 0;
-    c -= (c >= L) ? L : 0;
-    return ((unsigned)c < (unsigned)L) ? c : 0;   // only a non-finite position gets here; it is flagged
-
+    return axis_cell(lattice_X(x), S, L);
 }
 // The same rule in float32 without a conversion instruction (the solvent
 // passes).  With S an integer, floor((floor(x 2^20) - S) / 2^20) =
@@ -106,7 +105,6 @@ __device__ __forceinline__ double drift(double x, double v, double dt, double L,
 // exact for a constant force; with no force the plain drift.
 __device__ __forceinline__ float kick(float v, float h) { return __fadd_rn(v, h); }
 __device__ __forceinline__ double kick(double v, double h) { return __dadd_rn(v, h); }
-
 
 __device__ __forceinline__ void ld4(const float *p, float (&o)[4])
 {
