@@ -450,7 +450,8 @@ double solvent_bytes(const mpcd_ctx *c, int flags)
     else if (flags & (SOLV_COLLIDE | SOLV_BIN)) b += 3 * rs * n;  // r read
     if (flags & SOLV_COLLIDE) b += 2 * 3 * rs * n + C * c->param_bytes;   // v read+write, params
     else if (flags & SOLV_BIN) b += 3 * rs * n;              // v read
-    if (c->prm.rule == MPCD_AT) b += 4 * n;                    // tags
+    if (c->prm.rule == MPCD_AT)                              // tags; the normals kept, read and written
+        b += 4 * n + (flags & SOLV_COLLIDE ? 3 * rs * n : 0) + (flags & SOLV_BIN ? 3 * rs * n : 0);
     if (flags & SOLV_BIN) b += C * c->nw * 8.0;              // sums written once
     return b;
 }
@@ -695,10 +696,11 @@ int do_sort(mpcd_ctx *c, int canonical, cudaStream_t s, bool from_words = false)
 int k_ang(mpcd_ctx *c, int phase, cudaStream_t s)
 {
     static const char *names[] = {"angular_collide", "angular_params", "angular_apply", "angular_stream"};
-    // algorithmic bytes: the solvent arrays each pass reads and writes, the cell
-    // words written or read once, the per-cell records
+    // algorithmic bytes: the solvent arrays each pass reads and writes (MPCD-AT: the
+    // tags and the normals kept too), the cell words written or read once, the
+    // per-cell records
     const double N = (double)c->Ns, C = (double)c->C, r = c->realsz;
-    const double rec = (double)angular_param_bytes(c->prm.precision), at = c->prm.rule == MPCD_AT ? 4 * N : 0;
+    const double rec = (double)angular_param_bytes(c->prm.precision), at = c->prm.rule == MPCD_AT ? N * (4 + 3 * r) : 0;
     const double words = c->B > 0 ? ANG_WORDS : AW_SOLVENT;
     const double bytes[] = {N * 9 * r + C * (c->param_bytes + AW_SOLVENT * 8.0) + at, C * (2.0 * words * 8 + rec),
                             N * 9 * r + C * rec, N * 12 * r + C * (rec + c->nw * 8.0) + at};
